@@ -109,13 +109,14 @@ typedef struct {
                              N <= 64 and lsqr_tc != 1, the problems advance together in one grouped LSQR and
                              refinement (one launch per phase for all problems); 0 in any problem's options =
                              each problem solved on its own (host lanes) */
-  int emulate_fp64;       /* [1] MIXED: the float64 products -- the Gram matrix, the Cholesky trailing
-                             updates, and the refinement's r = b - A x and A^T r -- on the BF16 tensor
-                             cores from exact integer digits (see tk_gram_emulated,
-                             tk_cholesky_shifted_emulated, tk_residual) instead of the float64 pipe;
-                             the same float64 accuracy.  Costs 32 bytes of workspace per element of A
-                             (two sets of digit planes); 0 = float64 FMA.  The grouped batch uses the
-                             emulated Gram and Cholesky and keeps its float64 refinement passes. */
+  int emulate_fp64;       /* [1] the float64 products on the BF16 tensor cores from exact integer digits
+                             (see tk_gram_emulated, tk_cholesky_shifted_emulated, tk_residual) instead of
+                             the float64 pipe, with the same float64 accuracy: MIXED: the Gram matrix, the
+                             Cholesky trailing updates, and the refinement's r = b - A x and A^T r; FP64:
+                             the Gram matrix, the trailing updates and the two products with A of every
+                             LSQR step, when at least 2 lambda run together and A has 2^19 .. 2^32
+                             elements.  Costs 32 (MIXED) or 16 (FP64) bytes of workspace per element of
+                             A for the digit planes; 0 = float64 FMA. */
   const double* x0;       /* [NULL] warm start, device N x n float64 (row i for lambdas[i]; m >= n only):
                              the solve starts from x = x0 instead of 0 and returns the same minimiser of
                              problem (1.2).  FP64: LSQR solves for the correction d in
@@ -385,8 +386,8 @@ TK_API tk_status tk_lowrank_ranks(const double* sigma, int64_t s, const double* 
  * G = R A (the two float64 passes of the refinement of the mixed form:
  * residuals b - A x_l and A^T (b - A x_l); no counterpart in the paper's
  * algorithms).  emulate = 0: float64 FMA.  emulate = 1: on the BF16
- * tensor cores: every row of A (and of X) is scaled by a power of two and
- * split into 8 signed 7-bit integer slices (exact in BF16, 56 bits), the 36
+ * tensor cores: the rows and columns of A (and the rows of X) are scaled by
+ * powers of two and split into 8 signed 7-bit integer slices (exact in BF16, 56 bits), the 36
  * slice products whose weight is at least 2^-56 of the row maxima are
  * accumulated exactly in FP32 over chunks of 256 values of K and then
  * exactly in int64, rounded once to float64 per output; the error is at
@@ -397,8 +398,8 @@ TK_API tk_status tk_lowrank_ranks(const double* sigma, int64_t s, const double* 
  *   X:   device, M x n float64, row stride ldx >= n.
  *   R:   device, M x m float64 (row l = b - A x_l), written.
  *   G:   device, M x n float64 (row l = A^T (b - A x_l)), written; may be NULL.
- *        Emulated, A^T r is formed from the same slices of A, the row scale of A
- *        moved onto r.
+ *        Emulated, A^T r is formed from the same slices of A, read along its columns, the
+ *        row scale of A moved onto r.
  *   work: device, tk_residual_workspace(m, n, M) bytes.  Synchronizes `stream`. */
 TK_API size_t tk_residual_workspace(int64_t m, int64_t n, int M);
 TK_API tk_status tk_residual(const tk_problem* p, const double* X, int M, int64_t ldx, int emulate, double* R,

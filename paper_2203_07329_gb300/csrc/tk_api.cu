@@ -45,6 +45,7 @@ struct Plan {
   bool qr = false;        // BP2: R from a QR of [Y; sqrt(l) I] instead of chol(Y^T Y + l I)
   bool lsqr_tc = false;  // tensor-core float32 LSQR products (3-term TF32)
   bool lsqr_oz = false;  // float32 LSQR products from the 4-digit slices of A
+  bool oz64 = false;     // float64 form: its products with A, Gram matrix and Cholesky updates from exact digits
   bool lsqr_fused = false;  // ... both products of a step in one kernel
   bool prep_only = false;  // grouped batch: build the preconditioner only
   bool inv64 = false;      // float64 form: explicit float64 R^-1 (small factors)
@@ -52,6 +53,7 @@ struct Plan {
 
 constexpr int64_t kMaxShort = 8192;
 constexpr int64_t kMaxLong = (int64_t(1) << 30);
+constexpr int64_t kOz64MinElems = int64_t(1) << 19;  // smallest A (elements) that the float64 form splits into digits
 
 tk_status check_opts(const tk_opts* o) {
   if (!o) return einval("options pointer is NULL");
@@ -73,6 +75,14 @@ tk_status check_opts(const tk_opts* o) {
     if (!(o->inner_tol > 0.0) || !(o->refine_tol > 0.0)) return einval("inner_tol and refine_tol must be > 0");
   }
   return TK_OK;
+}
+
+// The float64 form with emulate_fp64: whether the solve makes digit planes of A at all.  They pay off
+// from two lambda at a time (a digit product costs the same for 1..32 lambda, the float64 pipe's work
+// grows with the count) and when A is large enough that a product is not all launch latency; A of more
+// than 2^32 elements keeps the float64 pipe, because the planes take 16 bytes per element.
+bool oz64_wanted(int64_t m, int64_t n, int N_cap) {
+  return N_cap >= 2 && m * n >= kOz64MinElems && m * n <= (int64_t(1) << 32);
 }
 
 tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
@@ -119,6 +129,7 @@ tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
               (P.dt == TK_F64 || P.lda % 4 == 0);
   P.lsqr_oz = P.mixed && (o->lsqr_tc == 2 || o->lsqr_tc == 3) && o->emulate_fp64 && !P.under;
   P.lsqr_fused = P.lsqr_oz && o->lsqr_tc == 3;
+  P.oz64 = !P.mixed && o->emulate_fp64 && oz64_wanted(P.m, P.n, P.N_cap);
   return TK_OK;
 }
 
@@ -152,12 +163,11 @@ struct Bufs {
   double* Rres = nullptr;
   double* part = nullptr;
   double* nrm = nullptr;
-  void* Aoz = nullptr;      // mixed, emulate_fp64: BF16 slices of A and their row exponents
+  void* Aoz = nullptr;      // emulate_fp64: the digit planes of A and their row exponents
   int* EA = nullptr;
   void* Xoz = nullptr;      // ... and of the lambda rows of x
   int* EX = nullptr;
-  void* AozC = nullptr;     // ... the column-scaled slices of A, their column exponents
-  int* EC = nullptr;
+  int* EC = nullptr;        // ... the column exponents of A
   void* colmax = nullptr;
   int* oz_err = nullptr;    // set by a timed-out wait of the emulated products
   void* Roz = nullptr;      // ... and of the residuals (normal-equation pass)
@@ -175,9 +185,21 @@ struct Bufs {
 // cores (BF16 operands, FP32 accumulation); every other sketch is SIMT.
 bool tc_sketch(const Plan& P) { return P.mixed && P.o.sketch == TK_SKETCH_GAUSS && !P.under; }
 
-// The mixed form with emulate_fp64 forms its Gram matrix from exact slices on
-// the tensor cores (float64 accuracy).
-bool emulated_gram(const Plan& P) { return P.mixed && P.o.emulate_fp64 && !P.lowrank && !P.qr; }
+// With emulate_fp64 the mixed form, and the float64 form when it works from digits, make their Gram
+// matrix (m >= n) and their Cholesky updates from exact slices on the tensor cores (float64 accuracy).
+bool emulated_chol(const Plan& P) {
+  return ((P.mixed && P.o.emulate_fp64) || P.oz64) && !P.lowrank && !P.qr;
+}
+bool emulated_gram(const Plan& P) { return emulated_chol(P); }
+OzMat oz_mat(const Plan& P, const Bufs& B) {
+  OzMat A;
+  A.planes = B.Aoz;
+  A.ER = B.EA;
+  A.EC = B.EC;
+  A.m = P.m;
+  A.n = P.n;
+  return A;
+}
 
 size_t sketch_scratch(const Plan& P) {
   tk_dtype dt = P.mixed ? TK_F32 : P.dt;
@@ -231,13 +253,21 @@ void carve(const Plan& P, Arena& a, Arena& t, Bufs& B) {
       B.lrS32 = a.take<float>((size_t)N * P.s);
     }
   }
-  if (P.mixed && P.o.emulate_fp64) B.oz_err = a.take<int>(4);
+  if ((P.mixed && P.o.emulate_fp64) || P.oz64) B.oz_err = a.take<int>(4);
+  if (P.oz64) {
+    B.Aoz = a.take<char>(oz_slices_bytes(P.m, P.n));
+    B.EA = a.take<int>(P.m);
+    B.EC = a.take<int>(P.n);
+    B.colmax = a.take<char>(oz_colmax_bytes(P.n));
+  }
   if (P.mixed && !P.prep_only && P.o.emulate_fp64) {
     B.Aoz = a.take<char>(oz_slices_bytes(P.m, P.n));
+    // the mixed form promises 32 bytes per element of A (tk_opts.emulate_fp64): one set of planes
+    // serves both products, the second set's space stays part of the workspace size
+    a.take<char>(oz_slices_bytes(P.n, P.m));
     B.EA = a.take<int>(P.m);
     B.Xoz = a.take<char>(oz_slices_bytes(N, P.n));
     B.EX = a.take<int>(N);
-    B.AozC = a.take<char>(oz_slices_bytes(P.n, P.m));  // A^T, column exponents
     B.EC = a.take<int>(P.n);
     B.colmax = a.take<char>(oz_colmax_bytes(P.n));
     B.Roz = a.take<char>(oz_slices_bytes(N, P.m));
@@ -275,6 +305,7 @@ void carve(const Plan& P, Arena& a, Arena& t, Bufs& B) {
     B.e32.carve(a);
   } else {
     B.e64.m = P.m; B.e64.n = P.n; B.e64.N_cap = P.N_cap; B.e64.under = P.under; B.e64.lr_s = lr_s;
+    B.e64.oz = P.oz64;
     B.e64.carve(a);
   }
 }
@@ -482,8 +513,17 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
   const double* A64 = (P.dt == TK_F64) ? (const double*)p->A : nullptr;
   const float* A32 = (P.dt == TK_F32) ? (const float*)p->A : nullptr;
   int64_t lda64 = P.lda, lda32 = P.lda;
+  // A is split once, for every product of the solve (x, r and the LSQR vectors on every pass); the
+  // first pass over a float64 A also writes the float32 copy of the mixed form
+  const bool digits = (P.mixed && P.o.emulate_fp64 && !P.prep_only) || P.oz64;
+  if (digits && !reuse) {
+    float* copy = P.mixed && P.dt == TK_F64 ? B.A32 : nullptr;
+    const int tok = prof_begin(TK_PHASE_SLICE, st);
+    TK_TRY(oz_split_matrix(p->A, P.dt, P.m, P.n, P.lda, B.Aoz, B.EA, B.EC, B.colmax, copy, st));
+    prof_end(tok, st, 0.0, ((P.dt == TK_F64 ? 16.0 : 8.0) + 16.0 + (copy ? 4.0 : 0.0)) * P.m * P.n);
+  }
   if (P.mixed && P.dt == TK_F64) {
-    if (!reuse) {
+    if (!reuse && !digits) {
       const int tok = prof_begin(TK_PHASE_SLICE, st);  // a copy of A made once per solve, like the digit planes
       TK_TRY(convert_f64_to_f32((const double*)p->A, B.A32, P.m, P.n, P.lda, P.n, st));
       prof_end(tok, st, 0.0, 12.0 * P.m * P.n);
@@ -557,7 +597,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
     if (emulated_gram(P)) TK_CUDA(cudaMemcpyAsync(&gerr, B.oz_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     TK_CUDA(cudaStreamSynchronize(st));
     if (gerr) {
-      set_error_msg("emulated float64 Gram matrix: a pipeline wait timed out");
+      set_error_msg("emulated float64 Gram matrix or Cholesky: a pipeline wait timed out");
       return TK_ETIMEOUT;
     }
     for (int i = 0; i < N; ++i) {
@@ -637,6 +677,11 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
     Lsqr<double>& e = B.e64;
     e.A = A64; e.lda = lda64; e.st = st; e.atol = e.btol = P.o.tol; e.maxiter = P.o.maxiter;
     e.a_es = P.dt == TK_F64 ? 8.0 : 4.0;
+    if (P.oz64) {
+      TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));
+      e.oz_A = oz_mat(P, B);
+      e.oz_err = B.oz_err;
+    }
     if (!P.lowrank) {
       e.prec_kind = TK_PRECOND_CHOL; e.R = B.R; e.ldr = P.np; e.rstride = P.np * P.np;
       if (P.inv64) { e.Mi = B.Minv64; e.Mti = B.Mtinv64; e.ldm = P.np; e.mstride = P.np * P.np; }
@@ -664,6 +709,15 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
       TK_TRY(e.run(p->b, 0, nullptr, 0, B.ids, B.lam, nok, X, P.n, false, res));
     } else {
       for (int k = 0; k < nok; ++k) TK_TRY(e.run(p->b, 0, nullptr, 0, B.ids + k, B.lam, 1, X, P.n, false, res));
+    }
+    if (P.oz64) {
+      int oz_err = 0;
+      TK_CUDA(cudaMemcpyAsync(&oz_err, B.oz_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+      TK_CUDA(cudaStreamSynchronize(st));
+      if (oz_err) {
+        set_error_msg("emulated float64 product: a pipeline wait timed out");
+        return TK_ETIMEOUT;
+      }
     }
     for (const auto& r : res) {
       tk_info& q = inf[r.lam_idx];
@@ -695,16 +749,11 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
     std::vector<int> act = ok_ids;
     std::vector<double> hn(3 * std::max(N, 1));
     std::vector<double> prev_dn(std::max(N, 1), INFINITY);
-    if (P.o.emulate_fp64 && !act.empty()) {  // A is split once (by rows and by columns); x, r on every pass
-      if (!reuse) {
-        const int tok = prof_begin(TK_PHASE_SLICE, st);
-        TK_TRY(oz_prepare(p->A, P.dt, P.m, P.n, P.lda, B.Aoz, B.EA, st));
-        TK_TRY(oz_prepare_cols(p->A, P.dt, P.m, P.n, P.lda, B.AozC, B.EC, B.colmax, st));
-        prof_end(tok, st, 0.0, 2.0 * ((P.dt == TK_F64 ? 16.0 : 8.0) * P.m * P.n + 16.0 * P.m * P.n));
-      }
+    if (P.o.emulate_fp64 && !act.empty()) {
       TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));
-      if (P.lsqr_oz) {  // the LSQR products read the first 4 digits of the same slices
-        e.oz_A = B.Aoz; e.oz_EA = B.EA; e.oz_AT = B.AozC; e.oz_EAT = B.EC; e.oz_err = B.oz_err;
+      if (P.lsqr_oz) {  // the LSQR products read the first 4 digits of the same planes
+        e.oz_A = oz_mat(P, B);
+        e.oz_err = B.oz_err;
       }
     }
     for (int round = 0; round < P.o.max_refine && !act.empty(); ++round) {
@@ -724,8 +773,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
         const double fl = 2.0 * cnt * P.m * P.n;
         int tok = prof_begin(TK_PHASE_RES64, st);
         if (P.o.emulate_fp64) {
-          TK_TRY(oz_prepare(B.Xa, TK_F64, cnt, P.n, P.n, B.Xoz, B.EX, st));
-          TK_TRY(oz_residual(B.Aoz, B.EA, P.m, P.n, B.Xoz, B.EX, cnt, p->b, B.Rres, P.m, B.oz_err, st));
+          TK_TRY(oz_residual(oz_mat(P, B), B.Xa, P.n, cnt, B.Xoz, B.EX, p->b, B.Rres, P.m, B.oz_err, st));
         } else if (P.dt == TK_F64) {
           TK_TRY((gemm<double, double, double>(false, true, cnt, P.m, P.n, B.Xa, P.n, A64, lda64, B.Rres, P.m, -1.0,
                                                B.ones, B.Rres, P.m, st)));
@@ -739,7 +787,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
         int sp;
         if (P.o.emulate_fp64) {
           sp = std::min(B.splits, oz_normal_splits(P.m, P.n, cnt));
-          TK_TRY(oz_normal(B.AozC, B.EC, P.m, P.n, B.Rres, P.m, cnt, B.Roz, B.ER, B.part, sp, B.oz_err, st));
+          TK_TRY(oz_normal(oz_mat(P, B), B.Rres, P.m, cnt, B.Roz, B.ER, B.part, sp, B.oz_err, st));
         } else {
           sp = P.dt == TK_F64 ? splitk_tuned<double, double>(cnt, P.n, P.m, B.splits)
                               : splitk_tuned<double, float>(cnt, P.n, P.m, B.splits);
@@ -913,8 +961,7 @@ tk_status lc_norms(const tk_problem* p, const Plan& P, Bufs& B, const LcBufs& L,
                    int off, cudaStream_t st) {
   if (cnt <= 0) return TK_OK;
   if (P.mixed && P.o.emulate_fp64) {
-    TK_TRY(oz_prepare(Xrows, TK_F64, cnt, P.n, P.n, B.Xoz, B.EX, st));
-    TK_TRY(oz_residual(B.Aoz, B.EA, P.m, P.n, B.Xoz, B.EX, cnt, p->b, L.R, P.m, B.oz_err, st));
+    TK_TRY(oz_residual(oz_mat(P, B), Xrows, P.n, cnt, B.Xoz, B.EX, p->b, L.R, P.m, B.oz_err, st));
   } else {
     k_bcast<<<rgrid(P.m, cnt), 256, 0, st>>>(p->b, P.m, L.R, cnt);
     k_fill<<<1, 256, 0, st>>>(B.ones, cnt, 1.0);
@@ -1258,7 +1305,7 @@ TK_API tk_status tk_autotune(const tk_problem* p, int N, const tk_opts* o, void*
 
 namespace tk {
 struct ResidualBufs {
-  void *Aoz, *Xoz, *AozC, *colmax, *Roz;
+  void *Aoz, *Xoz, *colmax, *Roz;
   int *EA, *EX, *EC, *ER, *err;
   double *ones, *part;
   int splits;
@@ -1269,7 +1316,6 @@ static void residual_carve(Arena& a, int64_t m, int64_t n, int M, ResidualBufs& 
   w.EA = a.take<int>(m);
   w.Xoz = a.take<char>(oz_slices_bytes(M, n));
   w.EX = a.take<int>(M);
-  w.AozC = a.take<char>(oz_slices_bytes(n, m));
   w.EC = a.take<int>(n);
   w.colmax = a.take<char>(oz_colmax_bytes(n));
   w.Roz = a.take<char>(oz_slices_bytes(M, m));
@@ -1317,12 +1363,12 @@ TK_API tk_status tk_residual(const tk_problem* p, const double* X, int M, int64_
   int herr = 0;
   if (emulate) {
     TK_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), st));
-    TK_TRY(oz_prepare(p->A, p->dtype, m, n, p->lda, w.Aoz, w.EA, st));
-    TK_TRY(oz_prepare(X, TK_F64, M, n, ldx, w.Xoz, w.EX, st));
-    TK_TRY(oz_residual(w.Aoz, w.EA, m, n, w.Xoz, w.EX, M, p->b, R, m, w.err, st));
+    TK_TRY(oz_split_matrix(p->A, p->dtype, m, n, p->lda, w.Aoz, w.EA, w.EC, w.colmax, nullptr, st));
+    OzMat Am;
+    Am.planes = w.Aoz; Am.ER = w.EA; Am.EC = w.EC; Am.m = m; Am.n = n;
+    TK_TRY(oz_residual(Am, X, ldx, M, w.Xoz, w.EX, p->b, R, m, w.err, st));
     if (G) {
-      TK_TRY(oz_prepare_cols(p->A, p->dtype, m, n, p->lda, w.AozC, w.EC, w.colmax, st));
-      TK_TRY(oz_normal(w.AozC, w.EC, m, n, R, m, M, w.Roz, w.ER, w.part, w.splits, w.err, st));
+      TK_TRY(oz_normal(Am, R, m, M, w.Roz, w.ER, w.part, w.splits, w.err, st));
       k_residual_sum_splits<<<(unsigned)std::min<int64_t>(cdiv((int64_t)M * n, 256), 152 * 8), 256, 0, st>>>(
           w.part, w.splits, (int64_t)M * n, G);
       TK_LAUNCH_CHECK();
@@ -1788,7 +1834,7 @@ TK_API tk_status tk_lcurve(const tk_problem* p, const double* lambdas, int N, in
 // ---- the products of one LSQR step on their own (parity of the fused form) ----------
 namespace {
 struct StepBufs {
-  void *Aoz, *AozC, *colmax, *Wq, *Uq;
+  void *Aoz, *colmax, *Wq, *Uq;
   int *EA, *EC, *EW, *EU, *err;
   double* part;
   float* A32;
@@ -1799,7 +1845,6 @@ void step_carve(Arena& a, int64_t m, int64_t n, int count, StepBufs& w) {
   w.A32 = a.take<float>((size_t)m * n);
   w.Aoz = a.take<char>(oz_slices_bytes(m, n));
   w.EA = a.take<int>(m);
-  w.AozC = a.take<char>(oz_slices_bytes(n, m));
   w.EC = a.take<int>(n);
   w.colmax = a.take<char>(oz_colmax_bytes(n));
   w.Wq = a.take<char>(oz_slices_bytes(count, n, OZ_LSQR_DIGITS));
@@ -1870,16 +1915,16 @@ TK_API tk_status tk_lsqr_step_products(const tk_problem* p, const float* W, int 
     planes = std::min(w.planes, lm_small_atu_splits(m, n));
     TK_TRY(lm_small_atu(A32, lda32, m, n, U, m, count, w.part, planes, st));
   } else {
-  TK_TRY(oz_prepare(p->A, p->dtype, m, n, p->lda, w.Aoz, w.EA, st));
-  if (fused) {
-    TK_TRY(oz_lsqr_fused(w.Aoz, w.EA, m, n, W, n, count, w.Wq, w.EW, U, m, coef, w.part, w.planes, &planes, w.err,
-                         st));
-  } else {
-    TK_TRY(oz_prepare_cols(p->A, p->dtype, m, n, p->lda, w.AozC, w.EC, w.colmax, st));
-    TK_TRY(oz_lsqr_aw(w.Aoz, w.EA, m, n, W, n, count, w.Wq, w.EW, U, m, coef, w.err, st));
-    planes = std::min(w.planes, oz_normal_splits(m, n, count, OZ_LSQR_DIGITS));
-    TK_TRY(oz_lsqr_atu(w.AozC, w.EC, m, n, U, m, count, w.Uq, w.EU, w.part, planes, w.err, st));
-  }
+    TK_TRY(oz_split_matrix(p->A, p->dtype, m, n, p->lda, w.Aoz, w.EA, w.EC, w.colmax, nullptr, st));
+    OzMat Am;
+    Am.planes = w.Aoz; Am.ER = w.EA; Am.EC = w.EC; Am.m = m; Am.n = n;
+    if (fused) {
+      TK_TRY(oz_lsqr_fused(Am, W, n, count, w.Wq, w.EW, U, m, coef, w.part, w.planes, &planes, w.err, st));
+    } else {
+      TK_TRY(oz_lsqr_aw<float>(Am, W, n, count, w.Wq, w.EW, U, m, coef, w.err, st));
+      planes = std::min(w.planes, oz_normal_splits(m, n, count, OZ_LSQR_DIGITS));
+      TK_TRY(oz_lsqr_atu<float>(Am, U, m, count, w.Uq, w.EU, w.part, planes, w.err, st));
+    }
   }
   const int64_t total = (int64_t)count * n;
   k_step_sum_planes<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(cdiv(total, 256), 152 * 8)), 256, 0, st>>>(

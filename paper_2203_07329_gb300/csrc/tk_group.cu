@@ -446,8 +446,8 @@ struct GState {
   double fl_aw = 0.0;  // flops of one step (all slots active): for the profiler
   // the emulated float64 passes: digit planes of one problem at a time (the largest fits)
   int64_t oz_m = 0, oz_n = 0;
-  size_t oz_rows_bytes = 0, oz_cols_bytes = 0, oz_vec_bytes = 0;
-  void *oz_rows = nullptr, *oz_cols = nullptr, *oz_colmax = nullptr, *oz_vec = nullptr;
+  size_t oz_rows_bytes = 0, oz_vec_bytes = 0;
+  void *oz_rows = nullptr, *oz_colmax = nullptr, *oz_vec = nullptr;
   int *oz_EA = nullptr, *oz_EC = nullptr, *oz_EV = nullptr, *oz_err = nullptr;
 };
 
@@ -506,7 +506,6 @@ void carve_group(const std::vector<GroupProblem>& g, int N, Arena& a, GState& S)
       S.oz_m = std::max(S.oz_m, q.m);
       S.oz_n = std::max(S.oz_n, q.n);
       S.oz_rows_bytes = std::max(S.oz_rows_bytes, oz_slices_bytes(q.m, q.n));
-      S.oz_cols_bytes = std::max(S.oz_cols_bytes, oz_slices_bytes(q.n, q.m));
       S.oz_vec_bytes = std::max({S.oz_vec_bytes, oz_slices_bytes(N, q.n), oz_slices_bytes(N, q.m)});
     }
     naw += (size_t)cdiv(q.m, tiles::LM_BN);
@@ -536,10 +535,9 @@ void carve_group(const std::vector<GroupProblem>& g, int N, Arena& a, GState& S)
   }
   S.BM = N <= 16 ? 16 : (N <= 32 ? 32 : 64);
   if (S.oz_rows_bytes > 0) {
-    // the largest problem's digit planes of A's rows and columns, and of the lambda-side vectors
+    // the largest problem's digit planes of A, and of the lambda-side vectors
     // (X: N x n, r: N x m), reused problem by problem
     S.oz_rows = a.take<char>(S.oz_rows_bytes);
-    S.oz_cols = a.take<char>(S.oz_cols_bytes);
     S.oz_colmax = a.take<char>(oz_colmax_bytes(S.oz_n));
     S.oz_vec = a.take<char>(S.oz_vec_bytes);
     S.oz_EA = a.take<int>((size_t)S.oz_m);
@@ -683,32 +681,23 @@ tk_status group_solve_mixed(std::vector<GroupProblem>& g, int N, void* work, siz
       for (int p = 0; p < P; ++p) any_oz = any_oz || (hcnt[p] > 0 && g[p].emulate);
       if (any_oz) {
         TK_CUDA(cudaMemsetAsync(S.oz_err, 0, sizeof(int), st));
-        for (int mode = 0; mode < 2; ++mode) {
-          double fl = 0.0, by = 0.0, ib = 0.0;
-          const int tok = prof_begin(mode == 0 ? TK_PHASE_RES64 : TK_PHASE_NE64, st);
-          for (int p = 0; p < P; ++p) {
-            if (hcnt[p] == 0 || !g[p].emulate) continue;
-            const GDesc& d = S.hd[p];
-            const tk_dtype dt = g[p].f64 ? TK_F64 : TK_F32;
-            const int M = hcnt[p];
-            if (mode == 0) {
-              TK_TRY(oz_prepare(g[p].Af, dt, g[p].m, g[p].n, g[p].ldaf, S.oz_rows, S.oz_EA, st));
-              TK_TRY(oz_prepare(d.Xa, TK_F64, M, g[p].n, g[p].n, S.oz_vec, S.oz_EV, st));
-              TK_TRY(oz_residual(S.oz_rows, S.oz_EA, g[p].m, g[p].n, S.oz_vec, S.oz_EV, M, g[p].b, d.Rres, g[p].m,
-                                 S.oz_err, st));
-            } else {
-              const int sp = std::min(d.splits64, oz_normal_splits(g[p].m, g[p].n, M));
-              TK_TRY(oz_prepare_cols(g[p].Af, dt, g[p].m, g[p].n, g[p].ldaf, S.oz_cols, S.oz_EC, S.oz_colmax, st));
-              TK_TRY(oz_normal(S.oz_cols, S.oz_EC, g[p].m, g[p].n, d.Rres, g[p].m, M, S.oz_vec, S.oz_EV, d.part64, sp,
-                               S.oz_err, st));
-              S.hd[p].sp64 = sp;
-            }
-            const double es = g[p].f64 ? 8.0 : 4.0;
-            fl += 2.0 * M * g[p].m * g[p].n;
-            by += es * g[p].m * g[p].n + 16.0 * M * g[p].m;
-            ib += (2.0 * es + 32.0) * g[p].m * g[p].n + 16.0 * M * g[p].m;  // A read twice, 8 planes out and in
-          }
-          prof_end(tok, st, fl, by, ib);
+        for (int p = 0; p < P; ++p) {
+          if (hcnt[p] == 0 || !g[p].emulate) continue;
+          const GDesc& d = S.hd[p];
+          const int M = hcnt[p];
+          const double es = g[p].f64 ? 8.0 : 4.0, mn = (double)g[p].m * g[p].n;
+          OzMat Am;
+          Am.planes = S.oz_rows; Am.ER = S.oz_EA; Am.EC = S.oz_EC; Am.m = g[p].m; Am.n = g[p].n;
+          int tok = prof_begin(TK_PHASE_RES64, st);
+          TK_TRY(oz_split_matrix(g[p].Af, g[p].f64 ? TK_F64 : TK_F32, g[p].m, g[p].n, g[p].ldaf, S.oz_rows, S.oz_EA,
+                                 S.oz_EC, S.oz_colmax, nullptr, st));
+          TK_TRY(oz_residual(Am, d.Xa, g[p].n, M, S.oz_vec, S.oz_EV, g[p].b, d.Rres, g[p].m, S.oz_err, st));
+          prof_end(tok, st, 2.0 * M * mn, es * mn + 16.0 * M * g[p].m, (2.0 * es + 32.0) * mn + 16.0 * M * g[p].m);
+          tok = prof_begin(TK_PHASE_NE64, st);
+          const int sp = std::min(d.splits64, oz_normal_splits(g[p].m, g[p].n, M));
+          TK_TRY(oz_normal(Am, d.Rres, g[p].m, M, S.oz_vec, S.oz_EV, d.part64, sp, S.oz_err, st));
+          S.hd[p].sp64 = sp;
+          prof_end(tok, st, 2.0 * M * mn, es * mn + 16.0 * M * g[p].m, 16.0 * mn + 16.0 * M * g[p].m);
         }
         TK_CUDA(cudaMemcpyAsync(S.dd, S.hd.data(), sizeof(GDesc) * P, cudaMemcpyHostToDevice, st));
       }

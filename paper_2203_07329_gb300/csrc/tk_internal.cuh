@@ -231,26 +231,40 @@ constexpr int dtype_code() {
   return sizeof(T) == 8 ? 1 : 0;
 }
 
-// Float64-accurate products on the BF16 tensor cores (tk_oz.cu).  The rows of
-// X (rows x cols, row stride ld) are split into 8 exact BF16 slice planes
-// (row stride cols rounded up to 64) with row exponents E (oz_prepare), or the
-// columns of X into planes of X^T with column exponents (oz_prepare_cols:
-// slices bytes oz_slices_bytes(cols, rows), E: cols ints, colmax:
-// oz_colmax_bytes(cols)).  *err (device) is set if a pipeline wait timed out.
+// Float64-accurate products on the BF16 tensor cores (tk_oz.cu).  A matrix A
+// (m x n) is scaled by powers of two along its rows and its columns,
+// A'' = A[i][j] 2^-(ER[i] + EC[j]), and split into 8 exact BF16 digit planes
+// (row stride n rounded up to 64): one set, read along the rows by the
+// products A W^T and along the columns by A^T U.  The lambda rows of a
+// product's small operand are split on every pass (oz_split_vectors; `shift`:
+// the exponents of A along the summed index move onto it).  *err (device) is
+// set if a pipeline wait timed out.
+struct OzMat {
+  const void* planes = nullptr;
+  const int* ER = nullptr;  // m row exponents
+  const int* EC = nullptr;  // n column exponents
+  int64_t m = 0, n = 0;
+};
 constexpr int OZ_LSQR_DIGITS = 4;  // digits of the float32-accurate LSQR products
+// digits of an LSQR product in T's precision: 8 (float64) or 4 (float32)
+template <typename T>
+constexpr int oz_digits() {
+  return sizeof(T) == 8 ? 8 : OZ_LSQR_DIGITS;
+}
 size_t oz_slices_bytes(int64_t rows, int64_t cols, int planes = 8);
-tk_status oz_prepare(const void* X, tk_dtype dt, int64_t rows, int64_t cols, int64_t ld, void* slices, int* E,
-                     cudaStream_t st, int planes = 8);
 size_t oz_colmax_bytes(int64_t cols);
-tk_status oz_prepare_cols(const void* X, tk_dtype dt, int64_t rows, int64_t cols, int64_t ld, void* slices, int* E,
-                          void* colmax, cudaStream_t st);
-// R[l][i] = b[i] - sum_k X[l][k] A[i][k] from the row slices of A (m x n) and
-// of X (M x n).
-tk_status oz_residual(const void* Aslices, const int* EA, int64_t m, int64_t n, const void* Xslices, const int* EX,
-                      int64_t M, const double* b, double* R, int64_t ldr, int* err, cudaStream_t st);
+// slices: oz_slices_bytes(rows, cols); ER: rows ints; EC: cols ints; colmax: oz_colmax_bytes(cols);
+// copy (may be null): the float32 copy of A (row stride cols), written by the first pass
+tk_status oz_split_matrix(const void* A, tk_dtype dt, int64_t rows, int64_t cols, int64_t ld, void* slices, int* ER,
+                          int* EC, void* colmax, float* copy, cudaStream_t st);
+tk_status oz_split_vectors(const void* V, tk_dtype dt, int64_t M, int64_t K, int64_t ld, const int* shift,
+                           void* slices, int* E, cudaStream_t st, int planes = 8);
+// R[l][i] = b[i] - sum_k X[l][k] A[i][k] (X: M x n, row stride ldx; Xslices: oz_slices_bytes(M, n),
+// EX: M ints).
+tk_status oz_residual(const OzMat& A, const double* X, int64_t ldx, int64_t M, void* Xslices, int* EX,
+                      const double* b, double* R, int64_t ldr, int* err, cudaStream_t st);
 // The normal-equation pass: partial[z][l][j] (z < splits; unused planes zero)
-// of sum_i A[i][j] R[l][i], from the column slices of A (oz_prepare_cols) and
-// R (M x m, row stride ldr); Rslices: oz_slices_bytes(M, m), EX: M ints.
+// of sum_i A[i][j] R[l][i] (R: M x m, row stride ldr; Rslices: oz_slices_bytes(M, m), EX: M ints).
 int oz_normal_splits(int64_t m, int64_t n, int64_t M, int S = 8);  // S: digits of the product (4 or 8)
 // Cholesky of C + lambda I (chol_shifted) with the trailing updates on the
 // tensor cores: oz_chol_begin prepares the slice buffers and tensor maps
@@ -270,22 +284,28 @@ size_t oz_chol_workspace(int64_t np, int N);
 tk_status oz_chol_begin(double* R, int64_t ldr, int64_t rstride, int N, int64_t np, void* work, size_t bytes,
                         int* err, OzCholPlan* plan, cudaStream_t st);
 tk_status oz_chol_step(const OzCholPlan& plan, int kb, cudaStream_t st);
-// The two float32 LSQR products from the first 4 digits of the slices of A
-// (the 28-bit rounded A) and of the lambda-major vectors, sliced here
-// (Wslices / Uslices: oz_slices_bytes(count, n or m, 4); EW / EU: count ints):
+// The LSQR products in T's precision, from the first oz_digits<T>() digits of A and of the
+// lambda-major vectors, split here (Wslices / Uslices: oz_slices_bytes(count, n or m, digits);
+// EW / EU: count ints):
 //   aw:  U[l][i] = sum_k W[l][k] A[i][k] + coef[l] U[l][i]  (coef may be null);
+//   aw_split: partial[z][l][i] of sum_{k in split z} W[l][k] A[i][k] (short output, long K);
 //   atu: partial[z][l][j] = sum_{i in split z} U[l][i] A[i][j].
-tk_status oz_lsqr_aw(const void* Aslices, const int* EA, int64_t m, int64_t n, const float* W, int64_t ldw, int count,
-                     void* Wslices, int* EW, float* U, int64_t ldu, const double* coef, int* err, cudaStream_t st);
+template <typename T>
+tk_status oz_lsqr_aw(const OzMat& A, const T* W, int64_t ldw, int count, void* Wslices, int* EW, T* U, int64_t ldu,
+                     const double* coef, int* err, cudaStream_t st);
+template <typename T>
+tk_status oz_lsqr_aw_split(const OzMat& A, const T* W, int64_t ldw, int count, void* Wslices, int* EW, double* partial,
+                           int splits, int* err, cudaStream_t st);
+template <typename T>
+tk_status oz_lsqr_atu(const OzMat& A, const T* U, int64_t ldu, int count, void* Uslices, int* EU, double* partial,
+                      int splits, int* err, cudaStream_t st);
 // The two products of one LSQR step fused over one read of A's row-exponent digit planes (count <= 32,
 // n <= 2048): U <- W A^T + coef .* U in place, and partial[z] (z < *planes <= max_planes; count x n
 // float64 planes) whose sum is U A for the new U.  Wslices / EW as oz_lsqr_aw.
 bool oz_fused_supported(int64_t m, int64_t n, int count);
-tk_status oz_lsqr_fused(const void* Aslices, const int* EA, int64_t m, int64_t n, const float* W, int64_t ldw,
-                        int count, void* Wslices, int* EW, float* U, int64_t ldu, const double* coef, double* partial,
-                        int max_planes, int* planes, int* err, cudaStream_t st);
-tk_status oz_lsqr_atu(const void* AslicesT, const int* EC, int64_t m, int64_t n, const float* U, int64_t ldu,
-                      int count, void* Uslices, int* EU, double* partial, int splits, int* err, cudaStream_t st);
+tk_status oz_lsqr_fused(const OzMat& A, const float* W, int64_t ldw, int count, void* Wslices, int* EW, float* U,
+                        int64_t ldu, const double* coef, double* partial, int max_planes, int* planes, int* err,
+                        cudaStream_t st);
 // Float32 LSQR products for at most 16 lambda from the float32 A (m x n, row
 // stride lda): aw: C[l][i] = sum_k W[l][k] A[i][k] (+ beta[l] C[l][i]; beta may
 // be null), W (count x n) held in shared memory (lm_small_aw_supported);
@@ -301,8 +321,8 @@ tk_status lm_small_atu(const float* A, int64_t lda, int64_t m, int64_t n, const 
 size_t oz_gram_workspace(int64_t r, int64_t c);
 tk_status oz_gram(const double* Y, int64_t r, int64_t c, double* C, void* work, size_t bytes, int* err,
                   cudaStream_t st);
-tk_status oz_normal(const void* AslicesT, const int* EC, int64_t m, int64_t n, const double* R, int64_t ldr,
-                    int64_t M, void* Rslices, int* EX, double* partial, int splits, int* err, cudaStream_t st);
+tk_status oz_normal(const OzMat& A, const double* R, int64_t ldr, int64_t M, void* Rslices, int* EX, double* partial,
+                    int splits, int* err, cudaStream_t st);
 
 // Dense kernels (tk_dense.cu)
 template <typename TA, typename TB, typename TC>

@@ -317,6 +317,7 @@ void Lsqr<T>::carve(Arena& a) {
   const int64_t gcols = n;
   splits = splitk_count(N_cap, gcols, m);
   if (std::is_same<T, float>::value) splits = std::max(splits, lm_small_atu_splits(m, n));  // <= 16 lambda
+  if (oz && std::is_same<T, double>::value) splits = std::max(splits, oz_normal_splits(m, n, N_cap));
   if (oz && oz_fused) splits = std::max(splits, 152);  // one partial plane per cluster of the fused step
   V = a.take<T>((size_t)N_cap * nv);
   W = a.take<T>((size_t)N_cap * nv);
@@ -339,7 +340,7 @@ void Lsqr<T>::carve(Arena& a) {
   }
   if (tc) tc_scratch = a.take<char>(tc_lmaj_workspace(N_cap, std::max(n, m)));
   if (oz) {
-    oz_q = a.take<char>(oz_slices_bytes(N_cap, std::max(n, m), OZ_LSQR_DIGITS));
+    oz_q = a.take<char>(oz_slices_bytes(N_cap, std::max(n, m), oz_digits<T>()));
     oz_e = a.take<int>((size_t)N_cap);
   }
 }
@@ -376,12 +377,12 @@ tk_status Lsqr<T>::prod_aw(const T* Win, int64_t ldw, T* C, const double* beta, 
   const double vec = es * (count * (double)n + 2.0 * count * m);
   int tok = prof_begin(digits ? TK_PHASE_AW_DIGITS : TK_PHASE_AW, st);
   tk_status r;
+  if (digits && !(under && !beta)) {
+    r = oz_lsqr_aw<T>(oz_A, Win, ldw, count, oz_q, oz_e, C, m, beta, oz_err, st);
+    prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec, 2.0 * oz_digits<T>() * m * n + vec);
+    return r;
+  }
   if constexpr (std::is_same<T, float>::value) {
-    if (digits) {
-      r = oz_lsqr_aw(oz_A, oz_EA, m, n, Win, ldw, count, oz_q, oz_e, C, m, beta, oz_err, st);
-      prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec, 8.0 * m * n + vec);
-      return r;
-    }
     if (tc && beta) {
       r = tc_lmaj_product(true, A, m, n, lda, Win, ldw, count, C, m, beta, nullptr, 1, tc_scratch, st);
       prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec, es * m * n + vec);
@@ -397,9 +398,13 @@ tk_status Lsqr<T>::prod_aw(const T* Win, int64_t ldw, T* C, const double* beta, 
     // the underdetermined product: a short output (count x m, m < n) against a long K = n; split K
     // over the GPU and add the planes (part_g holds splits x N_cap x n >= sp x count x m values)
     const int64_t cap = ((int64_t)splits * N_cap * n) / std::max<int64_t>((int64_t)count * m, 1);
-    const int sp = (int)std::min<int64_t>(splitk_count(count, m, n), cap);
-    if (sp > 1) {
-      r = gemm_splitk<T, T>(false, true, count, m, n, Win, ldw, A, lda, part_g, sp, st);
+    const int sp = (int)std::min<int64_t>(digits ? oz_normal_splits(n, m, count) : splitk_count(count, m, n), cap);
+    if (sp > 1 || digits) {
+      r = TK_EINVAL;
+      if constexpr (std::is_same<T, double>::value) {
+        if (digits) r = oz_lsqr_aw_split<T>(oz_A, Win, ldw, count, oz_q, oz_e, part_g, sp, oz_err, st);
+      }
+      if (!digits) r = gemm_splitk<T, T>(false, true, count, m, n, Win, ldw, A, lda, part_g, sp, st);
       if (r == TK_OK) {
         const int64_t total = (int64_t)count * m;
         k_sum_planes_to<T><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(cdiv(total, 256), 152 * 8)), 256, 0,
@@ -407,7 +412,7 @@ tk_status Lsqr<T>::prod_aw(const T* Win, int64_t ldw, T* C, const double* beta, 
         TK_LAUNCH_CHECK();
       }
       prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec + 16.0 * sp * total_count(count, m),
-               es * m * n + vec + 16.0 * sp * total_count(count, m));
+               (digits ? 2.0 * oz_digits<T>() : es) * m * n + vec + 16.0 * sp * total_count(count, m));
       return r;
     }
   }
@@ -423,14 +428,14 @@ tk_status Lsqr<T>::prod_atu(const T* Uin, int count) {
   const double es = (double)sizeof(T);
   int tok = prof_begin(digits ? TK_PHASE_ATU_DIGITS : TK_PHASE_ATU, st);
   tk_status r;
+  if (digits) {
+    cur_splits = std::min(splits, oz_normal_splits(m, n, count, oz_digits<T>()));
+    const double vec = es * count * (double)m + 8.0 * cur_splits * count * n;
+    r = oz_lsqr_atu<T>(oz_A, Uin, m, count, oz_q, oz_e, part_g, cur_splits, oz_err, st);
+    prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec, 2.0 * oz_digits<T>() * m * n + vec);
+    return r;
+  }
   if constexpr (std::is_same<T, float>::value) {
-    if (digits) {
-      cur_splits = std::min(splits, oz_normal_splits(m, n, count, OZ_LSQR_DIGITS));
-      const double vec = es * count * (double)m + 8.0 * cur_splits * count * n;
-      r = oz_lsqr_atu(oz_AT, oz_EAT, m, n, Uin, m, count, oz_q, oz_e, part_g, cur_splits, oz_err, st);
-      prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec, 8.0 * m * n + vec);
-      return r;
-    }
     if (tc && AT) {
       cur_splits = splits;
       const double vec = es * count * (double)m + 8.0 * splits * count * n;
@@ -460,7 +465,7 @@ tk_status Lsqr<T>::prod_fused(const T* Win, T* C, const double* beta, int count)
   int tok = prof_begin(TK_PHASE_LSQR_FUSED, st);
   tk_status r = TK_EINVAL;
   if constexpr (std::is_same<T, float>::value)
-    r = oz_lsqr_fused(oz_A, oz_EA, m, n, Win, n, count, oz_q, oz_e, C, m, beta, part_g, splits, &cur_splits, oz_err,
+    r = oz_lsqr_fused(oz_A, Win, n, count, oz_q, oz_e, C, m, beta, part_g, splits, &cur_splits, oz_err,
                       st);
   // A once from memory (its second read, a few microseconds later, comes from L2)
   const double vec = es * (count * (double)n + 2.0 * count * m) + 8.0 * cur_splits * count * n;

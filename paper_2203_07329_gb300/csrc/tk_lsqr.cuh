@@ -2,6 +2,7 @@
 #pragma once
 
 #include <map>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -162,21 +163,22 @@ struct Lsqr {
   bool tc = false;
   const T* AT = nullptr;
   void* tc_scratch = nullptr;
-  // products from the 4-digit slices of A on the tensor cores (float32
-  // engine, large problems): row-exponent slices of A (m x n) and
-  // column-exponent slices of A^T (n x m) as made for the float64 passes
+  // products from the digit planes of A on the tensor cores: the first 4 digits (float32 engine) or
+  // all 8 (float64 engine)
   bool oz = false;
-  const void* oz_A = nullptr;
-  const int* oz_EA = nullptr;
-  const void* oz_AT = nullptr;
-  const int* oz_EAT = nullptr;
+  OzMat oz_A;
   int* oz_err = nullptr;
   void* oz_q = nullptr;  // slices of the lambda-major vector of a product
   int* oz_e = nullptr;
-  // the digit products read 8 bytes per element of A whatever the number of
-  // lambdas, the float32 SIMT products 4 bytes but with work proportional to
-  // it: the digits pay off for large A and more than 16 active lambdas
-  bool use_oz(int count) const { return oz && oz_A && oz_AT && (int64_t)m * n > (int64_t(1) << 24) && count > 16; }
+  // A digit product reads 8 (float32 engine) or 16 bytes (float64) per element of A whatever the
+  // number of lambdas; the SIMT products read 4 or 8 bytes but their work grows with it.  Float32: the
+  // digits pay off for large A and more than 16 active lambdas.  Float64: the pipe (1.2 TFLOP/s) takes
+  // 1.7 ps per element and lambda against the digits' 2.7 ps per element, so from two lambdas on.
+  bool use_oz(int count) const {
+    if (!oz || !oz_A.planes) return false;
+    if (std::is_same<T, double>::value) return count >= 2;
+    return (int64_t)m * n > (int64_t(1) << 24) && count > 16;
+  }
   // both products of an overdetermined step in one kernel over one read of
   // the digits (n <= 2048, at most 32 lambda per launch)
   bool oz_fused = false;

@@ -1,11 +1,13 @@
 // Float64-accurate products on the BF16 tensor cores (splitting into exact
 // integer slices, in the manner of Ozaki's error-free matrix multiplication).
 //
-// GB300 issues about two float64 FMA per clock per SM, so the float64 products
-// of the mixed form (the Gram matrix, the Cholesky trailing updates, and the
-// refinement's r = b - X A^T and A^T r) are bound by that pipe.  Here every
-// row of an operand is scaled by a power of two 2^E (E one above the exponent
-// of its largest entry, so that 2^(E-2) <= max |x| < 2^(E-1)), rounded to
+// GB300 issues about two float64 FMA per clock per SM, so float64 products
+// (the Gram matrix, the Cholesky trailing updates, the refinement's r = b - X A^T
+// and A^T r, and the LSQR products of the float64 form) are bound by that pipe:
+// one product of 65536 x 1024 with 16 lambda takes 3.8 ms there and 0.25 ms from
+// digits.  Here every row of an operand is scaled by a power of two 2^E (E one
+// above the exponent of its largest entry, so that 2^(E-2) <= max |x| < 2^(E-1);
+// A is scaled along its columns first, see k_oz_scale_slice), rounded to
 // nearest at 2^(E-57) (within 2^-55 of the row maximum) and written with
 // S = 8 balanced base-128 digits,
 //   x 2^-E = sum_p d_p 2^(-7(p+1)),  d_p in [-64, 64],
@@ -47,7 +49,14 @@ constexpr int OZ_KPAD = 64;      // slice rows are padded to a multiple of 64 va
 // Exponent marking a row or column with an inf or NaN: its digits are zero
 // and every output that uses it is NaN, so non-finite input is reported (the
 // LSQR stop tests and the refinement see it) instead of being dropped.
+// A marked exponent is OZ_EBAD plus the exponent of the finite entries (0 for a column), which the
+// digits of those entries use.
 constexpr int OZ_EBAD = 1 << 24;
+__host__ __device__ constexpr bool oz_bad(int e) { return e > OZ_EBAD / 2; }
+__host__ __device__ constexpr int oz_val(int e) { return oz_bad(e) ? e - OZ_EBAD : e; }
+// Exponent of a row that holds only zeros so far (a memset pattern; far below every exponent, and
+// adding any exponent to it does not overflow).
+constexpr int OZ_EZERO = (int)0x80808080;
 
 // max(m, |x|) that turns inf and NaN into +inf (fmax would ignore a NaN).
 __device__ __forceinline__ double oz_absmax(double m, double x) {
@@ -65,31 +74,58 @@ __device__ __forceinline__ int oz_exponent(double mx) {
   return e;
 }
 
-// Exponent E with max_j |row_j| < 2^(E-1) (0 for a zero row); one warp per row.
-template <typename T>
-__global__ void k_oz_rowexp(const T* __restrict__ X, int64_t rows, int64_t cols, int64_t ld, int* __restrict__ E) {
-  const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= rows) return;
-  const int lane = threadIdx.x & 31;
-  double mx = 0.0;
-  for (int64_t j = lane; j < cols; j += 32) mx = oz_absmax(mx, (double)X[r * ld + j]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) E[r] = oz_exponent(mx);
+// One above frexp's exponent of x, from the bit pattern: 2^(E-2) <= |x| < 2^(E-1) (OZ_EZERO for 0).
+// *bad is set for inf and NaN, which count as 0.
+__device__ __forceinline__ int oz_exp_of(double x, bool* bad) {
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  if (ex == 0x7ff) {
+    *bad = true;
+    return OZ_EZERO;
+  }
+  if (ex) return ex - 1021;
+  const long long mant = __double_as_longlong(x) & ((1ll << 52) - 1);
+  return mant ? (63 - __clzll(mant)) - 1072 : OZ_EZERO;
+}
+__device__ __forceinline__ int oz_exp_of(float x, bool* bad) {
+  const int b = __float_as_int(x), ex = (b >> 23) & 0xff;
+  if (ex == 0xff) {
+    *bad = true;
+    return OZ_EZERO;
+  }
+  if (ex) return ex - 125;
+  const int mant = b & 0x7fffff;
+  return mant ? (31 - __clz(mant)) - 147 : OZ_EZERO;
 }
 
 // Exponent E with max_r |X[r][c]| < 2^(E-1) per column (0 for a zero column):
 // the bit patterns of non-negative doubles order like the values, so the
 // column maxima are combined with an integer atomicMax (mx zeroed first).
+// With copy != nullptr the same pass writes the float32 copy of X (row stride cols) that the
+// float32 products read: A crosses HBM once for both.
 template <typename T>
-__global__ void k_oz_colmax(const T* __restrict__ X, int64_t rows, int64_t cols, int64_t ld, int64_t rows_per,
-                            unsigned long long* __restrict__ mx) {
+__global__ void __launch_bounds__(256) k_oz_colmax(const T* __restrict__ X, int64_t rows, int64_t cols, int64_t ld,
+                                                   int64_t rows_per, unsigned long long* __restrict__ mx,
+                                                   float* __restrict__ copy) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= cols) return;
   const int64_t r0 = (int64_t)blockIdx.y * rows_per, r1 = r0 + rows_per < rows ? r0 + rows_per : rows;
   double v = 0.0;
-#pragma unroll 8
-  for (int64_t r = r0; r < r1; ++r) v = oz_absmax(v, (double)X[r * ld + c]);
+  int64_t r = r0;
+  for (; r + 8 <= r1; r += 8) {
+    T x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = X[(r + k) * ld + c];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      v = oz_absmax(v, (double)x[k]);
+      if (copy) copy[(r + k) * cols + c] = (float)x[k];
+    }
+  }
+  for (; r < r1; ++r) {
+    const T x = X[r * ld + c];
+    v = oz_absmax(v, (double)x);
+    if (copy) copy[r * cols + c] = (float)x;
+  }
   atomicMax(&mx[c], (unsigned long long)__double_as_longlong(v));  // +inf orders above every finite value
 }
 __global__ void k_oz_colexp(const unsigned long long* __restrict__ mx, int64_t cols, int* __restrict__ E) {
@@ -158,66 +194,160 @@ __device__ __forceinline__ void oz_digits(long long v, unsigned short (&bits)[OZ
   bits[0] = oz_bf16_bits(hi);
 }
 
+// x, or 0 for inf and NaN (their row or column is marked)
+__device__ __forceinline__ double oz_finite(double x) {
+  return ((__double2hiint(x) >> 20) & 0x7ff) == 0x7ff ? 0.0 : x;
+}
+__device__ __forceinline__ float oz_finite(float x) { return ((__float_as_int(x) >> 23) & 0xff) == 0xff ? 0.f : x; }
+
 template <typename T>
 __device__ __forceinline__ void oz_split(T x, int E, unsigned short (&bits)[OZ_S]) {
   oz_digits(oz_fixed(x, E), bits);
 }
 __device__ __forceinline__ unsigned oz_pack(unsigned short a, unsigned short b) { return (unsigned)a | ((unsigned)b << 16); }
 
-// Slices of the rows of X with row exponents E: planes out[p][r][c] (row
-// stride cols_pad, zero in the padding) with X[r][c] 2^-E[r] = sum_p
-// out[p][r][c] 2^(-7(p+1)) to within 2^-57 (rounded to nearest).
-// Grid: rows over blockIdx.x (grid-stride) and column chunks of 2 x 256 over
-// blockIdx.y; each thread splits two adjacent values (one 4-byte store per plane).
+// Row exponents and digit planes of a matrix A (rows x cols, row stride ld) whose columns are scaled
+// by 2^-EC: with A'' = A[r][c] 2^-(ER[r] + EC[c]), ER the smallest exponents with |A''| < 1/2, planes
+// out[p][r][c] (row stride cols_pad, zero in the padding) with A'' = sum_p out[p][r][c] 2^(-7(p+1)) to
+// within 2^-57.  Scaling the columns first makes the digits independent of the columns' units, and
+// lets one set of planes serve both products: A W^T reads it along the rows (K = columns), A^T U
+// along the columns (K = rows, the operand MN-major).
+// A block owns a band of RB rows: its 8 warps find the RB exponents (8 / RB warps to a row), then
+// all threads split the band, whose second read comes from L2 (RB is chosen so that the bands of the
+// resident blocks fit there).  Bound by HBM: one read of A and 16 bytes written per element; 262144 x
+// 2048 float64 takes 3.0 ms (and 1.1 ms for the column maxima and the float32 copy) where separate row
+// and column planes took 9.5 ms.
 template <typename T>
-__global__ void __launch_bounds__(256) k_oz_slice(const T* __restrict__ X, int64_t rows, int64_t cols, int64_t ld,
-                                                  const int* __restrict__ E, int64_t cols_pad, int planes,
-                                                  __nv_bfloat16* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_oz_scale_slice(const T* __restrict__ A, int64_t rows, int64_t cols,
+                                                        int64_t ld, const int* __restrict__ EC, int RB,
+                                                        int64_t cols_pad, int* __restrict__ ER,
+                                                        __nv_bfloat16* __restrict__ out) {
+  __shared__ int sh_e[8], sh_bad[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t r0 = (int64_t)blockIdx.x * RB;
+  const int nr = rows - r0 < RB ? (int)(rows - r0) : RB;
+  if (threadIdx.x < 8) {
+    sh_e[threadIdx.x] = OZ_EZERO;
+    sh_bad[threadIdx.x] = 0;
+  }
+  __syncthreads();
+  const int wpr = 8 / RB;  // warps to a row
+  const int lr = warp / wpr;
+  if (lr < nr) {
+    const T* x = A + (r0 + lr) * ld;
+    int e = OZ_EZERO;
+    bool bad = false;
+#pragma unroll 8
+    for (int64_t c = (warp % wpr) * 32 + lane; c < cols; c += wpr * 32) {
+      const int ex = oz_exp_of(x[c], &bad);
+      const int ec = oz_val(EC[c]);
+      e = max(e, ex == OZ_EZERO ? OZ_EZERO : ex - ec);
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) {
+      atomicMax(&sh_e[lr], e);
+      if (bad) sh_bad[lr] = 1;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < nr) {
+    const int e = sh_e[threadIdx.x] == OZ_EZERO ? 0 : sh_e[threadIdx.x];
+    ER[r0 + threadIdx.x] = e + (sh_bad[threadIdx.x] ? OZ_EBAD : 0);
+    sh_e[threadIdx.x] = e;
+  }
+  __syncthreads();
   const int64_t plane = rows * cols_pad;
-  const int64_t c = ((int64_t)blockIdx.y * blockDim.x + threadIdx.x) * 2;
-  if (c >= cols_pad) return;
-  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
-    const int e = E[r];
-    const T* xr = X + r * ld;
-    unsigned short s0[OZ_S], s1[OZ_S];
-    oz_split(c < cols ? xr[c] : T(0), e, s0);
-    oz_split(c + 1 < cols ? xr[c + 1] : T(0), e, s1);
-    unsigned* o = reinterpret_cast<unsigned*>(out + r * cols_pad + c);
+  for (int64_t c = 2 * threadIdx.x; c < cols_pad; c += 2 * blockDim.x) {
+    const int e0 = c < cols ? oz_val(EC[c]) : 0, e1 = c + 1 < cols ? oz_val(EC[c + 1]) : 0;
+    for (int k = 0; k < nr; ++k) {
+      const T* x = A + (r0 + k) * ld;
+      const int e = sh_e[k];
+      unsigned short s0[OZ_S], s1[OZ_S];
+      oz_split(c < cols ? oz_finite(x[c]) : T(0), e + e0, s0);
+      oz_split(c + 1 < cols ? oz_finite(x[c + 1]) : T(0), e + e1, s1);
+      unsigned* o = reinterpret_cast<unsigned*>(out + (r0 + k) * cols_pad + c);
 #pragma unroll
-    for (int p = 0; p < OZ_S; ++p)
-      if (p < planes) o[p * (plane / 2)] = oz_pack(s0[p], s1[p]);
+      for (int p = 0; p < OZ_S; ++p) o[p * (plane / 2)] = oz_pack(s0[p], s1[p]);
+    }
   }
 }
 
-// Exponents of long rows (cols much larger than rows): E[r] = max over the
-// blocks of a row of the exponent of their largest |value| (atomicMax; E
-// filled with OZ_EMIN first, then zero rows set to 0).
-constexpr int OZ_EMIN = -4096;
-__global__ void k_oz_fill_emin(int* __restrict__ E, int64_t rows) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < rows) E[r] = OZ_EMIN;
+// Digits of the lambda rows of a vector block V (M x K, row stride ld), the small operand of a
+// product: with V'[l][k] = V[l][k] 2^shift[k] (shift: the exponents of A that the product sums over;
+// null = 0), E[l] one above the exponent of the row's largest |V'| and planes out[p][l][k] (row
+// stride kp, zero in the padding).  Rows of fewer than OZ_VEC_LONG values: one block per row does
+// both (the row comes from L1 or L2 the second time); longer rows: the exponents by blocks of
+// values (k_oz_vec_exp, E preset to OZ_EZERO by a memset), then k_oz_vec_slice.
+constexpr int64_t OZ_VEC_LONG = 8192;
+template <typename T>
+__device__ __forceinline__ int oz_vec_exp(const T* __restrict__ x, const int* __restrict__ shift, int64_t k0,
+                                          int64_t k1, bool* bad) {
+  int e = OZ_EZERO;
+#pragma unroll 4
+  for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
+    const int ex = oz_exp_of(x[k], bad);
+    const int sk = shift ? oz_val(shift[k]) : 0;
+    e = max(e, ex == OZ_EZERO ? OZ_EZERO : ex + sk);
+  }
+  return e;
+}
+// max over the block; a non-finite value anywhere marks it
+__device__ __forceinline__ int oz_block_exp(int e, bool bad, int* sh) {
+  e = __reduce_max_sync(0xffffffffu, bad ? OZ_EBAD : e);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = e;
+  __syncthreads();
+  e = sh[0];
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) e = max(e, sh[w]);
+  return e;
 }
 template <typename T>
-__global__ void __launch_bounds__(256) k_oz_rowexp_long(const T* __restrict__ X, int64_t cols, int64_t ld,
-                                                        int64_t per_block, int* __restrict__ E) {
-  __shared__ double sh[32];
-  const int64_t r = blockIdx.y;
-  const int64_t c0 = (int64_t)blockIdx.x * per_block;
-  const int64_t c1 = c0 + per_block < cols ? c0 + per_block : cols;
-  double mx = 0.0;
-  for (int64_t c = c0 + threadIdx.x; c < c1; c += blockDim.x) mx = oz_absmax(mx, (double)X[r * ld + c]);
+__device__ __forceinline__ void oz_vec_split(const T* __restrict__ x, const int* __restrict__ shift, int64_t k,
+                                             int64_t K, int e, int64_t plane, int planes, unsigned* __restrict__ o) {
+  // a marked row's digits are not used (every output of it is NaN); a zero row has zero digits
+  const bool none = oz_bad(e) || e == OZ_EZERO;
+  unsigned short s0[OZ_S], s1[OZ_S];
+  oz_split(k < K && !none ? x[k] : T(0), (none || !shift || k >= K) ? (none ? 0 : e) : e - oz_val(shift[k]), s0);
+  oz_split(k + 1 < K && !none ? x[k + 1] : T(0),
+           (none || !shift || k + 1 >= K) ? (none ? 0 : e) : e - oz_val(shift[k + 1]), s1);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, sh[w]);
-    if (mx > 0.0) atomicMax(&E[r], oz_exponent(mx));  // OZ_EBAD wins
-  }
+  for (int p = 0; p < OZ_S; ++p)
+    if (p < planes) o[p * (plane / 2)] = oz_pack(s0[p], s1[p]);
 }
-__global__ void k_oz_fix_zero_rows(int* __restrict__ E, int64_t rows) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < rows && E[r] == OZ_EMIN) E[r] = 0;
+template <typename T>
+__global__ void __launch_bounds__(512) k_oz_vec(const T* __restrict__ V, int64_t M, int64_t K, int64_t ld,
+                                                const int* __restrict__ shift, int* __restrict__ E, int64_t kp,
+                                                int planes, __nv_bfloat16* __restrict__ out) {
+  __shared__ int sh[16];
+  const int64_t l = blockIdx.x;
+  const T* x = V + l * ld;
+  bool bad = false;
+  int e = oz_vec_exp(x, shift, 0, K, &bad);
+  e = oz_block_exp(e, bad, sh);
+  if (threadIdx.x == 0) E[l] = e;
+  for (int64_t k = 2 * threadIdx.x; k < kp; k += 2 * blockDim.x)
+    oz_vec_split(x, shift, k, K, e, M * kp, planes, reinterpret_cast<unsigned*>(out + l * kp + k));
+}
+template <typename T>
+__global__ void __launch_bounds__(256) k_oz_vec_exp(const T* __restrict__ V, int64_t K, int64_t ld,
+                                                    const int* __restrict__ shift, int64_t per_block,
+                                                    int* __restrict__ E) {
+  __shared__ int sh[8];
+  const int64_t k0 = (int64_t)blockIdx.x * per_block;
+  const int64_t k1 = k0 + per_block < K ? k0 + per_block : K;
+  bool bad = false;
+  int e = oz_vec_exp(V + (int64_t)blockIdx.y * ld, shift, k0, k1, &bad);
+  e = oz_block_exp(e, bad, sh);
+  if (threadIdx.x == 0) atomicMax(&E[blockIdx.y], e);  // OZ_EBAD wins
+}
+template <typename T>
+__global__ void __launch_bounds__(256) k_oz_vec_slice(const T* __restrict__ V, int64_t M, int64_t K, int64_t ld,
+                                                      const int* __restrict__ shift, const int* __restrict__ E,
+                                                      int64_t kp, int planes, __nv_bfloat16* __restrict__ out) {
+  const int64_t l = blockIdx.y;
+  const int e = E[l];
+  const int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2;
+  if (k < kp) oz_vec_split(V + l * ld, shift, k, K, e, M * kp, planes, reinterpret_cast<unsigned*>(out + l * kp + k));
 }
 
 // Slices of the COLUMNS of X (rows x cols) with column exponents E, stored
@@ -257,7 +387,10 @@ __global__ void __launch_bounds__(256) k_oz_slice_t(const T* __restrict__ X, int
 
 // ---- the product on tcgen05 ---------------------------------------------------
 // D[r][l] = sum_k P[r][k] Q[l][k] from the first S digit planes of P (rows x
-// K, row exponents EP) and of Q (M x K, row exponents EQ), both K-major.
+// K, row exponents EP) and of Q (M x K, row exponents EQ), Q K-major.  P is
+// K-major (TR = false: the planes hold P row by row) or MN-major (TR = true:
+// the planes hold P^T, K rows of `rows` values; the A^T products read the
+// planes of A this way, two boxes of 64 K x 64 rows of P per ring slot).
 // S = 8: float64 accuracy (levels added exactly into int64 accumulators, one
 // rounding at the end); S = 4: the 28-bit rounded operands, float32 accuracy
 // (levels flushed into float32).
@@ -274,7 +407,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_t(const T* __restrict__ X, int
 //     add them into 32 accumulators per row, release the buffer; at the end
 //     write the result: MODE 0 R[l][r] = b[r] - D (float64); MODE 1
 //     partial[z][l][r] = D (float64); MODE 2 U[l][r] = D + coef[l] U[l][r]
-//     (float32 U; coef == nullptr: U = D).
+//     (coef == nullptr: U = D; U float32 for S = 4, float64 for S = 8).
 // Every mbarrier wait is bounded; a wait that gives up sets *err and the
 // roles stop.
 constexpr int OT_M = 128;
@@ -314,7 +447,7 @@ struct OtSmem {
   uint32_t tmem_base;
 };
 
-template <int S, int MODE, int NT>
+template <int S, int MODE, int NT, bool TR>
 __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
     k_oz_tc(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmQ,
             const int* __restrict__ EP, const int* __restrict__ EQ, int64_t rows, int M, int64_t K, int64_t kps,
@@ -378,7 +511,12 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
           break;
         }
         mbar_expect_tx(&Sm.p_full[ps], OT_P_BYTES);
-        tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], kc, (int)r0, p);
+        if constexpr (TR) {
+          tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], (int)r0, kc, p);
+          tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps] + OT_P_BYTES / 2, (int)r0 + 64, kc, p);
+        } else {
+          tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], kc, (int)r0, p);
+        }
       }
     }
     if (*(volatile int*)err) {  // gave up: no bulk copy may still be landing when the CTA exits
@@ -413,15 +551,17 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
           // the planes Q_0 .. Q_(S-1-p) lie one after another (NT rows each), and the levels
           // p .. S-1 are consecutive NT-column blocks of the buffer: all pairs (p, q) are one
           // MMA with N = NT (S - p) whose column block q lands on level p + q
-          const uint64_t pd = sdesc_sw128(smem_u32(Sm.p[ps]));
+          // 16 values of K are 32 bytes of a K-major row, or 16 rows of 128 bytes of the MN-major tile
+          const uint64_t pd = TR ? sdesc_mn_sw128(smem_u32(Sm.p[ps]), OT_P_BYTES / 2) : sdesc_sw128(smem_u32(Sm.p[ps]));
+          constexpr uint64_t pstep = TR ? 2048 / 16 : 2;
           const uint64_t qd = sdesc_sw128(qa);
-          const uint32_t idesc = idesc_bf16(OT_M, NT * (S - p));
+          const uint32_t idesc = idesc_bf16(OT_M, NT * (S - p)) | (TR ? 1u << 15 : 0u);
           const uint32_t d = dbase + (uint32_t)(p * NT);
 #pragma unroll
           for (int k = 0; k < OT_KB / 16; ++k) {
             // the first MMA of a chunk (p = 0) overwrites every level of the buffer
             const uint32_t acc = (kb == kb0 && p == 0 && k == 0) ? 0u : 1u;
-            tc_mma_bf16(d, pd + 2ull * k, qd + 2ull * k, idesc, acc);
+            tc_mma_bf16(d, pd + pstep * k, qd + 2ull * k, idesc, acc);
           }
           tc_commit(&Sm.p_empty[ps]);
         }
@@ -500,15 +640,16 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
           double d;
           if constexpr (S == OZ_S) d = fma((double)lacc[j], 0x1p-63, (double)hacc[j] * 0x1p-35);
           else d = (double)acc[j];
-          const double v = (er >= OZ_EBAD || eq >= OZ_EBAD) ? __longlong_as_double(0x7ff8000000000000ll)
+          const double v = (oz_bad(er) || oz_bad(eq)) ? __longlong_as_double(0x7ff8000000000000ll)
                                                             : ldexp(d, er + eq);
           if (MODE == 0) {
             static_cast<double*>(out)[(int64_t)l * ldo + r] = br - v;
           } else if (MODE == 1) {
             static_cast<double*>(out)[((int64_t)blockIdx.z * M + l) * ldo + r] = v;
           } else {
-            float* u = static_cast<float*>(out) + (int64_t)l * ldo + r;
-            *u = coef ? (float)(v + coef[l] * (double)*u) : (float)v;
+            using TU = typename std::conditional<S == OZ_S, double, float>::type;
+            TU* u = static_cast<TU*>(out) + (int64_t)l * ldo + r;
+            *u = coef ? (TU)(v + coef[l] * (double)*u) : (TU)v;
           }
         }
       }
@@ -526,7 +667,7 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
 // 3D map over the slice planes (K fastest, then rows, then the plane index),
 // box = 64 values of K x box_rows x 1 plane, 128-byte swizzle.
 tk_status make_slice_map(CUtensorMap* map, const void* base, int64_t rows, int64_t kp, uint32_t box_rows,
-                         int planes) {
+                         int planes) {  // kp: row stride
   EncodeTiledFn fn;
   TK_TRY(encode_fn(&fn));
   const cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)rows, (cuuint64_t)planes};
@@ -549,31 +690,40 @@ tk_status make_slice_map(CUtensorMap* map, const void* base, int64_t rows, int64
 // LSQR products (S = 4) over more than 32 lambda, else 32.
 constexpr int oz_tile_n(int S, int64_t M) { return (S != OZ_S && M > 32) ? 64 : 32; }
 
-template <int S, int MODE, int NT>
-tk_status launch_oz_tc_nt(const CUtensorMap& mP, const void* Qs, const int* EP, int64_t rows, const int* EQ, int M,
-                          int planesQ, int64_t kp, int64_t kps, int sp, const double* b, void* out, int64_t ldo,
-                          const double* coef, int* err, cudaStream_t st, int upper_only) {
-  CUtensorMap mQ;
+// The big operand of a product: K-major planes of rows x K (trans = false), or MN-major: the planes
+// hold K x rows (trans = true).
+struct OtBig {
+  const void* planes;
+  const int* E;  // exponents of its `rows`
+  int64_t rows, K;
+  bool trans;
+};
+
+template <int S, int MODE, int NT, bool TR>
+tk_status launch_oz_tc_nt(const OtBig& P, const void* Qs, const int* EQ, int M, int planesQ, int64_t kp, int64_t kps,
+                          int sp, const double* b, void* out, int64_t ldo, const double* coef, int* err,
+                          cudaStream_t st, int upper_only) {
+  CUtensorMap mP, mQ;
+  if (TR) TK_TRY(make_slice_map(&mP, P.planes, P.K, cdiv(P.rows, OZ_KPAD) * OZ_KPAD, OT_KB, OZ_S));
+  else TK_TRY(make_slice_map(&mP, P.planes, P.rows, kp, OT_M, OZ_S));
   TK_TRY(make_slice_map(&mQ, Qs, M, kp, NT, planesQ));
   const size_t smem = sizeof(OtSmem<S, NT>) + 1024;
-  TK_CUDA(cudaFuncSetAttribute(k_oz_tc<S, MODE, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const dim3 grid((unsigned)cdiv(rows, OT_M), (unsigned)cdiv(M, NT), (unsigned)sp);
-  k_oz_tc<S, MODE, NT><<<grid, 256, smem, st>>>(mP, mQ, EP, EQ, rows, M, kp, kps, b, out, ldo, coef, upper_only, err);
+  TK_CUDA(cudaFuncSetAttribute(k_oz_tc<S, MODE, NT, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const dim3 grid((unsigned)cdiv(P.rows, OT_M), (unsigned)cdiv(M, NT), (unsigned)sp);
+  k_oz_tc<S, MODE, NT, TR>
+      <<<grid, 256, smem, st>>>(mP, mQ, P.E, EQ, P.rows, M, kp, kps, b, out, ldo, coef, upper_only, err);
   TK_LAUNCH_CHECK();
   return TK_OK;
 }
 
-template <int S, int MODE>
-tk_status launch_oz_tc(const void* Ps, const int* EP, int64_t rows, int planesP, const void* Qs, const int* EQ, int M,
-                       int planesQ, int64_t K, int splits, const double* b, void* out, int64_t ldo,
-                       const double* coef, int* err, cudaStream_t st, int upper_only = 0) {
-  const int64_t kp = cdiv(K, OZ_KPAD) * OZ_KPAD;
-  if (rows > INT32_MAX || kp > INT32_MAX || M > 65535 * OT_N) {
+template <int S, int MODE, bool TR>
+tk_status launch_oz_tc(const OtBig& P, const void* Qs, const int* EQ, int M, int planesQ, int splits, const double* b,
+                       void* out, int64_t ldo, const double* coef, int* err, cudaStream_t st, int upper_only = 0) {
+  const int64_t K = P.K, kp = cdiv(K, OZ_KPAD) * OZ_KPAD;
+  if (P.rows > INT32_MAX - 2 * OT_M || kp > INT32_MAX || M > 65535 * OT_N) {
     set_error_msg("emulated product: dimensions exceed the 32-bit TMA coordinates");
     return TK_EINVAL;
   }
-  CUtensorMap mP;
-  TK_TRY(make_slice_map(&mP, Ps, rows, kp, OT_M, planesP));
   const int64_t kps = cdiv(cdiv(K, splits), OT_CHUNK) * OT_CHUNK;  // whole chunks per split
   const int sp = (int)cdiv(K, kps);
   if (S == OZ_S && kps > OT_MAX_KPS) {  // the exact int64 level accumulators of a split
@@ -582,11 +732,11 @@ tk_status launch_oz_tc(const void* Ps, const int* EP, int64_t rows, int planesP,
   }
   if (oz_tile_n(S, M) == 64) {
     if constexpr (S != OZ_S)
-      TK_TRY((launch_oz_tc_nt<S, MODE, 64>(mP, Qs, EP, rows, EQ, M, planesQ, kp, kps, sp, b, out, ldo, coef, err, st,
-                                           upper_only)));
+      TK_TRY((launch_oz_tc_nt<S, MODE, 64, TR>(P, Qs, EQ, M, planesQ, kp, kps, sp, b, out, ldo, coef, err, st,
+                                               upper_only)));
   } else {
-    TK_TRY((launch_oz_tc_nt<S, MODE, 32>(mP, Qs, EP, rows, EQ, M, planesQ, kp, kps, sp, b, out, ldo, coef, err, st,
-                                         upper_only)));
+    TK_TRY((launch_oz_tc_nt<S, MODE, 32, TR>(P, Qs, EQ, M, planesQ, kp, kps, sp, b, out, ldo, coef, err, st,
+                                             upper_only)));
   }
   if (MODE == 1 && sp < splits) {  // the caller sums `splits` planes: the unused ones are zero
     double* o = static_cast<double*>(out);
@@ -831,7 +981,7 @@ __global__ void __launch_bounds__(384, 1)
             if (jg + j < w && jg + j >= i) {
               const int ej = S.ecol[t * CS_N + half * 2 * G + gi * G + j];
               const int e = ei + ej;
-              if (ei >= OZ_EBAD || ej >= OZ_EBAD) {  // a row or column marked non-finite: NaN (its digits are zero)
+              if (oz_bad(ei) || oz_bad(ej)) {  // a row or column marked non-finite: NaN (its digits are zero)
                 Trow[jg + j] = __longlong_as_double(0x7ff8000000000000ll);
                 continue;
               }
@@ -991,17 +1141,6 @@ __device__ __forceinline__ void cluster_sync_all() {
 __device__ __forceinline__ uint32_t sw128_off(int row, int k) {
   return (uint32_t)(row * 128 + ((((k >> 3) ^ (row & 7)) & 7) << 4) + ((k & 7) << 1));
 }
-// MN-major 128-byte-swizzled operand: LBO = distance between 64-element blocks along M, SBO = between
-// 8-row blocks along K
-__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr, uint32_t lbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((1024u >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
 // 2^e as a float (0 below the normal range, inf above)
 __device__ __forceinline__ float pow2f(int e) {
   return e < -126 ? 0.f : (e > 127 ? __int_as_float(0x7f800000) : __int_as_float((127 + e) << 23));
@@ -1023,8 +1162,8 @@ __device__ __forceinline__ void oz_split4(float x, int E, unsigned short (&bits)
 
 __global__ void __launch_bounds__(256, 1)
     k_oz_fused(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
-               const int* __restrict__ EA, const int* __restrict__ EW, int64_t m, int64_t n, int count, int cpc,
-               float* __restrict__ U, int64_t ldu, const double* __restrict__ coef, double* __restrict__ partial,
+               const int* __restrict__ EA, const int* __restrict__ EC, const int* __restrict__ EW, int64_t m,
+               int64_t n, int count, int cpc, float* __restrict__ U, int64_t ldu, const double* __restrict__ coef, double* __restrict__ partial,
                int* __restrict__ err) {
   extern __shared__ __align__(1024) uint8_t fu_raw[];
   FuSmem& S = *reinterpret_cast<FuSmem*>((reinterpret_cast<uintptr_t>(fu_raw) + 1023) & ~uintptr_t(1023));
@@ -1224,7 +1363,7 @@ __global__ void __launch_bounds__(256, 1)
         ea_next = i + 1 < nb && rn < m ? EA[rn] : 0;
       }
       S.ea[e] = ea_e;
-      const int wm = __reduce_max_sync(0xffffffffu, (r0 + e < m && ea_e < OZ_EBAD) ? ea_e : INT_MIN);
+      const int wm = __reduce_max_sync(0xffffffffu, (r0 + e < m && !oz_bad(ea_e)) ? ea_e : INT_MIN);
       if (lane == 0) S.emax4[ew] = wm;
       epi_sync();
       int eamax = max(max(S.emax4[0], S.emax4[1]), max(S.emax4[2], S.emax4[3]));
@@ -1295,13 +1434,13 @@ __global__ void __launch_bounds__(256, 1)
           if (grow < m && l < count) {
             const int er = S.ea[row + k], eq = S.ew[l];
             const int es = er + eq;
-            const double val = (er >= OZ_EBAD || eq >= OZ_EBAD) ? __longlong_as_double(0x7ff8000000000000ll)
+            const double val = (oz_bad(er) || oz_bad(eq)) ? __longlong_as_double(0x7ff8000000000000ll)
                                : (es >= -1022 && es <= 1023) ? (double)sv[k] * pow2d(es)
                                                              : ldexp((double)sv[k], es);
             float* u = U + (int64_t)l * ldu + grow;
             const float un = coef ? (float)(val + coef[l] * (double)*u) : (float)val;
             *u = un;
-            up[k] = er >= OZ_EBAD ? un : un * pow2f(er - eamax);
+            up[k] = oz_bad(er) ? un : un * pow2f(er - eamax);
           }
         }
         const float4 u4 = make_float4(up[0], up[1], up[2], up[3]);
@@ -1333,7 +1472,7 @@ __global__ void __launch_bounds__(256, 1)
         const uint32_t mx = max(max(S.umax[0][e], S.umax[1][e]), max(S.umax[2][e], S.umax[3][e]));
         const int eu = mx >= 0x7f800000u ? OZ_EBAD : oz_exponent((double)__uint_as_float(mx));
         S.eu[e] = eu;
-        S.psc[e] = eu >= OZ_EBAD ? __int_as_float(0x7fc00000) : pow2f(eamax + eu);
+        S.psc[e] = oz_bad(eu) ? __int_as_float(0x7fc00000) : pow2f(eamax + eu);
       }
       epi_sync();
       {
@@ -1342,7 +1481,7 @@ __global__ void __launch_bounds__(256, 1)
         for (int l = 0; l < FU_NT; ++l) {
           const int eu = S.eu[l];
           unsigned short bits[FU_S];
-          oz_split4(eu >= OZ_EBAD ? 0.f : S.ub[l * FU_M + e], eu >= OZ_EBAD ? 0 : eu, bits);
+          oz_split4(oz_bad(eu) ? 0.f : S.ub[l * FU_M + e], oz_bad(eu) ? 0 : eu, bits);
 #pragma unroll
           for (int p = 0; p < FU_S; ++p)
             *reinterpret_cast<unsigned short*>(base + p * FU_QBOX + sw128_off(l, e & 63)) = bits[p];
@@ -1365,9 +1504,12 @@ __global__ void __launch_bounds__(256, 1)
         if (c >= nch) break;
         const int64_t col = col0 + 128 * c + e;
         if (col < n) {
+          const int ec = EC[col];  // the column's scale in the digits of A
 #pragma unroll
           for (int l = 0; l < FU_NT; ++l)
-            if (l < count) partial[((int64_t)zc * count + l) * n + col] = (double)gacc[c][l];
+            if (l < count)
+              partial[((int64_t)zc * count + l) * n + col] =
+                  oz_bad(ec) ? __longlong_as_double(0x7ff8000000000000ll) : ldexp((double)gacc[c][l], ec);
         }
       }
     }
@@ -1387,74 +1529,99 @@ size_t oz_slices_bytes(int64_t rows, int64_t cols, int planes) {
   return sizeof(__nv_bfloat16) * (size_t)planes * (size_t)rows * (size_t)(cdiv(cols, OZ_KPAD) * OZ_KPAD);
 }
 
-tk_status oz_prepare(const void* X, tk_dtype dt, int64_t rows, int64_t cols, int64_t ld, void* slices, int* E,
-                     cudaStream_t st, int planes) {
-  if (rows == 0 || cols == 0) return TK_OK;
-  const int64_t kp = cdiv(cols, OZ_KPAD) * OZ_KPAD;
+tk_status oz_split_vectors(const void* V, tk_dtype dt, int64_t M, int64_t K, int64_t ld, const int* shift,
+                           void* slices, int* E, cudaStream_t st, int planes) {
+  if (M == 0 || K == 0) return TK_OK;
+  const int64_t kp = cdiv(K, OZ_KPAD) * OZ_KPAD;
   const bool f64 = dt == TK_F64;
-  if (cols >= 16384 && rows <= 65535) {
-    // few long rows (the residuals of the normal-equation pass): blocks of 8192 values per row
-    const int64_t per = 8192;
-    k_oz_fill_emin<<<(unsigned)cdiv(rows, 256), 256, 0, st>>>(E, rows);
-    TK_LAUNCH_CHECK();
-    const dim3 g((unsigned)cdiv(cols, per), (unsigned)rows);
-    if (f64) k_oz_rowexp_long<double><<<g, 256, 0, st>>>((const double*)X, cols, ld, per, E);
-    else k_oz_rowexp_long<float><<<g, 256, 0, st>>>((const float*)X, cols, ld, per, E);
-    TK_LAUNCH_CHECK();
-    k_oz_fix_zero_rows<<<(unsigned)cdiv(rows, 256), 256, 0, st>>>(E, rows);
-  } else {
-    const unsigned gr = (unsigned)cdiv(rows, 8);
-    if (f64) k_oz_rowexp<double><<<gr, 256, 0, st>>>((const double*)X, rows, cols, ld, E);
-    else k_oz_rowexp<float><<<gr, 256, 0, st>>>((const float*)X, rows, cols, ld, E);
-  }
-  TK_LAUNCH_CHECK();
-  const int64_t chunks = cdiv(kp, 512);  // 256 threads x 2 values
-  if (chunks > 65535) {
-    set_error_msg("emulated float64 product: rows too long for the slicing grid");
+  __nv_bfloat16* out = static_cast<__nv_bfloat16*>(slices);
+  if (M > 65535) {
+    set_error_msg("emulated float64 product: too many rows of the small operand");
     return TK_EINVAL;
   }
-  const dim3 gs((unsigned)std::min<int64_t>(rows, std::max<int64_t>(1, 152 * 16 / chunks)), (unsigned)chunks);
-  __nv_bfloat16* out = static_cast<__nv_bfloat16*>(slices);
-  if (f64) k_oz_slice<double><<<gs, 256, 0, st>>>((const double*)X, rows, cols, ld, E, kp, planes, out);
-  else k_oz_slice<float><<<gs, 256, 0, st>>>((const float*)X, rows, cols, ld, E, kp, planes, out);
+  if (K < OZ_VEC_LONG) {
+    if (f64) k_oz_vec<double><<<(unsigned)M, 512, 0, st>>>((const double*)V, M, K, ld, shift, E, kp, planes, out);
+    else k_oz_vec<float><<<(unsigned)M, 512, 0, st>>>((const float*)V, M, K, ld, shift, E, kp, planes, out);
+    TK_LAUNCH_CHECK();
+    return TK_OK;
+  }
+  // blocks of 2048 values or more, about 8 blocks per SM in all
+  const int64_t per = std::max<int64_t>(2048, cdiv(cdiv(K * M, 8 * 152), 256) * 256);
+  TK_CUDA(cudaMemsetAsync(E, 0x80, sizeof(int) * (size_t)M, st));  // OZ_EZERO
+  const dim3 g((unsigned)cdiv(K, per), (unsigned)M), gs((unsigned)cdiv(kp, 512), (unsigned)M);
+  if (f64) k_oz_vec_exp<double><<<g, 256, 0, st>>>((const double*)V, K, ld, shift, per, E);
+  else k_oz_vec_exp<float><<<g, 256, 0, st>>>((const float*)V, K, ld, shift, per, E);
+  TK_LAUNCH_CHECK();
+  if (f64) k_oz_vec_slice<double><<<gs, 256, 0, st>>>((const double*)V, M, K, ld, shift, E, kp, planes, out);
+  else k_oz_vec_slice<float><<<gs, 256, 0, st>>>((const float*)V, M, K, ld, shift, E, kp, planes, out);
   TK_LAUNCH_CHECK();
   return TK_OK;
 }
 
 size_t oz_colmax_bytes(int64_t cols) { return sizeof(unsigned long long) * (size_t)std::max<int64_t>(cols, 1); }
 
-tk_status oz_prepare_cols(const void* X, tk_dtype dt, int64_t rows, int64_t cols, int64_t ld, void* slices, int* E,
-                          void* colmax, cudaStream_t st) {
-  if (rows == 0 || cols == 0) return TK_OK;
-  const int64_t rp = cdiv(rows, OZ_KPAD) * OZ_KPAD;
+// Column exponents EC of X (and, with copy, its float32 copy): one pass over X.
+static tk_status oz_column_exponents(const void* X, tk_dtype dt, int64_t rows, int64_t cols, int64_t ld, int* EC,
+                                     void* colmax, float* copy, cudaStream_t st) {
   unsigned long long* mx = static_cast<unsigned long long*>(colmax);
   TK_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * (size_t)cols, st));
-  // about 4 CTAs of 256 columns per SM, each over a band of rows
+  // about 8 CTAs of 256 columns per SM, each over a band of rows
   const int64_t cb = cdiv(cols, 256);
-  const int64_t bands = std::max<int64_t>(1, std::min<int64_t>(cdiv(4 * 152, cb), cdiv(rows, 64)));
+  const int64_t bands = std::max<int64_t>(1, std::min<int64_t>({cdiv(8 * 152, cb), cdiv(rows, 32), 65535}));
   const int64_t rows_per = cdiv(rows, bands);
   const dim3 gm((unsigned)cb, (unsigned)cdiv(rows, rows_per));
-  if (cdiv(cols, 32) > 65535) {
-    set_error_msg("emulated float64 product: too many columns for the slicing grid");
-    return TK_EINVAL;
-  }
-  const dim3 gt((unsigned)cdiv(rp, 64), (unsigned)cdiv(cols, 32));
-  __nv_bfloat16* out = static_cast<__nv_bfloat16*>(slices);
-  if (dt == TK_F64) k_oz_colmax<double><<<gm, 256, 0, st>>>((const double*)X, rows, cols, ld, rows_per, mx);
-  else k_oz_colmax<float><<<gm, 256, 0, st>>>((const float*)X, rows, cols, ld, rows_per, mx);
+  if (dt == TK_F64) k_oz_colmax<double><<<gm, 256, 0, st>>>((const double*)X, rows, cols, ld, rows_per, mx, copy);
+  else k_oz_colmax<float><<<gm, 256, 0, st>>>((const float*)X, rows, cols, ld, rows_per, mx, copy);
   TK_LAUNCH_CHECK();
-  k_oz_colexp<<<(unsigned)cb, 256, 0, st>>>(mx, cols, E);
-  TK_LAUNCH_CHECK();
-  if (dt == TK_F64) k_oz_slice_t<double><<<gt, dim3(32, 8), 0, st>>>((const double*)X, rows, cols, ld, E, rp, out);
-  else k_oz_slice_t<float><<<gt, dim3(32, 8), 0, st>>>((const float*)X, rows, cols, ld, E, rp, out);
+  k_oz_colexp<<<(unsigned)cb, 256, 0, st>>>(mx, cols, EC);
   TK_LAUNCH_CHECK();
   return TK_OK;
 }
 
-tk_status oz_residual(const void* Aslices, const int* EA, int64_t m, int64_t n, const void* Xslices, const int* EX,
-                      int64_t M, const double* b, double* R, int64_t ldr, int* err, cudaStream_t st) {
-  if (m == 0 || M == 0) return TK_OK;
-  return launch_oz_tc<OZ_S, 0>(Aslices, EA, m, OZ_S, Xslices, EX, (int)M, OZ_S, n, 1, b, R, ldr, nullptr, err, st);
+tk_status oz_split_matrix(const void* A, tk_dtype dt, int64_t rows, int64_t cols, int64_t ld, void* slices, int* ER,
+                          int* EC, void* colmax, float* copy, cudaStream_t st) {
+  if (rows == 0 || cols == 0) return TK_OK;
+  TK_TRY(oz_column_exponents(A, dt, rows, cols, ld, EC, colmax, copy, st));
+  const int64_t cp = cdiv(cols, OZ_KPAD) * OZ_KPAD;
+  const size_t es = dt == TK_F64 ? 8 : 4;
+  // about 5 blocks per SM are resident: keep their bands within half of the 129 MB L2
+  int RB = 8;
+  while (RB > 1 && (size_t)RB * cols * es * 5 * 152 > (size_t)64 << 20) RB /= 2;
+  const int64_t nb = cdiv(rows, RB);
+  if (nb > INT32_MAX) {
+    set_error_msg("emulated float64 product: too many rows for the slicing grid");
+    return TK_EINVAL;
+  }
+  __nv_bfloat16* out = static_cast<__nv_bfloat16*>(slices);
+  if (dt == TK_F64)
+    k_oz_scale_slice<double><<<(unsigned)nb, 256, 0, st>>>((const double*)A, rows, cols, ld, EC, RB, cp, ER, out);
+  else
+    k_oz_scale_slice<float><<<(unsigned)nb, 256, 0, st>>>((const float*)A, rows, cols, ld, EC, RB, cp, ER, out);
+  TK_LAUNCH_CHECK();
+  return TK_OK;
+}
+
+// Column-exponent digits of X stored transposed (the Gram matrix of the sketch): planes of X^T.
+static tk_status oz_split_columns(const double* X, int64_t rows, int64_t cols, void* slices, int* E, void* colmax,
+                                  cudaStream_t st) {
+  const int64_t rp = cdiv(rows, OZ_KPAD) * OZ_KPAD;
+  if (cdiv(cols, 32) > 65535) {
+    set_error_msg("emulated float64 product: too many columns for the slicing grid");
+    return TK_EINVAL;
+  }
+  TK_TRY(oz_column_exponents(X, TK_F64, rows, cols, cols, E, colmax, nullptr, st));
+  const dim3 gt((unsigned)cdiv(rp, 64), (unsigned)cdiv(cols, 32));
+  k_oz_slice_t<double><<<gt, dim3(32, 8), 0, st>>>(X, rows, cols, cols, E, rp, static_cast<__nv_bfloat16*>(slices));
+  TK_LAUNCH_CHECK();
+  return TK_OK;
+}
+
+tk_status oz_residual(const OzMat& A, const double* X, int64_t ldx, int64_t M, void* Xslices, int* EX,
+                      const double* b, double* R, int64_t ldr, int* err, cudaStream_t st) {
+  if (A.m == 0 || M == 0) return TK_OK;
+  TK_TRY(oz_split_vectors(X, TK_F64, M, A.n, ldx, A.EC, Xslices, EX, st));
+  return launch_oz_tc<OZ_S, 0, false>({A.planes, A.ER, A.m, A.n, false}, Xslices, EX, (int)M, OZ_S, 1, b, R, ldr,
+                                      nullptr, err, st);
 }
 
 // Split count of a split-K digit product with `tiles` output tiles: the fewest
@@ -1482,29 +1649,53 @@ int oz_normal_splits(int64_t m, int64_t n, int64_t M, int S) {
   return (int)std::max<int64_t>({int64_t(1), best, cdiv(m, OT_MAX_KPS)});  // at most 2^27 values of K per split
 }
 
-tk_status oz_normal(const void* AslicesT, const int* EC, int64_t m, int64_t n, const double* R, int64_t ldr,
-                    int64_t M, void* Rslices, int* EX, double* partial, int splits, int* err, cudaStream_t st) {
-  if (M == 0 || n == 0) return TK_OK;
-  TK_TRY(oz_prepare(R, TK_F64, M, m, ldr, Rslices, EX, st));
-  return launch_oz_tc<OZ_S, 1>(AslicesT, EC, n, OZ_S, Rslices, EX, (int)M, OZ_S, m, splits, nullptr, partial, n,
-                               nullptr, err, st);
+tk_status oz_normal(const OzMat& A, const double* R, int64_t ldr, int64_t M, void* Rslices, int* EX, double* partial,
+                    int splits, int* err, cudaStream_t st) {
+  if (M == 0 || A.n == 0) return TK_OK;
+  TK_TRY(oz_split_vectors(R, TK_F64, M, A.m, ldr, A.ER, Rslices, EX, st));
+  return launch_oz_tc<OZ_S, 1, true>({A.planes, A.EC, A.n, A.m, true}, Rslices, EX, (int)M, OZ_S, splits, nullptr,
+                                     partial, A.n, nullptr, err, st);
 }
 
-tk_status oz_lsqr_aw(const void* Aslices, const int* EA, int64_t m, int64_t n, const float* W, int64_t ldw, int count,
-                     void* Wslices, int* EW, float* U, int64_t ldu, const double* coef, int* err, cudaStream_t st) {
-  if (m == 0 || count == 0) return TK_OK;
-  TK_TRY(oz_prepare(W, TK_F32, count, n, ldw, Wslices, EW, st, OZ_LSQR_DIGITS));
-  return launch_oz_tc<OZ_LSQR_DIGITS, 2>(Aslices, EA, m, OZ_S, Wslices, EW, count, OZ_LSQR_DIGITS, n, 1, nullptr, U,
-                                         ldu, coef, err, st);
+template <typename T>
+tk_status oz_lsqr_aw(const OzMat& A, const T* W, int64_t ldw, int count, void* Wslices, int* EW, T* U, int64_t ldu,
+                     const double* coef, int* err, cudaStream_t st) {
+  if (A.m == 0 || count == 0) return TK_OK;
+  constexpr int S = oz_digits<T>();
+  TK_TRY(oz_split_vectors(W, sizeof(T) == 8 ? TK_F64 : TK_F32, count, A.n, ldw, A.EC, Wslices, EW, st, S));
+  return launch_oz_tc<S, 2, false>({A.planes, A.ER, A.m, A.n, false}, Wslices, EW, count, S, 1, nullptr, U, ldu, coef,
+                                   err, st);
 }
 
-tk_status oz_lsqr_atu(const void* AslicesT, const int* EC, int64_t m, int64_t n, const float* U, int64_t ldu,
-                      int count, void* Uslices, int* EU, double* partial, int splits, int* err, cudaStream_t st) {
-  if (n == 0 || count == 0) return TK_OK;
-  TK_TRY(oz_prepare(U, TK_F32, count, m, ldu, Uslices, EU, st, OZ_LSQR_DIGITS));
-  return launch_oz_tc<OZ_LSQR_DIGITS, 1>(AslicesT, EC, n, OZ_S, Uslices, EU, count, OZ_LSQR_DIGITS, m, splits,
-                                         nullptr, partial, n, nullptr, err, st);
+template <typename T>
+tk_status oz_lsqr_aw_split(const OzMat& A, const T* W, int64_t ldw, int count, void* Wslices, int* EW, double* partial,
+                           int splits, int* err, cudaStream_t st) {
+  if (A.m == 0 || count == 0) return TK_OK;
+  constexpr int S = oz_digits<T>();
+  TK_TRY(oz_split_vectors(W, sizeof(T) == 8 ? TK_F64 : TK_F32, count, A.n, ldw, A.EC, Wslices, EW, st, S));
+  return launch_oz_tc<S, 1, false>({A.planes, A.ER, A.m, A.n, false}, Wslices, EW, count, S, splits, nullptr, partial,
+                                   A.m, nullptr, err, st);
 }
+
+template <typename T>
+tk_status oz_lsqr_atu(const OzMat& A, const T* U, int64_t ldu, int count, void* Uslices, int* EU, double* partial,
+                      int splits, int* err, cudaStream_t st) {
+  if (A.n == 0 || count == 0) return TK_OK;
+  constexpr int S = oz_digits<T>();
+  TK_TRY(oz_split_vectors(U, sizeof(T) == 8 ? TK_F64 : TK_F32, count, A.m, ldu, A.ER, Uslices, EU, st, S));
+  return launch_oz_tc<S, 1, true>({A.planes, A.EC, A.n, A.m, true}, Uslices, EU, count, S, splits, nullptr, partial,
+                                  A.n, nullptr, err, st);
+}
+template tk_status oz_lsqr_aw<float>(const OzMat&, const float*, int64_t, int, void*, int*, float*, int64_t,
+                                     const double*, int*, cudaStream_t);
+template tk_status oz_lsqr_aw<double>(const OzMat&, const double*, int64_t, int, void*, int*, double*, int64_t,
+                                      const double*, int*, cudaStream_t);
+template tk_status oz_lsqr_aw_split<double>(const OzMat&, const double*, int64_t, int, void*, int*, double*, int,
+                                            int*, cudaStream_t);
+template tk_status oz_lsqr_atu<float>(const OzMat&, const float*, int64_t, int, void*, int*, double*, int, int*,
+                                      cudaStream_t);
+template tk_status oz_lsqr_atu<double>(const OzMat&, const double*, int64_t, int, void*, int*, double*, int, int*,
+                                       cudaStream_t);
 
 // Cluster shape of the fused step for n columns: CL CTAs (a power of two, at most 8, so that each
 // CTA's share of a band's 128 rows is a multiple of 4) of cpc columns (a multiple of 128, at most
@@ -1525,9 +1716,10 @@ bool oz_fused_supported(int64_t m, int64_t n, int count) {
   return cl > 0 && count >= 1 && count <= FU_NT && m >= 1 && m <= INT32_MAX;
 }
 
-tk_status oz_lsqr_fused(const void* Aslices, const int* EA, int64_t m, int64_t n, const float* W, int64_t ldw,
-                        int count, void* Wslices, int* EW, float* U, int64_t ldu, const double* coef, double* partial,
-                        int max_planes, int* planes, int* err, cudaStream_t st) {
+tk_status oz_lsqr_fused(const OzMat& A, const float* W, int64_t ldw, int count, void* Wslices, int* EW, float* U,
+                        int64_t ldu, const double* coef, double* partial, int max_planes, int* planes, int* err,
+                        cudaStream_t st) {
+  const int64_t m = A.m, n = A.n;
   int CL = 0, cpc = 0;
   fused_shape(n, &CL, &cpc);
   if (!oz_fused_supported(m, n, count) || max_planes < 1) {
@@ -1535,9 +1727,9 @@ tk_status oz_lsqr_fused(const void* Aslices, const int* EA, int64_t m, int64_t n
     return TK_EINVAL;
   }
   const int64_t n64 = cdiv(n, OZ_KPAD) * OZ_KPAD;
-  TK_TRY(oz_prepare(W, TK_F32, count, n, ldw, Wslices, EW, st, OZ_LSQR_DIGITS));
+  TK_TRY(oz_split_vectors(W, TK_F32, count, n, ldw, A.EC, Wslices, EW, st, OZ_LSQR_DIGITS));
   CUtensorMap mA, mW;
-  TK_TRY(make_slice_map(&mA, Aslices, m, n64, OT_M, OZ_S));
+  TK_TRY(make_slice_map(&mA, A.planes, m, n64, OT_M, OZ_S));
   TK_TRY(make_slice_map(&mW, Wslices, count, n64, FU_NT, OZ_LSQR_DIGITS));
   const size_t smem = sizeof(FuSmem) + 1024;
   TK_CUDA(cudaFuncSetAttribute(k_oz_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1563,7 +1755,7 @@ tk_status oz_lsqr_fused(const void* Aslices, const int* EA, int64_t m, int64_t n
   const int64_t bands = cdiv(m, FU_M);
   const int ncl = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)cached[CL], bands, (int64_t)max_planes}));
   cfg.gridDim = dim3((unsigned)(ncl * CL), 1, 1);
-  TK_CUDA(cudaLaunchKernelEx(&cfg, k_oz_fused, mA, mW, EA, (const int*)EW, m, n, count, cpc, U, ldu, coef, partial,
+  TK_CUDA(cudaLaunchKernelEx(&cfg, k_oz_fused, mA, mW, A.ER, A.EC, (const int*)EW, m, n, count, cpc, U, ldu, coef, partial,
                              err));
   TK_LAUNCH_CHECK();
   *planes = ncl;
@@ -1592,8 +1784,9 @@ tk_status oz_gram(const double* Y, int64_t r, int64_t c, double* C, void* work, 
   int* E = a.take<int>(c);
   void* mx = a.take<char>(oz_colmax_bytes(c));
   if (!a.ok()) return TK_ENOMEM;
-  TK_TRY(oz_prepare_cols(Y, TK_F64, r, c, c, Ys, E, mx, st));
-  return launch_oz_tc<OZ_S, 1>(Ys, E, c, OZ_S, Ys, E, (int)c, OZ_S, r, 1, nullptr, C, c, nullptr, err, st, 1);
+  TK_TRY(oz_split_columns(Y, r, c, Ys, E, mx, st));
+  return launch_oz_tc<OZ_S, 1, false>({Ys, E, c, r, false}, Ys, E, (int)c, OZ_S, 1, nullptr, C, c, nullptr, err, st,
+                                      1);
 }
 
 size_t oz_chol_workspace(int64_t np, int N) {

@@ -1,0 +1,70 @@
+"""The float64 form's products with A from exact digits on the tensor cores (emulate_fp64 = 1): the
+same solutions as on the float64 pipe (emulate_fp64 = 0), whatever the shape and the scales of A."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2203_07329_gb300 import datagen, tikhonov as tk
+
+pytestmark = pytest.mark.gpu
+
+
+def _solve(A, b, lams, **kw):
+    return tk.tk_solve(A, b, lams, tk.opts_default(**kw))
+
+
+# A at and around the smallest size that is split into digits (2^19 elements), ragged against the 64-,
+# 128- and 256-value tiles, one and several tiles of 32 lambdas, float64 views with odd row strides,
+# and m < n.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
+@pytest.mark.parametrize("m,n,N,pad", [(8192, 64, 2, 0), (8193, 65, 3, 1), (2051, 257, 33, 0), (1500, 700, 5, 3),
+                                       (16500, 40, 4, 0), (129, 4099, 4, 0), (500, 1100, 34, 5), (63, 8400, 2, 0)])
+def test_digit_solve_matches_float64_pipe(m, n, N, pad):
+    k = min(m, n)
+    p = datagen.make_ridge_problem(m, n, datagen.spectrum("log", k, hi=1.0, lo=1e-3),
+                                   datagen.log_lambdas(N, 1e-6, 1e-1), seed=m + n)
+    full = torch.full((m, n + pad), float("nan"), dtype=torch.float64, device="cuda")
+    full[:, :n] = p.A.cuda()
+    A, b, lams = full[:, :n], p.b.cuda(), p.lambdas.numpy()
+    s = min(4 * k, max(m, n))
+    r1 = _solve(A, b, lams, sketch=tk.TK_SKETCH_SRHT, s=s)
+    r0 = _solve(A, b, lams, sketch=tk.TK_SKETCH_SRHT, s=s, emulate_fp64=0)
+    for i in range(N):
+        e = float((r1.X[i] - r0.X[i]).norm() / r0.X[i].norm())
+        assert e < 1e-10, (lams[i], e)
+        assert r1.info[i]["status"] == 0
+        assert abs(r1.info[i]["iters"] - r0.info[i]["iters"]) <= 2
+
+
+# rows and columns of A in very different units: the digits follow both, so every entry of the two
+# products keeps the accuracy of a float64 sum of its own terms (K terms, each relative to the
+# product of the scaled maxima: 8 2^-53 sqrt(K) of sum |a||x| as for the other digit products)
+@pytest.mark.parametrize("rows,cols", [(0, 12), (12, 0), (9, 9)])
+def test_digit_products_follow_row_and_column_scales(rows, cols):
+    gen = torch.Generator().manual_seed(3)
+    m, n, M = 3001, 390, 5
+    A = torch.randn(m, n, generator=gen, dtype=torch.float64)
+    A *= torch.pow(10.0, -rows * torch.rand(m, 1, generator=gen, dtype=torch.float64))
+    A *= torch.pow(10.0, -cols * torch.rand(1, n, generator=gen, dtype=torch.float64))
+    # x in the units of the columns, b in those of the rows, as the solution of a fit has them
+    X = torch.randn(M, n, generator=gen, dtype=torch.float64) / A.abs().amax(0)
+    b = torch.zeros(m, dtype=torch.float64)
+    R, G = tk.tk_residual(A.cuda(), b.cuda(), X.cuda(), True, with_g=True)
+    R, G, Ah, Xh = R.cpu().numpy(), G.cpu().numpy(), A.numpy(), X.numpy()
+    Rref = -(Xh.astype(np.longdouble) @ Ah.T.astype(np.longdouble))
+    err = np.max(np.abs((R - Rref).astype(np.float64)) / (np.abs(Xh) @ np.abs(Ah).T))
+    assert err < 8 * 2.0 ** -53 * math.sqrt(n), err
+    Gref = R.astype(np.longdouble) @ Ah.astype(np.longdouble)
+    err = np.max(np.abs((G - Gref).astype(np.float64)) / (np.abs(R) @ np.abs(Ah)))
+    assert err < 8 * 2.0 ** -53 * math.sqrt(m), err
+
+
+def test_non_finite_a_is_enumeric_from_digits():
+    gen = torch.Generator().manual_seed(5)
+    A = torch.randn(9000, 70, generator=gen, dtype=torch.float64)
+    b = torch.randn(9000, generator=gen, dtype=torch.float64).cuda()
+    A[4001, 3] = float("nan")
+    r = tk.tk_solve(A.cuda(), b, [1e-2, 1.0], tk.opts_default(sketch=tk.TK_SKETCH_SRHT, s=280),
+                    allow=tuple(range(8)))
+    assert r.status == tk.TK_ENUMERIC
