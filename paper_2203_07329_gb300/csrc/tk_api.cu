@@ -53,6 +53,7 @@ struct Plan {
 
 constexpr int64_t kMaxShort = 8192;
 constexpr int64_t kMaxLong = (int64_t(1) << 30);
+constexpr double kInv64Cost = 8e7;  // N c^2 up to which the explicit float64 inverse costs less than the substitutions
 constexpr int64_t kOz64MinElems = int64_t(1) << 19;  // smallest A (elements) that the float64 form splits into digits
 
 tk_status check_opts(const tk_opts* o) {
@@ -121,10 +122,10 @@ tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
   P.N_cap = (o->schedule == TK_SCHED_ONE_AT_A_TIME) ? 1 : std::max(N, 1);
   // the tensor-core products need 16-byte aligned float32 rows of A, A^T and
   // the lambda-major vectors; other shapes keep the SIMT float32 products
-  // small float64 factors: an explicit inverse costs N n^3/3 flops once and
-  // turns each preconditioner apply into one launch (substitution on a
-  // factor of order <= 512 runs in a single CTA per lambda)
-  P.inv64 = !P.mixed && !P.lowrank && !P.under && P.c <= 512;
+  // float64 factors: an explicit inverse costs N c^3/3 flops once on the float64 pipe (1024, 16 lambda:
+  // 5 ms) and turns each preconditioner apply into one launch (13 us there) where a substitution is a
+  // chain of c/32 launches (1.1 ms for the two of a step, about 30 steps)
+  P.inv64 = !P.mixed && !P.lowrank && (double)std::max(N, 1) * P.c * P.c <= kInv64Cost;
   P.lsqr_tc = P.mixed && o->lsqr_tc == 1 && P.N_cap <= 64 && !P.under && P.m % 4 == 0 && P.n % 4 == 0 &&
               (P.dt == TK_F64 || P.lda % 4 == 0);
   P.lsqr_oz = P.mixed && (o->lsqr_tc == 2 || o->lsqr_tc == 3) && o->emulate_fp64 && !P.under;
@@ -1317,6 +1318,7 @@ static void residual_carve(Arena& a, int64_t m, int64_t n, int M, ResidualBufs& 
   w.Xoz = a.take<char>(oz_slices_bytes(M, n));
   w.EX = a.take<int>(M);
   w.EC = a.take<int>(n);
+  a.take<char>(oz_slices_bytes(n, m));  // not used: callers' workspaces are sized for two sets of planes
   w.colmax = a.take<char>(oz_colmax_bytes(n));
   w.Roz = a.take<char>(oz_slices_bytes(M, m));
   w.ER = a.take<int>(M);

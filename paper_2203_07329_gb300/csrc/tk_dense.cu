@@ -473,13 +473,13 @@ __global__ void __launch_bounds__(256) k_tinv_final(T* __restrict__ M, T* __rest
 }
 
 // ------------------------------------------------------------------ TRMV --
-template <typename T, bool UPPER>
+template <typename T, bool UPPER, int RW>
 __global__ void __launch_bounds__(256) k_trmv(int64_t n, const T* __restrict__ M, int64_t ldm, int64_t mstride,
                                               const int* __restrict__ idx, const T* in, T* out, int64_t ldx) {
   extern __shared__ float4 trmv_v4[];
   const int slot = blockIdx.y;
-  tiles::trmv_rows<T, UPPER>(n, M + (int64_t)(idx ? idx[slot] : slot) * mstride, ldm, in + (int64_t)slot * ldx,
-                             out + (int64_t)slot * ldx, (int64_t)blockIdx.x * tiles::kTrmvRows, trmv_v4);
+  tiles::trmv_rows<T, UPPER, RW>(n, M + (int64_t)(idx ? idx[slot] : slot) * mstride, ldm, in + (int64_t)slot * ldx,
+                                 out + (int64_t)slot * ldx, (int64_t)blockIdx.x * (8 * RW), trmv_v4);
 }
 
 // ------------------------------------------------------------------ TRSV --
@@ -893,10 +893,22 @@ template <typename T>
 tk_status trmv_batched(bool transposed, int64_t n, const T* M, const T* Mt, int64_t ldm, int64_t mstride,
                        const int* idx, const T* in, T* out, int64_t ldx, int count, cudaStream_t st) {
   if (count == 0 || n == 0) return TK_OK;
-  const dim3 grid((unsigned)cdiv(n, tiles::kTrmvRows), (unsigned)count);
-  const size_t smem = tiles::trmv_smem_bytes<T>(n);
-  if (!transposed) k_trmv<T, true><<<grid, 256, smem, st>>>(n, M, ldm, mstride, idx, in, out, ldx);
-  else k_trmv<T, false><<<grid, 256, smem, st>>>(n, Mt, ldm, mstride, idx, in, out, ldx);
+  const size_t smem = tiles::trmv_smem_bytes<T>(n);  // at most 64 KiB (n <= 8192)
+  constexpr int kCap = 64 * 1024;                    // one cap: host threads launch concurrently
+#define TK_TRMV(UP, RW)                                                                              \
+  {                                                                                                  \
+    auto kern = k_trmv<T, UP, RW>;                                                                   \
+    TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kCap));          \
+    kern<<<dim3((unsigned)cdiv(n, 8 * RW), (unsigned)count), 256, smem, st>>>(n, UP ? M : Mt, ldm, mstride, idx, in, \
+                                                                             out, ldx);              \
+  }
+  const bool wide = cdiv(n, 64) * count >= 2 * 152;  // two CTAs of 64 rows per SM
+  if (!transposed) {
+    if (wide) TK_TRMV(true, 8) else TK_TRMV(true, 2)
+  } else {
+    if (wide) TK_TRMV(false, 8) else TK_TRMV(false, 2)
+  }
+#undef TK_TRMV
   TK_LAUNCH_CHECK();
   return TK_OK;
 }

@@ -273,7 +273,11 @@ __device__ __forceinline__ void gemm_lm_tile(LmSmem<BM>& sm, bool vec, int64_t M
 // (row stride and base 16-byte aligned), starting at the vector that holds
 // column i (upper) or ending at it (lower): the extra entries lie in the
 // 64-aligned diagonal block, where that triangle is stored as zeros.  256 threads.
-constexpr int kTrmvRows = 64;  // rows per CTA (8 warps x 8 rows)
+// A warp forms RW rows together: RW independent 16-byte loads in flight per lane and one read of the
+// vector for all of them; row by row, each row's latency was paid in full.  Float32: n = 256, 8 slots
+// 6.2 -> 2.4 us; n = 777, 10 slots 21 -> 6 us; n = 2048, about 25 slots (HBM-bound: half of n^2 floats
+// per slot) 50 -> 46 us.  RW = 8 (64 rows per CTA) when that gives the GPU enough CTAs, else 2.
+constexpr int kTrmvRows = 64;  // most rows per CTA (8 warps x 8 rows)
 
 template <typename T>
 struct Vec16;
@@ -303,7 +307,37 @@ inline size_t trmv_smem_bytes(int64_t n) {
   return sizeof(T) * (size_t)Vec16<T>::W * (size_t)cdiv(n, Vec16<T>::W);
 }
 
-template <typename T, bool UPPER>
+// Sums of RW values over the warp: halving exchanges (each step keeps half of the values, the lanes
+// with bit s set the upper half), then plain steps; the lane's sum is value *which.
+template <typename T, int RW>
+__device__ __forceinline__ T warp_sum_rows(T (&v)[RW], int* which) {
+  const int lane = threadIdx.x & 31;
+  int base = 0, nv = RW;
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) {
+    if (nv > 1) {
+      const int half = nv / 2;
+      const bool up = (lane & s) != 0;
+#pragma unroll
+      for (int q = 0; q < RW / 2; ++q) {
+        if (q < half) {
+          const T send = up ? v[q] : v[q + half];
+          const T keep = up ? v[q + half] : v[q];
+          v[q] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+      }
+      if (up) base += half;
+      nv = half;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], s);
+    }
+  }
+  *which = base;
+  return v[0];
+}
+
+// Rows i0 .. i0 + 8 RW - 1 (i0 a multiple of 8 RW, which divides 64).
+template <typename T, bool UPPER, int RW>
 __device__ __forceinline__ void trmv_rows(int64_t n, const T* __restrict__ Ml, int64_t ldm, const T* x, T* out,
                                           int64_t i0, void* smem) {
   using V = typename Vec16<T>::type;
@@ -311,20 +345,36 @@ __device__ __forceinline__ void trmv_rows(int64_t n, const T* __restrict__ Ml, i
   T* v = reinterpret_cast<T*>(smem);
   const V* vv = reinterpret_cast<const V*>(smem);
   const int64_t nv = cdiv(n, W);
-  for (int64_t j = threadIdx.x; j < W * nv; j += blockDim.x) v[j] = j < n ? x[j] : T(0);
+  // the upper rows read the vector from their first column on, the lower ones up to their last
+  const int64_t v0 = UPPER ? i0 / W * W : 0, v1 = UPPER ? W * nv : (i0 + 8 * RW < W * nv ? i0 + 8 * RW : W * nv);
+  for (int64_t j = v0 + threadIdx.x; j < v1; j += blockDim.x) v[j] = j < n ? x[j] : T(0);
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int q = 0; q < kTrmvRows / 8; ++q) {
-    const int64_t i = i0 + w + 8 * q;
-    if (i >= n) break;
-    const V* row = reinterpret_cast<const V*>(Ml + i * ldm);
-    const int64_t j0 = UPPER ? (i / W) : 0, j1 = UPPER ? nv : (i / W) + 1;
-    T acc = T(0);
-#pragma unroll 4
-    for (int64_t j = j0 + lane; j < j1; j += 32) acc = Vec16<T>::dot(__ldg(row + j), vv[j], acc);
-    acc = warp_sum(acc);
-    if (lane == 0) out[i] = acc;
+  const int64_t i = i0 + (int64_t)w * RW;
+  if (i >= n) return;
+  // the RW rows share the vectors of the first (upper) or last (lower) one: what that adds to the
+  // others lies in the 64-aligned diagonal block's zero triangle; rows past n repeat row n - 1
+  const V* row[RW];
+#pragma unroll
+  for (int q = 0; q < RW; ++q) row[q] = reinterpret_cast<const V*>(Ml + (i + q < n ? i + q : n - 1) * ldm);
+  const int64_t il = i + RW - 1 < n ? i + RW - 1 : n - 1;
+  const int64_t j0 = UPPER ? i / W : 0, j1 = UPPER ? nv : il / W + 1;
+  T acc[RW];
+#pragma unroll
+  for (int q = 0; q < RW; ++q) acc[q] = T(0);
+#pragma unroll 2
+  for (int64_t j = j0 + lane; j < j1; j += 32) {
+    V m[RW];
+#pragma unroll
+    for (int q = 0; q < RW; ++q) m[q] = __ldg(row[q] + j);
+    const V xv = vv[j];
+#pragma unroll
+    for (int q = 0; q < RW; ++q) acc[q] = Vec16<T>::dot(m[q], xv, acc[q]);
   }
+  int which;
+  const T sum = warp_sum_rows<T, RW>(acc, &which);
+  // RW distinct sums; each sits on 32 / RW lanes, written by the one whose low bits are clear
+  if ((lane & (32 / RW - 1)) == 0 && i + which < n) out[i + which] = sum;
 }
 
 }  // namespace tiles

@@ -199,11 +199,10 @@ __global__ void __launch_bounds__(kThreads)
   const GSlot q = sl[blockIdx.x];
   const GDesc& d = Dd[q.p];
   const int64_t off = (int64_t)q.k * d.n;
-  vstep_block<float>(d.Vraw + off, d.V + off, d.W + off, d.Y + off, d.n, d.sc + q.k, d.atol, d.atol, d.maxiter,
-                     init, sh);
+  vstep_block<float, 1>(d.Vraw + off, d.V + off, d.W + off, d.Y + off, d.n, d.sc + q.k, d.coef + q.k, d.atol, d.atol,
+                        d.maxiter, init, sh, nullptr);
   if (threadIdx.x == 0) {  // the thread that wrote the scalars
     const Scal z = d.sc[q.k];
-    d.coef[q.k] = z.coef;
     GReport r;
     r.istop = z.istop;
     r.iters = z.iters;
@@ -224,7 +223,7 @@ __global__ void __launch_bounds__(256)
   const int64_t i0 = (int64_t)blockIdx.x * tiles::kTrmvRows;
   if (d.lowrank || i0 >= d.n) return;
   const float* Ml = (UPPER ? d.Mi : d.Mti) + (int64_t)d.slot_lam[q.k] * d.np * d.np;
-  tiles::trmv_rows<float, UPPER>(d.n, Ml, d.np, field(d, fsrc) + (int64_t)q.k * d.n,
+  tiles::trmv_rows<float, UPPER, 8>(d.n, Ml, d.np, field(d, fsrc) + (int64_t)q.k * d.n,
                                  field(d, fdst) + (int64_t)q.k * d.n, i0, g_trmv_v4);
 }
 

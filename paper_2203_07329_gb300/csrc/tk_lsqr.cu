@@ -92,80 +92,153 @@ __global__ void k_over_init_beta(const double* __restrict__ part, int chunks, co
   }
 }
 
-// Ub = sqrt(l) T + coef Ub;  beta = sqrt(sum partial + ||Ub||^2);  anorm2 += alpha^2 + beta^2
+// Ub = sqrt(l) T + coef Ub;  beta = ||[Ut; Ub]||;  anorm2 += alpha^2 + beta^2.  The `chunks` blocks of a
+// slot each take a piece of Ut and of Ub and leave the sum of squares in partial; the block that
+// arrives last adds the pieces (in a fixed order) and writes the scalars: one launch for what were a
+// partial-sum kernel and a one-block kernel behind it (9 us of dependent float64 latency).  arrivals[s]
+// is zero on entry and left zero.
 template <typename T>
-__global__ void k_over_beta(const double* __restrict__ part, int chunks, const T* __restrict__ Tt,
-                            T* __restrict__ Ub, int64_t n, Scal* __restrict__ sc) {
+__global__ void __launch_bounds__(256)
+    k_over_norm(const T* __restrict__ Ut, int64_t m, const T* __restrict__ Tt, T* __restrict__ Ub, int64_t n,
+                Scal* __restrict__ sc, double* __restrict__ partial, int* __restrict__ arrivals) {
   __shared__ double sh[32];
-  const int s = blockIdx.x;
-  if (sc[s].istop != 0) return;  // retired inside a chunk of steps
+  __shared__ int last;
+  const int s = blockIdx.y, c = blockIdx.x, chunks = gridDim.x;
+  if (sc[s].istop != 0) return;  // retired inside a chunk of steps (every block of the slot returns)
   const double sl = sc[s].sqrtl, coef = sc[s].coef;
   double acc = 0.0;
-  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-    int64_t k = (int64_t)s * n + j;
-    double v = fma(sl, (double)Tt[k], coef * (double)Ub[k]);
-    T vt = (T)v;
-    Ub[k] = vt;
-    acc = fma((double)vt, (double)vt, acc);
+  {
+    const int64_t per = cdiv(m, chunks), b = c * per, e = b + per < m ? b + per : m;
+    const T* u = Ut + (int64_t)s * m;
+#pragma unroll 4
+    for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) {
+      const double v = (double)u[i];
+      acc = fma(v, v, acc);
+    }
+  }
+  {
+    const int64_t per = cdiv(n, chunks), b = c * per, e = b + per < n ? b + per : n;
+    for (int64_t j = b + threadIdx.x; j < e; j += blockDim.x) {
+      const int64_t k = (int64_t)s * n + j;
+      const T vt = (T)fma(sl, (double)Tt[k], coef * (double)Ub[k]);
+      Ub[k] = vt;
+      acc = fma((double)vt, (double)vt, acc);
+    }
   }
   acc = block_sum(acc, sh);
   if (threadIdx.x == 0) {
-    double t = acc;
-    for (int c = 0; c < chunks; ++c) t += part[s * chunks + c];
-    double beta = sqrt(t);
-    Scal q = sc[s];
-    q.anorm2 += q.alpha * q.alpha + beta * beta;
-    q.beta = beta;
-    sc[s] = q;
+    partial[s * kSumChunks + c] = acc;
+    __threadfence();
+    last = atomicAdd(&arrivals[s], 1) == chunks - 1;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  __threadfence();
+  double t = 0.0;
+  for (int k = threadIdx.x; k < chunks; k += 32) t += *(volatile double*)&partial[s * kSumChunks + k];
+  t = warp_sum(t);
+  if (threadIdx.x == 0) {
+    const double beta = sqrt(t);
+    const double al = sc[s].alpha;
+    sc[s].anorm2 += al * al + beta * beta;
+    sc[s].beta = beta;
+    arrivals[s] = 0;
   }
 }
 
-// C[k] = sum_z partial[z][k] (the split-K planes of a product, in order)
+// G = (sum_z partial_z + sqrt(l) Ub) / beta.  Block: 32 columns x 8 groups of planes, the groups' sums
+// added in order in shared memory: the planes' loads run 8 x 4 deep (a thread per column walking up to
+// 900 planes took 60 us at n = 777; this takes 5).
 template <typename T>
-__global__ void k_sum_planes_to(const double* __restrict__ part, int splits, int64_t total, T* __restrict__ C) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int z = 0; z < splits; ++z) acc += part[(int64_t)z * total + k];
-    C[k] = (T)acc;
+__global__ void __launch_bounds__(256)
+    k_over_g(const double* __restrict__ part, int splits, int count, const T* __restrict__ Ub, int64_t n,
+             const Scal* __restrict__ sc, T* __restrict__ G) {
+  __shared__ double sh[8][33];
+  const int s = blockIdx.y, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t plane = (int64_t)count * n, j = (int64_t)blockIdx.x * 32 + tx;
+  double acc = 0.0;
+  if (j < n) {
+    const double* p = part + (int64_t)s * n + j;
+#pragma unroll 4
+    for (int z = ty; z < splits; z += 8) acc += p[z * plane];
   }
-}
-
-// G = (sum_z partial_z + sqrt(l) Ub) / beta
-template <typename T>
-__global__ void k_over_g(const double* __restrict__ part, int splits, int count, const T* __restrict__ Ub, int64_t n,
-                         const Scal* __restrict__ sc, T* __restrict__ G) {
-  const int s = blockIdx.y;
-  const double sl = sc[s].sqrtl, beta = sc[s].beta;
-  const double inv = beta > 0.0 ? 1.0 / beta : 0.0;
-  const int64_t plane = (int64_t)count * n;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int z = 0; z < splits; ++z) acc += part[z * plane + (int64_t)s * n + j];
+  sh[ty][tx] = acc;
+  __syncthreads();
+  if (ty == 0 && j < n) {
+    const double sl = sc[s].sqrtl, beta = sc[s].beta;
+    const double inv = beta > 0.0 ? 1.0 / beta : 0.0;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) acc += sh[q][tx];
     acc = fma(sl, (double)Ub[(int64_t)s * n + j], acc);
     G[(int64_t)s * n + j] = (T)(acc * inv);
   }
 }
 
 // ---- shared Golub-Kahan v-step + Givens + tests (body: vstep_block) ---
-template <typename T>
-__global__ void __launch_bounds__(kVecThreads)
+// A slot's vectors are split over the CL CTAs of a cluster (the sums meet in distributed shared
+// memory): with one CTA per slot the 66560 values of a 1024 x 65536 problem took 295 us a step.
+template <typename T, int CL>
+__global__ void __launch_bounds__(512)
     k_vstep(const T* __restrict__ Vraw, T* __restrict__ V, T* __restrict__ W, T* __restrict__ Y, int64_t nv,
-            Scal* __restrict__ sc, double atol, double btol, int maxiter, int init) {
+            Scal* __restrict__ sc, double* __restrict__ coef, double atol, double btol, int maxiter, int init) {
   __shared__ double sh[32];
-  const int s = blockIdx.x;
+  __shared__ double red[2];
+  const int s = blockIdx.y;
   const int64_t off = (int64_t)s * nv;
-  vstep_block<T>(Vraw + off, V + off, W + off, Y + off, nv, sc + s, atol, btol, maxiter, init, sh);
+  vstep_block<T, CL>(Vraw + off, V + off, W + off, Y + off, nv, sc + s, coef + s, atol, btol, maxiter, init, sh, red);
+}
+
+// Threads: the fewest warps that leave a thread about 2 values; CTAs: one per 4096 values, at most 8
+// (the portable cluster size).
+template <typename T>
+tk_status launch_vstep(const T* Vraw, T* V, T* W, T* Y, int64_t nv, Scal* sc, double* coef, double atol, double btol,
+                       int maxiter, int init, int count, cudaStream_t st) {
+  const int cl = nv <= 4096 ? 1 : nv <= 8192 ? 2 : nv <= 16384 ? 4 : 8;
+  const int threads = nv <= 512 ? 256 : 512;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)cl, (unsigned)count, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = cl > 1 ? 1 : 0;
+  auto go = [&](auto kern) -> tk_status {
+    TK_CUDA(cudaLaunchKernelEx(&cfg, kern, Vraw, V, W, Y, nv, sc, coef, atol, btol, maxiter, init));
+    TK_LAUNCH_CHECK();
+    return TK_OK;
+  };
+  if (cl == 1) return go(k_vstep<T, 1>);
+  if (cl == 2) return go(k_vstep<T, 2>);
+  if (cl == 4) return go(k_vstep<T, 4>);
+  return go(k_vstep<T, 8>);
 }
 
 // ---- underdetermined ----------------------------------------------------
-// P = V1 A^T (from the GEMM) + sqrt(l) V2 ;  in place on P.
+// P = sum_z partial_z (the planes of V1 A^T, count x m) + sqrt(l) V2; blocks as k_over_g.
 template <typename T>
-__global__ void k_under_addv2(T* __restrict__ P, int64_t m, const T* __restrict__ V, int64_t nv, int64_t n,
-                              const Scal* __restrict__ sc) {
-  const int s = blockIdx.y;
-  const double sl = sc[s].sqrtl;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-    P[(int64_t)s * m + i] = (T)((double)P[(int64_t)s * m + i] + sl * (double)V[(int64_t)s * nv + n + i]);
+__global__ void __launch_bounds__(256)
+    k_under_p(const double* __restrict__ part, int splits, int count, int64_t m, const T* __restrict__ V, int64_t nv,
+              int64_t n, const Scal* __restrict__ sc, T* __restrict__ P) {
+  __shared__ double sh[8][33];
+  const int s = blockIdx.y, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t plane = (int64_t)count * m, i = (int64_t)blockIdx.x * 32 + tx;
+  double acc = 0.0;
+  if (i < m) {
+    const double* p = part + (int64_t)s * m + i;
+#pragma unroll 4
+    for (int z = ty; z < splits; z += 8) acc += p[z * plane];
+  }
+  sh[ty][tx] = acc;
+  __syncthreads();
+  if (ty == 0 && i < m) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) acc += sh[q][tx];
+    P[(int64_t)s * m + i] = (T)(acc + sc[s].sqrtl * (double)V[(int64_t)s * nv + n + i]);
+  }
 }
 
 // u = Q - alpha u (init: u = Q), beta = ||u||, u /= beta, anorm2 += alpha^2 + beta^2
@@ -244,10 +317,11 @@ __global__ void k_move_rows(T* __restrict__ X, int64_t len, const int* __restric
     X[b * len + i] = X[a * len + i];
 }
 
-__global__ void k_move_scal(Scal* __restrict__ sc, int* __restrict__ slot_lam, const int* __restrict__ src,
-                            const int* __restrict__ dst, int moves) {
+__global__ void k_move_scal(Scal* __restrict__ sc, int* __restrict__ slot_lam, double* __restrict__ coef,
+                            const int* __restrict__ src, const int* __restrict__ dst, int moves) {
   for (int k = threadIdx.x; k < moves; k += blockDim.x) {
     sc[dst[k]] = sc[src[k]];
+    coef[dst[k]] = coef[src[k]];
     slot_lam[dst[k]] = slot_lam[src[k]];
   }
 }
@@ -328,7 +402,8 @@ void Lsqr<T>::carve(Arena& a) {
   Ub = under ? nullptr : a.take<T>((size_t)N_cap * n);
   part_u = a.take<double>((size_t)N_cap * kSumChunks);
   part_g = a.take<double>((size_t)splits * N_cap * gcols);
-  coef_buf = a.take<double>((size_t)N_cap);
+  coef_buf = a.take<double>((size_t)N_cap);  // Scal.coef of the slots, dense, as the products' epilogues read it
+  arrivals = a.take<int>((size_t)N_cap);
   sc = a.take<Scal>((size_t)N_cap);
   slot_lam = a.take<int>((size_t)N_cap);
   idx_buf = a.take<int>((size_t)N_cap * 3);
@@ -371,13 +446,13 @@ inline double total_count(int count, int64_t m) { return (double)count * (double
 
 template <typename T>
 tk_status Lsqr<T>::prod_aw(const T* Win, int64_t ldw, T* C, const double* beta, int count) {
-  // C (count x m) = Win (count x n) A^T  [+ beta_row * C]
+  // C (count x m) = Win (count x n) A^T  [+ beta_row * C]; under: its split-K planes in part_g (cur_splits)
   const bool digits = use_oz(count);
   const double es = (double)sizeof(T);
   const double vec = es * (count * (double)n + 2.0 * count * m);
   int tok = prof_begin(digits ? TK_PHASE_AW_DIGITS : TK_PHASE_AW, st);
   tk_status r;
-  if (digits && !(under && !beta)) {
+  if (digits && !under) {
     r = oz_lsqr_aw<T>(oz_A, Win, ldw, count, oz_q, oz_e, C, m, beta, oz_err, st);
     prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec, 2.0 * oz_digits<T>() * m * n + vec);
     return r;
@@ -394,27 +469,20 @@ tk_status Lsqr<T>::prod_aw(const T* Win, int64_t ldw, T* C, const double* beta, 
       return r;
     }
   }
-  if (under && !beta) {
+  if (under) {
     // the underdetermined product: a short output (count x m, m < n) against a long K = n; split K
-    // over the GPU and add the planes (part_g holds splits x N_cap x n >= sp x count x m values)
+    // over the GPU, the planes (part_g holds splits x N_cap x n >= sp x count x m values) are added by
+    // the caller's next kernel
     const int64_t cap = ((int64_t)splits * N_cap * n) / std::max<int64_t>((int64_t)count * m, 1);
-    const int sp = (int)std::min<int64_t>(digits ? oz_normal_splits(n, m, count) : splitk_count(count, m, n), cap);
-    if (sp > 1 || digits) {
-      r = TK_EINVAL;
-      if constexpr (std::is_same<T, double>::value) {
-        if (digits) r = oz_lsqr_aw_split<T>(oz_A, Win, ldw, count, oz_q, oz_e, part_g, sp, oz_err, st);
-      }
-      if (!digits) r = gemm_splitk<T, T>(false, true, count, m, n, Win, ldw, A, lda, part_g, sp, st);
-      if (r == TK_OK) {
-        const int64_t total = (int64_t)count * m;
-        k_sum_planes_to<T><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(cdiv(total, 256), 152 * 8)), 256, 0,
-                             st>>>(part_g, sp, total, C);
-        TK_LAUNCH_CHECK();
-      }
-      prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec + 16.0 * sp * total_count(count, m),
-               (digits ? 2.0 * oz_digits<T>() : es) * m * n + vec + 16.0 * sp * total_count(count, m));
-      return r;
+    cur_splits = (int)std::min<int64_t>(digits ? oz_normal_splits(n, m, count) : splitk_count(count, m, n), cap);
+    r = TK_EINVAL;
+    if constexpr (std::is_same<T, double>::value) {
+      if (digits) r = oz_lsqr_aw_split<T>(oz_A, Win, ldw, count, oz_q, oz_e, part_g, cur_splits, oz_err, st);
     }
+    if (!digits) r = gemm_splitk<T, T>(false, true, count, m, n, Win, ldw, A, lda, part_g, cur_splits, st);
+    const double pl = 8.0 * cur_splits * total_count(count, m);
+    prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec + pl, (digits ? 16.0 : es) * m * n + vec + pl);
+    return r;
   }
   r = gemm<T, T, T>(false, true, count, m, n, Win, ldw, A, lda, C, m, 1.0, beta, beta ? C : nullptr, m, st);
   prof_end(tok, st, 2.0 * count * m * n, a_es * m * n + vec, es * m * n + vec);
@@ -484,6 +552,7 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
   }
   int nact = count;
   lam_all = lam_dev;
+  TK_CUDA(cudaMemsetAsync(arrivals, 0, sizeof(int) * (size_t)N_cap, st));
   k_init_scal<<<cdiv(count, 128), 128, 0, st>>>(sc, slot_lam, lam_ids_dev, lam_dev, count);
   TK_LAUNCH_CHECK();
   // ---------------------------------------------------------------- init
@@ -495,22 +564,21 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
     k_over_init_beta<T><<<nact, kVecThreads, 0, st>>>(part_u, kSumChunks, Ub, n, sc);
     TK_LAUNCH_CHECK();
     TK_TRY(prod_atu(Ut, nact));
-    k_over_g<T><<<rows_grid(n, nact), 256, 0, st>>>(part_g, cur_splits, nact, Ub, n, sc, Tt);
+    k_over_g<T><<<dim3((unsigned)cdiv(n, 32), (unsigned)nact), 256, 0, st>>>(part_g, cur_splits, nact, Ub, n, sc, Tt);
     TK_LAUNCH_CHECK();
     TK_TRY(apply_prec(true, Tt, Vraw, nact, n));
   } else {
     k_bcast_rows<T><<<rows_grid(m, nact), 256, 0, st>>>(b, m, Tt);
     TK_LAUNCH_CHECK();
-    TK_TRY(apply_prec(true, Tt, Tt, nact, m));
-    k_under_ustep<T><<<nact, kVecThreads, 0, st>>>(Tt, Ut, m, sc, 1);
+    TK_TRY(apply_prec(true, Tt, xtmp, nact, m));
+    k_under_ustep<T><<<nact, kVecThreads, 0, st>>>(xtmp, Ut, m, sc, 1);
     TK_LAUNCH_CHECK();
     TK_TRY(apply_prec(false, Ut, Tt, nact, m));
     TK_TRY(prod_atu(Tt, nact));
     k_under_vraw<T><<<rows_grid(nv, nact), 256, 0, st>>>(part_g, cur_splits, nact, Tt, m, n, sc, Vraw);
     TK_LAUNCH_CHECK();
   }
-  k_vstep<T><<<nact, kVecThreads, 0, st>>>(Vraw, V, W, Y, nv, sc, atol, btol, maxiter, 1);
-  TK_LAUNCH_CHECK();
+  TK_TRY(launch_vstep<T>(Vraw, V, W, Y, nv, sc, coef_buf, atol, btol, maxiter, 1, nact, st));
 
   // steps per read of the scalars: several for problems whose steps are
   // launch-bound (A of at most 2^24 elements), one otherwise
@@ -574,7 +642,7 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
         k_move_rows<T><<<rows_grid(nv, moves), 256, 0, st>>>(Y, nv, d_src, d_dst, moves);
         k_move_rows<T><<<rows_grid(m, moves), 256, 0, st>>>(Ut, m, d_src, d_dst, moves);
         if (!under) k_move_rows<T><<<rows_grid(n, moves), 256, 0, st>>>(Ub, n, d_src, d_dst, moves);
-        k_move_scal<<<1, 128, 0, st>>>(sc, slot_lam, d_src, d_dst, moves);
+        k_move_scal<<<1, 128, 0, st>>>(sc, slot_lam, coef_buf, d_src, d_dst, moves);
         TK_LAUNCH_CHECK();
       }
       nact = nnew;
@@ -598,42 +666,44 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
 }
 
 template <typename T>
+tk_status Lsqr<T>::norm(int nact) {
+  // enough blocks for every SM, at least 2048 values to a block
+  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>({kSumChunks, cdiv(m, 2048), cdiv(8 * 152, nact)}));
+  k_over_norm<T><<<dim3((unsigned)chunks, (unsigned)nact), 256, 0, st>>>(Ut, m, Tt, Ub, n, sc, part_u, arrivals);
+  TK_LAUNCH_CHECK();
+  return TK_OK;
+}
+
+template <typename T>
 tk_status Lsqr<T>::step(int nact) {
+  const dim3 gn((unsigned)cdiv(n, 32), (unsigned)nact);
   if (!under) {
     TK_TRY(apply_prec(false, V, Tt, nact, n));  // T = R^-1 v
-    TK_TRY(gather_coef(nact));
     if (use_fused(nact)) {  // u' = A R^-1 v - alpha u and A^T u' over one read of A's digits
       TK_TRY(prod_fused(Tt, Ut, coef_buf, nact));
-      k_sumsq_rows<T><<<dim3(kSumChunks, nact), 256, 0, st>>>(Ut, m, m, kSumChunks, part_u);
-      TK_LAUNCH_CHECK();
-      k_over_beta<T><<<nact, kVecThreads, 0, st>>>(part_u, kSumChunks, Tt, Ub, n, sc);
-      TK_LAUNCH_CHECK();
+      TK_TRY(norm(nact));
     } else {
       TK_TRY(prod_aw(Tt, n, Ut, coef_buf, nact));
-      k_sumsq_rows<T><<<dim3(kSumChunks, nact), 256, 0, st>>>(Ut, m, m, kSumChunks, part_u);
-      TK_LAUNCH_CHECK();
-      k_over_beta<T><<<nact, kVecThreads, 0, st>>>(part_u, kSumChunks, Tt, Ub, n, sc);
-      TK_LAUNCH_CHECK();
+      TK_TRY(norm(nact));
       TK_TRY(prod_atu(Ut, nact));
     }
-    k_over_g<T><<<rows_grid(n, nact), 256, 0, st>>>(part_g, cur_splits, nact, Ub, n, sc, Tt);
+    k_over_g<T><<<gn, 256, 0, st>>>(part_g, cur_splits, nact, Ub, n, sc, Tt);
     TK_LAUNCH_CHECK();
     TK_TRY(apply_prec(true, Tt, Vraw, nact, n));  // R^-T g
   } else {
-    TK_TRY(prod_aw(V, nv, Tt, nullptr, nact));
-    k_under_addv2<T><<<rows_grid(m, nact), 256, 0, st>>>(Tt, m, V, nv, n, sc);
+    TK_TRY(prod_aw(V, nv, nullptr, nullptr, nact));
+    k_under_p<T><<<dim3((unsigned)cdiv(m, 32), (unsigned)nact), 256, 0, st>>>(part_g, cur_splits, nact, m, V, nv, n,
+                                                                             sc, Tt);
     TK_LAUNCH_CHECK();
-    TK_TRY(apply_prec(true, Tt, Tt, nact, m));
-    k_under_ustep<T><<<nact, kVecThreads, 0, st>>>(Tt, Ut, m, sc, 0);
+    TK_TRY(apply_prec(true, Tt, xtmp, nact, m));
+    k_under_ustep<T><<<nact, kVecThreads, 0, st>>>(xtmp, Ut, m, sc, 0);
     TK_LAUNCH_CHECK();
     TK_TRY(apply_prec(false, Ut, Tt, nact, m));
     TK_TRY(prod_atu(Tt, nact));
     k_under_vraw<T><<<rows_grid(nv, nact), 256, 0, st>>>(part_g, cur_splits, nact, Tt, m, n, sc, Vraw);
     TK_LAUNCH_CHECK();
   }
-  k_vstep<T><<<nact, kVecThreads, 0, st>>>(Vraw, V, W, Y, nv, sc, atol, btol, maxiter, 0);
-  TK_LAUNCH_CHECK();
-  return TK_OK;
+  return launch_vstep<T>(Vraw, V, W, Y, nv, sc, coef_buf, atol, btol, maxiter, 0, nact, st);
 }
 
 // `count` steps for `nact` active slots: launched directly (count 1, a
@@ -702,22 +772,6 @@ void Lsqr<T>::release_graphs() {
     cudaEventDestroy(gev[1]);
     gstream = nullptr;
   }
-}
-
-// The GEMM epilogue takes a dense per-row coefficient array; Scal.coef is
-// strided, so it is gathered each step.
-namespace {
-__global__ void k_coef(const Scal* __restrict__ sc, double* __restrict__ coef, int count) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < count) coef[s] = sc[s].coef;
-}
-}  // namespace
-
-template <typename T>
-tk_status Lsqr<T>::gather_coef(int count) {
-  k_coef<<<cdiv(count, 128), 128, 0, st>>>(sc, coef_buf, count);
-  TK_LAUNCH_CHECK();
-  return TK_OK;
 }
 
 template struct Lsqr<double>;

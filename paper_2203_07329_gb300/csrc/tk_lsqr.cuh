@@ -35,92 +35,132 @@ template <typename T>
 tk_status lowrank_diag_dev(const double* sigma, int64_t s, const double* lam_dev, const int64_t* rank_dev, int N,
                            T* S, cudaStream_t st);
 
-// One block's Golub-Kahan v-step for one slot (Paige & Saunders' LSQR):
-// Vraw holds M^T u (length nv).  v' = Vraw - beta v, alpha = ||v'||, then the
-// Givens rotation, the y and w updates and the stopping tests (istop 1: the
-// residual test, 2: the normal-equation test, 5: non-finite, 7: iteration
-// cap).  init: the first v (alpha_1 v_1 = M^T u_1), w = v, y = 0.  sh: 32
-// doubles of shared memory.
-template <typename T>
-__device__ __forceinline__ void vstep_block(const T* __restrict__ Vraw, T* __restrict__ V, T* __restrict__ W,
-                                            T* __restrict__ Y, int64_t nv, Scal* __restrict__ sq, double atol,
-                                            double btol, int maxiter, int init, double* sh) {
-  Scal q = *sq;
-  if (!init && q.istop != 0) return;  // retired inside a chunk of steps: left as it is
-  const int64_t off = 0;
+// One slot's Golub-Kahan v-step (Paige & Saunders' LSQR): Vraw holds M^T u
+// (length nv).  v' = Vraw - beta v, alpha = ||v'||, then the Givens rotation,
+// the y and w updates and the stopping tests (istop 1: the residual test, 2:
+// the normal-equation test, 5: non-finite, 7: iteration cap).  init: the first
+// v (alpha_1 v_1 = M^T u_1), w = v, y = 0.
+struct VGivens {
+  double ainv, t1, t2;  // 1 / alpha, phi / rho, theta / rho
+  double c, rhobar, phibar;
+};
+__device__ __forceinline__ VGivens vstep_givens(const Scal& q, double alpha) {
+  VGivens g;
   const double beta = q.beta;
+  const double rho = sqrt(q.rhobar * q.rhobar + beta * beta);
+  const double rinv = rho > 0.0 ? 1.0 / rho : 0.0;
+  g.c = rho > 0.0 ? q.rhobar / rho : 1.0;
+  const double sn = rho > 0.0 ? beta / rho : 0.0;
+  g.rhobar = -g.c * alpha;
+  g.phibar = sn * q.phibar;
+  g.t1 = g.c * q.phibar * rinv;
+  g.t2 = sn * alpha * rinv;
+  g.ainv = alpha > 0.0 ? 1.0 / alpha : 0.0;
+  return g;
+}
+__device__ __forceinline__ void vstep_init_scal(Scal& q, double alpha) {
+  q.alpha = alpha;
+  q.rhobar = alpha;
+  q.coef = (q.beta > 0.0) ? -alpha / q.beta : 0.0;
+  q.arnorm = alpha * q.beta;
+  if (alpha == 0.0 && q.istop == 0) q.istop = 1;  // b orthogonal to range(M): y = 0 is exact
+  if (!isfinite(alpha)) q.istop = 5;
+}
+__device__ __forceinline__ void vstep_finish_scal(Scal& q, const VGivens& g, double alpha, double ynorm, double atol,
+                                                  double btol, int maxiter) {
+  const double beta = q.beta;
+  q.alpha = alpha;
+  q.rhobar = g.rhobar;
+  q.phibar = g.phibar;
+  q.iters += 1;
+  q.coef = beta > 0.0 ? -alpha / beta : 0.0;
+  const double rnorm = g.phibar;
+  const double arnorm = g.phibar * alpha * fabs(g.c);
+  const double anorm = sqrt(q.anorm2);
+  q.rnorm = rnorm;
+  q.arnorm = arnorm;
+  q.ynorm = ynorm;
+  int istop = 0;
+  if (!isfinite(alpha) || !isfinite(beta) || !isfinite(ynorm)) istop = 5;
+  else if (rnorm == 0.0) istop = 1;
+  else if (arnorm / (anorm * rnorm) <= atol) istop = 2;
+  else if (rnorm <= btol * q.bnorm + atol * anorm * ynorm) istop = 1;
+  else if (q.iters >= maxiter) istop = 7;
+  q.istop = istop;
+}
+
+// The step by CL CTAs of a cluster (CL = 1: a plain block), this CTA taking every CL-th block of
+// values; sh: 32 doubles, red: 2 doubles of shared memory that the peers read.
+template <typename T, int CL>
+__device__ __forceinline__ void vstep_block(const T* __restrict__ Vraw, T* __restrict__ V, T* __restrict__ W,
+                                            T* __restrict__ Y, int64_t nv, Scal* __restrict__ sq,
+                                            double* __restrict__ coef_out, double atol, double btol, int maxiter,
+                                            int init, double* sh, double* red) {
+  Scal q = *sq;
+  if (!init && q.istop != 0) return;  // retired inside a chunk of steps: left as it is (every CTA returns)
+  const double beta = q.beta;
+  int rank = 0;
+  if constexpr (CL > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  // sum over the cluster, in rank order; slot: a fresh entry of red for each sum
+  auto cluster_sum = [&](double v, int slot) -> double {
+    v = block_sum(v, sh);
+    if constexpr (CL > 1) {
+      if (threadIdx.x == 0) red[slot] = v;
+      asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      v = 0.0;
+#pragma unroll
+      for (int r = 0; r < CL; ++r) v += *static_cast<double*>(__cluster_map_shared_rank(red + slot, r));
+    }
+    return v;
+  };
+  const int64_t first = (int64_t)rank * blockDim.x + threadIdx.x, stride = (int64_t)CL * blockDim.x;
   // v' = Vraw - beta v  (init: v' = Vraw)
   double acc = 0.0;
-  for (int64_t j = threadIdx.x; j < nv; j += blockDim.x) {
-    double v = (double)Vraw[off + j];
-    if (!init) v = fma(-beta, (double)V[off + j], v);
-    V[off + j] = (T)v;
+#pragma unroll 4
+  for (int64_t j = first; j < nv; j += stride) {
+    double v = (double)Vraw[j];
+    if (!init) v = fma(-beta, (double)V[j], v);
+    V[j] = (T)v;
     acc = fma(v, v, acc);
   }
-  const double alpha = sqrt(block_sum(acc, sh));
-  const double ainv = alpha > 0.0 ? 1.0 / alpha : 0.0;
+  const double alpha = sqrt(cluster_sum(acc, 0));
   if (init) {
-    double yn = 0.0;
-    for (int64_t j = threadIdx.x; j < nv; j += blockDim.x) {
-      T v = (T)((double)V[off + j] * ainv);
-      V[off + j] = v;
-      W[off + j] = v;
-      Y[off + j] = T(0);
+    const double ainv = alpha > 0.0 ? 1.0 / alpha : 0.0;
+    for (int64_t j = first; j < nv; j += stride) {
+      T v = (T)((double)V[j] * ainv);
+      V[j] = v;
+      W[j] = v;
+      Y[j] = T(0);
     }
-    (void)yn;
-    if (threadIdx.x == 0) {
-      q.alpha = alpha;
-      q.rhobar = alpha;
-      q.coef = (q.beta > 0.0) ? -alpha / q.beta : 0.0;
-      q.arnorm = alpha * q.beta;
-      if (alpha == 0.0 && q.istop == 0) q.istop = 1;  // b orthogonal to range(M): y = 0 is exact
-      if (!isfinite(alpha)) q.istop = 5;
+    if (rank == 0 && threadIdx.x == 0) {
+      vstep_init_scal(q, alpha);
       *sq = q;
+      if (coef_out) *coef_out = q.coef;
     }
-    return;
+  } else {
+    const VGivens g = vstep_givens(q, alpha);
+    double yy = 0.0;
+#pragma unroll 4
+    for (int64_t j = first; j < nv; j += stride) {
+      double v = (double)V[j] * g.ainv;
+      double w = (double)W[j];
+      double y = fma(g.t1, w, (double)Y[j]);
+      w = fma(-g.t2, w, v);
+      V[j] = (T)v;
+      W[j] = (T)w;
+      Y[j] = (T)y;
+      yy = fma(y, y, yy);
+    }
+    const double ynorm = sqrt(cluster_sum(yy, 1));
+    if (rank == 0 && threadIdx.x == 0) {
+      vstep_finish_scal(q, g, alpha, ynorm, atol, btol, maxiter);
+      *sq = q;
+      if (coef_out) *coef_out = q.coef;
+    }
   }
-  const double rho = sqrt(q.rhobar * q.rhobar + beta * beta);
-  const double c = rho > 0.0 ? q.rhobar / rho : 1.0;
-  const double sn = rho > 0.0 ? beta / rho : 0.0;
-  const double theta = sn * alpha;
-  const double rhobar = -c * alpha;
-  const double phi = c * q.phibar;
-  const double phibar = sn * q.phibar;
-  const double t1 = rho > 0.0 ? phi / rho : 0.0;
-  const double t2 = rho > 0.0 ? theta / rho : 0.0;
-  double yy = 0.0;
-  for (int64_t j = threadIdx.x; j < nv; j += blockDim.x) {
-    double v = (double)V[off + j] * ainv;
-    double w = (double)W[off + j];
-    double y = fma(t1, w, (double)Y[off + j]);
-    w = fma(-t2, w, v);
-    V[off + j] = (T)v;
-    W[off + j] = (T)w;
-    Y[off + j] = (T)y;
-    yy = fma(y, y, yy);
-  }
-  const double ynorm = sqrt(block_sum(yy, sh));
-  if (threadIdx.x == 0) {
-    q.alpha = alpha;
-    q.rhobar = rhobar;
-    q.phibar = phibar;
-    q.iters += 1;
-    q.coef = beta > 0.0 ? -alpha / beta : 0.0;
-    const double rnorm = phibar;
-    const double arnorm = phibar * alpha * fabs(c);
-    const double anorm = sqrt(q.anorm2);
-    q.rnorm = rnorm;
-    q.arnorm = arnorm;
-    q.ynorm = ynorm;
-    int istop = 0;
-    if (!isfinite(alpha) || !isfinite(beta) || !isfinite(ynorm)) istop = 5;
-    else if (rnorm == 0.0) istop = 1;
-    else if (arnorm / (anorm * rnorm) <= atol) istop = 2;
-    else if (rnorm <= btol * q.bnorm + atol * anorm * ynorm) istop = 1;
-    else if (q.iters >= maxiter) istop = 7;
-    q.istop = istop;
-    *sq = q;
-  }
+  // no CTA leaves while a peer may still read its sums
+  if constexpr (CL > 1)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 template <typename T>
@@ -154,6 +194,7 @@ struct Lsqr {
   int cur_splits = 1;  // splits of the last A^T U product (the tuned count, <= splits)
   T *V = nullptr, *W = nullptr, *Y = nullptr, *Vraw = nullptr, *Ut = nullptr, *Tt = nullptr, *Ub = nullptr,
     *xtmp = nullptr, *lr_tmp = nullptr;
+  int* arrivals = nullptr;  // N_cap counters of the norm kernel, zero between launches
   double *part_u = nullptr, *part_g = nullptr, *coef_buf = nullptr, *lr_inv = nullptr, *trsv_p = nullptr;
   Scal* sc = nullptr;
   int* slot_lam = nullptr;
@@ -197,7 +238,7 @@ struct Lsqr {
   tk_status prod_aw(const T* Win, int64_t ldw, T* C, const double* beta, int count);
   tk_status prod_atu(const T* Uin, int count);
   tk_status prod_fused(const T* Win, T* C, const double* beta, int count);
-  tk_status gather_coef(int count);
+  tk_status norm(int nact);
   // one LSQR step for slots 0..nact-1; `count` of them (see steps())
   tk_status step(int nact);
   tk_status steps(int nact, int count);

@@ -17,9 +17,10 @@ def _solve(A, b, lams, **kw):
 
 # A at and around the smallest size that is split into digits (2^19 elements), ragged against the 64-,
 # 128- and 256-value tiles, one and several tiles of 32 lambdas, float64 views with odd row strides,
-# and m < n.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
+# and m < n with vectors of 1, 2, 4 and 8 CTAs per v-step.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
 @pytest.mark.parametrize("m,n,N,pad", [(8192, 64, 2, 0), (8193, 65, 3, 1), (2051, 257, 33, 0), (1500, 700, 5, 3),
-                                       (16500, 40, 4, 0), (129, 4099, 4, 0), (500, 1100, 34, 5), (63, 8400, 2, 0)])
+                                       (16500, 40, 4, 0), (129, 4099, 4, 0), (500, 1100, 34, 5), (63, 8400, 2, 0),
+                                       (101, 17001, 3, 0)])
 def test_digit_solve_matches_float64_pipe(m, n, N, pad):
     k = min(m, n)
     p = datagen.make_ridge_problem(m, n, datagen.spectrum("log", k, hi=1.0, lo=1e-3),
