@@ -664,6 +664,13 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
       gp->svd_Y = B.Y;
       gp->svd_scratch = B.svd;
       gp->svd_bytes = B.svd_bytes;
+      SvdJob j;
+      j.Y = B.Y;
+      j.s = P.s;
+      j.n = P.c;
+      j.scratch = B.svd;
+      j.scratch_bytes = B.svd_bytes;
+      TK_TRY(jacobi_svd_begin(j, st));
     }
     for (int i = 0; i < N; ++i) gp->inf[i] = inf[i];
     TK_CUDA(cudaStreamSynchronize(st));  // the build scratch is reused by the lane's next problem

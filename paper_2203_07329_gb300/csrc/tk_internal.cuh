@@ -379,10 +379,11 @@ template <typename TR, typename TX>
 tk_status trsv_batched(bool transposed, int64_t n, const TR* R, int64_t ldr, int64_t rstride, const int* idx,
                        const TX* Xin, TX* X, int64_t ldx, int count, double* pbuf, cudaStream_t st);
 
-// Low rank (tk_lowrank.cu)
+// One-sided Jacobi SVDs (tk_svd.cu)
 size_t svd_workspace(int64_t s, int64_t n);
-// Many one-sided Jacobi SVDs at once (grouped batch): every round of the
-// circle schedule is one launch over the pairs of all matrices still rotating.
+// Many SVDs at once (grouped batch): jacobi_svd_begin starts a matrix on its own (the orthogonal start,
+// into its scratch, on the stream of the lane that sketched it); then every round of the circle
+// schedule is one launch over the block pairs of all matrices still rotating.
 struct SvdJob {
   const double* Y = nullptr;  // s x n (read only)
   int64_t s = 0, n = 0;
@@ -391,10 +392,8 @@ struct SvdJob {
   void* scratch = nullptr;    // svd_workspace(s, n) bytes
   size_t scratch_bytes = 0;
   int sweeps = 0;             // out
-  double* W = nullptr;        // carved from scratch
-  double* nrm = nullptr;
-  int* perm = nullptr;
 };
+tk_status jacobi_svd_begin(SvdJob& q, cudaStream_t st);
 size_t svd_grouped_workspace(const std::vector<SvdJob>& jobs);
 tk_status jacobi_svd_grouped(std::vector<SvdJob>& jobs, void* work, size_t work_bytes, cudaStream_t st);
 tk_status jacobi_svd(const double* Y, int64_t s, int64_t n, double* sigma, double* V, int* sweeps_host, Arena& ar,
