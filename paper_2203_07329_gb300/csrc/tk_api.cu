@@ -79,12 +79,11 @@ tk_status check_opts(const tk_opts* o) {
 }
 
 // The float64 form with emulate_fp64: whether the solve makes digit planes of A at all.  They pay off
-// from two lambda at a time (a digit product costs the same for 1..32 lambda, the float64 pipe's work
-// grows with the count) and when A is large enough that a product is not all launch latency; A of more
-// than 2^32 elements keeps the float64 pipe, because the planes take 16 bytes per element.
-bool oz64_wanted(int64_t m, int64_t n, int N_cap) {
-  return N_cap >= 2 && m * n >= kOz64MinElems && m * n <= (int64_t(1) << 32);
-}
+// when A is large enough that a product is not all launch latency (4096 x 256, 8 lambda: 20 us from
+// digits, 37 on the float64 pipe; a single lambda of 30000 x 1000: 105 us against 560, the pipe's
+// smallest tile being 8 rows); A of more than 2^32 elements keeps the float64 pipe, because the planes
+// take 16 bytes per element.
+bool oz64_wanted(int64_t m, int64_t n) { return m * n >= kOz64MinElems && m * n <= (int64_t(1) << 32); }
 
 tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
   if (!p) return einval("problem pointer is NULL");
@@ -130,7 +129,7 @@ tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
               (P.dt == TK_F64 || P.lda % 4 == 0);
   P.lsqr_oz = P.mixed && (o->lsqr_tc == 2 || o->lsqr_tc == 3) && o->emulate_fp64 && !P.under;
   P.lsqr_fused = P.lsqr_oz && o->lsqr_tc == 3;
-  P.oz64 = !P.mixed && o->emulate_fp64 && oz64_wanted(P.m, P.n, P.N_cap);
+  P.oz64 = !P.mixed && o->emulate_fp64 && oz64_wanted(P.m, P.n);
   return TK_OK;
 }
 
@@ -202,8 +201,18 @@ OzMat oz_mat(const Plan& P, const Bufs& B) {
   return A;
 }
 
+// The float64 form's Gaussian sketch from the digit planes of A (2 s L c flops on the float64 pipe
+// otherwise: 462 x 30000 x 1000 takes 31 ms there, 1.6 ms from digits).
+bool oz_gauss(const Plan& P) { return P.oz64 && P.o.sketch == TK_SKETCH_GAUSS && P.s <= 65535; }
+
 size_t sketch_scratch(const Plan& P) {
   tk_dtype dt = P.mixed ? TK_F32 : P.dt;
+  if (oz_gauss(P)) {
+    Arena a;
+    a.take<double>((size_t)P.s * P.L);
+    a.take<char>(oz_sketch_workspace(P.L, P.c, P.s));
+    return a.used + 512;
+  }
   if (tc_sketch(P)) return tc_sketch_workspace(P.L, P.c, P.s);
   if (P.o.sketch == TK_SKETCH_SRHT) return srht_rows_workspace(P.L, P.c, dt, P.s);
   if (P.o.sketch == TK_SKETCH_SPARSE) return sparse_rows_workspace(P.L, P.c, P.s);
@@ -413,6 +422,17 @@ inline dim3 rgrid(int64_t len, int rows) {
 tk_status do_sketch(const Plan& P, const void* A_sk, tk_dtype dt_sk, int64_t ld_sk, Bufs& B, cudaStream_t st) {
   const void* src = A_sk;
   int64_t ld = ld_sk;
+  if (oz_gauss(P)) {
+    Arena sa;
+    sa.base = B.scratch;
+    sa.cap = B.scratch_bytes;
+    double* G = sa.take<double>((size_t)P.s * P.L);
+    const size_t wb = oz_sketch_workspace(P.L, P.c, P.s);
+    char* w = sa.take<char>(wb);
+    if (!sa.ok()) return TK_ENOMEM;
+    TK_TRY(gauss_fill(P.o.seed, P.s, P.L, G, st));
+    return oz_sketch(oz_mat(P, B), P.under, G, P.s, B.Y, w, wb, B.oz_err, st);
+  }
   if (P.under) {
     TK_TRY(transpose(A_sk, dt_sk, P.m, P.n, ld_sk, B.AT, st));
     src = B.AT;
@@ -517,6 +537,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
   // A is split once, for every product of the solve (x, r and the LSQR vectors on every pass); the
   // first pass over a float64 A also writes the float32 copy of the mixed form
   const bool digits = (P.mixed && P.o.emulate_fp64 && !P.prep_only) || P.oz64;
+  if (digits) TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));
   if (digits && !reuse) {
     float* copy = P.mixed && P.dt == TK_F64 ? B.A32 : nullptr;
     const int tok = prof_begin(TK_PHASE_SLICE, st);
@@ -565,7 +586,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
   std::vector<int> ok_ids;
   if (!P.lowrank) {
     int tok = -1;
-    if (emulated_gram(P)) TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));
+    if (emulated_gram(P) && !digits) TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));  // grouped build
     if (!reuse && !P.qr) {
       tok = prof_begin(TK_PHASE_GRAM, st);
       if (emulated_gram(P)) {  // the Cholesky reads only j >= i
@@ -686,7 +707,6 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
     e.A = A64; e.lda = lda64; e.st = st; e.atol = e.btol = P.o.tol; e.maxiter = P.o.maxiter;
     e.a_es = P.dt == TK_F64 ? 8.0 : 4.0;
     if (P.oz64) {
-      TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));
       e.oz_A = oz_mat(P, B);
       e.oz_err = B.oz_err;
     }
@@ -758,7 +778,6 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
     std::vector<double> hn(3 * std::max(N, 1));
     std::vector<double> prev_dn(std::max(N, 1), INFINITY);
     if (P.o.emulate_fp64 && !act.empty()) {
-      TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));
       if (P.lsqr_oz) {  // the LSQR products read the first 4 digits of the same planes
         e.oz_A = oz_mat(P, B);
         e.oz_err = B.oz_err;

@@ -181,6 +181,7 @@ size_t srht_rows_workspace(int64_t L, int64_t cols, tk_dtype dt, int64_t s);
 tk_status gauss_rows(const void* A, tk_dtype dt, int64_t L, int64_t cols, int64_t ld, uint64_t seed, int64_t s,
                      double* Y, Arena& ar, cudaStream_t st);
 size_t gauss_rows_workspace(int64_t L, int64_t cols, tk_dtype dt, int64_t s);
+tk_status gauss_fill(uint64_t seed, int64_t s, int64_t L, double* G, cudaStream_t st);  // the s x L embedding itself
 // SRDCT (tk_sketch.cu): X = sqrt(Lp/s) S C D [I; 0], C the orthonormal DCT-II of length Lp.
 tk_status srdct_rows(const void* A, tk_dtype dt, int64_t L, int64_t cols, int64_t ld, uint64_t seed, int64_t s,
                      double* Y, Arena& ar, cudaStream_t st);
@@ -316,6 +317,12 @@ tk_status lm_small_aw(const float* A, int64_t lda, int64_t m, int64_t n, const f
 int lm_small_atu_splits(int64_t m, int64_t n);
 tk_status lm_small_atu(const float* A, int64_t lda, int64_t m, int64_t n, const float* U, int64_t ldu, int count,
                        double* partial, int splits, cudaStream_t st);
+// Y (s x c) = G A (m >= n: G s x m, c = n) or G A^T (under: G s x n, c = m) for an embedding G (float64,
+// s <= 65535) from the digit planes of A, float64-accurate; work: oz_sketch_workspace(L, c, s) bytes, L the
+// length of G's rows.
+size_t oz_sketch_workspace(int64_t L, int64_t c, int64_t s);
+tk_status oz_sketch(const OzMat& A, bool under, const double* G, int64_t s, double* Y, void* work, size_t bytes,
+                    int* err, cudaStream_t st);
 // C = Y^T Y (Y: r x c float64, row stride c), the upper triangle (j >= i) of
 // C (c x c) written, float64-accurate; work: oz_gram_workspace(r, c) bytes.
 size_t oz_gram_workspace(int64_t r, int64_t c);

@@ -437,7 +437,8 @@ tk_status Lsqr<T>::apply_prec(bool transposed, const T* in, T* out, int count, i
   }
   // Low rank: out = l^{-1/2}(in - V S V^T in); symmetric, so transposed is the same.
   int tok = prof_begin(TK_PHASE_PRECOND, st);
-  tk_status r = lr_apply<T>(count, len, lr_s, lrV, lrS, slot_lam, lam_all, in, out, lr_tmp, lr_inv, st);
+  tk_status r = lr_apply<T>(count, len, lr_s, lrV, lrS, slot_lam, lam_all, in, out, lr_tmp, lr_inv, part_g,
+                              (int64_t)splits * N_cap * n, st);
   prof_end(tok, st, 4.0 * count * len * lr_s, es * (len * lr_s + 2.0 * count * len));
   return r;
 }
@@ -609,7 +610,8 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
           if (Mi) TK_TRY(trmv_batched<T>(false, n, Mi, Mti, ldm, mstride, d_src, Vraw, xtmp, n, nr, st));
           else TK_TRY((trsv_batched<T, T>(false, n, R, ldr, rstride, d_src, Vraw, xtmp, n, nr, trsv_p, st)));
         } else {
-          TK_TRY(lr_apply<T>(nr, n, lr_s, lrV, lrS, d_src, lam_all, Vraw, xtmp, lr_tmp, lr_inv, st));
+          TK_TRY(lr_apply<T>(nr, n, lr_s, lrV, lrS, d_src, lam_all, Vraw, xtmp, lr_tmp, lr_inv, part_g,
+                                (int64_t)splits * N_cap * n, st));
         }
         xs = xtmp;
       }

@@ -23,10 +23,12 @@ struct LsqrResult {
 
 // Low-rank preconditioner apply (Section 3.1, eq. for R^-1):
 // out_k = l^{-1/2} (in_k - V diag(S_l) V^T in_k) for each listed row k, with
-// l = lam_idx[k]; V is n x s (row-major), S is N_lam x s (zero past s_l).
+// l = lam_idx[k]; V is n x s (row-major), S is N_lam x s (zero past s_l); part: part_len >= count s doubles of
+// scratch (the split sums of V^T in).
 template <typename T>
 tk_status lr_apply(int count, int64_t n, int64_t s, const T* V, const T* S, const int* lam_idx,
-                   const double* lam_dev, const T* in, T* out, T* tmp, double* invs, cudaStream_t st);
+                   const double* lam_dev, const T* in, T* out, T* tmp, double* invs, double* part, int64_t part_len,
+                   cudaStream_t st);
 
 // sd_i, s_i of Algorithm 3 step 5 (device in/out) and the S_i rows (step 7).
 tk_status lowrank_ranks_dev(const double* sigma, int64_t s, const double* lam_dev, int N, double alpha,
@@ -214,10 +216,11 @@ struct Lsqr {
   // A digit product reads 8 (float32 engine) or 16 bytes (float64) per element of A whatever the
   // number of lambdas; the SIMT products read 4 or 8 bytes but their work grows with it.  Float32: the
   // digits pay off for large A and more than 16 active lambdas.  Float64: the pipe (1.2 TFLOP/s) takes
-  // 1.7 ps per element and lambda against the digits' 2.7 ps per element, so from two lambdas on.
+  // 1.7 ps per element and lambda, the digits 2.7 ps per element, and the pipe's smallest tile does the
+  // work of 8 lambdas: always.
   bool use_oz(int count) const {
     if (!oz || !oz_A.planes) return false;
-    if (std::is_same<T, double>::value) return count >= 2;
+    if (std::is_same<T, double>::value) return true;
     return (int64_t)m * n > (int64_t(1) << 24) && count > 16;
   }
   // both products of an overdetermined step in one kernel over one read of

@@ -1762,6 +1762,55 @@ tk_status oz_lsqr_fused(const OzMat& A, const float* W, int64_t ldw, int count, 
   return TK_OK;
 }
 
+static int oz_sketch_splits(int64_t L, int64_t c, int64_t s) {
+  const int64_t tiles = cdiv(c, OT_M) * cdiv(s, OT_N);
+  return tiles >= 152 ? (int)cdiv(L, OT_MAX_KPS) : oz_normal_splits(L, c, s);
+}
+__global__ void k_oz_sum_planes(const double* __restrict__ part, int splits, int64_t total, double* __restrict__ Y) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
+    double acc = 0.0;
+#pragma unroll 4
+    for (int z = 0; z < splits; ++z) acc += part[(int64_t)z * total + k];
+    Y[k] = acc;
+  }
+}
+
+size_t oz_sketch_workspace(int64_t L, int64_t c, int64_t s) {
+  Arena a;
+  a.take<char>(oz_slices_bytes(s, L));
+  a.take<int>(s);
+  const int sp = oz_sketch_splits(L, c, s);
+  if (sp > 1) a.take<double>((size_t)sp * s * c);
+  return a.used + 256;
+}
+
+tk_status oz_sketch(const OzMat& A, bool under, const double* G, int64_t s, double* Y, void* work, size_t bytes,
+                    int* err, cudaStream_t st) {
+  const int64_t L = under ? A.n : A.m, c = under ? A.m : A.n;
+  if (s == 0 || c == 0) return TK_OK;
+  Arena a;
+  a.base = static_cast<char*>(work);
+  a.cap = bytes;
+  void* Gs = a.take<char>(oz_slices_bytes(s, L));
+  int* E = a.take<int>(s);
+  const int sp = oz_sketch_splits(L, c, s);
+  double* part = sp > 1 ? a.take<double>((size_t)sp * s * c) : nullptr;
+  if (!a.ok()) return TK_ENOMEM;
+  TK_TRY(oz_split_vectors(G, TK_F64, s, L, L, under ? A.EC : A.ER, Gs, E, st));
+  double* out = sp > 1 ? part : Y;
+  if (under)
+    TK_TRY((launch_oz_tc<OZ_S, 1, false>({A.planes, A.ER, A.m, A.n, false}, Gs, E, (int)s, OZ_S, sp, nullptr, out, c,
+                                         nullptr, err, st)));
+  else
+    TK_TRY((launch_oz_tc<OZ_S, 1, true>({A.planes, A.EC, A.n, A.m, true}, Gs, E, (int)s, OZ_S, sp, nullptr, out, c,
+                                        nullptr, err, st)));
+  if (sp > 1) {
+    k_oz_sum_planes<<<(unsigned)std::min<int64_t>(cdiv(s * c, 256), 152 * 8), 256, 0, st>>>(part, sp, s * c, Y);
+    TK_LAUNCH_CHECK();
+  }
+  return TK_OK;
+}
+
 size_t oz_gram_workspace(int64_t r, int64_t c) {
   Arena a;
   a.take<char>(oz_slices_bytes(c, r));

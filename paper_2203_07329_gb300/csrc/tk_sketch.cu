@@ -537,6 +537,13 @@ tk_status srht_rows(const void* A, tk_dtype dt, int64_t L, int64_t cols, int64_t
   return srht_impl<float, float>((const float*)A, L, cols, ld, seed, s, Y, ar, st);
 }
 
+tk_status gauss_fill(uint64_t seed, int64_t s, int64_t L, double* G, cudaStream_t st) {
+  if (s * L == 0) return TK_OK;
+  k_gauss_fill<double><<<grid_for(s * L, 256), 256, 0, st>>>(seed, s, L, 1.0 / sqrt((double)s), G);
+  TK_LAUNCH_CHECK();
+  return TK_OK;
+}
+
 tk_status gauss_rows(const void* A, tk_dtype dt, int64_t L, int64_t cols, int64_t ld, uint64_t seed, int64_t s,
                      double* Y, Arena& ar, cudaStream_t st) {
   if (dt == TK_F64) return gauss_impl<double, double>((const double*)A, L, cols, ld, seed, s, Y, ar, st);

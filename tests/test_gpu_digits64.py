@@ -18,7 +18,7 @@ def _solve(A, b, lams, **kw):
 # A at and around the smallest size that is split into digits (2^19 elements), ragged against the 64-,
 # 128- and 256-value tiles, one and several tiles of 32 lambdas, float64 views with odd row strides,
 # and m < n with vectors of 1, 2, 4 and 8 CTAs per v-step.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
-@pytest.mark.parametrize("m,n,N,pad", [(8192, 64, 2, 0), (8193, 65, 3, 1), (2051, 257, 33, 0), (1500, 700, 5, 3),
+@pytest.mark.parametrize("m,n,N,pad", [(8192, 64, 2, 0), (8192, 65, 1, 0), (8193, 65, 3, 1), (2051, 257, 33, 0), (1500, 700, 5, 3),
                                        (16500, 40, 4, 0), (129, 4099, 4, 0), (500, 1100, 34, 5), (63, 8400, 2, 0),
                                        (101, 17001, 3, 0)])
 def test_digit_solve_matches_float64_pipe(m, n, N, pad):
@@ -69,3 +69,18 @@ def test_non_finite_a_is_enumeric_from_digits():
     r = tk.tk_solve(A.cuda(), b, [1e-2, 1.0], tk.opts_default(sketch=tk.TK_SKETCH_SRHT, s=280),
                     allow=tuple(range(8)))
     assert r.status == tk.TK_ENUMERIC
+
+
+# the low-rank preconditioner's apply over slot counts around its groups of 8 slots, ragged rows and columns, and
+# more sketch rows than fit in shared memory with 8 slots (s > 2560): the same solutions as with the Cholesky one
+@pytest.mark.parametrize("m,n,s,N", [(3000, 301, 97, 1), (5001, 333, 120, 9), (2500, 257, 64, 17), (6000, 2600, 2570, 3)])
+def test_lowrank_apply_shapes(m, n, s, N):
+    p = datagen.make_ridge_problem(m, n, datagen.spectrum("exp", n, tau=n / 40.0), datagen.log_lambdas(N, 1e-3, 1.0),
+                                   seed=m)
+    A, b, lams = p.A.cuda(), p.b.cuda(), p.lambdas.numpy()
+    r1 = _solve(A, b, lams, sketch=tk.TK_SKETCH_GAUSS, s=s, precond=tk.TK_PRECOND_LOWRANK)
+    r0 = _solve(A, b, lams, sketch=tk.TK_SKETCH_GAUSS, s=min(4 * n, m), emulate_fp64=0)
+    for i in range(N):
+        e = float((r1.X[i] - r0.X[i]).norm() / r0.X[i].norm())
+        assert e < 1e-10, (lams[i], e)
+        assert r1.info[i]["status"] == 0
