@@ -1121,6 +1121,8 @@ tk_status batch_layout(const tk_problem* ps, int P, int N, const tk_opts* o, int
     gp[i].m = pl[i].m;
     gp[i].n = pl[i].n;
     gp[i].emulate = pl[i].o.emulate_fp64 ? 1 : 0;  // the digit scratch of the float64 passes
+    gp[i].lowrank = pl[i].lowrank;
+    gp[i].lr_s = pl[i].lowrank ? pl[i].s : 0;
   }
   L.scratch_off = off;
   off += L.scratch_per * (size_t)L.lanes;

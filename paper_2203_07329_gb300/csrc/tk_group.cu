@@ -5,14 +5,19 @@
 // 0..nact_p-1 contiguous (a retired slot is refilled by the problem's last
 // active one), lambda-major as in the single-problem engine.  One launch per
 // phase covers all problems:
-//   * the two float32 products with A run over a tile list (problem, column
-//     tile[, K split]); a tile multiplies every active lambda of its problem
-//     (the lambda-major tile body shared with the single-problem GEMM),
-//   * the per-slot kernels (norms, Golub-Kahan scalars, preconditioner apply)
+//   * the two float32 products with A run over a tile list (problem, rows of A;
+//     or columns and rows); a tile multiplies every active lambda of its problem:
+//     at most 16 with the bodies of tk_lm_body.cuh (the lambda-side operand on
+//     chip), more with the lambda-major tile body of the single-problem GEMM.
+//     The lists are rebuilt as slots retire, so that the problems still running
+//     always fill the GPU: the last of 16 problems (49060 x 210, 800 steps) ran
+//     its A^T U on 12 CTAs, 337 us a step, now 10,
+//   * the low-rank applies use the same bodies on V (n x s),
+//   * the per-slot kernels (norms, Golub-Kahan scalars, triangular applies)
 //     run over a slot list (problem, slot),
 //   * the float64 refinement passes (r = b - A x and A^T r - lambda x) run
 //     over tile lists of the generic GEMM tile body.
-// The host reads one small report per step to retire converged slots.
+// The host reads one small report per step (every 4 steps once they are short) to retire converged slots.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -21,6 +26,7 @@
 
 #include "tk_gemm_tiles.cuh"
 #include "tk_group.cuh"
+#include "tk_lm_body.cuh"
 #include "tk_lsqr.cuh"
 
 namespace tk {
@@ -30,6 +36,10 @@ constexpr int kThreads = 256;
 constexpr int64_t kKps = 4096;    // rows of A per K split of the float32 A^T U product
 constexpr int64_t kKps64 = 4096;  // rows of A per K split of the float64 A^T r pass
 constexpr int kBM64 = 32, kBN64 = 128;
+constexpr int kBetaChunks = 32;                // most blocks of a slot's norm
+constexpr int kSmallLambda = 16;               // products with at most 16 lambda: tk_lm_body.cuh
+constexpr size_t kAwSmem = 64 * 1024;          // W's column chunk of a k_g_aw block (3 blocks per SM)
+constexpr int kTargetTiles = 152 * 6;          // tiles of a product: 3 resident blocks per SM, 2 waves
 
 struct GDesc {
   int64_t m, n;
@@ -52,8 +62,8 @@ struct GDesc {
   int maxiter;
   // slot storage: row k of each N x n (or N x m) block belongs to local slot k
   float *V, *W, *Y, *Vraw, *Tt, *Ub, *Xt, *Ut;
-  double* part;  // splits x nact x n  (float32 A^T U partial sums)
-  int splits;
+  double* part;  // nsp x nact x n  (float32 A^T U partial sums)
+  float* lrT;    // low rank: N x s, the scaled V^T x
   double* coef;
   Scal* sc;
   int* slot_lam;
@@ -68,8 +78,8 @@ struct GDesc {
 struct GSlot {
   int p, k;
 };
-struct GTile {
-  int p, z, m0, pad;
+struct GTile {  // float64 passes: z, m0, n0 as k_g_gemm64; products: see k_g_aw, k_g_atu, k_g_lm
+  int p, z, m0, nl;
   int64_t n0;
 };
 struct GReport {
@@ -148,46 +158,84 @@ __global__ void __launch_bounds__(kThreads) k_g_init_beta(const GDesc* __restric
   }
 }
 
-// Tt = (sum_z part_z + sqrt(l) Ub) / beta   (the normalized A^T u part of M^T u)
-__global__ void k_g_over_g(const GDesc* __restrict__ Dd, const int* __restrict__ nact, const GSlot* __restrict__ sl) {
+// Tt = (sum_z part_z + sqrt(l) Ub) / beta   (the normalized A^T u part of M^T u); blocks of 32 columns x 8
+// groups of planes
+__global__ void __launch_bounds__(256)
+    k_g_over_g(const GDesc* __restrict__ Dd, const int* __restrict__ nact, const int* __restrict__ nsp,
+               const GSlot* __restrict__ sl) {
+  __shared__ double sh[8][33];
   const GSlot q = sl[blockIdx.y];
   const GDesc& d = Dd[q.p];
-  const double sq = d.sc[q.k].sqrtl, beta = d.sc[q.k].beta;
-  const double inv = beta > 0.0 ? 1.0 / beta : 0.0;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t j = (int64_t)blockIdx.x * 32 + tx;
+  if ((int64_t)blockIdx.x * 32 >= d.n) return;
   const int64_t plane = (int64_t)nact[q.p] * d.n;
-  const float* ub = d.Ub + (int64_t)q.k * d.n;
-  float* tt = d.Tt + (int64_t)q.k * d.n;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int z = 0; z < d.splits; ++z) acc += d.part[z * plane + (int64_t)q.k * d.n + j];
-    acc = fma(sq, (double)ub[j], acc);
-    tt[j] = (float)(acc * inv);
+  const int splits = nsp[q.p];
+  double acc = 0.0;
+  if (j < d.n) {
+    const double* p = d.part + (int64_t)q.k * d.n + j;
+#pragma unroll 4
+    for (int z = ty; z < splits; z += 8) acc += p[z * plane];
+  }
+  sh[ty][tx] = acc;
+  __syncthreads();
+  if (ty == 0 && j < d.n) {
+    const double sq = d.sc[q.k].sqrtl, beta = d.sc[q.k].beta;
+    const double inv = beta > 0.0 ? 1.0 / beta : 0.0;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) acc += sh[k][tx];
+    acc = fma(sq, (double)d.Ub[(int64_t)q.k * d.n + j], acc);
+    d.Tt[(int64_t)q.k * d.n + j] = (float)(acc * inv);
   }
 }
 
-// Ub = sqrt(l) Tt + coef Ub;  beta = ||[Ut; Ub]||;  anorm2 += alpha^2 + beta^2
-__global__ void __launch_bounds__(kThreads) k_g_beta(const GDesc* __restrict__ Dd, const GSlot* __restrict__ sl) {
+// Ub = sqrt(l) Tt + coef Ub;  beta = ||[Ut; Ub]||;  anorm2 += alpha^2 + beta^2: gridDim.x blocks to a slot,
+// the last to arrive adds their sums (as k_over_norm; arrivals and partial are indexed by the slot's
+// place in the list, arrivals zero on entry and left zero).
+__global__ void __launch_bounds__(kThreads)
+    k_g_beta(const GDesc* __restrict__ Dd, const GSlot* __restrict__ sl, double* __restrict__ partial,
+             int* __restrict__ arrivals) {
   __shared__ double sh[32];
-  const GSlot q = sl[blockIdx.x];
+  __shared__ int last;
+  const GSlot q = sl[blockIdx.y];
   const GDesc& d = Dd[q.p];
+  const int c = blockIdx.x, chunks = gridDim.x;
+  if (d.sc[q.k].istop != 0) return;  // retired inside a chunk of steps
   const double sq = d.sc[q.k].sqrtl, coef = d.sc[q.k].coef;
   const float* ut = d.Ut + (int64_t)q.k * d.m;
   const float* tt = d.Tt + (int64_t)q.k * d.n;
   float* ub = d.Ub + (int64_t)q.k * d.n;
   double acc = 0.0;
-  for (int64_t i = threadIdx.x; i < d.m; i += blockDim.x) acc = fma((double)ut[i], (double)ut[i], acc);
-  for (int64_t j = threadIdx.x; j < d.n; j += blockDim.x) {
-    const float v = (float)fma(sq, (double)tt[j], coef * (double)ub[j]);
-    ub[j] = v;
-    acc = fma((double)v, (double)v, acc);
+  {
+    const int64_t per = cdiv(d.m, chunks), b = c * per, e = b + per < d.m ? b + per : d.m;
+#pragma unroll 4
+    for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) acc = fma((double)ut[i], (double)ut[i], acc);
+  }
+  {
+    const int64_t per = cdiv(d.n, chunks), b = c * per, e = b + per < d.n ? b + per : d.n;
+    for (int64_t j = b + threadIdx.x; j < e; j += blockDim.x) {
+      const float v = (float)fma(sq, (double)tt[j], coef * (double)ub[j]);
+      ub[j] = v;
+      acc = fma((double)v, (double)v, acc);
+    }
   }
   acc = block_sum(acc, sh);
   if (threadIdx.x == 0) {
-    const double beta = sqrt(acc);
-    Scal z = d.sc[q.k];
-    z.anorm2 += z.alpha * z.alpha + beta * beta;
-    z.beta = beta;
-    d.sc[q.k] = z;
+    partial[blockIdx.y * kBetaChunks + c] = acc;
+    __threadfence();
+    last = atomicAdd(&arrivals[blockIdx.y], 1) == chunks - 1;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  __threadfence();
+  double t = threadIdx.x < chunks ? *(volatile double*)&partial[blockIdx.y * kBetaChunks + threadIdx.x] : 0.0;
+  t = warp_sum(t);
+  if (threadIdx.x == 0) {
+    Scal* z = d.sc + q.k;
+    const double beta = sqrt(t);
+    z->anorm2 += z->alpha * z->alpha + beta * beta;
+    z->beta = beta;
+    arrivals[blockIdx.y] = 0;
   }
 }
 
@@ -227,52 +275,121 @@ __global__ void __launch_bounds__(256)
                                  field(d, fdst) + (int64_t)q.k * d.n, i0, g_trmv_v4);
 }
 
-// Low-rank problems (Section 3.1): out = l^{-1/2} (x - V diag(S_l) V^T x),
-// symmetric, one CTA per slot; x and t = S_l V^T x / sqrt(l) in shared memory.
-__global__ void __launch_bounds__(256)
-    k_g_lr(const GDesc* __restrict__ Dd, const GSlot* __restrict__ sl, int fsrc, int fdst) {
-  extern __shared__ float g_lr_sm[];
-  const GSlot q = sl[blockIdx.x];
-  const GDesc& d = Dd[q.p];
-  if (!d.lowrank) return;
-  const int64_t n = d.n, s = d.lr_s;
-  const int l = d.slot_lam[q.k];
-  const float* x = field(d, fsrc) + (int64_t)q.k * n;
-  float* y = field(d, fdst) + (int64_t)q.k * n;
-  float* xs = g_lr_sm;
-  float* t = g_lr_sm + n;
-  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) xs[j] = x[j];
-  __syncthreads();
-  const double is = 1.0 / sqrt(d.lam[l]);
-  const float* V = d.lrV;
-  const float* S = d.lrS + (int64_t)l * s;
-  for (int64_t c = threadIdx.x; c < s; c += blockDim.x) {
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    int64_t i = 0;
-    for (; i + 3 < n; i += 4) {
-      a0 = fmaf(V[i * s + c], xs[i], a0);
-      a1 = fmaf(V[(i + 1) * s + c], xs[i + 1], a1);
-      a2 = fmaf(V[(i + 2) * s + c], xs[i + 2], a2);
-      a3 = fmaf(V[(i + 3) * s + c], xs[i + 3], a3);
-    }
-    for (; i < n; ++i) a0 = fmaf(V[i * s + c], xs[i], a0);
-    const float a = (a0 + a1) + (a2 + a3);
-    t[c] = (float)((double)a * (double)S[c] * is);
+// ---- the products over tile lists ---------------------------------------------
+// Ut = Tt A^T + coef .* Ut (LR = false) or, for low-rank problems (Section 3.1: out = l^{-1/2} (x - V
+// diag(S_l) V^T x)), dst = x / sqrt(l) - t V^T with t = lrT: tile = problem, rows n0 .. n0 + m0 - 1 of A
+// (or V); W (or t) in shared memory in chunks of columns.
+struct LrStore {
+  const float* x;
+  float* y;
+  int64_t n;
+  const double* lam;
+  const int* slot_lam;
+  bool first;
+  __device__ __forceinline__ void operator()(int l, int64_t i, float v) const {
+    float* o = y + (int64_t)l * n + i;
+    *o = first ? (float)((double)x[(int64_t)l * n + i] / sqrt(lam[slot_lam[l]]) - (double)v) : *o - v;
   }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int64_t i = w; i < n; i += nw) {
-    float acc = 0.f;
-    for (int64_t c = lane; c < s; c += 32) acc = fmaf(V[i * s + c], t[c], acc);
-    acc = warp_sum(acc);
-    if (lane == 0) y[i] = (float)(-(double)acc + is * (double)xs[i]);
+};
+// slots l0 .. l0 + M - 1 (M <= NL)
+template <int NL, bool LR>
+__device__ __forceinline__ void g_aw_tile(const GDesc& d, int l0, int M, int64_t r0, int64_t r1, int fsrc, int fdst,
+                                          float* ws) {
+  const float* A = LR ? d.lrV : d.A32;
+  const int64_t lda = LR ? d.lr_s : d.lda32, cols = LR ? d.lr_s : d.n, rows = LR ? d.n : d.m;
+  const float* W = (LR ? d.lrT : d.Tt) + l0 * cols;
+  const bool vec = ((uintptr_t)A % 16 == 0) && (lda % 4 == 0);
+  const int64_t fit = (int64_t)kAwSmem / (4 * NL) / 128 * 128;
+  const int64_t gb = r0 / lmb::kRows, ge = (r1 + lmb::kRows - 1) / lmb::kRows;
+  for (int64_t k0 = 0; k0 < cols; k0 += fit) {
+    const int64_t len = cols - k0 < fit ? cols - k0 : fit;
+    const int64_t n_pad = (len + 127) / 128 * 128;
+    __syncthreads();
+    lmb::load_w<NL>(ws, W + k0, cols, M, len, n_pad);
+    __syncthreads();
+    const int64_t g0 = gb + (threadIdx.x >> 5);
+    if constexpr (LR)
+      lmb::aw_rows<NL>(ws, n_pad, A + k0, lda, rows, len, M,
+                       LrStore{field(d, fsrc) + l0 * d.n, field(d, fdst) + l0 * d.n, d.n, d.lam, d.slot_lam + l0,
+                               k0 == 0},
+                       vec, g0, 8, ge);
+    else
+      lmb::aw_rows<NL>(ws, n_pad, A + k0, lda, rows, len, M,
+                       lmb::AwStore{d.Ut + l0 * d.m, d.m, d.coef + l0, k0 == 0}, vec, g0, 8, ge);
+  }
+}
+template <bool LR>
+__global__ void __launch_bounds__(256, 2)
+    k_g_aw(const GDesc* __restrict__ Dd, const int* __restrict__ nact, const GTile* __restrict__ tl, int fsrc,
+           int fdst) {
+  extern __shared__ __align__(16) float g_ws[];
+  const GTile t = tl[blockIdx.x];
+  const int M = nact[t.p];
+  if (M == 0) return;
+  const GDesc& d = Dd[t.p];
+  const int64_t rows = LR ? d.n : d.m, r1 = t.n0 + t.m0 < rows ? t.n0 + t.m0 : rows;
+  if (M <= 4) {
+    g_aw_tile<4, LR>(d, 0, M, t.n0, r1, fsrc, fdst, g_ws);
+  } else if (M <= 8) {
+    g_aw_tile<8, LR>(d, 0, M, t.n0, r1, fsrc, fdst, g_ws);
+  } else {
+    for (int l0 = 0; l0 < M; l0 += 16)  // more than 16 only on V
+      g_aw_tile<16, LR>(d, l0, M - l0 < 16 ? M - l0 : 16, t.n0, r1, fsrc, fdst, g_ws);
   }
 }
 
-// ---- the two products with A, over tile lists --------------------------------
-// TRANSB: Ut = Tt A^T + coef .* Ut (tile = problem, 256 rows of A).
-// else:   part_z = Ut A over rows [z kKps, (z+1) kKps) (tile = problem, 256
-//         columns, split z).
+// part_z = Ut A (LR = false) or x V: tile = problem, split z of m0 rows, columns from n0 (1024 of them,
+// or 512 for nl = 16: the list's lambda class, which the active count does not exceed).
+template <int NL, int CW, bool LR>
+__device__ __forceinline__ void g_atu_tile(const GDesc& d, int l0, int M, int Mall, const GTile& t, int fsrc,
+                                           void* sm) {
+  const float* A = LR ? d.lrV : d.A32;
+  const int64_t lda = LR ? d.lr_s : d.lda32, cols = LR ? d.lr_s : d.n, rows = LR ? d.n : d.m;
+  const bool vec = ((uintptr_t)A % 16 == 0) && (lda % 4 == 0);
+  const int64_t rb = (int64_t)t.z * t.m0, re = rb + t.m0 < rows ? rb + t.m0 : rows;
+  lmb::atu_cols<NL, CW>(*reinterpret_cast<lmb::AtuSmem<NL, CW>*>(sm), A, lda, cols,
+                        (LR ? field(d, fsrc) : d.Ut) + l0 * rows, rows, M, rb, re, t.n0,
+                        d.part + ((int64_t)t.z * Mall + l0) * cols, vec);
+}
+template <bool LR>
+__global__ void __launch_bounds__(256, 3)
+    k_g_atu(const GDesc* __restrict__ Dd, const int* __restrict__ nact, const GTile* __restrict__ tl, int fsrc) {
+  constexpr size_t kSm = sizeof(lmb::AtuSmem<8, 4>) > sizeof(lmb::AtuSmem<16, 2>) ? sizeof(lmb::AtuSmem<8, 4>)
+                                                                                  : sizeof(lmb::AtuSmem<16, 2>);
+  __shared__ __align__(16) unsigned char sm[kSm];
+  const GTile t = tl[blockIdx.x];
+  const int M = nact[t.p];
+  if (M == 0) return;
+  const GDesc& d = Dd[t.p];
+  if (t.nl == 4) {
+    g_atu_tile<4, 4, LR>(d, 0, M, M, t, fsrc, sm);
+  } else if (t.nl == 8) {
+    g_atu_tile<8, 4, LR>(d, 0, M, M, t, fsrc, sm);
+  } else {
+    for (int l0 = 0; l0 < M; l0 += 16)  // more than 16 only on V
+      g_atu_tile<16, 2, LR>(d, l0, M - l0 < 16 ? M - l0 : 16, M, t, fsrc, sm);
+  }
+}
+
+// t = S_l (V^T x) / sqrt(l) of a slot, from the split sums
+__global__ void __launch_bounds__(256)
+    k_g_lr_t(const GDesc* __restrict__ Dd, const int* __restrict__ nact, const int* __restrict__ nsp,
+             const GSlot* __restrict__ sl) {
+  const GSlot q = sl[blockIdx.y];
+  const GDesc& d = Dd[q.p];
+  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (!d.lowrank || j >= d.lr_s) return;
+  const int l = d.slot_lam[q.k];
+  const int64_t plane = (int64_t)nact[q.p] * d.lr_s;
+  const int splits = nsp[q.p];
+  double acc = 0.0;
+#pragma unroll 4
+  for (int z = 0; z < splits; ++z) acc += d.part[z * plane + (int64_t)q.k * d.lr_s + j];
+  d.lrT[(int64_t)q.k * d.lr_s + j] = (float)(acc * (double)d.lrS[(int64_t)l * d.lr_s + j] / sqrt(d.lam[l]));
+}
+
+// The lambda-major tiles (more than 16 lambda): TRANSB: Ut = Tt A^T + coef .* Ut (tile = problem, 256
+// rows of A); else part_z = Ut A over rows [z kKps, (z+1) kKps) (tile = problem, 256 columns, split z).
 template <bool TRANSB, int BM, int TM>
 __global__ void __launch_bounds__(256)
     k_g_lm(const GDesc* __restrict__ Dd, const int* __restrict__ nact, const GTile* __restrict__ tl) {
@@ -412,7 +529,7 @@ inline dim3 chunk_grid(int64_t len, int rows) {
 
 // ---- host side ---------------------------------------------------------------------
 struct Sizes {
-  int splits = 1, splits64 = 1;
+  int splits = 1, splits64 = 1;  // planes of part (N slots; more while fewer slots are active)
 };
 
 Sizes sizes_of(const GroupProblem& g) {
@@ -437,8 +554,16 @@ struct GState {
   GSlot* rslots = nullptr;  // retiring slots
   GMove* moves = nullptr;
   GReport* rep = nullptr;
-  GTile* t_aw = nullptr;
+  GTile* t_aw = nullptr;   // more than 16 lambda
   GTile* t_atu = nullptr;
+  GTile* s_tiles = nullptr;  // at most 16: the aw, atu, and low-rank V^T x and V t lists, one after another
+  size_t s_cap = 0;
+  int s_n[4] = {0, 0, 0, 0};
+  size_t s_off[4] = {0, 0, 0, 0};
+  int* nsp = nullptr;        // planes of part per problem, of the A^T U and of the low-rank product
+  double* beta_part = nullptr;
+  int* arrivals = nullptr;
+  int64_t max_s = 0;
   GTile* t_64 = nullptr;  // per-round float64 tiles (residual, then normal equations)
   int n_aw = 0, n_atu = 0;
   size_t cap64 = 0;
@@ -489,8 +614,11 @@ void carve_group(const std::vector<GroupProblem>& g, int N, Arena& a, GState& S)
     d.Ub = a.take<float>(vn);
     d.Xt = a.take<float>(vn);
     d.Ut = a.take<float>((size_t)N * q.m);
-    d.splits = z.splits;
     d.part = a.take<double>((size_t)z.splits * vn);
+    if (q.lowrank) {
+      d.lrT = a.take<float>((size_t)N * q.lr_s);
+      S.max_s = std::max(S.max_s, q.lr_s);
+    }
     d.coef = a.take<double>(N);
     d.sc = a.take<Scal>(N);
     d.slot_lam = a.take<int>(N);
@@ -527,6 +655,14 @@ void carve_group(const std::vector<GroupProblem>& g, int N, Arena& a, GState& S)
   S.t_aw = a.take<GTile>(std::max<size_t>(naw, 1));
   S.t_atu = a.take<GTile>(std::max<size_t>(natu, 1));
   S.t_64 = a.take<GTile>(std::max<size_t>(n64, 1));
+  // the small lists: about kTargetTiles tiles each, a ragged one per problem and column tile, and the
+  // splits of 4096 rows that are never exceeded
+  S.s_cap = 8 * kTargetTiles;
+  for (int p = 0; p < P; ++p) S.s_cap += 8 + (size_t)(cdiv(g[p].m, 4096) + cdiv(g[p].n, 4096) + 4) * cdiv(g[p].n, 512);
+  S.s_tiles = a.take<GTile>(S.s_cap);
+  S.nsp = a.take<int>((size_t)2 * std::max(P, 1));
+  S.beta_part = a.take<double>(ns * kBetaChunks);
+  S.arrivals = a.take<int>(ns);
   S.cap64 = n64;
   for (int p = 0; p < P; ++p) {
     S.hd[p].ids = S.ids_all + (size_t)p * N;
@@ -548,21 +684,31 @@ void carve_group(const std::vector<GroupProblem>& g, int N, Arena& a, GState& S)
 
 // ---- launch helpers ----------------------------------------------------------------
 tk_status launch_lm(const GState& S, bool transb, cudaStream_t st) {
+  if (transb && S.s_n[0]) {
+    TK_CUDA(cudaFuncSetAttribute(k_g_aw<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAwSmem));
+    k_g_aw<false><<<S.s_n[0], 256, kAwSmem, st>>>(S.dd, S.nact, S.s_tiles + S.s_off[0], 0, 0);
+    TK_LAUNCH_CHECK();
+  }
+  if (!transb && S.s_n[1]) {
+    k_g_atu<false><<<S.s_n[1], 256, 0, st>>>(S.dd, S.nact, S.s_tiles + S.s_off[1], 0);
+    TK_LAUNCH_CHECK();
+  }
   const GTile* tl = transb ? S.t_aw : S.t_atu;
   const int nt = transb ? S.n_aw : S.n_atu;
   if (nt == 0) return TK_OK;
 #define TK_GLM(TRB, BMV, TMV) k_g_lm<TRB, BMV, TMV><<<nt, 256, 0, st>>>(S.dd, S.nact, tl)
-  if (S.BM == 16) { if (transb) TK_GLM(true, 16, 2); else TK_GLM(false, 16, 2); }
-  else if (S.BM == 32) { if (transb) TK_GLM(true, 32, 4); else TK_GLM(false, 32, 4); }
+  if (S.BM == 32) { if (transb) TK_GLM(true, 32, 4); else TK_GLM(false, 32, 4); }
   else { if (transb) TK_GLM(true, 64, 8); else TK_GLM(false, 64, 8); }
 #undef TK_GLM
   TK_LAUNCH_CHECK();
   return TK_OK;
 }
 
-// Preconditioner apply over a slot list (both kinds; each kernel skips the other's slots).
-tk_status launch_prec(const GState& S, bool transposed, const GSlot* sl, int nsl, int fsrc, int fdst,
-                      bool any_chol, bool any_lr, cudaStream_t st) {
+// Preconditioner apply over a slot list: the triangular products skip the low-rank problems' slots; the
+// low-rank apply covers every active slot of the low-rank problems (their tile lists), `all` being the
+// list of all active slots.
+tk_status launch_prec(const GState& S, bool transposed, const GSlot* sl, int nsl, const GSlot* all, int nall, int fsrc,
+                      int fdst, bool any_chol, cudaStream_t st) {
   if (nsl == 0) return TK_OK;
   if (any_chol) {
     const dim3 grid((unsigned)cdiv(S.maxn, tiles::kTrmvRows), (unsigned)nsl);
@@ -571,8 +717,13 @@ tk_status launch_prec(const GState& S, bool transposed, const GSlot* sl, int nsl
     else k_g_trmv<false><<<grid, 256, smem, st>>>(S.dd, sl, fsrc, fdst);
     TK_LAUNCH_CHECK();
   }
-  if (any_lr) {
-    k_g_lr<<<nsl, 256, sizeof(float) * 2 * (size_t)S.maxn, st>>>(S.dd, sl, fsrc, fdst);
+  if (S.s_n[2]) {
+    k_g_atu<true><<<S.s_n[2], 256, 0, st>>>(S.dd, S.nact, S.s_tiles + S.s_off[2], fsrc);
+    TK_LAUNCH_CHECK();
+    k_g_lr_t<<<dim3((unsigned)cdiv(S.max_s, 256), (unsigned)nall), 256, 0, st>>>(S.dd, S.nact, S.nsp + S.P, all);
+    TK_LAUNCH_CHECK();
+    TK_CUDA(cudaFuncSetAttribute(k_g_aw<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAwSmem));
+    k_g_aw<true><<<S.s_n[3], 256, kAwSmem, st>>>(S.dd, S.nact, S.s_tiles + S.s_off[3], fsrc, fdst);
     TK_LAUNCH_CHECK();
   }
   return TK_OK;
@@ -603,32 +754,72 @@ tk_status group_solve_mixed(std::vector<GroupProblem>& g, int N, void* work, siz
     set_error_msg("workspace smaller than the grouped solve needs");
     return TK_ENOMEM;
   }
-  bool any_chol = false, any_lr = false;
+  bool any_chol = false;
   for (const auto& q : g) {
     if (q.n > kGroupMaxN) {
       set_error_msg("grouped solve: n above 4096");
       return TK_EINVAL;
     }
-    (q.lowrank ? any_lr : any_chol) = true;
+    any_chol = any_chol || !q.lowrank;
   }
   TK_CUDA(cudaMemcpyAsync(S.dd, S.hd.data(), sizeof(GDesc) * P, cudaMemcpyHostToDevice, st));
   k_g_fill<<<1, 64, 0, st>>>(S.ones, kGroupMaxLambda, 1.0);
   TK_LAUNCH_CHECK();
-  // tile lists of the float32 products over the problems that still have
-  // active slots (rebuilt when that set shrinks by a quarter: a retired
-  // problem's tiles would only launch CTAs that exit at once)
-  std::vector<GTile> t_aw, t_atu;
-  int tiled_problems = 0;
-  auto build_tiles = [&](const std::vector<int>& live) -> tk_status {
+  TK_CUDA(cudaMemsetAsync(S.arrivals, 0, sizeof(int) * (size_t)P * N, st));
+  // Tile lists of the products over the active slots (hact[p] of problem p), rebuilt as slots retire:
+  // row and split sizes such that each list has about kTargetTiles tiles whatever is still active (but
+  // at least 32 rows to an aw tile, 128 to an atu split, and no more planes than part holds: the planes
+  // have hact[p] rows, so fewer active slots allow more of them).
+  std::vector<GTile> t_aw, t_atu, ts[4];
+  std::vector<int> nsp_h(2 * (size_t)P);
+  int tiled_slots = 0;
+  auto build_tiles = [&](const std::vector<int>& hact) -> tk_status {
     t_aw.clear();
     t_atu.clear();
-    tiled_problems = 0;
+    for (auto& t : ts) t.clear();
+    tiled_slots = 0;
+    const auto nl_of = [](int M) { return M <= 4 ? 4 : (M <= 8 ? 8 : 16); };
+    const auto width = [](int nl) { return (int64_t)(nl == 16 ? 512 : 1024); };  // columns of an atu tile
+    double el[2] = {0.0, 0.0}, un[2] = {0.0, 0.0};  // elements of the aw lists, row-units of the atu lists
     for (int p = 0; p < P; ++p) {
-      if (!live[p]) continue;
-      ++tiled_problems;
-      for (int64_t n0 = 0; n0 < g[p].m; n0 += tiles::LM_BN) t_aw.push_back(GTile{p, 0, 0, 0, n0});
-      for (int64_t n0 = 0; n0 < g[p].n; n0 += tiles::LM_BN)
-        for (int z = 0; z < S.hd[p].splits; ++z) t_atu.push_back(GTile{p, z, 0, 0, n0});
+      const int M = hact[p];
+      if (M == 0) continue;
+      tiled_slots += M;
+      if (M <= kSmallLambda) {
+        el[0] += (double)g[p].m * g[p].n;
+        un[0] += (double)g[p].m * cdiv(g[p].n, width(nl_of(M)));
+      }
+      if (g[p].lowrank) {
+        el[1] += (double)g[p].n * g[p].lr_s;
+        un[1] += (double)g[p].n * cdiv(g[p].lr_s, width(nl_of(M)));
+      }
+    }
+    for (int p = 0; p < P; ++p) {
+      const int M = hact[p];
+      nsp_h[p] = nsp_h[P + p] = 0;
+      if (M == 0) continue;
+      const int nl = nl_of(M);
+      const int64_t cap = (int64_t)sizes_of(g[p]).splits * N * g[p].n;  // doubles of part
+      for (int f = 0; f < 2; ++f) {  // 0: A, 1: V of a low-rank problem
+        const int64_t rows = f ? g[p].n : g[p].m, cols = f ? g[p].lr_s : g[p].n;
+        if (f ? !g[p].lowrank : M > kSmallLambda) continue;
+        const int64_t per =
+            std::min<int64_t>(std::max<int64_t>(cdiv((int64_t)(el[f] / kTargetTiles), cols * 32) * 32, 32), 1 << 30);
+        for (int64_t r = 0; r < rows; r += per) ts[f ? 3 : 0].push_back(GTile{p, 0, (int)per, nl, r});
+        int64_t kps = std::max<int64_t>(cdiv((int64_t)(un[f] / kTargetTiles), 128) * 128, 128);
+        kps = std::max<int64_t>(std::min<int64_t>(kps, 4096), cdiv(cdiv(rows, std::max<int64_t>(cap / (M * cols), 1)), 128) * 128);
+        const int z = (int)cdiv(rows, kps);
+        nsp_h[f * P + p] = z;
+        for (int64_t c = 0; c < cols; c += width(nl))
+          for (int k = 0; k < z; ++k) ts[f ? 2 : 1].push_back(GTile{p, k, (int)kps, nl, c});
+      }
+      if (M > kSmallLambda) {
+        const int z = (int)cdiv(g[p].m, kKps);
+        nsp_h[p] = z;
+        for (int64_t n0 = 0; n0 < g[p].m; n0 += tiles::LM_BN) t_aw.push_back(GTile{p, 0, 0, 0, n0});
+        for (int64_t n0 = 0; n0 < g[p].n; n0 += tiles::LM_BN)
+          for (int k = 0; k < z; ++k) t_atu.push_back(GTile{p, k, 0, 0, n0});
+      }
     }
     S.n_aw = (int)t_aw.size();
     S.n_atu = (int)t_atu.size();
@@ -636,6 +827,20 @@ tk_status group_solve_mixed(std::vector<GroupProblem>& g, int N, void* work, siz
       TK_CUDA(cudaMemcpyAsync(S.t_aw, t_aw.data(), sizeof(GTile) * t_aw.size(), cudaMemcpyHostToDevice, st));
     if (!t_atu.empty())
       TK_CUDA(cudaMemcpyAsync(S.t_atu, t_atu.data(), sizeof(GTile) * t_atu.size(), cudaMemcpyHostToDevice, st));
+    size_t off = 0;
+    for (int k = 0; k < 4; ++k) {
+      S.s_off[k] = off;
+      S.s_n[k] = (int)ts[k].size();
+      if (off + ts[k].size() > S.s_cap) {
+        set_error_msg("grouped solve: product tile list overflow");
+        return TK_EINVAL;
+      }
+      if (!ts[k].empty())
+        TK_CUDA(cudaMemcpyAsync(S.s_tiles + off, ts[k].data(), sizeof(GTile) * ts[k].size(), cudaMemcpyHostToDevice,
+                                st));
+      off += ts[k].size();
+    }
+    TK_CUDA(cudaMemcpyAsync(S.nsp, nsp_h.data(), sizeof(int) * nsp_h.size(), cudaMemcpyHostToDevice, st));
     return TK_OK;
   };
   std::vector<std::vector<int>> act(P);
@@ -756,11 +961,7 @@ tk_status group_solve_mixed(std::vector<GroupProblem>& g, int N, void* work, siz
       mirror[p].assign(act[p].begin(), act[p].end());
     }
     TK_CUDA(cudaMemcpyAsync(S.nact, hnact.data(), sizeof(int) * P, cudaMemcpyHostToDevice, st));
-    {
-      std::vector<int> live(P);
-      for (int p = 0; p < P; ++p) live[p] = hnact[p] > 0;
-      TK_TRY(build_tiles(live));
-    }
+    TK_TRY(build_tiles(hnact));
     sl = rl;
     int nsl = nrl;
     k_g_init<<<chunk_grid(std::max<int64_t>(S.maxn, 1 << 14), nsl), 256, 0, st>>>(S.dd, S.rnd, round == 0);
@@ -794,11 +995,11 @@ tk_status group_solve_mixed(std::vector<GroupProblem>& g, int N, void* work, siz
       TK_TRY(launch_lm(S, false, st));
       prof_end(tok, st, fb.first, fb.second, fb.impl);
     }
-    k_g_over_g<<<chunk_grid(S.maxn, nsl), 256, 0, st>>>(S.dd, S.nact, S.rnd);
+    k_g_over_g<<<dim3((unsigned)cdiv(S.maxn, 32), (unsigned)nsl), 256, 0, st>>>(S.dd, S.nact, S.nsp, S.rnd);
     TK_LAUNCH_CHECK();
     {
       const int tok = prof_begin(TK_PHASE_PRECOND, st);
-      TK_TRY(launch_prec(S, true, S.rnd, nsl, F_TT, F_VRAW, any_chol, any_lr, st));
+      TK_TRY(launch_prec(S, true, S.rnd, nsl, S.rnd, nsl, F_TT, F_VRAW, any_chol, st));
       prof_end(tok, st, prec_flops(), 0.0);
     }
     k_g_vstep<<<nsl, kThreads, 0, st>>>(S.dd, S.rnd, 1, S.rep);
@@ -826,7 +1027,7 @@ tk_status group_solve_mixed(std::vector<GroupProblem>& g, int N, void* work, siz
         const int nr = (int)retire.size();
         TK_CUDA(cudaMemcpyAsync(S.rslots, retire.data(), sizeof(GSlot) * nr, cudaMemcpyHostToDevice, st));
         // x = R^-1 y of the retiring slots, written as the lambda's correction
-        TK_TRY(launch_prec(S, false, S.rslots, nr, F_Y, F_XT, any_chol, any_lr, st));
+        TK_TRY(launch_prec(S, false, S.rslots, nr, S.slots, nsl, F_Y, F_XT, any_chol, st));
         k_g_scatter<<<chunk_grid(S.maxn, nr), 256, 0, st>>>(S.dd, S.rslots);
         TK_LAUNCH_CHECK();
         // per problem: survivors beyond the new end move into holes below it
@@ -864,35 +1065,38 @@ tk_status group_solve_mixed(std::vector<GroupProblem>& g, int N, void* work, siz
         nsl = (int)sl.size();
         TK_CUDA(cudaMemcpyAsync(S.nact, hnact.data(), sizeof(int) * P, cudaMemcpyHostToDevice, st));
         if (nsl > 0) TK_CUDA(cudaMemcpyAsync(S.slots, sl.data(), sizeof(GSlot) * nsl, cudaMemcpyHostToDevice, st));
-        {
-          std::vector<int> live(P);
-          int nlive = 0;
-          for (int p = 0; p < P; ++p) nlive += (live[p] = hnact[p] > 0);
-          if (nlive > 0 && 4 * nlive <= 3 * tiled_problems) TK_TRY(build_tiles(live));
-        }
+        if (nsl > 0 && 8 * nsl <= 7 * tiled_slots) TK_TRY(build_tiles(hnact));
         TK_CUDA(cudaStreamSynchronize(st));  // host lists are reused
       }
       if (nsl == 0) break;
-      // ------------------------------------------------------------ one step
+      // ------------------------------------------- one step, or 4 short ones between two reports
+      // (a slot that converges inside stays as it is: its norm and v-step return at once)
       auto fb = step_flops();
-      int tok = prof_begin(TK_PHASE_PRECOND, st);
-      TK_TRY(launch_prec(S, false, S.slots, nsl, F_V, F_TT, any_chol, any_lr, st));  // T = R^-1 v
-      prof_end(tok, st, prec_flops(), 0.0);
-      tok = prof_begin(TK_PHASE_AW, st);
-      TK_TRY(launch_lm(S, true, st));  // Ut = T A^T - (alpha/beta) Ut
-      prof_end(tok, st, fb.first, fb.second, fb.impl);
-      k_g_beta<<<nsl, kThreads, 0, st>>>(S.dd, S.slots);
-      TK_LAUNCH_CHECK();
-      tok = prof_begin(TK_PHASE_ATU, st);
-      TK_TRY(launch_lm(S, false, st));  // part = Ut A
-      prof_end(tok, st, fb.first, fb.second, fb.impl);
-      k_g_over_g<<<chunk_grid(S.maxn, nsl), 256, 0, st>>>(S.dd, S.nact, S.slots);
-      TK_LAUNCH_CHECK();
-      tok = prof_begin(TK_PHASE_PRECOND, st);
-      TK_TRY(launch_prec(S, true, S.slots, nsl, F_TT, F_VRAW, any_chol, any_lr, st));  // R^-T g
-      prof_end(tok, st, prec_flops(), 0.0);
-      k_g_vstep<<<nsl, kThreads, 0, st>>>(S.dd, S.slots, 0, S.rep);
-      TK_LAUNCH_CHECK();
+      const int steps = fb.impl <= 256e6 ? 4 : 1;
+      int64_t max_m = 1;
+      for (int p = 0; p < P; ++p)
+        if (hnact[p]) max_m = std::max(max_m, g[p].m);
+      const unsigned chunks = (unsigned)std::min<int64_t>({(int64_t)kBetaChunks, cdiv(max_m, 2048), cdiv(8 * 152, nsl)});
+      for (int k = 0; k < steps; ++k) {
+        int tok = prof_begin(TK_PHASE_PRECOND, st);
+        TK_TRY(launch_prec(S, false, S.slots, nsl, S.slots, nsl, F_V, F_TT, any_chol, st));  // T = R^-1 v
+        prof_end(tok, st, prec_flops(), 0.0);
+        tok = prof_begin(TK_PHASE_AW, st);
+        TK_TRY(launch_lm(S, true, st));  // Ut = T A^T - (alpha/beta) Ut
+        prof_end(tok, st, fb.first, fb.second, fb.impl);
+        k_g_beta<<<dim3(chunks, (unsigned)nsl), kThreads, 0, st>>>(S.dd, S.slots, S.beta_part, S.arrivals);
+        TK_LAUNCH_CHECK();
+        tok = prof_begin(TK_PHASE_ATU, st);
+        TK_TRY(launch_lm(S, false, st));  // part = Ut A
+        prof_end(tok, st, fb.first, fb.second, fb.impl);
+        k_g_over_g<<<dim3((unsigned)cdiv(S.maxn, 32), (unsigned)nsl), 256, 0, st>>>(S.dd, S.nact, S.nsp, S.slots);
+        TK_LAUNCH_CHECK();
+        tok = prof_begin(TK_PHASE_PRECOND, st);
+        TK_TRY(launch_prec(S, true, S.slots, nsl, S.slots, nsl, F_TT, F_VRAW, any_chol, st));  // R^-T g
+        prof_end(tok, st, prec_flops(), 0.0);
+        k_g_vstep<<<nsl, kThreads, 0, st>>>(S.dd, S.slots, 0, S.rep);
+        TK_LAUNCH_CHECK();
+      }
     }
 
     // ---- x <- x + d and the stopping decisions

@@ -37,8 +37,8 @@ __global__ void __launch_bounds__(LM_AW_THREADS)
     __syncthreads();  // the previous chunk of W is no longer read
     lmb::load_w<NL>(lm_ws, W + k0, ldw, count, len, n_pad);
     __syncthreads();
-    lmb::aw_rows<NL>(lm_ws, n_pad, A + k0, lda, m, len, count, C, ldc, beta, vec,
-                     (int64_t)blockIdx.x * nwarps + (threadIdx.x >> 5), (int64_t)gridDim.x * nwarps, groups, k0 == 0);
+    lmb::aw_rows<NL>(lm_ws, n_pad, A + k0, lda, m, len, count, lmb::AwStore{C, ldc, beta, k0 == 0}, vec,
+                     (int64_t)blockIdx.x * nwarps + (threadIdx.x >> 5), (int64_t)gridDim.x * nwarps, groups);
   }
 }
 
@@ -47,11 +47,11 @@ template <int NL, int CW>
 __global__ void __launch_bounds__(lmb::kAtuThreads, 3)
     k_lm_atu(const float* __restrict__ A, int64_t lda, int64_t m, int64_t n, const float* __restrict__ U, int64_t ldu,
              int count, int64_t rows_per, double* __restrict__ partial, bool vec) {
-  __shared__ __align__(16) float us[lmb::kAtuRB][NL];
+  __shared__ __align__(16) lmb::AtuSmem<NL, CW> S;
   const int64_t z = blockIdx.x;
   const int64_t rb = z * rows_per, re = rb + rows_per < m ? rb + rows_per : m;
-  const int64_t c = (int64_t)blockIdx.y * (CW * lmb::kAtuThreads) + CW * threadIdx.x;
-  lmb::atu_cols<NL, CW>(us, A, lda, m, n, U, ldu, count, rb, re, c, partial + z * (int64_t)count * n, vec);
+  lmb::atu_cols<NL, CW>(S, A, lda, n, U, ldu, count, rb, re, (int64_t)blockIdx.y * (CW * lmb::kAtuThreads),
+                        partial + z * (int64_t)count * n, vec);
 }
 
 int lm_nl(int count) { return count <= 4 ? 4 : (count <= 8 ? 8 : 16); }

@@ -2,18 +2,18 @@
 // the single-problem kernels (tk_lm.cu) and the grouped engine (tk_group.cu).
 // Both read the float32 A once in 16-byte vectors along its rows and keep the
 // lambda-side operand on chip:
-//  * aw_rows: C[l][i] = sum_k W[l][k] A[i][k] (+ beta_l C[l][i]; first = false:
-//    C[l][i] += the sum, for a later chunk of columns) for the 4-row
+//  * aw_rows: store(l, i, sum_k W[l][k] A[i][k]) for the 4-row
 //    groups g_first, g_first + g_stride, ... < g_end, one warp per group at a
 //    time; W (zero-padded to NL x n_pad) is in shared memory (load_w); each lane
 //    takes 4 consecutive k of every 128, the next 128 loaded while the current
 //    ones are used; the 4 NL dot products per lane are added across the warp by
 //    halving exchanges (each step keeps half of the values and adds the
 //    partner's other half), then written.
-//  * atu_cols: out[l][c + t] = sum over rows rb <= i < re of U[l][i] A[i][c + t]
-//    for the thread's CW columns (NL x CW accumulators, 8 rows' loads in flight);
-//    the rows' U values are staged in shared memory ([row][lambda], read as
-//    broadcasts).  Every thread of the block must call it (it synchronizes).
+//  * atu_cols: out[l][c] = sum over rows rb <= i < re of U[l][i] A[i][c] for the
+//    block's columns, CW per thread (NL x CW accumulators, 8 rows' loads in flight);
+//    a block with fewer columns than 256 CW splits its rows over groups of threads,
+//    whose sums meet in shared memory; the rows' U values are staged in shared memory
+//    ([row][lambda], read as broadcasts).  Every thread of the block must call it.
 #pragma once
 #include "tk_internal.cuh"
 
@@ -59,11 +59,25 @@ __device__ __forceinline__ void load_w(float* ws, const float* __restrict__ W, i
   }
 }
 
-template <int NL>
+// the store of an LSQR product: C[l][i] = v (+ beta_l C[l][i]), or += v for a later chunk of columns
+struct AwStore {
+  float* C;
+  int64_t ldc;
+  const double* beta;
+  bool first;
+  __device__ __forceinline__ void operator()(int l, int64_t i, float v) const {
+    float* c = C + (int64_t)l * ldc + i;
+    double val = (double)v;
+    if (!first) val += (double)*c;
+    else if (beta) val += beta[l] * (double)*c;
+    *c = (float)val;
+  }
+};
+
+template <int NL, typename Store>
 __device__ __forceinline__ void aw_rows(const float* ws, int64_t n_pad, const float* __restrict__ A, int64_t lda,
-                                        int64_t m, int64_t n, int count, float* C, int64_t ldc,
-                                        const double* __restrict__ beta, bool vec, int64_t g_first,
-                                        int64_t g_stride, int64_t g_end, bool first = true) {
+                                        int64_t m, int64_t n, int count, const Store& store, bool vec,
+                                        int64_t g_first, int64_t g_stride, int64_t g_end) {
   constexpr int LM_ROWS = kRows;
   const int lane = threadIdx.x & 31;
   const int nj = (int)(n_pad / 128);
@@ -135,12 +149,7 @@ __device__ __forceinline__ void aw_rows(const float* ws, int64_t n_pad, const fl
         if (t < nv) {
           const int q = qbase + t, r = q / NL, l = q % NL;
           const int64_t i = i0 + r;
-          if (i < m && l < count) {
-            double val = (double)v[t];
-            if (!first) val += (double)C[(int64_t)l * ldc + i];  // a later column chunk: add to the sum
-            else if (beta) val += beta[l] * (double)C[(int64_t)l * ldc + i];
-            C[(int64_t)l * ldc + i] = (float)val;
-          }
+          if (i < m && l < count) store(l, i, v[t]);
         }
       }
     }
@@ -164,28 +173,40 @@ __device__ __forceinline__ void loadv(const float* __restrict__ row, int64_t k, 
   for (int t = 0; t < CW; ++t) o[t] = k + t < len ? __ldg(row + k + t) : 0.f;
 }
 
-// CW columns per thread (4 for <= 8 lambda, 2 for 16: NL x CW accumulators), 8 rows' loads in flight
+// Shared memory of an atu block: the staged U values and the row groups' sums (4 lambda at a time).
 template <int NL, int CW>
-__device__ __forceinline__ void atu_cols(float (*us)[NL], const float* __restrict__ A, int64_t lda, int64_t m,
-                                         int64_t n, const float* __restrict__ U, int64_t ldu, int count, int64_t rb,
-                                         int64_t re, int64_t c, double* __restrict__ out, bool vec) {
+struct AtuSmem {
+  float us[kAtuRB][NL];
+  float red[4 * CW][kAtuThreads];
+};
+
+// The block's columns c0 .. c0 + CW kAtuThreads - 1 (those < n), rows rb .. re - 1.  CW columns per
+// thread (4 for <= 8 lambda, 2 for 16: NL x CW accumulators), 8 rows' loads in flight.
+template <int NL, int CW>
+__device__ __forceinline__ void atu_cols(AtuSmem<NL, CW>& S, const float* __restrict__ A, int64_t lda, int64_t n,
+                                         const float* __restrict__ U, int64_t ldu, int count, int64_t rb, int64_t re,
+                                         int64_t c0, double* __restrict__ out, bool vec) {
   constexpr int RU = 8;
-  constexpr int LM_ATU_RB = kAtuRB, LM_ATU_THREADS = kAtuThreads;
+  // cg threads across the columns (whole warps), rg groups of rows
+  const int64_t cols = n - c0 < (int64_t)CW * kAtuThreads ? n - c0 : (int64_t)CW * kAtuThreads;
+  const int cg = (int)((cols + 32 * CW - 1) / (32 * CW)) * 32, rg = kAtuThreads / cg;
+  const int g = threadIdx.x / cg;
+  const int64_t c = g < rg ? c0 + (int64_t)CW * (threadIdx.x % cg) : n;
   float acc[NL][CW];
 #pragma unroll
   for (int l = 0; l < NL; ++l)
 #pragma unroll
     for (int t = 0; t < CW; ++t) acc[l][t] = 0.f;
-  for (int64_t i0 = rb; i0 < re; i0 += LM_ATU_RB) {
-    const int nr = (int)(re - i0 < LM_ATU_RB ? re - i0 : LM_ATU_RB);
+  for (int64_t i0 = rb; i0 < re; i0 += kAtuRB) {
+    const int nr = (int)(re - i0 < kAtuRB ? re - i0 : kAtuRB);
     __syncthreads();  // the previous rows' U values are no longer read
-    for (int idx = threadIdx.x; idx < LM_ATU_RB * NL; idx += LM_ATU_THREADS) {
-      const int l = idx / LM_ATU_RB, r = idx % LM_ATU_RB;
-      us[r][l] = (l < count && r < nr) ? U[(int64_t)l * ldu + i0 + r] : 0.f;
+    for (int idx = threadIdx.x; idx < kAtuRB * NL; idx += kAtuThreads) {
+      const int l = idx / kAtuRB, r = idx % kAtuRB;
+      S.us[r][l] = (l < count && r < nr) ? U[(int64_t)l * ldu + i0 + r] : 0.f;
     }
     __syncthreads();
     if (c < n) {
-      for (int r = 0; r < nr; r += RU) {
+      for (int r = g * RU; r < nr; r += rg * RU) {
         float a[RU][CW];
 #pragma unroll
         for (int q = 0; q < RU; ++q) {
@@ -199,7 +220,7 @@ __device__ __forceinline__ void atu_cols(float (*us)[NL], const float* __restric
         for (int q = 0; q < RU; ++q) {
 #pragma unroll
           for (int l4 = 0; l4 < NL / 4; ++l4) {
-            const float4 u4 = *reinterpret_cast<const float4*>(&us[r + q][4 * l4]);
+            const float4 u4 = *reinterpret_cast<const float4*>(&S.us[r + q][4 * l4]);
             const float uu[4] = {u4.x, u4.y, u4.z, u4.w};
 #pragma unroll
             for (int t4 = 0; t4 < 4; ++t4)
@@ -210,13 +231,35 @@ __device__ __forceinline__ void atu_cols(float (*us)[NL], const float* __restric
       }
     }
   }
-  if (c < n) {
+  if (rg == 1) {
+    if (c < n) {
 #pragma unroll
-    for (int l = 0; l < NL; ++l) {
-      if (l < count) {
+      for (int l = 0; l < NL; ++l)
+        if (l < count) {
 #pragma unroll
-        for (int t = 0; t < CW; ++t)
-          if (c + t < n) out[(int64_t)l * n + c + t] = (double)acc[l][t];
+          for (int t = 0; t < CW; ++t)
+            if (c + t < n) out[(int64_t)l * n + c + t] = (double)acc[l][t];
+        }
+    }
+    return;
+  }
+#pragma unroll
+  for (int l4 = 0; l4 < NL / 4; ++l4) {
+    if (4 * l4 >= count) break;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int t = 0; t < CW; ++t) S.red[q * CW + t][threadIdx.x] = acc[4 * l4 + q][t];
+    __syncthreads();
+    // the groups' sums in order: (lambda, column) pairs over all threads
+    for (int idx = threadIdx.x; idx < 4 * CW * cg; idx += kAtuThreads) {
+      const int v = idx / cg, k = idx % cg, l = 4 * l4 + v / CW;
+      const int64_t cc = c0 + (int64_t)CW * k + v % CW;
+      if (l < count && cc < n) {
+        float t = S.red[v][k];
+        for (int q = 1; q < rg; ++q) t += S.red[v][k + q * cg];
+        out[(int64_t)l * n + cc] = (double)t;
       }
     }
   }
