@@ -202,45 +202,89 @@ __global__ void k_chol_init(const double* __restrict__ Cm, int64_t n, int64_t np
   }
 }
 
-// Factor the diagonal tile (kb, kb) of every lambda in shared memory
-// (right-looking within the tile).  A non-positive pivot records the global
+// 1 / d for a positive d: the float32 reciprocal and one third-order step (error e^3 with |e| < 2^-22).
+__device__ __forceinline__ double chol_recip(double d) {
+  if (!(d > 1e-36 && d < 1e36)) return 1.0 / d;  // beyond float32
+  const double w = (double)__frcp_rn((float)d);
+  const double e = fma(-d, w, 1.0);
+  return fma(w, fma(e, e, e), w);
+}
+
+// Factor the diagonal tile (kb, kb) of every lambda.  A non-positive pivot records the global
 // row + 1 in info[l] (first one only; its negative when the pivot is NaN, i.e.
 // non-finite input rather than a matrix that is not positive definite) and
 // continues with pivot 1.
+// One SM per lambda, bound by dependent float64 operations: a warp's instruction holds its quarter of
+// the SM's float64 pipe for 64 clocks.  So the tile is spread over 8 warps (thread: one column, the rows
+// of one residue mod 4, 16 values), the elimination runs on unnormalized rows (one reciprocal per
+// pivot, no root in the chain; r_jc = x_jc / sqrt(d_j) for all rows at the end), and there is one barrier
+// a column: between two barriers the warps that own the next row finish it, while the others still
+// subtract the row before.  98 us with a column's root, division and update one after another; now 67.
 __global__ void __launch_bounds__(256) k_chol_diag(double* __restrict__ R, int64_t ldr, int64_t rstride, int kb,
                                                    int* __restrict__ info) {
-  __shared__ double T[CB][CB + 1];
-  const int l = blockIdx.x;
+  __shared__ double row[CB][CB];  // the finished unnormalized rows
+  __shared__ double wv[CB];       // 1 / d_j
+  __shared__ int first;
+  const int l = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // warps 0-3: columns 32..63, rows mod 4 = 0..3; warps 4-7: columns 0..31, rows mod 4 = 1, 2, 3, 0 (the two
+  // warps of a residue on different quarters of the SM)
+  const bool hi = w < 4;
+  const int g = hi ? w : (w + 1) & 3, c = hi ? 32 + lane : lane;
   double* Rl = R + (int64_t)l * rstride + (int64_t)kb * CB * ldr + (int64_t)kb * CB;
-  for (int idx = threadIdx.x; idx < CB * CB; idx += blockDim.x) {
-    int i = idx / CB, j = idx % CB;
-    T[i][j] = Rl[(int64_t)i * ldr + j];
+  double x[CB / 4];  // rows 4 q + g
+#pragma unroll
+  for (int q = 0; q < CB / 4; ++q) x[q] = (hi || 4 * q + g < 32) ? Rl[(int64_t)(4 * q + g) * ldr + c] : 0.0;
+  if (threadIdx.x == 0) first = CB;
+  if (g == 0) row[0][c] = x[0];
+  __syncthreads();
+  double mp = 0.0;  // x_(j-1),c / d_(j-1)
+#pragma unroll
+  for (int j = 0; j < CB; ++j) {
+    // rows below 32 have no columns in the first half
+    if (j > 0 && (hi || j + 1 < 32)) mp = row[j - 1][c] * wv[j - 1];
+    if (g == ((j + 1) & 3) && j + 1 < CB && (hi || j + 1 < 32)) {
+      // this warp owns row j + 1: what row j - 1 leaves of it, then row j
+      constexpr int Q = CB / 4;
+      double v = x[((j + 1) >> 2) % Q];
+      if (j > 0) v = fma(-row[j - 1][j + 1], mp, v);
+      double d = row[j][j];
+      if (!(d > 0.0)) d = 1.0;
+      const double wj = chol_recip(d);
+      v = fma(-row[j][j + 1], row[j][c] * wj, v);
+      row[j + 1][c] = v;
+      if (c == CB - 1) wv[j] = wj;
+    }
+    if (j > 0) {
+#pragma unroll
+      for (int q = 0; q < CB / 4; ++q) {
+        // rows j + 1 (taken above) and earlier are finished
+        if (4 * q + 3 >= j + 2 && (hi || 4 * q < 32)) {
+          const int i = 4 * q + g;
+          if (4 * q >= j + 2 || i >= j + 2) x[q] = fma(-row[j - 1][i], mp, x[q]);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  // r_jc = x_jc / sqrt(d_j); the diagonal is sqrt(d_j)
+  if (threadIdx.x < CB) {
+    const double d = row[threadIdx.x][threadIdx.x];
+    const bool ok = d > 0.0;
+    if (!ok) atomicMin(&first, (int)threadIdx.x);
+    wv[threadIdx.x] = ok ? rsqrt(d) : 1.0;
   }
   __syncthreads();
-  for (int j = 0; j < CB; ++j) {
-    if (threadIdx.x == 0) {
-      double d = T[j][j];
-      if (!(d > 0.0)) {
-        if (info[l] == 0) info[l] = (d != d) ? -(kb * CB + j + 1) : kb * CB + j + 1;
-        d = 1.0;
-      }
-      T[j][j] = sqrt(d);
-    }
-    __syncthreads();
-    const double rjj = T[j][j];
-    for (int k = j + 1 + threadIdx.x; k < CB; k += blockDim.x) T[j][k] /= rjj;
-    __syncthreads();
-    // trailing update of the upper triangle: T[i][k] -= T[j][i] T[j][k], j < i <= k
-    const int rem = CB - j - 1;
-    for (int p = threadIdx.x; p < rem * rem; p += blockDim.x) {
-      int i = j + 1 + p / rem, k = j + 1 + p % rem;
-      if (k >= i) T[i][k] -= T[j][i] * T[j][k];
-    }
-    __syncthreads();
+  for (int idx = threadIdx.x; idx < CB * CB; idx += 256) {
+    const int i = idx / CB, k = idx % CB;
+    if (k < i) continue;
+    const double v = row[i][k], y = wv[i];
+    double r = v * y;
+    if (k == i) r = v > 0.0 ? fma(0.5 * y, fma(-r, r, v), r) : 1.0;
+    Rl[(int64_t)i * ldr + k] = r;
   }
-  for (int idx = threadIdx.x; idx < CB * CB; idx += blockDim.x) {
-    int i = idx / CB, j = idx % CB;
-    if (j >= i) Rl[(int64_t)i * ldr + j] = T[i][j];
+  if (threadIdx.x == 0 && first < CB && info[l] == 0) {
+    const double d = row[first][first];
+    info[l] = (d != d ? -1 : 1) * (kb * CB + first + 1);
   }
 }
 
@@ -274,6 +318,48 @@ __global__ void __launch_bounds__(CB) k_chol_trsm(double* __restrict__ R, int64_
   }
 #pragma unroll
   for (int i = 0; i < CB; ++i) Xg[(int64_t)i * ldr + c] = xr[i];
+}
+
+// The same for few tiles: a CTA solves 16 columns, the 8 half-warps of 4 warps holding the rows of one
+// residue mod 8 each, so that all four quarters of the SM's float64 pipe work and a tile is spread over
+// four SMs; one barrier a row (n = 256, 8 lambda: 77 us a panel, now 21).
+__global__ void __launch_bounds__(128) k_chol_trsm16(double* __restrict__ R, int64_t ldr, int64_t rstride, int kb) {
+  __shared__ double D[CB][CB + 1];
+  __shared__ double Dinv[CB];
+  __shared__ double xs[CB][16];
+  const int l = blockIdx.y, cc = threadIdx.x & 15, g = threadIdx.x >> 4;
+  double* Rl = R + (int64_t)l * rstride;
+  const double* Dg = Rl + (int64_t)kb * CB * ldr + (int64_t)kb * CB;
+  double* Xg = Rl + (int64_t)kb * CB * ldr + (int64_t)(kb + 1) * CB + 16 * (int64_t)blockIdx.x + cc;
+  double xr[CB / 8];  // rows 8 q + g
+#pragma unroll
+  for (int q = 0; q < CB / 8; ++q) xr[q] = Xg[(int64_t)(8 * q + g) * ldr];
+#pragma unroll 8
+  for (int idx = threadIdx.x; idx < CB * CB; idx += 128) D[idx / CB][idx % CB] = Dg[(int64_t)(idx / CB) * ldr + idx % CB];
+  if (threadIdx.x < CB) Dinv[threadIdx.x] = 1.0 / Dg[(int64_t)threadIdx.x * ldr + threadIdx.x];
+  __syncthreads();
+  if (g == 0) xs[0][cc] = xr[0] * Dinv[0];
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < CB; ++r) {
+    const double v = xs[r][cc];
+    // the next row first, then the rest behind it
+    if (r + 1 < CB && g == ((r + 1) & 7)) {
+      const int q = (r + 1) >> 3;
+      xs[r + 1][cc] = fma(-D[r][r + 1], v, xr[q % (CB / 8)]) * Dinv[r + 1];
+    }
+#pragma unroll
+    for (int q = 0; q < CB / 8; ++q)
+      if (8 * q + 7 >= r + 2) {
+        const int i = 8 * q + g;
+        if (8 * q >= r + 2 || i >= r + 2) xr[q] = fma(-D[r][i], v, xr[q]);
+      }
+    __syncthreads();
+  }
+  for (int idx = threadIdx.x; idx < CB * 16; idx += 128) {
+    const int i = idx / 16, k = idx % 16;
+    Rl[(int64_t)(kb * CB + i) * ldr + (int64_t)(kb + 1) * CB + 16 * (int64_t)blockIdx.x + k] = xs[i][k];
+  }
 }
 
 // Trailing update of tiles (ib, jb), kb < ib <= jb:
@@ -360,14 +446,17 @@ __global__ void __launch_bounds__(CB) k_tinv_diag(const double* __restrict__ R, 
   __shared__ double D[CB][CB + 1];
   const int kb = blockIdx.x, l = blockIdx.y, c = threadIdx.x;
   const double* Rg = R + (int64_t)l * rstride + (int64_t)kb * CB * ldr + (int64_t)kb * CB;
+  __shared__ double Dinv[CB];  // one division per row and tile, not one per row and column
+#pragma unroll 8
   for (int i = 0; i < CB; ++i) D[i][c] = Rg[(int64_t)i * ldr + c];
+  Dinv[c] = 1.0 / Rg[(int64_t)c * ldr + c];
   __syncthreads();
   double x[CB];
 #pragma unroll
   for (int r = 0; r < CB; ++r) x[r] = (r == c) ? 1.0 : 0.0;
 #pragma unroll
   for (int r = CB - 1; r >= 0; --r) {
-    x[r] = x[r] / D[r][r];
+    x[r] = x[r] * Dinv[r];
 #pragma unroll
     for (int q = 0; q < r; ++q) x[q] = fma(-D[q][r], x[r], x[q]);
   }
@@ -943,7 +1032,9 @@ tk_status chol_shifted(const double* Cm, int64_t n, const double* lambdas_dev, i
     k_chol_diag<<<N, 256, 0, st>>>(R, ldr, rstride, kb, info_dev);
     TK_LAUNCH_CHECK();
     if (r > 0) {
-      k_chol_trsm<<<dim3((unsigned)r, (unsigned)N), CB, 0, st>>>(R, ldr, rstride, kb);
+      // up to two tiles per SM: 16-column warps fill the GPU better
+      if ((int64_t)r * N <= 2 * 152) k_chol_trsm16<<<dim3((unsigned)(4 * r), (unsigned)N), 128, 0, st>>>(R, ldr, rstride, kb);
+      else k_chol_trsm<<<dim3((unsigned)r, (unsigned)N), CB, 0, st>>>(R, ldr, rstride, kb);
       TK_LAUNCH_CHECK();
     }
     prof_end(tok, st, (double)N * ((double)CB * CB * CB / 3.0 + (double)r * CB * CB * CB),

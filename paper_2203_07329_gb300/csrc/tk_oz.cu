@@ -821,6 +821,18 @@ __device__ __forceinline__ int level_int(uint32_t bits) {
   return __float_as_int(__fadd_rn(__uint_as_float(bits), 12582912.0f)) - 0x4B400000;
 }
 
+// 32 consecutive bytes (32-byte aligned) of global memory
+__device__ __forceinline__ void ld_global_v4(const double* p, double* v) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void st_global_v4(double* p, const double* v) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+               : "memory");
+}
+
 // 2^e as a double (e within the normal range).
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
 
@@ -951,15 +963,25 @@ __global__ void __launch_bounds__(384, 1)
     for (int t = 0; t < nt; ++t) {
       const int s = t & 1;
       const int64_t j0 = (int64_t)(t_first + t) * CS_N + half * 2 * G;
+      // a thread's 16 columns are 128 consecutive bytes of its row of T: four 32-byte loads and stores (whole
+      // sectors; element by element every 8-byte store was a partial sector write of its own: order 4096, 64
+      // lambda 2.51 ms a step on average, now 2.10; order 2048, 32 lambda 0.36, now 0.30).  Tiles on
+      // the diagonal (columns below the thread's row) and marked rows go element by element.
+      const bool full = i < w && j0 >= i;
       // T of the thread's 16 columns first: their loads do not wait for the products
       double tv[2][G];
+      if (full) {
 #pragma unroll
-      for (int gi = 0; gi < 2; ++gi)
+        for (int q = 0; q < 4; ++q) ld_global_v4(Trow + j0 + 4 * q, tv[q >> 1] + 4 * (q & 1));
+      } else {
 #pragma unroll
-        for (int j = 0; j < G; ++j) {
-          const int64_t col = j0 + gi * G + j;
-          tv[gi][j] = (i < w && col < w && col >= i) ? Trow[col] : 0.0;
-        }
+        for (int gi = 0; gi < 2; ++gi)
+#pragma unroll
+          for (int j = 0; j < G; ++j) {
+            const int64_t col = j0 + gi * G + j;
+            tv[gi][j] = (i < w && col < w && col >= i) ? Trow[col] : 0.0;
+          }
+      }
       if (!mbar_wait(&S.acc_full[s], (uint32_t)(t >> 1) & 1u, err)) break;
       tc_fence_after();
       const uint32_t base =
@@ -978,30 +1000,33 @@ __global__ void __launch_bounds__(384, 1)
         if (i < w) {
 #pragma unroll
           for (int j = 0; j < G; ++j) {
-            if (jg + j < w && jg + j >= i) {
-              const int ej = S.ecol[t * CS_N + half * 2 * G + gi * G + j];
-              const int e = ei + ej;
-              if (oz_bad(ei) || oz_bad(ej)) {  // a row or column marked non-finite: NaN (its digits are zero)
-                Trow[jg + j] = __longlong_as_double(0x7ff8000000000000ll);
-                continue;
-              }
-              const int a0 = level_int(v[0][j]) * 128 + level_int(v[1][j]);
-              const int a1 = level_int(v[2][j]) * 128 + level_int(v[3][j]);
-              const int b0 = level_int(v[4][j]) * 128 + level_int(v[5][j]);
-              const int b1 = level_int(v[6][j]) * 128 + level_int(v[7][j]);
-              const long long hi = (long long)a0 * 16384 + a1, lo = (long long)b0 * 16384 + b1;
-              // (hi 2^-35 + lo 2^-63) 2^e with the two scaled terms built exactly from the integers'
-              // bits; the sum and the subtraction are the only float64 operations (the same rounding
-              // as scaling the rounded sum, since a power of two scales exactly)
-              bool ok = true;
-              const double shi = i53_scaled(hi, e - 35, &ok), slo = i53_scaled(lo, e - 63, &ok);
-              if (ok) {
-                Trow[jg + j] = tv[gi][j] - (shi + slo);
-              } else {  // a scaled term outside the normal range: through the float64 pipe
-                const double vhi = (double)hi * 0x1p-35, vlo = (double)lo * 0x1p-63;  // exact
-                Trow[jg + j] = tv[gi][j] - (vhi + vlo) * (e >= -1022 && e <= 1023 ? pow2d(e) : ldexp(1.0, e));
-              }
+            const int ej = S.ecol[t * CS_N + half * 2 * G + gi * G + j];
+            const int e = ei + ej;
+            const int a0 = level_int(v[0][j]) * 128 + level_int(v[1][j]);
+            const int a1 = level_int(v[2][j]) * 128 + level_int(v[3][j]);
+            const int b0 = level_int(v[4][j]) * 128 + level_int(v[5][j]);
+            const int b1 = level_int(v[6][j]) * 128 + level_int(v[7][j]);
+            const long long hi = (long long)a0 * 16384 + a1, lo = (long long)b0 * 16384 + b1;
+            // (hi 2^-35 + lo 2^-63) 2^e with the two scaled terms built exactly from the integers'
+            // bits; the sum and the subtraction are the only float64 operations (the same rounding
+            // as scaling the rounded sum, since a power of two scales exactly)
+            bool ok = true;
+            const double shi = i53_scaled(hi, e - 35, &ok), slo = i53_scaled(lo, e - 63, &ok);
+            double r;
+            if (oz_bad(ei) || oz_bad(ej)) {  // a row or column marked non-finite: NaN (its digits are zero)
+              r = __longlong_as_double(0x7ff8000000000000ll);
+            } else if (ok) {
+              r = tv[gi][j] - (shi + slo);
+            } else {  // a scaled term outside the normal range: through the float64 pipe
+              const double vhi = (double)hi * 0x1p-35, vlo = (double)lo * 0x1p-63;  // exact
+              r = tv[gi][j] - (vhi + vlo) * (e >= -1022 && e <= 1023 ? pow2d(e) : ldexp(1.0, e));
             }
+            tv[gi][j] = r;
+            if (!full && jg + j < w && jg + j >= i) Trow[jg + j] = r;
+          }
+          if (full) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) st_global_v4(Trow + jg + 4 * q, tv[gi] + 4 * q);
           }
         }
       }
@@ -1847,7 +1872,7 @@ size_t oz_chol_workspace(int64_t np, int N) {
 
 tk_status oz_chol_begin(double* R, int64_t ldr, int64_t rstride, int N, int64_t np, void* work, size_t bytes,
                         int* err, OzCholPlan* plan, cudaStream_t st) {
-  if (np % 64 || (int64_t)N * OZ_S > 65535 || np > INT32_MAX) {
+  if (np % 64 || ldr % 4 || rstride % 4 || (uintptr_t)R % 32 || (int64_t)N * OZ_S > 65535 || np > INT32_MAX) {
     set_error_msg("emulated Cholesky: unsupported order or lambda count");
     return TK_EINVAL;
   }
