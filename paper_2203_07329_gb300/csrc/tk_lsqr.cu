@@ -581,9 +581,15 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
   }
   TK_TRY(launch_vstep<T>(Vraw, V, W, Y, nv, sc, coef_buf, atol, btol, maxiter, 1, nact, st));
 
-  // steps per read of the scalars: several for problems whose steps are
-  // launch-bound (A of at most 2^24 elements), one otherwise
-  chunk = ((int64_t)m * n <= (int64_t(1) << 24)) ? 4 : 1;
+  // Steps per read of the scalars: a read drains the GPU for about 15 us, a step takes 30 us (A of 2^20
+  // elements) to 300 us (2^26).  They are launched directly: a CUDA graph of four steps per active count
+  // cost more to instantiate than its few replays saved (4096 x 256 mixed, 8 lambda: 4.85 ms with
+  // graphs, 4.1 without).
+  const int64_t elems = (int64_t)m * n;
+  const int chunk = elems <= (int64_t(1) << 24) ? 4 : elems <= (int64_t(1) << 26) ? 2 : 1;
+  // Small problems keep finished slots in place until the products get cheaper without them (their cost
+  // goes by tiles of 4, 8, 16 and 32 lambda): a retirement is a dozen copies and launches.
+  const auto tile_class = [](size_t k) { return k <= 4 ? (k + 3) / 4 : k <= 8 ? size_t(2) : k <= 16 ? size_t(3) : 3 + (k + 31) / 32; };
   std::vector<Scal> hsc(N_cap);
   std::vector<int> hlam(N_cap);
   int* d_src = idx_buf;
@@ -595,7 +601,7 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
     TK_CUDA(cudaStreamSynchronize(st));
     std::vector<int> ret, keep;
     for (int s = 0; s < nact; ++s) (hsc[s].istop != 0 ? ret : keep).push_back(s);
-    if (!ret.empty()) {
+    if (!ret.empty() && (chunk == 1 || tile_class(keep.size()) < tile_class(nact))) {
       const int nr = (int)ret.size();
       TK_CUDA(cudaMemcpyAsync(d_ret, ret.data(), sizeof(int) * nr, cudaMemcpyHostToDevice, st));
       // x = R^-1 y (over) or x = z[0:n] (under)
@@ -652,17 +658,10 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
       TK_CUDA(cudaStreamSynchronize(st));
     }
     if (nact == 0) break;
-    // ------------------------------------------- `chunk` steps, one replay
-    // Small problems run several steps between two reads of the scalars (a
-    // slot that converges inside the chunk stays as it is: its kernels skip
-    // it), replayed from a CUDA graph captured once per active count.
-    const tk_status sr = steps(nact, chunk);
-    if (sr != TK_OK) {
-      release_graphs();
-      return sr;
-    }
+    // ------------------------------------------- `chunk` steps between two reads of the scalars (a
+    // slot that converges inside stays as it is: its norm and v-step return at once)
+    for (int c = 0; c < chunk; ++c) TK_TRY(step(nact));
   }
-  release_graphs();
   if (tc) TK_TRY(tc_lmaj_check(tc_scratch, N_cap, std::max(n, m), st));
   return TK_OK;
 }
@@ -706,74 +705,6 @@ tk_status Lsqr<T>::step(int nact) {
     TK_LAUNCH_CHECK();
   }
   return launch_vstep<T>(Vraw, V, W, Y, nv, sc, coef_buf, atol, btol, maxiter, 0, nact, st);
-}
-
-// `count` steps for `nact` active slots: launched directly (count 1, a
-// profiling run, or the tensor-core products), else replayed from a graph
-// captured the first time this active count is met.
-template <typename T>
-tk_status Lsqr<T>::steps(int nact, int count) {
-  if (count <= 1 || prof_enabled() || tc) {
-    for (int c = 0; c < count; ++c) TK_TRY(step(nact));
-    return TK_OK;
-  }
-  // graphs are captured and replayed on a stream of the engine's own (the
-  // caller's may be the legacy default stream, which cannot be captured),
-  // ordered after the caller's stream and before its next work by events
-  if (!gstream) {
-    TK_CUDA(cudaStreamCreateWithFlags(&gstream, cudaStreamNonBlocking));
-    TK_CUDA(cudaEventCreateWithFlags(&gev[0], cudaEventDisableTiming));
-    TK_CUDA(cudaEventCreateWithFlags(&gev[1], cudaEventDisableTiming));
-  }
-  auto it = graphs.find(nact);
-  if (it == graphs.end()) {
-    cudaStream_t caller = st;
-    st = gstream;
-    TK_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    tk_status r = TK_OK;
-    for (int c = 0; c < count && r == TK_OK; ++c) r = step(nact);
-    cudaGraph_t g = nullptr;
-    const cudaError_t ce = cudaStreamEndCapture(st, &g);
-    st = caller;
-    if (r != TK_OK) {
-      if (g) cudaGraphDestroy(g);
-      return r;
-    }
-    if (ce != cudaSuccess) {
-      set_error(ce, __FILE__, __LINE__);
-      return TK_ECUDA;
-    }
-    size_t nodes = 0;
-    cudaGraphGetNodes(g, nullptr, &nodes);
-    cudaGraphExec_t ge = nullptr;
-    const cudaError_t ie = cudaGraphInstantiate(&ge, g, 0);
-    cudaGraphDestroy(g);
-    if (ie != cudaSuccess) {
-      set_error(ie, __FILE__, __LINE__);
-      return TK_ECUDA;
-    }
-    it = graphs.emplace(nact, std::make_pair(ge, nodes)).first;
-  }
-  TK_CUDA(cudaEventRecord(gev[0], st));
-  TK_CUDA(cudaStreamWaitEvent(gstream, gev[0], 0));
-  TK_CUDA(cudaGraphLaunch(it->second.first, gstream));
-  TK_CUDA(cudaEventRecord(gev[1], gstream));
-  TK_CUDA(cudaStreamWaitEvent(st, gev[1], 0));
-  count_launches(it->second.second);
-  return TK_OK;
-}
-
-template <typename T>
-void Lsqr<T>::release_graphs() {
-  for (auto& kv : graphs) cudaGraphExecDestroy(kv.second.first);
-  graphs.clear();
-  if (gstream) {
-    cudaStreamSynchronize(gstream);
-    cudaStreamDestroy(gstream);
-    cudaEventDestroy(gev[0]);
-    cudaEventDestroy(gev[1]);
-    gstream = nullptr;
-  }
 }
 
 template struct Lsqr<double>;

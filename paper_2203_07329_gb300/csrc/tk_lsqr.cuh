@@ -1,9 +1,7 @@
 // Batched preconditioned LSQR engine (internal).
 #pragma once
 
-#include <map>
 #include <type_traits>
-#include <utility>
 #include <vector>
 
 #include "tk_internal.cuh"
@@ -242,14 +240,8 @@ struct Lsqr {
   tk_status prod_atu(const T* Uin, int count);
   tk_status prod_fused(const T* Win, T* C, const double* beta, int count);
   tk_status norm(int nact);
-  // one LSQR step for slots 0..nact-1; `count` of them (see steps())
+  // one LSQR step for slots 0..nact-1
   tk_status step(int nact);
-  tk_status steps(int nact, int count);
-  void release_graphs();
-  int chunk = 1;
-  std::map<int, std::pair<cudaGraphExec_t, size_t>> graphs;  // active count -> (replay, kernel nodes)
-  cudaStream_t gstream = nullptr;
-  cudaEvent_t gev[2] = {nullptr, nullptr};
 };
 
 }  // namespace tk
