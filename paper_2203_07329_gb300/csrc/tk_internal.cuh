@@ -30,6 +30,7 @@ void set_error_msg(const char* msg);
 // Every kernel launch of the library is followed by TK_LAUNCH_CHECK(), which
 // also counts it (tk_launch_count()).
 void count_launch();
+void count_launches(size_t n);  // n kernels of a replayed graph
 #define TK_LAUNCH_CHECK()   \
   do {                      \
     ::tk::count_launch();   \

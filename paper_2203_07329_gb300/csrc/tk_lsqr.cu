@@ -326,6 +326,11 @@ __global__ void k_move_scal(Scal* __restrict__ sc, int* __restrict__ slot_lam, d
   }
 }
 
+// Slots from .. to - 1 hold nothing any more: skipped by the norm and the v-step.
+__global__ void k_mark_done(Scal* __restrict__ sc, int from, int to) {
+  for (int k = from + threadIdx.x; k < to; k += blockDim.x) sc[k].istop = -1;
+}
+
 // X_out[lam] (+)= Xs[slot] for the listed slots (first n entries of rows of length ld)
 template <typename T>
 __global__ void k_scatter_out(const T* __restrict__ Xs, int64_t ld, int64_t n, const int* __restrict__ slots,
@@ -442,6 +447,10 @@ tk_status Lsqr<T>::apply_prec(bool transposed, const T* in, T* out, int count, i
   prof_end(tok, st, 4.0 * count * len * lr_s, es * (len * lr_s + 2.0 * count * len));
   return r;
 }
+
+// Largest A whose steps are replayed: beyond, a step takes a millisecond, and every retirement should
+// make the next step cheaper.
+constexpr int64_t kReplayMaxElems = int64_t(1) << 27;
 
 inline double total_count(int count, int64_t m) { return (double)count * (double)m; }
 
@@ -582,14 +591,33 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
   TK_TRY(launch_vstep<T>(Vraw, V, W, Y, nv, sc, coef_buf, atol, btol, maxiter, 1, nact, st));
 
   // Steps per read of the scalars: a read drains the GPU for about 15 us, a step takes 30 us (A of 2^20
-  // elements) to 300 us (2^26).  They are launched directly: a CUDA graph of four steps per active count
-  // cost more to instantiate than its few replays saved (4096 x 256 mixed, 8 lambda: 4.85 ms with
-  // graphs, 4.1 without).
+  // elements) to 300 us (2^26).
   const int64_t elems = (int64_t)m * n;
   const int chunk = elems <= (int64_t(1) << 24) ? 4 : elems <= (int64_t(1) << 26) ? 2 : 1;
-  // Small problems keep finished slots in place until the products get cheaper without them (their cost
-  // goes by tiles of 4, 8, 16 and 32 lambda): a retirement is a dozen copies and launches.
-  const auto tile_class = [](size_t k) { return k <= 4 ? (k + 3) / 4 : k <= 8 ? size_t(2) : k <= 16 ? size_t(3) : 3 + (k + 31) / 32; };
+  // The steps of a chunk are captured once per slot count and replayed: two dependent launches of a
+  // stream are 4.1 us apart at least, the kernels of a graph 1.5, and a step has 8 to 12 of them.  So that a
+  // few graphs serve the whole solve (all refinement rounds), the engine runs slot counts 4, 8, 16, 32,
+  // 64, ..: finished slots stay in place, skipped by the norm and the v-step, until the count falls into
+  // the next smaller class, which is also where the products get cheaper (tiles of 4, 8, 16, 32 lambda).
+  const bool replays = elems <= kReplayMaxElems && !prof_enabled() && !tc;
+  const auto slots_for = [&](int k) {
+    const int c = k <= 4 ? 4 : k <= 8 ? 8 : k <= 16 ? 16 : (k + 31) / 32 * 32;
+    return replays ? std::min(c, count) : k;
+  };
+  cudaStream_t caller = st;
+  if (replays) {  // on the replays' own stream, ordered behind the caller's work and before its next
+    if (!graphs.st) {
+      TK_CUDA(cudaStreamCreateWithFlags(&graphs.st, cudaStreamNonBlocking));
+      TK_CUDA(cudaEventCreateWithFlags(&graphs.ev, cudaEventDisableTiming));
+    }
+    TK_CUDA(cudaEventRecord(graphs.ev, st));
+    TK_CUDA(cudaStreamWaitEvent(graphs.st, graphs.ev, 0));
+    st = graphs.st;
+  }
+  struct Restore {
+    cudaStream_t &st, caller;
+    ~Restore() { st = caller; }
+  } restore{st, caller};
   std::vector<Scal> hsc(N_cap);
   std::vector<int> hlam(N_cap);
   int* d_src = idx_buf;
@@ -601,7 +629,12 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
     TK_CUDA(cudaStreamSynchronize(st));
     std::vector<int> ret, keep;
     for (int s = 0; s < nact; ++s) (hsc[s].istop != 0 ? ret : keep).push_back(s);
-    if (!ret.empty() && (chunk == 1 || tile_class(keep.size()) < tile_class(nact))) {
+    // slots whose solution was written are marked -1
+    for (size_t k = 0; k < ret.size();) {
+      if (hsc[ret[k]].istop < 0) ret.erase(ret.begin() + k);
+      else ++k;
+    }
+    if (!ret.empty() && (keep.empty() || slots_for((int)keep.size()) < nact)) {
       const int nr = (int)ret.size();
       TK_CUDA(cudaMemcpyAsync(d_ret, ret.data(), sizeof(int) * nr, cudaMemcpyHostToDevice, st));
       // x = R^-1 y (over) or x = z[0:n] (under)
@@ -634,13 +667,14 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
         r.arnorm = q.arnorm;
         results.push_back(r);
       }
-      // compaction: survivors beyond the new end move into holes below it
-      const int nnew = nact - nr;
+      // compaction: survivors beyond the new end move into holes below it; the slots from nkeep on are left
+      // marked -1
+      const int nkeep = (int)keep.size(), nnew = nkeep ? slots_for(nkeep) : 0;
       std::vector<int> holes, srcs;
-      for (int s : ret)
-        if (s < nnew) holes.push_back(s);
+      for (int s = 0; s < nkeep; ++s)
+        if (hsc[s].istop != 0) holes.push_back(s);
       for (int s : keep)
-        if (s >= nnew) srcs.push_back(s);
+        if (s >= nkeep) srcs.push_back(s);
       const int moves = (int)holes.size();
       if (moves > 0) {
         TK_CUDA(cudaMemcpyAsync(d_src, srcs.data(), sizeof(int) * moves, cudaMemcpyHostToDevice, st));
@@ -653,6 +687,10 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
         k_move_scal<<<1, 128, 0, st>>>(sc, slot_lam, coef_buf, d_src, d_dst, moves);
         TK_LAUNCH_CHECK();
       }
+      if (nnew > nkeep) {
+        k_mark_done<<<1, 128, 0, st>>>(sc, nkeep, nnew);
+        TK_LAUNCH_CHECK();
+      }
       nact = nnew;
       // the host copies of d_src/d_dst/d_ret must stay valid until the copies ran
       TK_CUDA(cudaStreamSynchronize(st));
@@ -660,7 +698,15 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
     if (nact == 0) break;
     // ------------------------------------------- `chunk` steps between two reads of the scalars (a
     // slot that converges inside stays as it is: its norm and v-step return at once)
-    for (int c = 0; c < chunk; ++c) TK_TRY(step(nact));
+    if (replays) {
+      TK_TRY(replay(nact, chunk));
+    } else {
+      for (int c = 0; c < chunk; ++c) TK_TRY(step(nact));
+    }
+  }
+  if (replays) {  // the caller's stream continues behind the replays
+    TK_CUDA(cudaEventRecord(graphs.ev, st));
+    TK_CUDA(cudaStreamWaitEvent(caller, graphs.ev, 0));
   }
   if (tc) TK_TRY(tc_lmaj_check(tc_scratch, N_cap, std::max(n, m), st));
   return TK_OK;
@@ -705,6 +751,41 @@ tk_status Lsqr<T>::step(int nact) {
     TK_LAUNCH_CHECK();
   }
   return launch_vstep<T>(Vraw, V, W, Y, nv, sc, coef_buf, atol, btol, maxiter, 0, nact, st);
+}
+
+// `count` steps for slots 0..nact-1 on graphs.st, captured the first time this slot count is met.
+template <typename T>
+tk_status Lsqr<T>::replay(int nact, int count) {
+  const StepGraphs::Entry* e = nullptr;
+  for (const auto& g : graphs.entries)
+    if (g.slots == nact) e = &g;
+  if (!e) {
+    TK_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+    tk_status r = TK_OK;
+    for (int c = 0; c < count && r == TK_OK; ++c) r = step(nact);
+    cudaGraph_t g = nullptr;
+    const cudaError_t ce = cudaStreamEndCapture(st, &g);
+    if (r != TK_OK || ce != cudaSuccess) {
+      if (g) cudaGraphDestroy(g);
+      if (r != TK_OK) return r;
+      set_error(ce, __FILE__, __LINE__);
+      return TK_ECUDA;
+    }
+    size_t nodes = 0;
+    cudaGraphGetNodes(g, nullptr, &nodes);
+    cudaGraphExec_t ge = nullptr;
+    const cudaError_t ie = cudaGraphInstantiate(&ge, g, 0);
+    cudaGraphDestroy(g);
+    if (ie != cudaSuccess) {
+      set_error(ie, __FILE__, __LINE__);
+      return TK_ECUDA;
+    }
+    graphs.entries.push_back({nact, ge, nodes});
+    e = &graphs.entries.back();
+  }
+  TK_CUDA(cudaGraphLaunch(e->exec, st));
+  count_launches(e->nodes);
+  return TK_OK;
 }
 
 template struct Lsqr<double>;

@@ -163,6 +163,28 @@ __device__ __forceinline__ void vstep_block(const T* __restrict__ Vraw, T* __res
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The replays of one solve: chunks of LSQR steps captured once per slot count, and the stream they run
+// on (the caller's may be the legacy default stream, which cannot be captured).
+struct StepGraphs {
+  cudaStream_t st = nullptr;
+  cudaEvent_t ev = nullptr;
+  struct Entry {
+    int slots;
+    cudaGraphExec_t exec;
+    size_t nodes;
+  };
+  std::vector<Entry> entries;
+  StepGraphs() = default;
+  StepGraphs(const StepGraphs&) = delete;
+  StepGraphs& operator=(const StepGraphs&) = delete;
+  ~StepGraphs() {
+    if (st) cudaStreamSynchronize(st);
+    for (auto& e : entries) cudaGraphExecDestroy(e.exec);
+    if (ev) cudaEventDestroy(ev);
+    if (st) cudaStreamDestroy(st);
+  }
+};
+
 template <typename T>
 struct Lsqr {
   // problem: A (m x n, row stride lda) in the compute type
@@ -240,8 +262,10 @@ struct Lsqr {
   tk_status prod_atu(const T* Uin, int count);
   tk_status prod_fused(const T* Win, T* C, const double* beta, int count);
   tk_status norm(int nact);
-  // one LSQR step for slots 0..nact-1
+  // one LSQR step for slots 0..nact-1; `count` of them, replayed from a graph
   tk_status step(int nact);
+  tk_status replay(int nact, int count);
+  StepGraphs graphs;
 };
 
 }  // namespace tk
