@@ -113,8 +113,9 @@ typedef struct {
                              (see tk_gram_emulated, tk_cholesky_shifted_emulated, tk_residual) instead of
                              the float64 pipe, with the same float64 accuracy: MIXED: the Gram matrix, the
                              Cholesky trailing updates, and the refinement's r = b - A x and A^T r; FP64:
-                             the Gram matrix, the trailing updates and the two products with A of every
-                             LSQR step (and the Gaussian sketch), when A has 2^19 .. 2^32 elements.  Costs 32 (MIXED) or 16 (FP64) bytes of workspace per element of
+                             the Gaussian sketch, the Gram matrix and the trailing updates when A has
+                             2^16 .. 2^32 elements, and the two products with A of every LSQR step when it
+                             has 2^19 or more.  Costs 32 (MIXED) or 16 (FP64) bytes of workspace per element of
                              A for the digit planes; 0 = float64 FMA. */
   const double* x0;       /* [NULL] warm start, device N x n float64 (row i for lambdas[i]; m >= n only):
                              the solve starts from x = x0 instead of 0 and returns the same minimiser of

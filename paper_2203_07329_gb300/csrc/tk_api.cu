@@ -54,7 +54,7 @@ struct Plan {
 constexpr int64_t kMaxShort = 8192;
 constexpr int64_t kMaxLong = (int64_t(1) << 30);
 constexpr double kInv64Cost = 8e7;  // N c^2 up to which the explicit float64 inverse costs less than the substitutions
-constexpr int64_t kOz64MinElems = int64_t(1) << 19;  // smallest A (elements) that the float64 form splits into digits
+constexpr int64_t kOz64MinElems = int64_t(1) << 16;  // smallest A (elements) that the float64 form splits into digits
 
 tk_status check_opts(const tk_opts* o) {
   if (!o) return einval("options pointer is NULL");
@@ -79,9 +79,8 @@ tk_status check_opts(const tk_opts* o) {
 }
 
 // The float64 form with emulate_fp64: whether the solve makes digit planes of A at all.  They pay off
-// when A is large enough that a product is not all launch latency (4096 x 256, 8 lambda: 20 us from
-// digits, 37 on the float64 pipe; a single lambda of 30000 x 1000: 105 us against 560, the pipe's
-// smallest tile being 8 rows); A of more than 2^32 elements keeps the float64 pipe, because the planes
+// for the Gaussian sketch, the Gram matrix and the Cholesky updates (2000 x 64: 25 us to make them, 400
+// us less work on the float64 pipe) and, for larger A, the LSQR products (use_oz); A of more than 2^32 elements keeps the float64 pipe, because the planes
 // take 16 bytes per element.
 bool oz64_wanted(int64_t m, int64_t n) { return m * n >= kOz64MinElems && m * n <= (int64_t(1) << 32); }
 
@@ -353,20 +352,35 @@ __global__ void k_gather_x(const double* __restrict__ X, int64_t n, const int* _
 }
 // g_k = sum_z partial - lambda_l x_l  (float64 normal-equation residual
 // A^T (b - A x) - lambda x of the k-th listed lambda); nrm[3k] = ||g_k||
-__global__ void k_ne_finish(const double* __restrict__ part, int splits, int count, int64_t n,
-                            const int* __restrict__ ids, const double* __restrict__ lam, const double* __restrict__ Xa,
-                            double* __restrict__ G, double* __restrict__ nrm) {
+// One block per lambda: 32 columns x 8 groups of planes at a time (a thread per column walking all planes
+// took 90 us at n = 777, 76 planes).
+__global__ void __launch_bounds__(1024)
+    k_ne_finish(const double* __restrict__ part, int splits, int count, int64_t n, const int* __restrict__ ids,
+                const double* __restrict__ lam, const double* __restrict__ Xa, double* __restrict__ G,
+                double* __restrict__ nrm) {
   __shared__ double sh[32];
-  const int k = blockIdx.x;
+  __shared__ double pl[8][129];
+  const int k = blockIdx.x, tx = threadIdx.x & 127, ty = threadIdx.x >> 7;
   const double lv = lam[ids[k]];
   const int64_t plane = (int64_t)count * n;
   double acc = 0.0;
-  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+  for (int64_t j0 = 0; j0 < n; j0 += 128) {
+    const int64_t j = j0 + tx;
     double g = 0.0;
-    for (int z = 0; z < splits; ++z) g += part[z * plane + (int64_t)k * n + j];
-    g = fma(-lv, Xa[(int64_t)k * n + j], g);
-    G[(int64_t)k * n + j] = g;
-    acc = fma(g, g, acc);
+    if (j < n) {
+#pragma unroll 4
+      for (int z = ty; z < splits; z += 8) g += part[z * plane + (int64_t)k * n + j];
+    }
+    pl[ty][tx] = g;
+    __syncthreads();
+    if (ty == 0 && j < n) {
+#pragma unroll
+      for (int q = 1; q < 8; ++q) g += pl[q][tx];
+      g = fma(-lv, Xa[(int64_t)k * n + j], g);
+      G[(int64_t)k * n + j] = g;
+      acc = fma(g, g, acc);
+    }
+    __syncthreads();
   }
   acc = block_sum(acc, sh);
   if (threadIdx.x == 0) nrm[3 * k] = sqrt(acc);
@@ -825,7 +839,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
         }
         prof_end(tok, st, fl, ea * P.m * P.n + 8.0 * (cnt * P.m + (double)sp * cnt * P.n),
                  (P.o.emulate_fp64 ? 16.0 : ea) * P.m * P.n + 8.0 * (cnt * P.m + (double)sp * cnt * P.n));
-        k_ne_finish<<<cnt, 256, 0, st>>>(B.part, sp, cnt, P.n, B.ids, B.lam, B.Xa, B.G, B.nrm);
+        k_ne_finish<<<cnt, 1024, 0, st>>>(B.part, sp, cnt, P.n, B.ids, B.lam, B.Xa, B.G, B.nrm);
         TK_LAUNCH_CHECK();
         // correction: min ||B d - [0; g/sqrt(l)]||, whose normal equations are
         // (A^T A + l I) d = g; the right-hand side shrinks with the error of x.
@@ -912,18 +926,16 @@ __global__ void k_lc_norms(const double* __restrict__ R, int64_t m, const double
 // Curvature on the ascending grid lam[0..N): kappa[0] = kappa[N-1] = 0; the
 // corner is the first largest interior kappa (*corner = -1 if N < 3).  With
 // nr > 0, also the second sweep: nr parameters log-spaced strictly between the
-// corner's neighbours.  One thread: N is a few dozen.
-__global__ void k_lc_curvature(const double* __restrict__ lam, const double* __restrict__ rn,
-                               const double* __restrict__ xn, int N, double* __restrict__ kappa,
-                               int* __restrict__ corner, int nr, double* __restrict__ next) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int i = 0; i < N; ++i) kappa[i] = 0.0;
-  if (N < 3) {
-    *corner = -1;
-    return;
-  }
-  int best = 1;
-  for (int k = 1; k < N - 1; ++k) {
+// corner's neighbours.  One block, a thread per point (one thread for all of
+// them took 390 us for 32 points).
+__global__ void __launch_bounds__(256)
+    k_lc_curvature(const double* __restrict__ lam, const double* __restrict__ rn, const double* __restrict__ xn, int N,
+                   double* __restrict__ kappa, int* __restrict__ corner, int nr, double* __restrict__ next) {
+  for (int k = threadIdx.x; k < N; k += blockDim.x) {
+    if (k == 0 || k == N - 1) {
+      kappa[k] = 0.0;
+      continue;
+    }
     const double t0 = log(lam[k - 1]), t1 = log(lam[k]), t2 = log(lam[k + 1]);
     const double h1 = t1 - t0, h2 = t2 - t1;
     const double p0 = log(rn[k - 1]), p1 = log(rn[k]), p2 = log(rn[k + 1]);
@@ -937,12 +949,24 @@ __global__ void k_lc_curvature(const double* __restrict__ lam, const double* __r
     const double ddq = __dmul_rn(v0, q0) + __dmul_rn(v1, q1) + __dmul_rn(v2, q2);
     const double den = pow(__dmul_rn(dp, dp) + __dmul_rn(dq, dq), 1.5);
     kappa[k] = den > 0.0 ? (__dmul_rn(dp, ddq) - __dmul_rn(ddp, dq)) / den : 0.0;
-    if (kappa[k] > kappa[best]) best = k;
   }
-  *corner = best;
-  if (nr > 0) {
+  __syncthreads();
+  __shared__ int best_s;
+  if (threadIdx.x == 0) {
+    int best = -1;
+    if (N >= 3) {
+      best = 1;
+      for (int k = 2; k < N - 1; ++k)
+        if (kappa[k] > kappa[best]) best = k;
+    }
+    *corner = best;
+    best_s = best;
+  }
+  __syncthreads();
+  const int best = best_s;
+  if (nr > 0 && best > 0) {
     const double a = log(lam[best - 1]), b = log(lam[best + 1]);
-    for (int j = 1; j <= nr; ++j) next[j - 1] = exp(a + (b - a) * (double)j / (double)(nr + 1));
+    for (int j = 1 + threadIdx.x; j <= nr; j += blockDim.x) next[j - 1] = exp(a + (b - a) * (double)j / (double)(nr + 1));
   }
 }
 
@@ -1802,7 +1826,7 @@ TK_API tk_status tk_lcurve(const tk_problem* p, const double* lambdas, int N, in
   if (s1 == TK_EINVAL || s1 == TK_ENOMEM || s1 == TK_ECUDA || s1 == TK_ETIMEOUT) return s1;
   TK_CUDA(cudaMemcpyAsync(L.lam, lam.data(), sizeof(double) * N, cudaMemcpyHostToDevice, st));
   TK_TRY(lc_norms(p, P, B, L, L.Xs, N, 0, st));
-  k_lc_curvature<<<1, 32, 0, st>>>(L.lam, L.rn, L.xn, N, L.kappa, L.corner, N_refine, L.next);
+  k_lc_curvature<<<1, 256, 0, st>>>(L.lam, L.rn, L.xn, N, L.kappa, L.corner, N_refine, L.next);
   TK_LAUNCH_CHECK();
   std::vector<double> next(std::max(N_refine, 1));
   tk_status s2 = TK_OK;
@@ -1828,7 +1852,7 @@ TK_API tk_status tk_lcurve(const tk_problem* p, const double* lambdas, int N, in
   k_lc_permute<<<1, 256, 0, st>>>(L.perm, Np, L.lam, L.lam_m);
   k_lc_permute<<<1, 256, 0, st>>>(L.perm, Np, L.rn, L.rn_m);
   k_lc_permute<<<1, 256, 0, st>>>(L.perm, Np, L.xn, L.xn_m);
-  k_lc_curvature<<<1, 32, 0, st>>>(L.lam_m, L.rn_m, L.xn_m, Np, L.kappa, L.corner, 0, nullptr);
+  k_lc_curvature<<<1, 256, 0, st>>>(L.lam_m, L.rn_m, L.xn_m, Np, L.kappa, L.corner, 0, nullptr);
   // X rows in the merged order
   TK_LAUNCH_CHECK();
   k_gather_x<<<rgrid(P.n, Np), 256, 0, st>>>(L.Xs, P.n, L.perm, X);

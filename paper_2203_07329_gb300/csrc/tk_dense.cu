@@ -438,38 +438,49 @@ __global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ R, int
 // right-looking in the not yet finished blocks of M (zero on entry).  Mt
 // receives M^T (its blocks above the diagonal are left unwritten).
 
-// M_kk = R_kk^-1: thread c back-substitutes column c of the identity.
+// M_kk = R_kk^-1: back substitution of the identity's columns, 16 of them per CTA (blockIdx.z); the half-warps
+// of 4 warps hold the rows of one residue mod 8 each, one barrier a row (as k_chol_trsm16: all quarters of
+// the float64 pipe; two warps with a column per thread took 83 us).
 template <typename T>
-__global__ void __launch_bounds__(CB) k_tinv_diag(const double* __restrict__ R, int64_t ldr, int64_t rstride,
-                                                  T* __restrict__ M, T* __restrict__ Mt, int64_t ldm,
-                                                  int64_t mstride) {
+__global__ void __launch_bounds__(128) k_tinv_diag(const double* __restrict__ R, int64_t ldr, int64_t rstride,
+                                                   T* __restrict__ M, T* __restrict__ Mt, int64_t ldm,
+                                                   int64_t mstride) {
   __shared__ double D[CB][CB + 1];
-  const int kb = blockIdx.x, l = blockIdx.y, c = threadIdx.x;
+  __shared__ double Dinv[CB];  // one division per row and tile
+  __shared__ double xs[CB][17];
+  const int kb = blockIdx.x, l = blockIdx.y, c0 = 16 * (int)blockIdx.z, cc = threadIdx.x & 15, g = threadIdx.x >> 4;
   const double* Rg = R + (int64_t)l * rstride + (int64_t)kb * CB * ldr + (int64_t)kb * CB;
-  __shared__ double Dinv[CB];  // one division per row and tile, not one per row and column
 #pragma unroll 8
-  for (int i = 0; i < CB; ++i) D[i][c] = Rg[(int64_t)i * ldr + c];
-  Dinv[c] = 1.0 / Rg[(int64_t)c * ldr + c];
-  __syncthreads();
-  double x[CB];
+  for (int idx = threadIdx.x; idx < CB * CB; idx += 128) D[idx / CB][idx % CB] = Rg[(int64_t)(idx / CB) * ldr + idx % CB];
+  if (threadIdx.x < CB) Dinv[threadIdx.x] = 1.0 / Rg[(int64_t)threadIdx.x * ldr + threadIdx.x];
+  double x[CB / 8];  // rows 8 q + g of column c0 + cc
 #pragma unroll
-  for (int r = 0; r < CB; ++r) x[r] = (r == c) ? 1.0 : 0.0;
+  for (int q = 0; q < CB / 8; ++q) x[q] = 8 * q + g == c0 + cc ? 1.0 : 0.0;
+  __syncthreads();
+  if (g == 7) xs[CB - 1][cc] = x[CB / 8 - 1] * Dinv[CB - 1];
+  __syncthreads();
 #pragma unroll
   for (int r = CB - 1; r >= 0; --r) {
-    x[r] = x[r] * Dinv[r];
+    const double v = xs[r][cc];
+    // the next row up first, then the rest behind it
+    if (r > 0 && g == ((r - 1) & 7)) {
+      const int q = (r - 1) >> 3;
+      xs[r - 1][cc] = fma(-D[r - 1][r], v, x[q < 0 ? 0 : q]) * Dinv[r - 1];
+    }
 #pragma unroll
-    for (int q = 0; q < r; ++q) x[q] = fma(-D[q][r], x[r], x[q]);
+    for (int q = 0; q < CB / 8; ++q)
+      if (8 * q <= r - 2) {
+        const int i = 8 * q + g;
+        if (i <= r - 2) x[q] = fma(-D[i][r], v, x[q]);
+      }
+    __syncthreads();
   }
-  __syncthreads();
-  T* Mg = M + (int64_t)l * mstride + (int64_t)kb * CB * ldm + (int64_t)kb * CB;
-#pragma unroll
-  for (int r = 0; r < CB; ++r) {
-    Mg[(int64_t)r * ldm + c] = (T)x[r];
-    D[r][c] = x[r];
+  T* Mg = M + (int64_t)l * mstride + (int64_t)kb * CB * ldm + (int64_t)kb * CB + c0;
+  T* Mtg = Mt + (int64_t)l * mstride + (int64_t)(kb * CB + c0) * ldm + (int64_t)kb * CB;
+  for (int idx = threadIdx.x; idx < CB * 16; idx += 128) {
+    Mg[(int64_t)(idx / 16) * ldm + idx % 16] = (T)xs[idx / 16][idx % 16];
+    Mtg[(int64_t)(idx / CB) * ldm + idx % CB] = (T)xs[idx % CB][idx / CB];
   }
-  __syncthreads();
-  T* Mtg = Mt + (int64_t)l * mstride + (int64_t)kb * CB * ldm + (int64_t)kb * CB;
-  for (int i = 0; i < CB; ++i) Mtg[(int64_t)i * ldm + c] = (T)D[c][i];
 }
 
 // S_{rb,cb} -= R_{rb,k} M_{k,cb} for rb < k <= cb (arithmetic in T; R read as float64).
@@ -964,7 +975,7 @@ tk_status tri_inverse(const double* R, int64_t n, int64_t ldr, int64_t rstride, 
   const int64_t np = cdiv(n, CB) * CB;
   const int nt = (int)(np / CB);
   TK_CUDA(cudaMemsetAsync(M, 0, sizeof(T) * (size_t)N * np * np, st));
-  k_tinv_diag<T><<<dim3((unsigned)nt, (unsigned)N), CB, 0, st>>>(R, ldr, rstride, M, Mt, np, np * np);
+  k_tinv_diag<T><<<dim3((unsigned)nt, (unsigned)N, CB / 16), 128, 0, st>>>(R, ldr, rstride, M, Mt, np, np * np);
   TK_LAUNCH_CHECK();
   for (int k = nt - 1; k >= 1; --k) {
     k_tinv_update<T><<<dim3((unsigned)(k * (nt - k)), (unsigned)N), 256, 0, st>>>(R, ldr, rstride, M, np, np * np,

@@ -133,6 +133,21 @@ __device__ __forceinline__ double gauss_entry(uint64_t seed, uint64_t k, double 
   return ((lane & 1) ? r * sn : r * cs) * inv_sqrt_s;
 }
 
+// Entries 4 g .. 4 g + 3 of the same stream: one Philox call, two Box-Muller pairs.
+__device__ __forceinline__ void gauss_entries4(uint64_t seed, uint64_t g, double inv_sqrt_s, double (&v)[4]) {
+  const uint4 w = philox(g, STREAM_GAUSS, seed);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const double u1 = ((double)(h ? w.z : w.x) + 1.0) * 2.3283064365386962890625e-10;
+    const double u2 = (double)(h ? w.w : w.y) * 2.3283064365386962890625e-10;
+    const double r = sqrt(-2.0 * log(u1));
+    double sn, cs;
+    sincospi(2.0 * u2, &sn, &cs);
+    v[2 * h] = (r * cs) * inv_sqrt_s;
+    v[2 * h + 1] = (r * sn) * inv_sqrt_s;
+  }
+}
+
 // -------------------------------------------------------------- reduce --
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {

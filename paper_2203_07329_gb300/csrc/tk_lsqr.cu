@@ -126,6 +126,14 @@ __global__ void __launch_bounds__(256)
     }
   }
   acc = block_sum(acc, sh);
+  if (chunks == 1) {
+    if (threadIdx.x == 0) {
+      const double beta = sqrt(acc), al = sc[s].alpha;
+      sc[s].anorm2 += al * al + beta * beta;
+      sc[s].beta = beta;
+    }
+    return;
+  }
   if (threadIdx.x == 0) {
     partial[s * kSumChunks + c] = acc;
     __threadfence();
@@ -714,8 +722,8 @@ tk_status Lsqr<T>::run(const double* b, int64_t ldbt, const double* bbot, int64_
 
 template <typename T>
 tk_status Lsqr<T>::norm(int nact) {
-  // enough blocks for every SM, at least 2048 values to a block
-  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>({kSumChunks, cdiv(m, 2048), cdiv(8 * 152, nact)}));
+  // enough blocks for every SM, at least 4096 values to a block (one block needs no second sum)
+  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>({kSumChunks, cdiv(m, 4096), cdiv(8 * 152, nact)}));
   k_over_norm<T><<<dim3((unsigned)chunks, (unsigned)nact), 256, 0, st>>>(Ut, m, Tt, Ub, n, sc, part_u, arrivals);
   TK_LAUNCH_CHECK();
   return TK_OK;

@@ -44,18 +44,19 @@ struct VGivens {
   double ainv, t1, t2;  // 1 / alpha, phi / rho, theta / rho
   double c, rhobar, phibar;
 };
-__device__ __forceinline__ VGivens vstep_givens(const Scal& q, double alpha) {
+// Roots and quotients through reciprocal roots: a float64 division or root is a dependent chain of a
+// dozen instructions on a slow pipe, and this is on the critical path of every step.
+__device__ __forceinline__ VGivens vstep_givens(const Scal& q, double alpha, double ainv) {
   VGivens g;
-  const double beta = q.beta;
-  const double rho = sqrt(q.rhobar * q.rhobar + beta * beta);
-  const double rinv = rho > 0.0 ? 1.0 / rho : 0.0;
-  g.c = rho > 0.0 ? q.rhobar / rho : 1.0;
-  const double sn = rho > 0.0 ? beta / rho : 0.0;
+  const double r2 = fma(q.rhobar, q.rhobar, q.beta * q.beta);
+  const double rinv = r2 > 0.0 ? rsqrt(r2) : 0.0;
+  g.c = r2 > 0.0 ? q.rhobar * rinv : 1.0;
+  const double sn = q.beta * rinv;
   g.rhobar = -g.c * alpha;
   g.phibar = sn * q.phibar;
   g.t1 = g.c * q.phibar * rinv;
   g.t2 = sn * alpha * rinv;
-  g.ainv = alpha > 0.0 ? 1.0 / alpha : 0.0;
+  g.ainv = ainv;
   return g;
 }
 __device__ __forceinline__ void vstep_init_scal(Scal& q, double alpha) {
@@ -83,7 +84,7 @@ __device__ __forceinline__ void vstep_finish_scal(Scal& q, const VGivens& g, dou
   int istop = 0;
   if (!isfinite(alpha) || !isfinite(beta) || !isfinite(ynorm)) istop = 5;
   else if (rnorm == 0.0) istop = 1;
-  else if (arnorm / (anorm * rnorm) <= atol) istop = 2;
+  else if (arnorm <= atol * (anorm * rnorm)) istop = 2;
   else if (rnorm <= btol * q.bnorm + atol * anorm * ynorm) istop = 1;
   else if (q.iters >= maxiter) istop = 7;
   q.istop = istop;
@@ -114,6 +115,8 @@ __device__ __forceinline__ void vstep_block(const T* __restrict__ Vraw, T* __res
     return v;
   };
   const int64_t first = (int64_t)rank * blockDim.x + threadIdx.x, stride = (int64_t)CL * blockDim.x;
+  __shared__ double bc[3];  // 1 / alpha, phi / rho, theta / rho from the first warp: every warp computing
+                            // them would queue for the float64 pipe (9.5 us a step at n = 256, now 6.3)
   // v' = Vraw - beta v  (init: v' = Vraw)
   double acc = 0.0;
 #pragma unroll 4
@@ -123,9 +126,22 @@ __device__ __forceinline__ void vstep_block(const T* __restrict__ Vraw, T* __res
     V[j] = (T)v;
     acc = fma(v, v, acc);
   }
-  const double alpha = sqrt(cluster_sum(acc, 0));
+  const double a2 = cluster_sum(acc, 0);
+  double alpha = 0.0;
+  VGivens g;
+  if (threadIdx.x < 32) {
+    alpha = sqrt(a2);
+    const double ainv = a2 > 0.0 ? rsqrt(a2) : 0.0;
+    g = vstep_givens(q, alpha, ainv);
+    if (threadIdx.x == 0) {
+      bc[0] = g.ainv;
+      bc[1] = g.t1;
+      bc[2] = g.t2;
+    }
+  }
+  __syncthreads();
+  const double ainv = bc[0], t1 = bc[1], t2 = bc[2];
   if (init) {
-    const double ainv = alpha > 0.0 ? 1.0 / alpha : 0.0;
     for (int64_t j = first; j < nv; j += stride) {
       T v = (T)((double)V[j] * ainv);
       V[j] = v;
@@ -138,21 +154,21 @@ __device__ __forceinline__ void vstep_block(const T* __restrict__ Vraw, T* __res
       if (coef_out) *coef_out = q.coef;
     }
   } else {
-    const VGivens g = vstep_givens(q, alpha);
     double yy = 0.0;
 #pragma unroll 4
     for (int64_t j = first; j < nv; j += stride) {
-      double v = (double)V[j] * g.ainv;
+      double v = (double)V[j] * ainv;
       double w = (double)W[j];
-      double y = fma(g.t1, w, (double)Y[j]);
-      w = fma(-g.t2, w, v);
+      double y = fma(t1, w, (double)Y[j]);
+      w = fma(-t2, w, v);
       V[j] = (T)v;
       W[j] = (T)w;
       Y[j] = (T)y;
       yy = fma(y, y, yy);
     }
-    const double ynorm = sqrt(cluster_sum(yy, 1));
+    const double y2 = cluster_sum(yy, 1);
     if (rank == 0 && threadIdx.x == 0) {
+      const double ynorm = sqrt(y2);
       vstep_finish_scal(q, g, alpha, ynorm, atol, btol, maxiter);
       *sq = q;
       if (coef_out) *coef_out = q.coef;
@@ -237,10 +253,11 @@ struct Lsqr {
   // number of lambdas; the SIMT products read 4 or 8 bytes but their work grows with it.  Float32: the
   // digits pay off for large A and more than 16 active lambdas.  Float64: the pipe (1.2 TFLOP/s) takes
   // 1.7 ps per element and lambda, the digits 2.7 ps per element, and the pipe's smallest tile does the
-  // work of 8 lambdas: always.
+  // work of 8 lambdas (a single lambda of 30000 x 1000: 560 us against 105; 4096 x 256, 8 lambda: 37 us
+  // against 20): whenever A has 2^19 elements (2000 x 64, one lambda: 15 us on the pipe, 20 from digits).
   bool use_oz(int count) const {
     if (!oz || !oz_A.planes) return false;
-    if (std::is_same<T, double>::value) return true;
+    if (std::is_same<T, double>::value) return (int64_t)m * n >= (int64_t(1) << 19);
     return (int64_t)m * n > (int64_t(1) << 24) && count > 16;
   }
   // both products of an overdetermined step in one kernel over one read of

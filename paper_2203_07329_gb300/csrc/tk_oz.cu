@@ -1836,11 +1836,21 @@ tk_status oz_sketch(const OzMat& A, bool under, const double* G, int64_t s, doub
   return TK_OK;
 }
 
+// Splits of the sum over the r rows of Y when the upper triangle's tiles (128 x 32) leave SMs idle.
+static int oz_gram_splits(int64_t r, int64_t c) {
+  int64_t tiles = 0;
+  for (int64_t i = 0; i < cdiv(c, OT_M); ++i) tiles += std::min<int64_t>(cdiv(c, OT_N), cdiv((i + 1) * OT_M, OT_N));
+  const int64_t want = tiles >= 152 ? 1 : 152 / tiles, maxs = std::max<int64_t>(1, r / (2 * OT_CHUNK));
+  return (int)std::max<int64_t>(std::min(want, maxs), cdiv(r, OT_MAX_KPS));
+}
+
 size_t oz_gram_workspace(int64_t r, int64_t c) {
   Arena a;
   a.take<char>(oz_slices_bytes(c, r));
   a.take<int>(c);
   a.take<char>(oz_colmax_bytes(c));
+  const int sp = oz_gram_splits(r, c);
+  if (sp > 1) a.take<double>((size_t)sp * c * c);
   return a.used + 256;
 }
 
@@ -1857,10 +1867,18 @@ tk_status oz_gram(const double* Y, int64_t r, int64_t c, double* C, void* work, 
   void* Ys = a.take<char>(oz_slices_bytes(c, r));
   int* E = a.take<int>(c);
   void* mx = a.take<char>(oz_colmax_bytes(c));
+  const int sp = oz_gram_splits(r, c);
+  double* part = sp > 1 ? a.take<double>((size_t)sp * c * c) : nullptr;
   if (!a.ok()) return TK_ENOMEM;
   TK_TRY(oz_split_columns(Y, r, c, Ys, E, mx, st));
-  return launch_oz_tc<OZ_S, 1, false>({Ys, E, c, r, false}, Ys, E, (int)c, OZ_S, 1, nullptr, C, c, nullptr, err, st,
-                                      1);
+  // n = 777, s = 12432: 0.47 ms in one piece on 100 of the 152 SMs, 0.18 in splits
+  TK_TRY((launch_oz_tc<OZ_S, 1, false>({Ys, E, c, r, false}, Ys, E, (int)c, OZ_S, sp, nullptr, sp > 1 ? part : C, c,
+                                       nullptr, err, st, 1)));
+  if (sp > 1) {  // (below the diagonal tiles the planes hold nothing: those sums are not read)
+    k_oz_sum_planes<<<(unsigned)std::min<int64_t>(cdiv(c * c, 256), 152 * 8), 256, 0, st>>>(part, sp, c * c, C);
+    TK_LAUNCH_CHECK();
+  }
+  return TK_OK;
 }
 
 size_t oz_chol_workspace(int64_t np, int N) {

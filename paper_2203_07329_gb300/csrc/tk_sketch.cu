@@ -374,12 +374,19 @@ tk_status srdct_impl(const TIn* A, int64_t L, int64_t cols, int64_t ld, uint64_t
   return TK_OK;
 }
 
+// Bound by the float64 pipe (logarithm, root, sine and cosine): four entries per thread share one Philox
+// call and two of each (an entry per thread: 1.84 ms for 462 x 30000).
 template <typename TC>
 __global__ void k_gauss_fill(uint64_t seed, int64_t s, int64_t L, double inv_sqrt_s, TC* __restrict__ G) {
-  int64_t total = s * L;
-  int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += stride)
-    G[k] = (TC)gauss_entry(seed, (uint64_t)k, inv_sqrt_s);
+  const int64_t total = s * L;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; 4 * g < total; g += stride) {
+    double v[4];
+    gauss_entries4(seed, (uint64_t)g, inv_sqrt_s, v);
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (4 * g + t < total) G[4 * g + t] = (TC)v[t];
+  }
 }
 
 template <typename T>
@@ -469,7 +476,7 @@ tk_status gauss_impl(const TIn* A, int64_t L, int64_t cols, int64_t ld, uint64_t
   double* part = splits > 1 ? ar.take<double>((size_t)splits * s * cols) : nullptr;
   if (!ar.ok()) return TK_ENOMEM;
   if (s == 0 || cols == 0) return TK_OK;
-  k_gauss_fill<TC><<<grid_for(s * L, 256), 256, 0, st>>>(seed, s, L, 1.0 / sqrt((double)s), G);
+  k_gauss_fill<TC><<<grid_for(cdiv(s * L, 4), 256), 256, 0, st>>>(seed, s, L, 1.0 / sqrt((double)s), G);
   TK_LAUNCH_CHECK();
   if (std::is_same<TC, double>::value) {
     if (splits > 1) {  // few output tiles: split the sum over the long axis, then add the planes
@@ -539,7 +546,7 @@ tk_status srht_rows(const void* A, tk_dtype dt, int64_t L, int64_t cols, int64_t
 
 tk_status gauss_fill(uint64_t seed, int64_t s, int64_t L, double* G, cudaStream_t st) {
   if (s * L == 0) return TK_OK;
-  k_gauss_fill<double><<<grid_for(s * L, 256), 256, 0, st>>>(seed, s, L, 1.0 / sqrt((double)s), G);
+  k_gauss_fill<double><<<grid_for(cdiv(s * L, 4), 256), 256, 0, st>>>(seed, s, L, 1.0 / sqrt((double)s), G);
   TK_LAUNCH_CHECK();
   return TK_OK;
 }

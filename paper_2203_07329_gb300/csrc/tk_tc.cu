@@ -144,25 +144,37 @@ __global__ void __launch_bounds__(128, 1)
 // G (s x ldk) BF16, entry (i, k) = N(0, 1/s) draw number i*m + k of Philox
 // stream 2 (the same counter convention as the float64 sketch, generated in
 // float32), zero for k >= m.
-__global__ void k_gauss_bf16(uint64_t seed, int64_t s, int64_t m, int64_t ldk, float inv_sqrt_s,
-                             __nv_bfloat16* __restrict__ G) {
-  const int64_t total = s * ldk;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / ldk, k = e - i * ldk;
-    float v = 0.f;
-    if (k < m) {
-      const uint64_t idx = (uint64_t)(i * m + k);
-      const uint4 w = philox(idx >> 2, STREAM_GAUSS, seed);
-      const int lane = (int)(idx & 3u);
-      const uint32_t a = (lane < 2) ? w.x : w.z, b = (lane < 2) ? w.y : w.w;
-      const float u1 = ((float)a + 1.0f) * 2.3283064365386962890625e-10f;
-      const float u2 = (float)b * 2.3283064365386962890625e-10f;
+// A thread makes the four entries of one Philox call (two Box-Muller pairs): grid.y over the rows, grid.x
+// over the calls that touch the row (the first and last are shared with its neighbours when m is not a
+// multiple of 4).  An entry per thread recomputed the call four times: 13.7 ms for 8192 x 262144.
+__global__ void __launch_bounds__(256) k_gauss_bf16(uint64_t seed, int64_t s, int64_t m, int64_t ldk, float inv_sqrt_s,
+                                                    __nv_bfloat16* __restrict__ G) {
+  for (int64_t i = blockIdx.y; i < s; i += gridDim.y) {
+    const int64_t i0 = i * m, g = (i0 >> 2) + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    __nv_bfloat16* row = G + i * ldk;
+    if (blockIdx.x == 0 && threadIdx.x < ldk - m) row[m + threadIdx.x] = __float2bfloat16_rn(0.f);
+    const int64_t k0 = 4 * g - i0;  // the row's column of the call's first entry (may start before it)
+    if (k0 >= m) continue;
+    const uint4 w = philox((uint64_t)g, STREAM_GAUSS, seed);
+    float v[4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float u1 = ((float)(h ? w.z : w.x) + 1.0f) * 2.3283064365386962890625e-10f;
+      const float u2 = (float)(h ? w.w : w.y) * 2.3283064365386962890625e-10f;
       const float r = sqrtf(-2.0f * logf(u1));
       float sn, cs;
       sincospif(2.0f * u2, &sn, &cs);
-      v = ((lane & 1) ? r * sn : r * cs) * inv_sqrt_s;
+      v[2 * h] = r * cs * inv_sqrt_s;
+      v[2 * h + 1] = r * sn * inv_sqrt_s;
     }
-    G[e] = __float2bfloat16_rn(v);
+    if ((k0 & 3) == 0 && k0 + 3 < m) {  // rows of ldk (a multiple of 8): 8-byte aligned
+      __nv_bfloat162 p[2] = {__floats2bfloat162_rn(v[0], v[1]), __floats2bfloat162_rn(v[2], v[3])};
+      *reinterpret_cast<uint2*>(row + k0) = *reinterpret_cast<uint2*>(p);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (k0 + t >= 0 && k0 + t < m) row[k0 + t] = __float2bfloat16_rn(v[t]);
+    }
   }
 }
 
@@ -440,8 +452,7 @@ tk_status tc_gauss_sketch(const void* A, tk_dtype dt, int64_t m, int64_t n, int6
     set_error_msg("tensor-core sketch: dimensions exceed the 32-bit TMA coordinates");
     return TK_EINVAL;
   }
-  const int64_t total = s * ldk;
-  k_gauss_bf16<<<(unsigned)std::min<int64_t>(cdiv(total, 256), 152 * 64), 256, 0, st>>>(
+  k_gauss_bf16<<<dim3((unsigned)cdiv(cdiv(m, 4) + 1, 256), (unsigned)std::min<int64_t>(s, 65535)), 256, 0, st>>>(
       seed, s, m, ldk, (float)(1.0 / sqrt((double)s)), G);
   TK_LAUNCH_CHECK();
   dim3 tg((unsigned)cdiv(n, 32), (unsigned)cdiv(ldk, 32));
