@@ -53,7 +53,12 @@ struct Plan {
 
 constexpr int64_t kMaxShort = 8192;
 constexpr int64_t kMaxLong = (int64_t(1) << 30);
-constexpr double kInv64Cost = 8e7;  // N c^2 up to which the explicit float64 inverse costs less than the substitutions
+// N c^2 up to which the float64 form makes the explicit inverse of its factors: it turns each preconditioner
+// apply into one launch (20 us at c = 1024, 16 lambda) where a substitution is a chain of c/32 launches
+// (1.1 ms for the two of a step, about 30 steps).  On the float64 pipe it costs N c^3/3 flops (6.9 ms there),
+// as much as the substitutions at c = 2048, 32 lambda; from digits a quarter of that, and the limit is its
+// memory (16 N c^2 bytes, 4 GiB).
+constexpr double kInv64Cost = 8e7, kInv64CostDigits = 2.7e8;
 constexpr int64_t kOz64MinElems = int64_t(1) << 16;  // smallest A (elements) that the float64 form splits into digits
 
 tk_status check_opts(const tk_opts* o) {
@@ -120,15 +125,13 @@ tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
   P.N_cap = (o->schedule == TK_SCHED_ONE_AT_A_TIME) ? 1 : std::max(N, 1);
   // the tensor-core products need 16-byte aligned float32 rows of A, A^T and
   // the lambda-major vectors; other shapes keep the SIMT float32 products
-  // float64 factors: an explicit inverse costs N c^3/3 flops once on the float64 pipe (1024, 16 lambda:
-  // 5 ms) and turns each preconditioner apply into one launch (13 us there) where a substitution is a
-  // chain of c/32 launches (1.1 ms for the two of a step, about 30 steps)
-  P.inv64 = !P.mixed && !P.lowrank && (double)std::max(N, 1) * P.c * P.c <= kInv64Cost;
   P.lsqr_tc = P.mixed && o->lsqr_tc == 1 && P.N_cap <= 64 && !P.under && P.m % 4 == 0 && P.n % 4 == 0 &&
               (P.dt == TK_F64 || P.lda % 4 == 0);
   P.lsqr_oz = P.mixed && (o->lsqr_tc == 2 || o->lsqr_tc == 3) && o->emulate_fp64 && !P.under;
   P.lsqr_fused = P.lsqr_oz && o->lsqr_tc == 3;
   P.oz64 = !P.mixed && o->emulate_fp64 && oz64_wanted(P.m, P.n);
+  P.inv64 = !P.mixed && !P.lowrank &&
+            (double)std::max(N, 1) * P.c * P.c <= (P.oz64 ? kInv64CostDigits : kInv64Cost);
   return TK_OK;
 }
 
@@ -190,6 +193,10 @@ bool emulated_chol(const Plan& P) {
   return ((P.mixed && P.o.emulate_fp64) || P.oz64) && !P.lowrank && !P.qr;
 }
 bool emulated_gram(const Plan& P) { return emulated_chol(P); }
+// ... and the off-diagonal blocks of the factors' inverse
+bool digit_inverse(const Plan& P) {
+  return !P.lowrank && (P.mixed ? P.o.emulate_fp64 != 0 : P.oz64 && P.inv64);
+}
 OzMat oz_mat(const Plan& P, const Bufs& B) {
   OzMat A;
   A.planes = B.Aoz;
@@ -301,6 +308,8 @@ void carve(const Plan& P, Arena& a, Arena& t, Bufs& B) {
   // the sketch's scratch is free again when the Gram matrix (or the BP2 factorization) is formed
   size_t sc = std::max(sketch_scratch(P), P.lowrank ? size_t(0) : gram_scratch_bytes(P.s, P.c));
   if (P.qr) sc = std::max(sc, bp2_workspace(P.s, P.c, N));
+  // and the inverse of the factors, after them
+  if (digit_inverse(P)) sc = std::max(sc, P.mixed ? tri_inverse_workspace<float>(P.np, N) : tri_inverse_workspace<double>(P.np, N));
   if (emulated_gram(P)) sc = std::max({sc, oz_gram_workspace(P.s, P.c), oz_chol_workspace(P.np, N)});
   B.scratch_bytes = sc;
   B.scratch = t.take<char>(sc);
@@ -551,7 +560,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
   // A is split once, for every product of the solve (x, r and the LSQR vectors on every pass); the
   // first pass over a float64 A also writes the float32 copy of the mixed form
   const bool digits = (P.mixed && P.o.emulate_fp64 && !P.prep_only) || P.oz64;
-  if (digits) TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));
+  if (B.oz_err) TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));
   if (digits && !reuse) {
     float* copy = P.mixed && P.dt == TK_F64 ? B.A32 : nullptr;
     const int tok = prof_begin(TK_PHASE_SLICE, st);
@@ -600,7 +609,6 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
   std::vector<int> ok_ids;
   if (!P.lowrank) {
     int tok = -1;
-    if (emulated_gram(P) && !digits) TK_CUDA(cudaMemsetAsync(B.oz_err, 0, sizeof(int), st));  // grouped build
     if (!reuse && !P.qr) {
       tok = prof_begin(TK_PHASE_GRAM, st);
       if (emulated_gram(P)) {  // the Cholesky reads only j >= i
@@ -643,12 +651,14 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
     if (P.mixed) {
       // the float32 LSQR applies R^-1 and R^-T as explicit float32 matrices
       tok = prof_begin(TK_PHASE_TRINV, st);
-      TK_TRY(tri_inverse<float>(B.R, P.c, P.np, P.np * P.np, N, B.Minv, B.Mtinv, st));
+      TK_TRY(tri_inverse<float>(B.R, P.c, P.np, P.np * P.np, N, B.Minv, B.Mtinv, digit_inverse(P) ? B.scratch : nullptr,
+                                B.scratch_bytes, B.oz_err, st));
       prof_end(tok, st, (double)N * P.c * P.c * P.c / 3.0, 4.0 * N * P.np * P.np * 3.0);
     }
     if (P.inv64) {
       tok = prof_begin(TK_PHASE_TRINV, st);
-      TK_TRY(tri_inverse<double>(B.R, P.c, P.np, P.np * P.np, N, B.Minv64, B.Mtinv64, st));
+      TK_TRY(tri_inverse<double>(B.R, P.c, P.np, P.np * P.np, N, B.Minv64, B.Mtinv64,
+                                 digit_inverse(P) ? B.scratch : nullptr, B.scratch_bytes, B.oz_err, st));
       prof_end(tok, st, (double)N * P.c * P.c * P.c / 3.0, 8.0 * N * P.np * P.np * 3.0);
     }
   } else if (!gp) {
@@ -708,7 +718,13 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
       TK_TRY(jacobi_svd_begin(j, st));
     }
     for (int i = 0; i < N; ++i) gp->inf[i] = inf[i];
+    int oz_err = 0;
+    if (B.oz_err) TK_CUDA(cudaMemcpyAsync(&oz_err, B.oz_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     TK_CUDA(cudaStreamSynchronize(st));  // the build scratch is reused by the lane's next problem
+    if (oz_err) {
+      set_error_msg("grouped build: a pipeline wait of an emulated product timed out");
+      return TK_ETIMEOUT;
+    }
     return TK_OK;
   }
   const int nok = (int)ok_ids.size();
@@ -854,7 +870,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
       TK_LAUNCH_CHECK();
       TK_CUDA(cudaMemcpyAsync(hn.data(), B.nrm, sizeof(double) * 3 * cnt, cudaMemcpyDeviceToHost, st));
       int oz_err = 0;
-      if (P.o.emulate_fp64 && (round > 0 || P.o.x0 || P.lsqr_oz))
+      if (P.o.emulate_fp64)
         TK_CUDA(cudaMemcpyAsync(&oz_err, B.oz_err, sizeof(int), cudaMemcpyDeviceToHost, st));
       TK_CUDA(cudaStreamSynchronize(st));
       if (oz_err) {

@@ -437,6 +437,10 @@ __global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ R, int
 // M_ic = M_ii S_ic with S_ic = -sum_{i<k<=c} R_ik M_kc, accumulated
 // right-looking in the not yet finished blocks of M (zero on entry).  Mt
 // receives M^T (its blocks above the diagonal are left unwritten).
+// On the SIMT pipes this way only the diagonal blocks of 256 are inverted (all of them at once); the
+// blocks beyond, most of the n^3 / 3, are products M12 = -M11 R12 M22 of doubling size from exact digits on
+// the tensor cores (float64, n = 1024, 16 lambda: 6.9 ms on the float64 pipe, now 1.7; float32, n = 4096, 64
+// lambda: 67 ms at 24 TFLOP/s, now 42; n = 2048, 32 lambda about 5 ms either way).
 
 // M_kk = R_kk^-1: back substitution of the identity's columns, 16 of them per CTA (blockIdx.z); the half-warps
 // of 4 warps hold the rows of one residue mod 8 each, one barrier a row (as k_chol_trsm16: all quarters of
@@ -487,11 +491,18 @@ __global__ void __launch_bounds__(128) k_tinv_diag(const double* __restrict__ R,
 template <typename T>
 __global__ void __launch_bounds__(256) k_tinv_update(const double* __restrict__ R, int64_t ldr, int64_t rstride,
                                                      T* __restrict__ M, int64_t ldm, int64_t mstride, int k,
-                                                     int nt) {
+                                                     int nt, int bt) {
+  // grid.z: blocks of bt tiles along the diagonal; k, nt (the tiles of this block) relative to the block
+  const int t0 = blockIdx.z * bt;
+  nt = nt - t0 < bt ? nt - t0 : bt;
+  if (k >= nt) return;
+  R += (int64_t)t0 * CB * (ldr + 1);
+  M += (int64_t)t0 * CB * (ldm + 1);
   constexpr int KC = 32;
   __shared__ T P[KC][CB + 4];  // P[kk][i] = R[rb*64 + i, k*64 + kc + kk]
   __shared__ T Q[KC][CB];      // Q[kk][j] = M[k*64 + kc + kk, cb*64 + j]
   const int l = blockIdx.y;
+  if ((int)blockIdx.x >= k * (nt - k)) return;
   const int rb = blockIdx.x / (nt - k), cb = k + blockIdx.x % (nt - k);
   const double* Pg = R + (int64_t)l * rstride + (int64_t)rb * CB * ldr + (int64_t)k * CB;
   T* Ml = M + (int64_t)l * mstride;
@@ -531,9 +542,13 @@ __global__ void __launch_bounds__(256) k_tinv_update(const double* __restrict__ 
 // precedes the barrier, every write follows it), and Mt_{cb,i} = M_{i,cb}^T.
 template <typename T>
 __global__ void __launch_bounds__(256) k_tinv_final(T* __restrict__ M, T* __restrict__ Mt, int64_t ldm,
-                                                    int64_t mstride, int i) {
+                                                    int64_t mstride, int i, int nt, int bt) {
   __shared__ T D[CB][CB + 1];
   const int l = blockIdx.y, cb = i + 1 + blockIdx.x;
+  const int t0 = blockIdx.z * bt;
+  if (t0 + cb >= nt) return;
+  M += (int64_t)t0 * CB * (ldm + 1);
+  Mt += (int64_t)t0 * CB * (ldm + 1);
   T* Ml = M + (int64_t)l * mstride;
   const T* Dg = Ml + (int64_t)i * CB * ldm + (int64_t)i * CB;
   T* Sg = Ml + (int64_t)i * CB * ldm + (int64_t)cb * CB;
@@ -969,25 +984,42 @@ template tk_status gemm_splitk<float, double>(bool, bool, int64_t, int64_t, int6
 template tk_status gemm_splitk<double, float>(bool, bool, int64_t, int64_t, int64_t, const double*, int64_t,
                                               const float*, int64_t, double*, int, cudaStream_t);
 
+constexpr int kTriBlock = 4;  // tiles of 64 of the blocks inverted on the SIMT pipes when the rest is products
+
 template <typename T>
-tk_status tri_inverse(const double* R, int64_t n, int64_t ldr, int64_t rstride, int N, T* M, T* Mt, cudaStream_t st) {
+size_t tri_inverse_workspace(int64_t n, int N) {
+  return oz_tri_workspace<T>(cdiv(n, CB) * CB, N, kTriBlock * CB);
+}
+template size_t tri_inverse_workspace<float>(int64_t, int);
+template size_t tri_inverse_workspace<double>(int64_t, int);
+
+template <typename T>
+tk_status tri_inverse(const double* R, int64_t n, int64_t ldr, int64_t rstride, int N, T* M, T* Mt, void* work,
+                      size_t bytes, int* err, cudaStream_t st) {
   if (N == 0 || n == 0) return TK_OK;
   const int64_t np = cdiv(n, CB) * CB;
   const int nt = (int)(np / CB);
   TK_CUDA(cudaMemsetAsync(M, 0, sizeof(T) * (size_t)N * np * np, st));
   k_tinv_diag<T><<<dim3((unsigned)nt, (unsigned)N, CB / 16), 128, 0, st>>>(R, ldr, rstride, M, Mt, np, np * np);
   TK_LAUNCH_CHECK();
-  for (int k = nt - 1; k >= 1; --k) {
-    k_tinv_update<T><<<dim3((unsigned)(k * (nt - k)), (unsigned)N), 256, 0, st>>>(R, ldr, rstride, M, np, np * np,
-                                                                                 k, nt);
+  const int bt = work ? std::min(kTriBlock, nt) : nt;
+  const unsigned nb = (unsigned)cdiv(nt, bt);
+  for (int k = bt - 1; k >= 1; --k) {
+    k_tinv_update<T><<<dim3((unsigned)(k * (bt - k)), (unsigned)N, nb), 256, 0, st>>>(R, ldr, rstride, M, np, np * np, k,
+                                                                                     nt, bt);
     TK_LAUNCH_CHECK();
-    k_tinv_final<T><<<dim3((unsigned)(nt - k), (unsigned)N), 256, 0, st>>>(M, Mt, np, np * np, k - 1);
+    k_tinv_final<T><<<dim3((unsigned)(bt - k), (unsigned)N, nb), 256, 0, st>>>(M, Mt, np, np * np, k - 1, nt, bt);
     TK_LAUNCH_CHECK();
   }
+  if (work)
+    for (int64_t h = (int64_t)kTriBlock * CB; h < np; h *= 2)
+      TK_TRY(oz_tri_level<T>(R, ldr, rstride, M, Mt, np, np * np, N, np, (int)h, work, bytes, err, st));
   return TK_OK;
 }
-template tk_status tri_inverse<float>(const double*, int64_t, int64_t, int64_t, int, float*, float*, cudaStream_t);
-template tk_status tri_inverse<double>(const double*, int64_t, int64_t, int64_t, int, double*, double*, cudaStream_t);
+template tk_status tri_inverse<float>(const double*, int64_t, int64_t, int64_t, int, float*, float*, void*, size_t, int*,
+                                      cudaStream_t);
+template tk_status tri_inverse<double>(const double*, int64_t, int64_t, int64_t, int, double*, double*, void*, size_t,
+                                       int*, cudaStream_t);
 
 template <typename T>
 tk_status trmv_batched(bool transposed, int64_t n, const T* M, const T* Mt, int64_t ldm, int64_t mstride,

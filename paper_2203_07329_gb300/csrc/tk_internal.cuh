@@ -332,6 +332,13 @@ tk_status lm_small_aw(const float* A, int64_t lda, int64_t m, int64_t n, const f
 int lm_small_atu_splits(int64_t m, int64_t n);
 tk_status lm_small_atu(const float* A, int64_t lda, int64_t m, int64_t n, const float* U, int64_t ldu, int count,
                        double* partial, int splits, cudaStream_t st);
+// Levels of the inverse of triangular factors (tri_inverse): M12 = -M11 R12 M22 for all pairs of h x h
+// diagonal blocks (h = h0, 2 h0, .. < n); work: oz_tri_workspace<T>(n, N, h0) bytes.
+template <typename T>
+tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* Mt, int64_t ldm, int64_t mstride, int N,
+                       int64_t n, int h, void* work, size_t bytes, int* err, cudaStream_t st);
+template <typename T>
+size_t oz_tri_workspace(int64_t n, int N, int h0);
 // Y (s x c) = G A (m >= n: G s x m, c = n) or G A^T (under: G s x n, c = m) for an embedding G (float64,
 // s <= 65535) from the digit planes of A, float64-accurate; work: oz_sketch_workspace(L, c, s) bytes, L the
 // length of G's rows.
@@ -384,8 +391,13 @@ tk_status chol_shifted(const double* C, int64_t n, const double* lambdas_dev, in
 // M = R^-1 (upper) and Mt = M^T (lower), arithmetic in T, for N factors R
 // (float64, padded order np = ceil(n/64)*64, row stride ldr, matrix stride
 // rstride); M and Mt: N x np x np, row stride np.
+// With work (tri_inverse_workspace<T>(n, N) bytes) and err the blocks beyond order 256 come from exact
+// digits on the tensor cores (err as the emulated products); work = null: all on the SIMT pipes.
 template <typename T>
-tk_status tri_inverse(const double* R, int64_t n, int64_t ldr, int64_t rstride, int N, T* M, T* Mt, cudaStream_t st);
+size_t tri_inverse_workspace(int64_t n, int N);
+template <typename T>
+tk_status tri_inverse(const double* R, int64_t n, int64_t ldr, int64_t rstride, int N, T* M, T* Mt, void* work,
+                      size_t bytes, int* err, cudaStream_t st);
 // out_k = M_l in_k (or Mt_l in_k when transposed) for slots k < count,
 // l = idx[k] (idx null: l = k); in/out vectors of length n at stride ldx
 // (out must not overlap in).

@@ -447,12 +447,23 @@ struct OtSmem {
   uint32_t tmem_base;
 };
 
+// MODE 3: many h x h products (h a multiple of 128), the blocks of a level of the triangular inverse:
+// batch z = (matrix, pair) holds rows z h .. z h + h - 1 of both operands' planes (K = h);
+// out[z / pairs * mstride + z % pairs * pstride + l ldo + r] = sign D, float64 (S = 8) or float32 (S = 4),
+// for l < min(h, n - (2 pair + 1) h).  Triangular operands skip the K they hold zeros in: tri 1: Q's row l
+// ends at k = l; tri 2: P's row r starts at k = r.
+struct OtTri {
+  int pairs, tri, h, n;
+  int64_t mstride, pstride;
+  double sign;
+};
+
 template <int S, int MODE, int NT, bool TR>
 __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
     k_oz_tc(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmQ,
             const int* __restrict__ EP, const int* __restrict__ EQ, int64_t rows, int M, int64_t K, int64_t kps,
             const double* __restrict__ b, void* __restrict__ out, int64_t ldo, const double* __restrict__ coef,
-            int upper_only, int* __restrict__ err) {
+            int upper_only, int* __restrict__ err, const OtTri tri) {
   using Acc = typename std::conditional<S == OZ_S, double, float>::type;
   constexpr uint32_t TMEM_COLS = 2 * S * NT;
   constexpr uint32_t QS_BYTES = OtCfg<S, NT>::QS_BYTES;
@@ -464,8 +475,19 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
   const int l0 = (int)blockIdx.y * NT;
   // a symmetric product (P = Q) needs out[l][r] for l <= r only
   if (upper_only && l0 > r0 + OT_M - 1) return;
-  const int64_t kbeg = (int64_t)blockIdx.z * kps;
-  const int64_t kend = K < kbeg + kps ? K : kbeg + kps;
+  int64_t kbeg = (int64_t)blockIdx.z * kps;
+  int64_t kend = K < kbeg + kps ? K : kbeg + kps;
+  int prow = 0;  // first row of the batch in the operands' planes and exponents
+  if constexpr (MODE == 3) {
+    const int left = tri.n - (2 * (int)(blockIdx.z % tri.pairs) + 1) * tri.h;
+    M = left < tri.h ? left : tri.h;
+    if (l0 >= M) return;
+    prow = (int)blockIdx.z * tri.h;
+    EP += prow;
+    EQ += prow;
+    kbeg = tri.tri == 2 ? r0 : 0;
+    kend = tri.tri == 1 && l0 + NT < K ? l0 + NT : K;
+  }
   const int nkb = kend > kbeg ? (int)((kend - kbeg + OT_KB - 1) / OT_KB) : 0;
   const int nch = (nkb + OT_KB_PER_CHUNK - 1) / OT_KB_PER_CHUNK;
 
@@ -502,7 +524,7 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
       const int qs = kb & 1;
       if (!mbar_wait(&Sm.q_empty[qs], ((uint32_t)(kb >> 1) & 1u) ^ 1u, err)) break;
       mbar_expect_tx(&Sm.q_full[qs], Q_BYTES);
-      for (int p = 0; p < S; ++p) tma_load_3d(&tmQ, &Sm.q_full[qs], Sm.q[qs] + p * QS_BYTES, kc, l0, p);
+      for (int p = 0; p < S; ++p) tma_load_3d(&tmQ, &Sm.q_full[qs], Sm.q[qs] + p * QS_BYTES, kc, prow + l0, p);
       ++gq;
       for (int p = 0; p < S; ++p, ++g) {
         const int ps = g % OtCfg<S, NT>::PST;
@@ -515,7 +537,7 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
           tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], (int)r0, kc, p);
           tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps] + OT_P_BYTES / 2, (int)r0 + 64, kc, p);
         } else {
-          tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], kc, (int)r0, p);
+          tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], kc, prow + (int)r0, p);
         }
       }
     }
@@ -646,6 +668,11 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
             static_cast<double*>(out)[(int64_t)l * ldo + r] = br - v;
           } else if (MODE == 1) {
             static_cast<double*>(out)[((int64_t)blockIdx.z * M + l) * ldo + r] = v;
+          } else if (MODE == 3) {
+            using TU = typename std::conditional<S == OZ_S, double, float>::type;
+            static_cast<TU*>(out)[(int64_t)(blockIdx.z / tri.pairs) * tri.mstride +
+                                  (int64_t)(blockIdx.z % tri.pairs) * tri.pstride + (int64_t)l * ldo + r] =
+                (TU)(tri.sign * v);
           } else {
             using TU = typename std::conditional<S == OZ_S, double, float>::type;
             TU* u = static_cast<TU*>(out) + (int64_t)l * ldo + r;
@@ -711,7 +738,7 @@ tk_status launch_oz_tc_nt(const OtBig& P, const void* Qs, const int* EQ, int M, 
   TK_CUDA(cudaFuncSetAttribute(k_oz_tc<S, MODE, NT, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const dim3 grid((unsigned)cdiv(P.rows, OT_M), (unsigned)cdiv(M, NT), (unsigned)sp);
   k_oz_tc<S, MODE, NT, TR>
-      <<<grid, 256, smem, st>>>(mP, mQ, P.E, EQ, P.rows, M, kp, kps, b, out, ldo, coef, upper_only, err);
+      <<<grid, 256, smem, st>>>(mP, mQ, P.E, EQ, P.rows, M, kp, kps, b, out, ldo, coef, upper_only, err, OtTri{});
   TK_LAUNCH_CHECK();
   return TK_OK;
 }
@@ -743,6 +770,50 @@ tk_status launch_oz_tc(const OtBig& P, const void* Qs, const int* EQ, int M, int
     TK_CUDA(cudaMemsetAsync(o + (int64_t)sp * M * ldo, 0, sizeof(double) * (size_t)(splits - sp) * M * ldo, st));
   }
   return TK_OK;
+}
+
+// ---- a level of the triangular inverse -----------------------------------------
+// Digit planes (row stride h) and row exponents of the blocks of a level: batch z = (matrix l, pair i),
+// row r: src + l mstride + i pstride + r ld, h values; rows or columns past the matrix (r or k >= n - edge,
+// edge = (2 i + 1) h, where row_edge / col_edge is set) and, with lower, the columns k > r are zero.
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_oz_block_rows(const T* __restrict__ src, int64_t mstride, int64_t pstride, int64_t ld, int pairs, int h, int n,
+                    int row_edge, int col_edge, int lower, int64_t rows, int planes, int* __restrict__ E,
+                    __nv_bfloat16* __restrict__ out) {
+  __shared__ int sh[8];
+  const int z = blockIdx.y, r = blockIdx.x;
+  const int left = n - (2 * (z % pairs) + 1) * h;
+  const T* x = src + (int64_t)(z / pairs) * mstride + (int64_t)(z % pairs) * pstride + (int64_t)r * ld;
+  int K = h;
+  if (col_edge && left < K) K = left;
+  if (lower && r + 1 < K) K = r + 1;
+  if (row_edge && r >= left) K = 0;
+  if (K < 0) K = 0;
+  bool bad = false;
+  int e = oz_vec_exp<T>(x, nullptr, 0, K, &bad);
+  e = oz_block_exp(e, bad, sh);
+  const int64_t row = (int64_t)z * h + r;
+  if (threadIdx.x == 0) E[row] = e;
+  unsigned* o = reinterpret_cast<unsigned*>(out + row * h);
+  for (int k = 2 * threadIdx.x; k < h; k += 2 * blockDim.x)
+    oz_vec_split<T>(x, nullptr, k, K, e, rows * h, planes, o + k / 2);
+}
+// M[a + r][a + h + l] = Mt[a + h + l][a + r] for the level's blocks (a = 2 i h): 32 x 32 tiles
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_oz_block_transpose(const T* __restrict__ Mt, T* __restrict__ M, int64_t ldm, int64_t mstride, int pairs, int h,
+                         int n) {
+  __shared__ T tile[32][33];
+  const int z = blockIdx.z, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t a = 2 * (int64_t)(z % pairs) * h;
+  const int64_t l0 = a + h + (int64_t)blockIdx.y * 32, r0 = a + (int64_t)blockIdx.x * 32;
+  if (l0 >= n) return;
+  const T* src = Mt + (int64_t)(z / pairs) * mstride;
+  T* dst = M + (int64_t)(z / pairs) * mstride;
+  for (int q = ty; q < 32; q += 8) tile[q][tx] = src[(l0 + q) * ldm + r0 + tx];
+  __syncthreads();
+  for (int q = ty; q < 32; q += 8) dst[(r0 + q) * ldm + l0 + tx] = tile[tx][q];
 }
 
 // ---- Cholesky trailing update -------------------------------------------------
@@ -1786,6 +1857,83 @@ tk_status oz_lsqr_fused(const OzMat& A, const float* W, int64_t ldw, int count, 
   *planes = ncl;
   return TK_OK;
 }
+
+// The level h of M = R^-1 (n a multiple of 64, h of 128): for every pair of diagonal blocks of M that are
+// finished, M12 = -M11 (R12 M22), both products from digits (T = double: 8, float64-accurate; T = float: 4,
+// the 28-bit rounded operands); Mt = M^T receives its block first.
+template <typename T>
+tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* Mt, int64_t ldm, int64_t mstride, int N,
+                       int64_t n, int h, void* work, size_t bytes, int* err, cudaStream_t st) {
+  constexpr int S = oz_digits<T>();
+  constexpr int NT = 32;
+  const int pairs = (int)cdiv(n - h, 2 * (int64_t)h);
+  if (pairs <= 0) return TK_OK;
+  const int64_t batch = (int64_t)N * pairs, rows = batch * h;
+  if (batch > 65535 || rows > INT32_MAX) {
+    set_error_msg("triangular inverse: too many blocks for one launch");
+    return TK_EINVAL;
+  }
+  Arena a;
+  a.base = static_cast<char*>(work);
+  a.cap = bytes;
+  __nv_bfloat16* Ps = a.take<__nv_bfloat16>((size_t)S * rows * h);
+  __nv_bfloat16* Qs = a.take<__nv_bfloat16>((size_t)S * rows * h);
+  int* EP = a.take<int>((size_t)rows);
+  int* EQ = a.take<int>((size_t)rows);
+  T* Tt = a.take<T>((size_t)rows * h);  // (R12 M22)^T
+  if (!a.ok()) return TK_ENOMEM;
+  CUtensorMap mP, mQ;
+  TK_TRY(make_slice_map(&mP, Ps, rows, h, OT_M, S));
+  TK_TRY(make_slice_map(&mQ, Qs, rows, h, NT, S));
+  const size_t smem = sizeof(OtSmem<S, NT>) + 1024;
+  TK_CUDA(cudaFuncSetAttribute(k_oz_tc<S, 3, NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const dim3 gs((unsigned)h, (unsigned)batch), g((unsigned)(h / OT_M), (unsigned)(h / NT), (unsigned)batch);
+  const int64_t pr = 2 * (int64_t)h;  // a pair's step along the diagonal
+  OtTri t{pairs, 1, h, (int)n, (int64_t)pairs * h * h, (int64_t)h * h, 1.0};
+  k_oz_block_rows<double><<<gs, 256, 0, st>>>(R + h, rstride, pr * (ldr + 1), ldr, pairs, h, (int)n, 0, 1, 0, rows, S,
+                                              EP, Ps);
+  TK_LAUNCH_CHECK();
+  k_oz_block_rows<T><<<gs, 256, 0, st>>>(Mt + h * (ldm + 1), mstride, pr * (ldm + 1), ldm, pairs, h, (int)n, 1, 1, 1,
+                                         rows, S, EQ, Qs);
+  TK_LAUNCH_CHECK();
+  k_oz_tc<S, 3, NT, false><<<g, 256, smem, st>>>(mP, mQ, EP, EQ, h, h, h, h, nullptr, Tt, h, nullptr, 0, err, t);
+  TK_LAUNCH_CHECK();
+  k_oz_block_rows<T><<<gs, 256, 0, st>>>(M, mstride, pr * (ldm + 1), ldm, pairs, h, (int)n, 0, 0, 0, rows, S, EP, Ps);
+  TK_LAUNCH_CHECK();
+  k_oz_block_rows<T><<<gs, 256, 0, st>>>(Tt, (int64_t)pairs * h * h, (int64_t)h * h, h, pairs, h, (int)n, 1, 0, 0, rows,
+                                         S, EQ, Qs);
+  TK_LAUNCH_CHECK();
+  t = OtTri{pairs, 2, h, (int)n, mstride, pr * (ldm + 1), -1.0};
+  k_oz_tc<S, 3, NT, false><<<g, 256, smem, st>>>(mP, mQ, EP, EQ, h, h, h, h, nullptr, Mt + h * ldm, ldm, nullptr, 0, err,
+                                                 t);
+  TK_LAUNCH_CHECK();
+  k_oz_block_transpose<T><<<dim3((unsigned)(h / 32), (unsigned)(h / 32), (unsigned)batch), 256, 0, st>>>(
+      Mt, M, ldm, mstride, pairs, h, (int)n);
+  TK_LAUNCH_CHECK();
+  return TK_OK;
+}
+template tk_status oz_tri_level<float>(const double*, int64_t, int64_t, float*, float*, int64_t, int64_t, int, int64_t,
+                                       int, void*, size_t, int*, cudaStream_t);
+template tk_status oz_tri_level<double>(const double*, int64_t, int64_t, double*, double*, int64_t, int64_t, int,
+                                        int64_t, int, void*, size_t, int*, cudaStream_t);
+
+template <typename T>
+size_t oz_tri_workspace(int64_t n, int N, int h0) {
+  size_t most = 0;
+  for (int64_t h = h0; h < n; h *= 2) {
+    const size_t rows = (size_t)N * cdiv(n - h, 2 * h) * h;
+    Arena a;
+    a.take<__nv_bfloat16>(oz_digits<T>() * rows * h);
+    a.take<__nv_bfloat16>(oz_digits<T>() * rows * h);
+    a.take<int>(rows);
+    a.take<int>(rows);
+    a.take<T>(rows * h);
+    most = std::max(most, a.used + 256);
+  }
+  return most;
+}
+template size_t oz_tri_workspace<float>(int64_t, int, int);
+template size_t oz_tri_workspace<double>(int64_t, int, int);
 
 static int oz_sketch_splits(int64_t L, int64_t c, int64_t s) {
   const int64_t tiles = cdiv(c, OT_M) * cdiv(s, OT_N);

@@ -17,10 +17,11 @@ def _solve(A, b, lams, **kw):
 
 # A at and around the smallest size that is split into digits (2^19 elements), ragged against the 64-,
 # 128- and 256-value tiles, one and several tiles of 32 lambdas, float64 views with odd row strides,
-# and m < n with vectors of 1, 2, 4 and 8 CTAs per v-step.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
+# the explicit inverse over one to three doubling levels with ragged last blocks (257 .. 1100 columns), and
+# m < n with vectors of 1, 2, 4 and 8 CTAs per v-step.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
 @pytest.mark.parametrize("m,n,N,pad", [(8192, 64, 2, 0), (8192, 65, 1, 0), (8193, 65, 3, 1), (2051, 257, 33, 0), (1500, 700, 5, 3),
                                        (16500, 40, 4, 0), (129, 4099, 4, 0), (500, 1100, 34, 5), (63, 8400, 2, 0),
-                                       (101, 17001, 3, 0)])
+                                       (101, 17001, 3, 0), (6000, 1100, 3, 0), (517, 4000, 2, 0)])
 def test_digit_solve_matches_float64_pipe(m, n, N, pad):
     k = min(m, n)
     p = datagen.make_ridge_problem(m, n, datagen.spectrum("log", k, hi=1.0, lo=1e-3),
@@ -59,6 +60,23 @@ def test_digit_products_follow_row_and_column_scales(rows, cols):
     Gref = R.astype(np.longdouble) @ Ah.astype(np.longdouble)
     err = np.max(np.abs((G - Gref).astype(np.float64)) / (np.abs(R) @ np.abs(Ah)))
     assert err < 8 * 2.0 ** -53 * math.sqrt(m), err
+
+
+# the same levels in float32 (the mixed form's preconditioner): refined to the float64 solution, with as
+# many iterations as the float32 pipe's inverse gives
+@pytest.mark.parametrize("n,N", [(256, 3), (300, 1), (513, 5), (1100, 3), (1290, 2)])
+def test_mixed_digit_inverse(n, N):
+    m = 4 * n + 17
+    p = datagen.make_ridge_problem(m, n, datagen.spectrum("log", n, hi=1.0, lo=1e-4),
+                                   datagen.log_lambdas(N, 1e-6, 1e-1), seed=n)
+    A, b, lams = p.A.cuda(), p.b.cuda(), p.lambdas.numpy()
+    kw = dict(sketch=tk.TK_SKETCH_GAUSS, s=3 * n, precision=tk.TK_PREC_MIXED)
+    r1 = _solve(A, b, lams, **kw)
+    r0 = _solve(A, b, lams, lsqr_tc=0, emulate_fp64=0, **kw)
+    for i in range(N):
+        e = float((r1.X[i] - r0.X[i]).norm() / r0.X[i].norm())
+        assert e < 2e-10, (lams[i], e)  # each within 1e-10 of the minimiser
+        assert r1.info[i]["iters"] <= 1.2 * r0.info[i]["iters"] + 3
 
 
 def test_non_finite_a_is_enumeric_from_digits():
