@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ R, int
 // receives M^T (its blocks above the diagonal are left unwritten).
 // On the SIMT pipes this way only the diagonal blocks of 256 are inverted (all of them at once); the
 // blocks beyond, most of the n^3 / 3, are products M12 = -M11 R12 M22 of doubling size from exact digits on
-// the tensor cores (float64, n = 1024, 16 lambda: 6.9 ms on the float64 pipe, now 1.7; float32, n = 4096, 64
-// lambda: 67 ms at 24 TFLOP/s, now 42; n = 2048, 32 lambda about 5 ms either way).
+// the tensor cores (float64, n = 1024, 16 lambda: 6.9 ms on the float64 pipe, now 1.5; float32, n = 4096, 64
+// lambda: 67 ms at 24 TFLOP/s, now 32; n = 2048, 32 lambda 5, now 3.8).
 
 // M_kk = R_kk^-1: back substitution of the identity's columns, 16 of them per CTA (blockIdx.z); the half-warps
 // of 4 warps hold the rows of one residue mod 8 each, one barrier a row (as k_chol_trsm16: all quarters of

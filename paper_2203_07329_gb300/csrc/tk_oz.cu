@@ -394,7 +394,11 @@ __global__ void __launch_bounds__(256) k_oz_slice_t(const T* __restrict__ X, int
 // S = 8: float64 accuracy (levels added exactly into int64 accumulators, one
 // rounding at the end); S = 4: the 28-bit rounded operands, float32 accuracy
 // (levels flushed into float32).
-// CTA: 128 rows of P x 32 rows of Q x one K split (blockIdx.z).
+// Tile: 128 rows of P x 32 (64) rows of Q x one K split.  A CTA per slot of the GPU runs through its tiles
+// with the rings and tensor-memory buffers going on from one to the next, so the last step of a tile (float64
+// arithmetic, reads of U) overlaps the products of the next (a CTA per tile: 4 digits, 64 lambda, 262144 x 4096
+// 1.85 ms, now 1.47 = 5.8 TB/s of planes; 32 lambda, 262144 x 2048 0.75, now 0.66; 8 digits, 65536 x 1024, 16
+// lambda 235 us, now 209, of which a quarter of the last of 3.4 rounds of tiles is idle).
 //   warp 0 (one lane): TMA producer -- per 64 values of K the S planes of Q
 //     (4 KiB each) into a 2-slot ring, then the S planes of P one by one
 //     (16 KiB each) into an 8-slot ring;
@@ -458,12 +462,19 @@ struct OtTri {
   double sign;
 };
 
+// 2^e as a double (e within the normal range).
+__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
+
+struct OtTiles {
+  uint32_t gx, gy, gz;
+};
+
 template <int S, int MODE, int NT, bool TR>
 __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
     k_oz_tc(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmQ,
             const int* __restrict__ EP, const int* __restrict__ EQ, int64_t rows, int M, int64_t K, int64_t kps,
             const double* __restrict__ b, void* __restrict__ out, int64_t ldo, const double* __restrict__ coef,
-            int upper_only, int* __restrict__ err, const OtTri tri) {
+            int upper_only, int* __restrict__ err, const OtTiles tiles, const OtTri tri) {
   using Acc = typename std::conditional<S == OZ_S, double, float>::type;
   constexpr uint32_t TMEM_COLS = 2 * S * NT;
   constexpr uint32_t QS_BYTES = OtCfg<S, NT>::QS_BYTES;
@@ -471,25 +482,42 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
   extern __shared__ __align__(1024) uint8_t ot_raw[];
   OtSmem<S, NT>& Sm = *reinterpret_cast<OtSmem<S, NT>*>((reinterpret_cast<uintptr_t>(ot_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t r0 = (int64_t)blockIdx.x * OT_M;
-  const int l0 = (int)blockIdx.y * NT;
-  // a symmetric product (P = Q) needs out[l][r] for l <= r only
-  if (upper_only && l0 > r0 + OT_M - 1) return;
-  int64_t kbeg = (int64_t)blockIdx.z * kps;
-  int64_t kend = K < kbeg + kps ? K : kbeg + kps;
-  int prow = 0;  // first row of the batch in the operands' planes and exponents
-  if constexpr (MODE == 3) {
-    const int left = tri.n - (2 * (int)(blockIdx.z % tri.pairs) + 1) * tri.h;
-    M = left < tri.h ? left : tri.h;
-    if (l0 >= M) return;
-    prow = (int)blockIdx.z * tri.h;
-    EP += prow;
-    EQ += prow;
-    kbeg = tri.tri == 2 ? r0 : 0;
-    kend = tri.tri == 1 && l0 + NT < K ? l0 + NT : K;
-  }
-  const int nkb = kend > kbeg ? (int)((kend - kbeg + OT_KB - 1) / OT_KB) : 0;
-  const int nch = (nkb + OT_KB_PER_CHUNK - 1) / OT_KB_PER_CHUNK;
+  // Tile t of the launch: gx row tiles x gy column tiles x gz splits (MODE 3: batches); false: nothing to do.
+  struct Tile {
+    int64_t r0, kbeg;
+    int l0, z, M, prow, nkb, nch;  // prow: first row of the batch in the operands' planes and exponents
+  };
+  const auto tile_at = [&](uint32_t t, Tile& T) -> bool {
+    const uint32_t q = t / tiles.gx;
+    // the row tile rotates with q: with gx a divisor of the grid a CTA would otherwise keep one row tile, and
+    // where the work of a tile depends on it (upper_only, MODE 3) the CTAs would end up unequal
+    T.r0 = (int64_t)((t - q * tiles.gx + q) % tiles.gx) * OT_M;
+    T.l0 = (int)(q % tiles.gy) * NT;
+    T.z = (int)(q / tiles.gy);
+    T.M = M;
+    T.prow = 0;
+    // a symmetric product (P = Q) needs out[l][r] for l <= r only
+    if (upper_only && T.l0 > T.r0 + OT_M - 1) return false;
+    int64_t kend;
+    if constexpr (MODE == 3) {
+      const int left = tri.n - (2 * (T.z % tri.pairs) + 1) * tri.h;
+      T.M = left < tri.h ? left : tri.h;
+      if (T.l0 >= T.M) return false;
+      T.prow = T.z * tri.h;
+      T.kbeg = tri.tri == 2 ? T.r0 : 0;
+      kend = tri.tri == 1 && T.l0 + NT < K ? T.l0 + NT : K;
+    } else {
+      T.kbeg = (int64_t)T.z * kps;
+      kend = K < T.kbeg + kps ? K : T.kbeg + kps;
+    }
+    T.nkb = kend > T.kbeg ? (int)((kend - T.kbeg + OT_KB - 1) / OT_KB) : 0;
+    T.nch = (T.nkb + OT_KB_PER_CHUNK - 1) / OT_KB_PER_CHUNK;
+    return true;
+  };
+  const uint32_t ntiles = tiles.gx * tiles.gy * tiles.gz;
+  Tile T;  // the first tile, found while the barriers and tensor memory are set up
+  bool has = tile_at(blockIdx.x, T);
+  const auto next_tile = [&](uint32_t t) { has = t < ntiles && tile_at(t, T); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < OtCfg<S, NT>::PST; ++s) {
@@ -517,79 +545,91 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
   const uint32_t tmem = Sm.tmem_base;
 
   if (warp == 0 && lane == 0) {
-    int g = 0, gq = 0;  // loads issued into the P ring and the Q ring
+    uint32_t g = 0, gq = 0;  // loads issued into the P ring and the Q ring, over all tiles
     bool live = true;
-    for (int kb = 0; kb < nkb && live; ++kb) {
-      const int kc = (int)(kbeg + (int64_t)kb * OT_KB);
-      const int qs = kb & 1;
-      if (!mbar_wait(&Sm.q_empty[qs], ((uint32_t)(kb >> 1) & 1u) ^ 1u, err)) break;
-      mbar_expect_tx(&Sm.q_full[qs], Q_BYTES);
-      for (int p = 0; p < S; ++p) tma_load_3d(&tmQ, &Sm.q_full[qs], Sm.q[qs] + p * QS_BYTES, kc, prow + l0, p);
-      ++gq;
-      for (int p = 0; p < S; ++p, ++g) {
-        const int ps = g % OtCfg<S, NT>::PST;
-        if (!mbar_wait(&Sm.p_empty[ps], ((uint32_t)(g / OtCfg<S, NT>::PST) & 1u) ^ 1u, err)) {
+    for (uint32_t t = blockIdx.x; t < ntiles && live; next_tile(t += gridDim.x)) {
+      if (!has) continue;
+      for (int kb = 0; kb < T.nkb && live; ++kb, ++gq) {
+        const int kc = (int)(T.kbeg + (int64_t)kb * OT_KB);
+        const int qs = gq & 1;
+        if (!mbar_wait(&Sm.q_empty[qs], ((gq >> 1) & 1u) ^ 1u, err)) {
           live = false;
           break;
         }
-        mbar_expect_tx(&Sm.p_full[ps], OT_P_BYTES);
-        if constexpr (TR) {
-          tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], (int)r0, kc, p);
-          tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps] + OT_P_BYTES / 2, (int)r0 + 64, kc, p);
-        } else {
-          tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], kc, prow + (int)r0, p);
+        mbar_expect_tx(&Sm.q_full[qs], Q_BYTES);
+        for (int p = 0; p < S; ++p) tma_load_3d(&tmQ, &Sm.q_full[qs], Sm.q[qs] + p * QS_BYTES, kc, T.prow + T.l0, p);
+        for (int p = 0; p < S; ++p, ++g) {
+          const int ps = g % OtCfg<S, NT>::PST;
+          if (!mbar_wait(&Sm.p_empty[ps], ((g / OtCfg<S, NT>::PST) & 1u) ^ 1u, err)) {
+            live = false;
+            break;
+          }
+          mbar_expect_tx(&Sm.p_full[ps], OT_P_BYTES);
+          if constexpr (TR) {
+            tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], (int)T.r0, kc, p);
+            tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps] + OT_P_BYTES / 2, (int)T.r0 + 64, kc, p);
+          } else {
+            tma_load_3d(&tmP, &Sm.p_full[ps], Sm.p[ps], kc, T.prow + (int)T.r0, p);
+          }
         }
       }
     }
     if (*(volatile int*)err) {  // gave up: no bulk copy may still be landing when the CTA exits
-      tma_drain_ring(Sm.p_full, OtCfg<S, NT>::PST, g);
-      tma_drain_ring(Sm.q_full, 2, gq);
+      tma_drain_ring(Sm.p_full, OtCfg<S, NT>::PST, (int)g);
+      tma_drain_ring(Sm.q_full, 2, (int)gq);
     }
   } else if (warp == 1 && lane == 0) {
-    int g = 0;
+    uint32_t g = 0, gq = 0, gc = 0;  // planes of P, of Q and chunks used, over all tiles
     bool live = true;
-    for (int c = 0; c < nch && live; ++c) {
-      const int bsel = c & 1, use = c >> 1;
-      if (use > 0 && !mbar_wait(&Sm.acc_empty[bsel], (uint32_t)(use - 1) & 1u, err)) break;
-      tc_fence_after();
-      const uint32_t dbase = tmem + (uint32_t)(bsel * S * NT);
-      const int kb0 = OT_KB_PER_CHUNK * c;
-      const int kb_end = nkb < kb0 + OT_KB_PER_CHUNK ? nkb : kb0 + OT_KB_PER_CHUNK;
-      for (int kb = kb0; kb < kb_end && live; ++kb) {
-        const int qs = kb & 1;
-        if (!mbar_wait(&Sm.q_full[qs], (uint32_t)(kb >> 1) & 1u, err)) {
+    for (uint32_t t = blockIdx.x; t < ntiles && live; next_tile(t += gridDim.x)) {
+      if (!has) continue;
+      for (int c = 0; c < T.nch && live; ++c, ++gc) {
+        const uint32_t bsel = gc & 1, use = gc >> 1;
+        if (use > 0 && !mbar_wait(&Sm.acc_empty[bsel], (use - 1) & 1u, err)) {
           live = false;
           break;
         }
         tc_fence_after();
-        const uint32_t qa = smem_u32(Sm.q[qs]);
-        for (int p = 0; p < S; ++p, ++g) {
-          const int ps = g % OtCfg<S, NT>::PST;
-          if (!mbar_wait(&Sm.p_full[ps], (uint32_t)(g / OtCfg<S, NT>::PST) & 1u, err)) {
+        const uint32_t dbase = tmem + bsel * S * NT;
+        const int kb0 = OT_KB_PER_CHUNK * c;
+        const int kb_end = T.nkb < kb0 + OT_KB_PER_CHUNK ? T.nkb : kb0 + OT_KB_PER_CHUNK;
+        for (int kb = kb0; kb < kb_end && live; ++kb, ++gq) {
+          const uint32_t qs = gq & 1;
+          if (!mbar_wait(&Sm.q_full[qs], (gq >> 1) & 1u, err)) {
             live = false;
             break;
           }
           tc_fence_after();
-          // the planes Q_0 .. Q_(S-1-p) lie one after another (NT rows each), and the levels
-          // p .. S-1 are consecutive NT-column blocks of the buffer: all pairs (p, q) are one
-          // MMA with N = NT (S - p) whose column block q lands on level p + q
-          // 16 values of K are 32 bytes of a K-major row, or 16 rows of 128 bytes of the MN-major tile
-          const uint64_t pd = TR ? sdesc_mn_sw128(smem_u32(Sm.p[ps]), OT_P_BYTES / 2) : sdesc_sw128(smem_u32(Sm.p[ps]));
-          constexpr uint64_t pstep = TR ? 2048 / 16 : 2;
-          const uint64_t qd = sdesc_sw128(qa);
-          const uint32_t idesc = idesc_bf16(OT_M, NT * (S - p)) | (TR ? 1u << 15 : 0u);
-          const uint32_t d = dbase + (uint32_t)(p * NT);
+          const uint32_t qa = smem_u32(Sm.q[qs]);
+          for (int p = 0; p < S; ++p, ++g) {
+            const int ps = g % OtCfg<S, NT>::PST;
+            if (!mbar_wait(&Sm.p_full[ps], (g / OtCfg<S, NT>::PST) & 1u, err)) {
+              live = false;
+              break;
+            }
+            tc_fence_after();
+            // the planes Q_0 .. Q_(S-1-p) lie one after another (NT rows each), and the levels
+            // p .. S-1 are consecutive NT-column blocks of the buffer: all pairs (p, q) are one
+            // MMA with N = NT (S - p) whose column block q lands on level p + q
+            // 16 values of K are 32 bytes of a K-major row, or 16 rows of 128 bytes of the MN-major tile
+            const uint32_t pa = smem_u32(Sm.p[ps]);
+            const uint64_t pd = TR ? sdesc_mn_sw128(pa, OT_P_BYTES / 2) : sdesc_sw128(pa);
+            constexpr uint64_t pstep = TR ? 2048 / 16 : 2;
+            const uint64_t qd = sdesc_sw128(qa);
+            const uint32_t idesc = idesc_bf16(OT_M, NT * (S - p)) | (TR ? 1u << 15 : 0u);
+            const uint32_t d = dbase + (uint32_t)(p * NT);
 #pragma unroll
-          for (int k = 0; k < OT_KB / 16; ++k) {
-            // the first MMA of a chunk (p = 0) overwrites every level of the buffer
-            const uint32_t acc = (kb == kb0 && p == 0 && k == 0) ? 0u : 1u;
-            tc_mma_bf16(d, pd + pstep * k, qd + 2ull * k, idesc, acc);
+            for (int k = 0; k < OT_KB / 16; ++k) {
+              // the first MMA of a chunk (p = 0) overwrites every level of the buffer
+              const uint32_t acc = (kb == kb0 && p == 0 && k == 0) ? 0u : 1u;
+              tc_mma_bf16(d, pd + pstep * k, qd + 2ull * k, idesc, acc);
+            }
+            tc_commit(&Sm.p_empty[ps]);
           }
-          tc_commit(&Sm.p_empty[ps]);
+          if (live) tc_commit(&Sm.q_empty[qs]);
         }
-        if (live) tc_commit(&Sm.q_empty[qs]);
+        if (live) tc_commit(&Sm.acc_full[bsel]);
       }
-      if (live) tc_commit(&Sm.acc_full[bsel]);
     }
     if (*(volatile int*)err) {  // gave up: wait for the MMAs issued before tensor memory is freed
       tc_commit(&Sm.mma_drain);
@@ -597,86 +637,116 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
     }
   } else if (warp >= 4) {
     const int ew = warp - 4;
-    // S = 8 (float64-accurate): the chunk's 8 exact level sums (|L_t| <= (t+1) 2^20, so L0 128 + L1 and
-    // the like fit an int) are added exactly into two int64 accumulators per column, hi += L0 2^21 +
-    // L1 2^14 + L2 2^7 + L3 and lo likewise from L4 .. L7 (value = hi 2^-35 + lo 2^-63; each under 2^44 per
-    // chunk, so exact for K <= 2^27 per split), 8 columns at a time -- integer work, off GB300's slow float64
-    // pipe -- and turned into one double at the end.  S = 4: float32 accumulators.
-    Acc acc[S == OZ_S ? 1 : NT];
-    long long hacc[S == OZ_S ? NT : 1], lacc[S == OZ_S ? NT : 1];
-#pragma unroll
-    for (int j = 0; j < (S == OZ_S ? 1 : NT); ++j) acc[j] = Acc(0);
-#pragma unroll
-    for (int j = 0; j < (S == OZ_S ? NT : 1); ++j) hacc[j] = lacc[j] = 0;
+    uint32_t gc = 0;  // chunks read, over all tiles
     bool ok = true;
-    for (int c = 0; c < nch; ++c) {
-      const int bsel = c & 1, use = c >> 1;
-      if (!mbar_wait(&Sm.acc_full[bsel], (uint32_t)use & 1u, err)) {
-        ok = false;
-        break;
+    for (uint32_t t = blockIdx.x; t < ntiles && ok; next_tile(t += gridDim.x)) {
+      if (!has) continue;
+      // what the last step needs besides the sums, on its way while the products are formed
+      const int64_t r = T.r0 + ew * 32 + lane;
+      const bool mine = r < rows;
+      const int er = mine ? EP[T.prow + r] : 0;
+      const double br = MODE == 0 && mine ? b[r] : 0.0;
+      int eqv[NT / 32];  // of column 32 h + lane
+      double cv[NT / 32];
+#pragma unroll
+      for (int h = 0; h < NT / 32; ++h) {
+        const int l = T.l0 + 32 * h + lane;
+        eqv[h] = l < T.M ? EQ[T.prow + l] : 0;
+        cv[h] = MODE == 2 && coef && l < T.M ? coef[l] : 0.0;
       }
-      tc_fence_after();
-      const uint32_t base = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(bsel * S * NT);
-      if constexpr (S == OZ_S) {
+      // S = 8 (float64-accurate): the chunk's 8 exact level sums (|L_t| <= (t+1) 2^20, so L0 128 + L1 and
+      // the like fit an int) are added exactly into two int64 accumulators per column, hi += L0 2^21 +
+      // L1 2^14 + L2 2^7 + L3 and lo likewise from L4 .. L7 (value = hi 2^-35 + lo 2^-63; each under 2^44 per
+      // chunk, so exact for K <= 2^27 per split), 8 columns at a time -- integer work, off GB300's slow float64
+      // pipe -- and turned into one double at the end.  S = 4: float32 accumulators.
+      Acc acc[S == OZ_S ? 1 : NT];
+      long long hacc[S == OZ_S ? NT : 1], lacc[S == OZ_S ? NT : 1];
 #pragma unroll
-        for (int g = 0; g < NT / 8; ++g) {
-          uint32_t v[OZ_S][8];
+      for (int j = 0; j < (S == OZ_S ? 1 : NT); ++j) acc[j] = Acc(0);
 #pragma unroll
-          for (int t = 0; t < OZ_S; ++t) tmem_ld8_nowait(base + (uint32_t)(t * NT + 8 * g), v[t]);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            int L[OZ_S];
-#pragma unroll
-            for (int t = 0; t < OZ_S; ++t) L[t] = __float2int_rz(__uint_as_float(v[t][j]));  // exact integers
-            hacc[8 * g + j] += (long long)(L[0] * 128 + L[1]) * 16384 + (L[2] * 128 + L[3]);
-            lacc[8 * g + j] += (long long)(L[4] * 128 + L[5]) * 16384 + (L[6] * 128 + L[7]);
-          }
+      for (int j = 0; j < (S == OZ_S ? NT : 1); ++j) hacc[j] = lacc[j] = 0;
+      for (int c = 0; c < T.nch; ++c, ++gc) {
+        const uint32_t bsel = gc & 1, use = gc >> 1;
+        if (!__all_sync(0xffffffffu, mbar_wait(&Sm.acc_full[bsel], use & 1u, err))) {
+          ok = false;
+          break;
         }
-      } else {
-#pragma unroll 1
-        for (int t = S - 1; t >= 0; --t) {  // smallest level first
+        tc_fence_after();
+        const uint32_t base = tmem + ((uint32_t)(ew * 32) << 16) + bsel * S * NT;
+        if constexpr (S == OZ_S) {
 #pragma unroll
-          for (int h = 0; h < NT / 32; ++h) {
-            uint32_t v[32];
-            tmem_ld32_nowait(base + (uint32_t)(t * NT + 32 * h), v);
+          for (int g = 0; g < NT / 8; ++g) {
+            uint32_t v[OZ_S][8];
+#pragma unroll
+            for (int t = 0; t < OZ_S; ++t) tmem_ld8_nowait(base + (uint32_t)(t * NT + 8 * g), v[t]);
             tmem_wait_ld();
-            const float sc = __int_as_float((127 - 7 * (t + 2)) << 23);  // 2^(-7(t+2)), exact
 #pragma unroll
-            for (int j = 0; j < 32; ++j) acc[32 * h + j] = fmaf(__uint_as_float(v[j]), sc, acc[32 * h + j]);
+            for (int j = 0; j < 8; ++j) {
+              int L[OZ_S];
+#pragma unroll
+              for (int t = 0; t < OZ_S; ++t) L[t] = __float2int_rz(__uint_as_float(v[t][j]));  // exact integers
+              hacc[8 * g + j] += (long long)(L[0] * 128 + L[1]) * 16384 + (L[2] * 128 + L[3]);
+              lacc[8 * g + j] += (long long)(L[4] * 128 + L[5]) * 16384 + (L[6] * 128 + L[7]);
+            }
+          }
+        } else {
+#pragma unroll 1
+          for (int t = S - 1; t >= 0; --t) {  // smallest level first
+#pragma unroll
+            for (int h = 0; h < NT / 32; ++h) {
+              uint32_t v[32];
+              tmem_ld32_nowait(base + (uint32_t)(t * NT + 32 * h), v);
+              tmem_wait_ld();
+              const float sc = __int_as_float((127 - 7 * (t + 2)) << 23);  // 2^(-7(t+2)), exact
+#pragma unroll
+              for (int j = 0; j < 32; ++j) acc[32 * h + j] = fmaf(__uint_as_float(v[j]), sc, acc[32 * h + j]);
+            }
           }
         }
+        tc_fence_before();
+        mbar_arrive(&Sm.acc_empty[bsel]);
       }
-      tc_fence_before();
-      mbar_arrive(&Sm.acc_empty[bsel]);
-    }
-    const int64_t r = r0 + ew * 32 + lane;
-    if (ok && r < rows) {
-      const int er = EP[r];
-      const double br = MODE == 0 ? b[r] : 0.0;
+      if (ok) {
+        using TU = typename std::conditional<S == OZ_S, double, float>::type;
+        constexpr int G = S == OZ_S ? 4 : 8;  // U is read G columns ahead: one by one a load waits for the last store
+        TU uv[G];
 #pragma unroll
-      for (int j = 0; j < NT; ++j) {
-        const int l = l0 + j;
-        if (l < M) {
-          const int eq = EQ[l];
+        for (int j = 0; j < NT; ++j) {
+          const int l = T.l0 + j;
+          const int eq = __shfl_sync(0xffffffffu, eqv[j / 32], j % 32), e = er + eq;
+          const double cf = MODE == 2 ? __shfl_sync(0xffffffffu, cv[j / 32], j % 32) : 0.0;
+          if (MODE == 2 && j % G == 0 && coef) {
+#pragma unroll
+            for (int q = 0; q < G; ++q)
+              uv[q] = mine && l + q < T.M ? static_cast<const TU*>(out)[(int64_t)(l + q) * ldo + r] : TU(0);
+          }
+          if (!mine || l >= T.M) continue;
+          const bool bad = oz_bad(er) || oz_bad(eq);
+          if constexpr (MODE == 3 && S != OZ_S) {
+            // a float32 result needs no float64 arithmetic: one scaling by a power of two, rounded once
+            const float sg = (float)tri.sign * acc[j];
+            static_cast<float*>(out)[(int64_t)(T.z / tri.pairs) * tri.mstride +
+                                     (int64_t)(T.z % tri.pairs) * tri.pstride + (int64_t)l * ldo + r] =
+                bad ? __int_as_float(0x7fc00000)
+                    : (e >= -126 && e <= 127 ? sg * __int_as_float((127 + e) << 23) : ldexpf(sg, e));
+            continue;
+          }
           double d;
           if constexpr (S == OZ_S) d = fma((double)lacc[j], 0x1p-63, (double)hacc[j] * 0x1p-35);
           else d = (double)acc[j];
-          const double v = (oz_bad(er) || oz_bad(eq)) ? __longlong_as_double(0x7ff8000000000000ll)
-                                                            : ldexp(d, er + eq);
+          const double v = bad ? __longlong_as_double(0x7ff8000000000000ll)
+                               : (e >= -1022 && e <= 1023 ? d * pow2d(e) : ldexp(d, e));
           if (MODE == 0) {
             static_cast<double*>(out)[(int64_t)l * ldo + r] = br - v;
           } else if (MODE == 1) {
-            static_cast<double*>(out)[((int64_t)blockIdx.z * M + l) * ldo + r] = v;
+            static_cast<double*>(out)[((int64_t)T.z * T.M + l) * ldo + r] = v;
           } else if (MODE == 3) {
-            using TU = typename std::conditional<S == OZ_S, double, float>::type;
-            static_cast<TU*>(out)[(int64_t)(blockIdx.z / tri.pairs) * tri.mstride +
-                                  (int64_t)(blockIdx.z % tri.pairs) * tri.pstride + (int64_t)l * ldo + r] =
+            static_cast<TU*>(out)[(int64_t)(T.z / tri.pairs) * tri.mstride +
+                                  (int64_t)(T.z % tri.pairs) * tri.pstride + (int64_t)l * ldo + r] =
                 (TU)(tri.sign * v);
           } else {
-            using TU = typename std::conditional<S == OZ_S, double, float>::type;
             TU* u = static_cast<TU*>(out) + (int64_t)l * ldo + r;
-            *u = coef ? (TU)(v + coef[l] * (double)*u) : (TU)v;
+            *u = coef ? (TU)(v + cf * (double)uv[j % G]) : (TU)v;
           }
         }
       }
@@ -689,6 +759,12 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
+}
+
+// One CTA per slot of the GPU at most
+template <int S, int NT>
+unsigned ot_grid(const OtTiles& t) {
+  return (unsigned)std::min<int64_t>((int64_t)t.gx * t.gy * t.gz, 152 * OtCfg<S, NT>::CTAS_PER_SM);
 }
 
 // 3D map over the slice planes (K fastest, then rows, then the plane index),
@@ -736,9 +812,15 @@ tk_status launch_oz_tc_nt(const OtBig& P, const void* Qs, const int* EQ, int M, 
   TK_TRY(make_slice_map(&mQ, Qs, M, kp, NT, planesQ));
   const size_t smem = sizeof(OtSmem<S, NT>) + 1024;
   TK_CUDA(cudaFuncSetAttribute(k_oz_tc<S, MODE, NT, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const dim3 grid((unsigned)cdiv(P.rows, OT_M), (unsigned)cdiv(M, NT), (unsigned)sp);
+  const OtTiles tl{(uint32_t)cdiv(P.rows, OT_M), (uint32_t)cdiv(M, NT), (uint32_t)sp};
+  if ((double)tl.gx * tl.gy * tl.gz > 2e9) {
+    set_error_msg("digit product: too many tiles for one launch");
+    return TK_EINVAL;
+  }
+  // (half a symmetric product's tiles are skipped: the hardware's own order shares those out better)
+  const unsigned grid = upper_only ? tl.gx * tl.gy * tl.gz : ot_grid<S, NT>(tl);
   k_oz_tc<S, MODE, NT, TR>
-      <<<grid, 256, smem, st>>>(mP, mQ, P.E, EQ, P.rows, M, kp, kps, b, out, ldo, coef, upper_only, err, OtTri{});
+      <<<grid, 256, smem, st>>>(mP, mQ, P.E, EQ, P.rows, M, kp, kps, b, out, ldo, coef, upper_only, err, tl, OtTri{});
   TK_LAUNCH_CHECK();
   return TK_OK;
 }
@@ -903,9 +985,6 @@ __device__ __forceinline__ void st_global_v4(double* p, const double* v) {
   asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
                : "memory");
 }
-
-// 2^e as a double (e within the normal range).
-__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
 
 // v 2^s as a double, built from the integer's bits with integer instructions
 // only (GB300's float64 pipe is the bottleneck of the update's epilogue):
@@ -1869,7 +1948,7 @@ tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* M
   const int pairs = (int)cdiv(n - h, 2 * (int64_t)h);
   if (pairs <= 0) return TK_OK;
   const int64_t batch = (int64_t)N * pairs, rows = batch * h;
-  if (batch > 65535 || rows > INT32_MAX) {
+  if (batch > 65535 || rows > INT32_MAX || (double)rows * h > 2e9 * OT_M * NT) {
     set_error_msg("triangular inverse: too many blocks for one launch");
     return TK_EINVAL;
   }
@@ -1887,7 +1966,9 @@ tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* M
   TK_TRY(make_slice_map(&mQ, Qs, rows, h, NT, S));
   const size_t smem = sizeof(OtSmem<S, NT>) + 1024;
   TK_CUDA(cudaFuncSetAttribute(k_oz_tc<S, 3, NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const dim3 gs((unsigned)h, (unsigned)batch), g((unsigned)(h / OT_M), (unsigned)(h / NT), (unsigned)batch);
+  const dim3 gs((unsigned)h, (unsigned)batch);
+  const OtTiles tl{(uint32_t)(h / OT_M), (uint32_t)(h / NT), (uint32_t)batch};
+  const unsigned g = ot_grid<S, NT>(tl);
   const int64_t pr = 2 * (int64_t)h;  // a pair's step along the diagonal
   OtTri t{pairs, 1, h, (int)n, (int64_t)pairs * h * h, (int64_t)h * h, 1.0};
   k_oz_block_rows<double><<<gs, 256, 0, st>>>(R + h, rstride, pr * (ldr + 1), ldr, pairs, h, (int)n, 0, 1, 0, rows, S,
@@ -1896,7 +1977,7 @@ tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* M
   k_oz_block_rows<T><<<gs, 256, 0, st>>>(Mt + h * (ldm + 1), mstride, pr * (ldm + 1), ldm, pairs, h, (int)n, 1, 1, 1,
                                          rows, S, EQ, Qs);
   TK_LAUNCH_CHECK();
-  k_oz_tc<S, 3, NT, false><<<g, 256, smem, st>>>(mP, mQ, EP, EQ, h, h, h, h, nullptr, Tt, h, nullptr, 0, err, t);
+  k_oz_tc<S, 3, NT, false><<<g, 256, smem, st>>>(mP, mQ, EP, EQ, h, h, h, h, nullptr, Tt, h, nullptr, 0, err, tl, t);
   TK_LAUNCH_CHECK();
   k_oz_block_rows<T><<<gs, 256, 0, st>>>(M, mstride, pr * (ldm + 1), ldm, pairs, h, (int)n, 0, 0, 0, rows, S, EP, Ps);
   TK_LAUNCH_CHECK();
@@ -1904,8 +1985,8 @@ tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* M
                                          S, EQ, Qs);
   TK_LAUNCH_CHECK();
   t = OtTri{pairs, 2, h, (int)n, mstride, pr * (ldm + 1), -1.0};
-  k_oz_tc<S, 3, NT, false><<<g, 256, smem, st>>>(mP, mQ, EP, EQ, h, h, h, h, nullptr, Mt + h * ldm, ldm, nullptr, 0, err,
-                                                 t);
+  k_oz_tc<S, 3, NT, false>
+      <<<g, 256, smem, st>>>(mP, mQ, EP, EQ, h, h, h, h, nullptr, Mt + h * ldm, ldm, nullptr, 0, err, tl, t);
   TK_LAUNCH_CHECK();
   k_oz_block_transpose<T><<<dim3((unsigned)(h / 32), (unsigned)(h / 32), (unsigned)batch), 256, 0, st>>>(
       Mt, M, ldm, mstride, pairs, h, (int)n);

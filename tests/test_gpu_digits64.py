@@ -17,11 +17,12 @@ def _solve(A, b, lams, **kw):
 
 # A at and around the smallest size that is split into digits (2^19 elements), ragged against the 64-,
 # 128- and 256-value tiles, one and several tiles of 32 lambdas, float64 views with odd row strides,
-# the explicit inverse over one to three doubling levels with ragged last blocks (257 .. 1100 columns), and
-# m < n with vectors of 1, 2, 4 and 8 CTAs per v-step.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
+# the explicit inverse over one to three doubling levels with ragged last blocks (257 .. 1100 columns), more
+# row tiles than SMs (60001 rows: a CTA's rings and buffers run on over several tiles), and m < n with vectors of 1, 2, 4 and 8 CTAs per v-step.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
 @pytest.mark.parametrize("m,n,N,pad", [(8192, 64, 2, 0), (8192, 65, 1, 0), (8193, 65, 3, 1), (2051, 257, 33, 0), (1500, 700, 5, 3),
                                        (16500, 40, 4, 0), (129, 4099, 4, 0), (500, 1100, 34, 5), (63, 8400, 2, 0),
-                                       (101, 17001, 3, 0), (6000, 1100, 3, 0), (517, 4000, 2, 0)])
+                                       (101, 17001, 3, 0), (6000, 1100, 3, 0), (517, 4000, 2, 0),
+                                       (60001, 130, 3, 0)])
 def test_digit_solve_matches_float64_pipe(m, n, N, pad):
     k = min(m, n)
     p = datagen.make_ridge_problem(m, n, datagen.spectrum("log", k, hi=1.0, lo=1e-3),
@@ -64,9 +65,10 @@ def test_digit_products_follow_row_and_column_scales(rows, cols):
 
 # the same levels in float32 (the mixed form's preconditioner): refined to the float64 solution, with as
 # many iterations as the float32 pipe's inverse gives
-@pytest.mark.parametrize("n,N", [(256, 3), (300, 1), (513, 5), (1100, 3), (1290, 2)])
-def test_mixed_digit_inverse(n, N):
-    m = 4 * n + 17
+# (the last two: 20 and 40 lambdas over more row tiles than the GPU has slots for)
+@pytest.mark.parametrize("n,N,m", [(256, 3, 1041), (300, 1, 1217), (513, 5, 2069), (1100, 3, 4417), (1290, 2, 5177),
+                                   (100, 20, 80001), (100, 40, 80001)])
+def test_mixed_digits(n, N, m):
     p = datagen.make_ridge_problem(m, n, datagen.spectrum("log", n, hi=1.0, lo=1e-4),
                                    datagen.log_lambdas(N, 1e-6, 1e-1), seed=n)
     A, b, lams = p.A.cuda(), p.b.cuda(), p.lambdas.numpy()
