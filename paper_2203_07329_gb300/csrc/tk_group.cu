@@ -309,12 +309,12 @@ __device__ __forceinline__ void g_aw_tile(const GDesc& d, int l0, int M, int64_t
     __syncthreads();
     const int64_t g0 = gb + (threadIdx.x >> 5);
     if constexpr (LR)
-      lmb::aw_rows<NL>(ws, n_pad, A + k0, lda, rows, len, M,
+      lmb::aw_rows<NL, lmb::kRows>(ws, n_pad, A + k0, lda, rows, len, M,
                        LrStore{field(d, fsrc) + l0 * d.n, field(d, fdst) + l0 * d.n, d.n, d.lam, d.slot_lam + l0,
                                k0 == 0},
                        vec, g0, 8, ge);
     else
-      lmb::aw_rows<NL>(ws, n_pad, A + k0, lda, rows, len, M,
+      lmb::aw_rows<NL, lmb::kRows>(ws, n_pad, A + k0, lda, rows, len, M,
                        lmb::AwStore{d.Ut + l0 * d.m, d.m, d.coef + l0, k0 == 0}, vec, g0, 8, ge);
   }
 }
@@ -348,7 +348,7 @@ __device__ __forceinline__ void g_atu_tile(const GDesc& d, int l0, int M, int Ma
   const bool vec = ((uintptr_t)A % 16 == 0) && (lda % 4 == 0);
   const int64_t rb = (int64_t)t.z * t.m0, re = rb + t.m0 < rows ? rb + t.m0 : rows;
   lmb::atu_cols<NL, CW>(*reinterpret_cast<lmb::AtuSmem<NL, CW>*>(sm), A, lda, cols,
-                        (LR ? field(d, fsrc) : d.Ut) + l0 * rows, rows, M, rb, re, t.n0,
+                        (LR ? field(d, fsrc) : d.Ut) + l0 * rows, rows, M, rb, re, t.n0, CW * lmb::kAtuThreads,
                         d.part + ((int64_t)t.z * Mall + l0) * cols, vec);
 }
 template <bool LR>

@@ -18,7 +18,9 @@ def _solve(A, b, lams, **kw):
 # A at and around the smallest size that is split into digits (2^19 elements), ragged against the 64-,
 # 128- and 256-value tiles, one and several tiles of 32 lambdas, float64 views with odd row strides,
 # the explicit inverse over one to three doubling levels with ragged last blocks (257 .. 1100 columns), more
-# row tiles than SMs (60001 rows: a CTA's rings and buffers run on over several tiles), and m < n with vectors of 1, 2, 4 and 8 CTAs per v-step.  Both forms solve to the float64 accuracy of the problem (condition about 1e3: 1e-10).
+# row tiles than SMs (60001 rows: a CTA's rings and buffers run on over several tiles), and m < n with vectors
+# of 1, 2, 4 and 8 CTAs per v-step.  Both forms solve to the float64 accuracy of the problem (condition about
+# 1e3: 1e-10).
 @pytest.mark.parametrize("m,n,N,pad", [(8192, 64, 2, 0), (8192, 65, 1, 0), (8193, 65, 3, 1), (2051, 257, 33, 0), (1500, 700, 5, 3),
                                        (16500, 40, 4, 0), (129, 4099, 4, 0), (500, 1100, 34, 5), (63, 8400, 2, 0),
                                        (101, 17001, 3, 0), (6000, 1100, 3, 0), (517, 4000, 2, 0),
