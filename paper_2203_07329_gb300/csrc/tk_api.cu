@@ -309,7 +309,8 @@ void carve(const Plan& P, Arena& a, Arena& t, Bufs& B) {
   size_t sc = std::max(sketch_scratch(P), P.lowrank ? size_t(0) : gram_scratch_bytes(P.s, P.c));
   if (P.qr) sc = std::max(sc, bp2_workspace(P.s, P.c, N));
   // and the inverse of the factors, after them
-  if (digit_inverse(P)) sc = std::max(sc, P.mixed ? tri_inverse_workspace<float>(P.np, N) : tri_inverse_workspace<double>(P.np, N));
+  if (digit_inverse(P))
+    sc = std::max(sc, P.mixed ? tri_inverse_workspace<float>(P.np, N) : tri_inverse_workspace<double>(P.np, N));
   if (emulated_gram(P)) sc = std::max({sc, oz_gram_workspace(P.s, P.c), oz_chol_workspace(P.np, N)});
   B.scratch_bytes = sc;
   B.scratch = t.take<char>(sc);
@@ -870,7 +871,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
       TK_LAUNCH_CHECK();
       TK_CUDA(cudaMemcpyAsync(hn.data(), B.nrm, sizeof(double) * 3 * cnt, cudaMemcpyDeviceToHost, st));
       int oz_err = 0;
-      if (P.o.emulate_fp64)
+      if (P.o.emulate_fp64 && (round > 0 || P.o.x0 || P.lsqr_oz || P.np > 256))  // a product from digits has run
         TK_CUDA(cudaMemcpyAsync(&oz_err, B.oz_err, sizeof(int), cudaMemcpyDeviceToHost, st));
       TK_CUDA(cudaStreamSynchronize(st));
       if (oz_err) {

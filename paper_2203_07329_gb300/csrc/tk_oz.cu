@@ -397,8 +397,8 @@ __global__ void __launch_bounds__(256) k_oz_slice_t(const T* __restrict__ X, int
 // Tile: 128 rows of P x 32 (64) rows of Q x one K split.  A CTA per slot of the GPU runs through its tiles
 // with the rings and tensor-memory buffers going on from one to the next, so the last step of a tile (float64
 // arithmetic, reads of U) overlaps the products of the next (a CTA per tile: 4 digits, 64 lambda, 262144 x 4096
-// 1.85 ms, now 1.47 = 5.8 TB/s of planes; 32 lambda, 262144 x 2048 0.75, now 0.66; 8 digits, 65536 x 1024, 16
-// lambda 235 us, now 209, of which a quarter of the last of 3.4 rounds of tiles is idle).
+// 1.85 ms, now 1.44 = 5.9 TB/s of planes; 32 lambda, 262144 x 2048 0.75, now 0.65; 8 digits, 65536 x 1024, 16
+// lambda 235 us, now 201, of which a quarter of the last of 3.4 rounds of tiles is idle).
 //   warp 0 (one lane): TMA producer -- per 64 values of K the S planes of Q
 //     (4 KiB each) into a 2-slot ring, then the S planes of P one by one
 //     (16 KiB each) into an 8-slot ring;
@@ -488,12 +488,18 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
     int l0, z, M, prow, nkb, nch;  // prow: first row of the batch in the operands' planes and exponents
   };
   const auto tile_at = [&](uint32_t t, Tile& T) -> bool {
-    const uint32_t q = t / tiles.gx;
-    // the row tile rotates with q: with gx a divisor of the grid a CTA would otherwise keep one row tile, and
-    // where the work of a tile depends on it (upper_only, MODE 3) the CTAs would end up unequal
-    T.r0 = (int64_t)((t - q * tiles.gx + q) % tiles.gx) * OT_M;
-    T.l0 = (int)(q % tiles.gy) * NT;
-    T.z = (int)(q / tiles.gy);
+    uint32_t x = t, y = 0;
+    T.z = 0;
+    if (t >= tiles.gx) {
+      // the row tile rotates with q: with gx a divisor of the grid a CTA would otherwise keep one row tile, and
+      // where the work of a tile depends on it (upper_only, MODE 3) the CTAs would end up unequal
+      const uint32_t q = t / tiles.gx;
+      x = (t - q * tiles.gx + q) % tiles.gx;
+      y = q % tiles.gy;
+      T.z = (int)(q / tiles.gy);
+    }
+    T.r0 = (int64_t)x * OT_M;
+    T.l0 = (int)y * NT;
     T.M = M;
     T.prow = 0;
     // a symmetric product (P = Q) needs out[l][r] for l <= r only
@@ -708,45 +714,53 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
       }
       if (ok) {
         using TU = typename std::conditional<S == OZ_S, double, float>::type;
-        constexpr int G = S == OZ_S ? 4 : 8;  // U is read G columns ahead: one by one a load waits for the last store
-        TU uv[G];
+        // G columns at a time: U is read G ahead (one by one a load waits for the last store), and the
+        // columns' float64 arithmetic overlaps
+        constexpr int G = S == OZ_S ? 4 : 8;
+        const double sign = MODE == 3 ? tri.sign : 1.0;
+        // the tile's first value: row r of its column l0
+        TU* o = nullptr;
+        double* o64 = nullptr;
+        if (MODE == 0) o64 = static_cast<double*>(out) + (int64_t)T.l0 * ldo + r;
+        else if (MODE == 1) o64 = static_cast<double*>(out) + ((int64_t)T.z * T.M + T.l0) * ldo + r;
+        else if (MODE == 2) o = static_cast<TU*>(out) + (int64_t)T.l0 * ldo + r;
+        else
+          o = static_cast<TU*>(out) + (int64_t)(T.z / tri.pairs) * tri.mstride +
+              (int64_t)(T.z % tri.pairs) * tri.pstride + (int64_t)T.l0 * ldo + r;
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-          const int l = T.l0 + j;
-          const int eq = __shfl_sync(0xffffffffu, eqv[j / 32], j % 32), e = er + eq;
-          const double cf = MODE == 2 ? __shfl_sync(0xffffffffu, cv[j / 32], j % 32) : 0.0;
-          if (MODE == 2 && j % G == 0 && coef) {
+        for (int j0 = 0; j0 < NT; j0 += G) {
+          const int left = T.M - T.l0 - j0;  // columns from here
+          if (left <= 0) break;
+          TU uv[G];
+          if (MODE == 2 && coef) {
 #pragma unroll
-            for (int q = 0; q < G; ++q)
-              uv[q] = mine && l + q < T.M ? static_cast<const TU*>(out)[(int64_t)(l + q) * ldo + r] : TU(0);
+            for (int q = 0; q < G; ++q) uv[q] = mine && q < left ? o[(int64_t)(j0 + q) * ldo] : TU(0);
           }
-          if (!mine || l >= T.M) continue;
-          const bool bad = oz_bad(er) || oz_bad(eq);
-          if constexpr (MODE == 3 && S != OZ_S) {
-            // a float32 result needs no float64 arithmetic: one scaling by a power of two, rounded once
-            const float sg = (float)tri.sign * acc[j];
-            static_cast<float*>(out)[(int64_t)(T.z / tri.pairs) * tri.mstride +
-                                     (int64_t)(T.z % tri.pairs) * tri.pstride + (int64_t)l * ldo + r] =
-                bad ? __int_as_float(0x7fc00000)
-                    : (e >= -126 && e <= 127 ? sg * __int_as_float((127 + e) << 23) : ldexpf(sg, e));
-            continue;
-          }
-          double d;
-          if constexpr (S == OZ_S) d = fma((double)lacc[j], 0x1p-63, (double)hacc[j] * 0x1p-35);
-          else d = (double)acc[j];
-          const double v = bad ? __longlong_as_double(0x7ff8000000000000ll)
-                               : (e >= -1022 && e <= 1023 ? d * pow2d(e) : ldexp(d, e));
-          if (MODE == 0) {
-            static_cast<double*>(out)[(int64_t)l * ldo + r] = br - v;
-          } else if (MODE == 1) {
-            static_cast<double*>(out)[((int64_t)T.z * T.M + l) * ldo + r] = v;
-          } else if (MODE == 3) {
-            static_cast<TU*>(out)[(int64_t)(T.z / tri.pairs) * tri.mstride +
-                                  (int64_t)(T.z % tri.pairs) * tri.pstride + (int64_t)l * ldo + r] =
-                (TU)(tri.sign * v);
-          } else {
-            TU* u = static_cast<TU*>(out) + (int64_t)l * ldo + r;
-            *u = coef ? (TU)(v + cf * (double)uv[j % G]) : (TU)v;
+#pragma unroll
+          for (int q = 0; q < G; ++q) {
+            const int j = j0 + q;
+            const int eq = __shfl_sync(0xffffffffu, eqv[j / 32], j % 32), e = er + eq;
+            const bool bad = oz_bad(er) || oz_bad(eq);
+            if constexpr (MODE == 3 && S != OZ_S) {
+              // a float32 result needs no float64 arithmetic: one scaling by a power of two, rounded once
+              const float sg = (float)sign * acc[j];
+              const float v = bad ? __int_as_float(0x7fc00000)
+                                  : (e >= -126 && e <= 127 ? sg * __int_as_float((127 + e) << 23) : ldexpf(sg, e));
+              if (mine && q < left) o[(int64_t)j * ldo] = v;
+            } else {
+              double d;
+              if constexpr (S == OZ_S) d = fma((double)lacc[j], 0x1p-63, (double)hacc[j] * 0x1p-35);
+              else d = (double)acc[j];
+              const double v = bad ? __longlong_as_double(0x7ff8000000000000ll)
+                                   : (e >= -1022 && e <= 1023 ? d * pow2d(e) : ldexp(d, e));
+              const double cf = MODE == 2 ? __shfl_sync(0xffffffffu, cv[j / 32], j % 32) : 0.0;
+              if (mine && q < left) {
+                if (MODE == 0) o64[(int64_t)j * ldo] = br - v;
+                else if (MODE == 1) o64[(int64_t)j * ldo] = v;
+                else if (MODE == 3) o[(int64_t)j * ldo] = (TU)(sign * v);
+                else o[(int64_t)j * ldo] = coef ? (TU)(v + cf * (double)uv[q]) : (TU)v;
+              }
+            }
           }
         }
       }
