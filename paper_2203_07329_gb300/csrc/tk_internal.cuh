@@ -287,8 +287,8 @@ int oz_normal_splits(int64_t m, int64_t n, int64_t M, int S = 8);  // S: digits 
 // (work: oz_chol_workspace(np, N) bytes), oz_chol_step(kb) replaces the
 // float64 update of block step kb.
 struct OzCholPlan {
-  CUtensorMap mP;
-  CUtensorMap mQ;
+  CUtensorMap mP, mQ;        // the planes of a block row of 64
+  CUtensorMap mP256, mQ256;  // of a panel of 256 rows
   double* R = nullptr;
   int64_t ldr = 0, rstride = 0, np = 0;
   int N = 0;

@@ -465,12 +465,40 @@ struct OtTri {
 // 2^e as a double (e within the normal range).
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
 
+// v 2^s as a double, built from the integer's bits with integer instructions
+// only (GB300's float64 pipe is the bottleneck of the update's epilogue):
+// exact for |v| < 2^53.  *ok = false when the result would not be a normal
+// double (the caller then takes the float64 route).
+__device__ __forceinline__ double i53_scaled(long long v, int s, bool* ok) {
+  if (v == 0) return 0.0;
+  const unsigned long long sg = v < 0 ? (1ull << 63) : 0ull;
+  const unsigned long long a = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
+  const int p = 63 - __clzll((long long)a);  // a in [2^p, 2^(p+1)), p <= 52
+  const int ex = p + s + 1023;
+  if (ex < 1 || ex > 2046) {
+    *ok = false;
+    return 0.0;
+  }
+  const unsigned long long mant = (a << (52 - p)) & ((1ull << 52) - 1);
+  return __longlong_as_double((long long)(sg | ((unsigned long long)ex << 52) | mant));
+}
+
 struct OtTiles {
   uint32_t gx, gy, gz;
 };
 
+// Threads of the result's warps.  MODE 4 has one chunk of products per tile, so reading a tile's sums out of
+// tensor memory and scaling them into T takes longer than the products: 8 warps (order 4096, 64 lambda: 4 warps,
+// each with its 32 columns' sums in registers and T read behind them, 4.35 ms a panel on average, now 3.39).
+template <int MODE>
+constexpr int ot_epi = MODE == 4 ? 256 : 128;
+
+// MODE 4: the trailing update of a Cholesky panel of 256 rows, for every lambda: T[l][r] -= D for r >= l, T the
+// w x w trailing block (rows ldo apart, lambda z at out + z mstride), P = Q = the panel's planes (lambda z's
+// columns at rows z h; K = 256).  Tiles: the blocks of 128 x 128 on and above the diagonal, 4 tiles of 32 each.
+
 template <int S, int MODE, int NT, bool TR>
-__global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
+__global__ void __launch_bounds__(128 + ot_epi<MODE>, OtCfg<S, NT>::CTAS_PER_SM)
     k_oz_tc(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmQ,
             const int* __restrict__ EP, const int* __restrict__ EQ, int64_t rows, int M, int64_t K, int64_t kps,
             const double* __restrict__ b, void* __restrict__ out, int64_t ldo, const double* __restrict__ coef,
@@ -490,7 +518,14 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
   const auto tile_at = [&](uint32_t t, Tile& T) -> bool {
     uint32_t x = t, y = 0;
     T.z = 0;
-    if (t >= tiles.gx) {
+    if constexpr (MODE == 4) {
+      const uint32_t per = tiles.gx, q = t / per, b = (t - q * per) / 4;
+      T.z = (int)q;
+      x = (uint32_t)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
+      while (x * (x + 1) / 2 > b) --x;
+      while ((x + 1) * (x + 2) / 2 <= b) ++x;
+      y = 4 * (b - x * (x + 1) / 2) + t % 4;  // (per is a multiple of 4)
+    } else if (t >= tiles.gx) {
       // the row tile rotates with q: with gx a divisor of the grid a CTA would otherwise keep one row tile, and
       // where the work of a tile depends on it (upper_only, MODE 3) the CTAs would end up unequal
       const uint32_t q = t / tiles.gx;
@@ -512,6 +547,11 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
       T.prow = T.z * tri.h;
       T.kbeg = tri.tri == 2 ? T.r0 : 0;
       kend = tri.tri == 1 && T.l0 + NT < K ? T.l0 + NT : K;
+    } else if constexpr (MODE == 4) {
+      if (T.l0 >= M) return false;
+      T.prow = T.z * tri.h;
+      T.kbeg = 0;
+      kend = K;
     } else {
       T.kbeg = (int64_t)T.z * kps;
       kend = K < T.kbeg + kps ? K : T.kbeg + kps;
@@ -534,7 +574,7 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
       mbar_init(&Sm.q_full[s], 1);
       mbar_init(&Sm.q_empty[s], 1);
       mbar_init(&Sm.acc_full[s], 1);
-      mbar_init(&Sm.acc_empty[s], 128);
+      mbar_init(&Sm.acc_empty[s], ot_epi<MODE>);
     }
     mbar_init(&Sm.mma_drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -641,7 +681,59 @@ __global__ void __launch_bounds__(256, OtCfg<S, NT>::CTAS_PER_SM)
       tc_commit(&Sm.mma_drain);
       mbar_drain(&Sm.mma_drain, 0u);
     }
-  } else if (warp >= 4) {
+  } else if (MODE == 4 && warp >= 4) {
+    // warps 4-7 the first 16 columns of a tile, warps 8-11 the others; T before the products are done
+    const int ew = warp & 3, half = (warp - 4) >> 2;
+    uint32_t gc = 0;
+    bool ok = true;
+    for (uint32_t t = blockIdx.x; t < ntiles && ok; next_tile(t += gridDim.x)) {
+      if (!has) continue;
+      const int64_t r = T.r0 + ew * 32 + lane;
+      const int l0 = T.l0 + 16 * half, left = T.M - l0;
+      const int er = r < rows ? EP[T.prow + r] : 0;
+      const int eqv = lane < 16 && lane < left ? EQ[T.prow + l0 + lane] : 0;
+      double* o = static_cast<double*>(out) + (int64_t)T.z * tri.mstride + (int64_t)l0 * ldo + r;
+      double tv[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) tv[j] = r < rows && j < left && r >= l0 + j ? o[(int64_t)j * ldo] : 0.0;
+      const uint32_t bsel = gc & 1, use = gc >> 1;
+      ++gc;
+      if (!__all_sync(0xffffffffu, mbar_wait(&Sm.acc_full[bsel], use & 1u, err))) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t base = tmem + ((uint32_t)(ew * 32) << 16) + bsel * S * NT + 16 * half;
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        uint32_t v[OZ_S][8];
+#pragma unroll
+        for (int q = 0; q < OZ_S; ++q) tmem_ld8_nowait(base + (uint32_t)(q * NT + 8 * g), v[q]);
+        tmem_wait_ld();
+        if (g == 1) {
+          tc_fence_before();
+          mbar_arrive(&Sm.acc_empty[bsel]);  // every sum of the thread's columns is in registers
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int j = 8 * g + q;
+          int L[OZ_S];
+#pragma unroll
+          for (int p = 0; p < OZ_S; ++p) L[p] = __float2int_rz(__uint_as_float(v[p][q]));  // exact integers
+          const long long hi = (long long)(L[0] * 128 + L[1]) * 16384 + (L[2] * 128 + L[3]);
+          const long long lo = (long long)(L[4] * 128 + L[5]) * 16384 + (L[6] * 128 + L[7]);
+          const int eq = __shfl_sync(0xffffffffu, eqv, j), e = er + eq;
+          // the two scaled terms from the integers' bits: the float64 pipe only adds and subtracts
+          bool fine = true;
+          const double shi = i53_scaled(hi, e - 35, &fine), slo = i53_scaled(lo, e - 63, &fine);
+          double d = shi + slo;
+          if (oz_bad(er) || oz_bad(eq)) d = __longlong_as_double(0x7ff8000000000000ll);
+          else if (!fine) d = ldexp(fma((double)lo, 0x1p-63, (double)hi * 0x1p-35), e);
+          if (r < rows && j < left && r >= l0 + j) o[(int64_t)j * ldo] = tv[j] - d;
+        }
+      }
+    }
+  } else if (MODE != 4 && warp >= 4) {
     const int ew = warp - 4;
     uint32_t gc = 0;  // chunks read, over all tiles
     bool ok = true;
@@ -961,6 +1053,47 @@ __global__ void __launch_bounds__(256) k_oz_panel_slice(const double* __restrict
   }
 }
 
+// The panel's planes for the products of 256 rows: block row kb0 .. kb0 + 3, columns c from (kb0 + 4) 64 on, one
+// exponent per column, planes [p][lambda np + c][256].
+constexpr size_t kPanelSmem = 256 * 33 * sizeof(double);
+__global__ void __launch_bounds__(256) k_oz_panel256(const double* __restrict__ R, int64_t ldr, int64_t rstride,
+                                                     int64_t np, int kb0, int64_t rows, __nv_bfloat16* __restrict__ out,
+                                                     int* __restrict__ EC) {
+  extern __shared__ double panel[];  // [256][33]
+  __shared__ double part[8][32];
+  __shared__ int ex[32];
+  const int l = blockIdx.y, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t c0 = (int64_t)(kb0 + 4) * 64, w = np - c0;
+  const int64_t ct = (int64_t)blockIdx.x * 32;
+  const double* Rl = R + (int64_t)l * rstride + (int64_t)kb0 * 64 * ldr + c0 + ct;
+  double mx = 0.0;
+  for (int k = ty; k < 256; k += 8) {
+    const double v = ct + tx < w ? Rl[(int64_t)k * ldr + tx] : 0.0;
+    panel[k * 33 + tx] = v;
+    mx = oz_absmax(mx, v);
+  }
+  part[ty][tx] = mx;
+  __syncthreads();
+  if (ty == 0) {
+    for (int q = 1; q < 8; ++q) mx = oz_absmax(mx, part[q][tx]);
+    ex[tx] = oz_exponent(mx);
+    if (ct + tx < w) EC[(int64_t)l * np + ct + tx] = ex[tx];
+  }
+  __syncthreads();
+  unsigned* o = reinterpret_cast<unsigned*>(out);
+  for (int idx = threadIdx.x; idx < 32 * 128; idx += blockDim.x) {
+    const int cc = idx >> 7, k = 2 * (idx & 127);
+    if (ct + cc < w) {
+      unsigned short s0[OZ_S], s1[OZ_S];
+      oz_split(panel[k * 33 + cc], ex[cc], s0);
+      oz_split(panel[(k + 1) * 33 + cc], ex[cc], s1);
+#pragma unroll
+      for (int p = 0; p < OZ_S; ++p)
+        o[(((int64_t)p * rows + (int64_t)l * np + ct + cc) * 256 + k) / 2] = oz_pack(s0[p], s1[p]);
+    }
+  }
+}
+
 constexpr int CS_M = 128;                        // rows of a CTA's slab
 constexpr int CS_N = 32;                         // columns of one tile
 constexpr int CS_TILES = 8;                      // column tiles per CTA
@@ -1000,24 +1133,6 @@ __device__ __forceinline__ void st_global_v4(double* p, const double* v) {
                : "memory");
 }
 
-// v 2^s as a double, built from the integer's bits with integer instructions
-// only (GB300's float64 pipe is the bottleneck of the update's epilogue):
-// exact for |v| < 2^53.  *ok = false when the result would not be a normal
-// double (the caller then takes the float64 route).
-__device__ __forceinline__ double i53_scaled(long long v, int s, bool* ok) {
-  if (v == 0) return 0.0;
-  const unsigned long long sg = v < 0 ? (1ull << 63) : 0ull;
-  const unsigned long long a = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
-  const int p = 63 - __clzll((long long)a);  // a in [2^p, 2^(p+1)), p <= 52
-  const int ex = p + s + 1023;
-  if (ex < 1 || ex > 2046) {
-    *ok = false;
-    return 0.0;
-  }
-  const unsigned long long mant = (a << (52 - p)) & ((1ull << 52) - 1);
-  return __longlong_as_double((long long)(sg | ((unsigned long long)ex << 52) | mant));
-}
-
 // Grid: (row slabs of 128, chunks of 8 column tiles of 32, lambda) over the
 // w x w trailing block.  Slab i0 needs the tiles j0 >= i0 (j >= i); a CTA
 // whose chunk holds none exits at once.  The slab's digit planes are loaded
@@ -1029,8 +1144,8 @@ __device__ __forceinline__ double i53_scaled(long long v, int s, bool* ok) {
 // exact integers), scaled by 2^(E_i + E_j).
 __global__ void __launch_bounds__(384, 1)
     k_oz_syrk(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmQ,
-              const int* __restrict__ EC, int64_t np, int kb, double* __restrict__ R, int64_t ldr, int64_t rstride,
-              int* __restrict__ err) {
+              const int* __restrict__ EC, int64_t np, int kb, int rem, double* __restrict__ R, int64_t ldr,
+              int64_t rstride, int* __restrict__ err) {
   extern __shared__ __align__(1024) uint8_t cs_raw[];
   CsSmem& S = *reinterpret_cast<CsSmem*>((reinterpret_cast<uintptr_t>(cs_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1110,8 +1225,9 @@ __global__ void __launch_bounds__(384, 1)
     // of a lane quarter split each tile's 32 columns: warps 4-7 the first 16, warps 8-11 the last 16
     const int ew = warp & 3, half = (warp - 4) >> 2;
     const int64_t i = i0 + ew * 32 + lane;
+    const bool mine = i < rem;  // (rem <= w)
     const int* El = EC + (int64_t)l * np;
-    const int ei = i < w ? El[i] : 0;
+    const int ei = mine ? El[i] : 0;
     double* Trow = R + (int64_t)l * rstride + (c0 + i) * ldr + c0;
     // the exponents of the CTA's columns, once, in shared memory (the epilogue warps only)
     for (int c = (int)threadIdx.x - 128; c < CS_TILES * CS_N; c += 256) {
@@ -1131,7 +1247,7 @@ __global__ void __launch_bounds__(384, 1)
       // sectors; element by element every 8-byte store was a partial sector write of its own: order 4096, 64
       // lambda 2.51 ms a step on average, now 2.10; order 2048, 32 lambda 0.36, now 0.30).  Tiles on
       // the diagonal (columns below the thread's row) and marked rows go element by element.
-      const bool full = i < w && j0 >= i;
+      const bool full = mine && j0 >= i;
       // T of the thread's 16 columns first: their loads do not wait for the products
       double tv[2][G];
       if (full) {
@@ -1143,7 +1259,7 @@ __global__ void __launch_bounds__(384, 1)
 #pragma unroll
           for (int j = 0; j < G; ++j) {
             const int64_t col = j0 + gi * G + j;
-            tv[gi][j] = (i < w && col < w && col >= i) ? Trow[col] : 0.0;
+            tv[gi][j] = (mine && col < w && col >= i) ? Trow[col] : 0.0;
           }
       }
       if (!mbar_wait(&S.acc_full[s], (uint32_t)(t >> 1) & 1u, err)) break;
@@ -1161,7 +1277,7 @@ __global__ void __launch_bounds__(384, 1)
           tc_fence_before();
           mbar_arrive(&S.acc_empty[s]);  // every level of the thread's columns is in registers
         }
-        if (i < w) {
+        if (mine) {
 #pragma unroll
           for (int j = 0; j < G; ++j) {
             const int ej = S.ecol[t * CS_N + half * 2 * G + gi * G + j];
@@ -2126,7 +2242,7 @@ tk_status oz_gram(const double* Y, int64_t r, int64_t c, double* C, void* work, 
 
 size_t oz_chol_workspace(int64_t np, int N) {
   Arena a;
-  a.take<__nv_bfloat16>((size_t)N * OZ_S * np * 64);
+  a.take<__nv_bfloat16>((size_t)N * OZ_S * np * (np > 256 ? 256 : 64));
   a.take<int>((size_t)N * np);
   return a.used + 256;
 }
@@ -2141,7 +2257,7 @@ tk_status oz_chol_begin(double* R, int64_t ldr, int64_t rstride, int N, int64_t 
   a.base = static_cast<char*>(work);
   a.cap = bytes;
   const size_t sb = sizeof(__nv_bfloat16) * (size_t)N * OZ_S * np * 64;
-  plan->slices = a.take<__nv_bfloat16>((size_t)N * OZ_S * np * 64);
+  plan->slices = a.take<__nv_bfloat16>((size_t)N * OZ_S * np * (np > 256 ? 256 : 64));
   plan->EC = a.take<int>((size_t)N * np);
   if (!a.ok()) return TK_ENOMEM;
   plan->R = R;
@@ -2169,19 +2285,54 @@ tk_status oz_chol_begin(double* R, int64_t ldr, int64_t rstride, int N, int64_t 
     }
   }
   TK_CUDA(cudaFuncSetAttribute(k_oz_syrk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(CsSmem) + 1024)));
+  if (np > 256) {
+    // the same memory, as the planes of a panel of 256 rows
+    const int64_t rows = (int64_t)N * np;
+    if (rows > INT32_MAX - 2 * OT_M || (double)N * np * np > 2e9 * OT_M * OT_N) {
+      set_error_msg("emulated Cholesky: unsupported order or lambda count");
+      return TK_EINVAL;
+    }
+    TK_TRY(make_slice_map(&plan->mP256, plan->slices, rows, 256, OT_M, OZ_S));
+    TK_TRY(make_slice_map(&plan->mQ256, plan->slices, rows, 256, OT_N, OZ_S));
+    TK_CUDA(cudaFuncSetAttribute(k_oz_tc<OZ_S, 4, 32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(OtSmem<OZ_S, 32>) + 1024)));
+    TK_CUDA(cudaFuncSetAttribute(k_oz_panel256, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPanelSmem));
+  }
   return TK_OK;
 }
 
+// Right-looking in panels of 4 block rows: after block row kb the rest of its panel (rem rows, all columns
+// right of it) takes the product of its 64 rows; after the panel's last one the whole trailing block takes the
+// product of the panel's 256 rows.  A trailing element is then read, scaled and written once per 256 rows
+// instead of once per 64, which is what bounded the update (the float64 pipe and the integer work of an
+// element's flush, not the products): order 4096, 64 lambda 138 ms for all updates of 64 rows, now 73; order
+// 2048, 32 lambda 10.3, now 6.7; order 1024, 16 lambda 1.25, now 1.10.
 tk_status oz_chol_step(const OzCholPlan& plan, int kb, cudaStream_t st) {
   const int64_t w = plan.np - (int64_t)(kb + 1) * 64;
   if (w <= 0) return TK_OK;
+  const int64_t rem = std::min<int64_t>(w, (3 - kb % 4) * 64);
+  if (rem == 0) {
+    const int kb0 = kb - 3;
+    const int64_t rows = (int64_t)plan.N * plan.np, c0 = (int64_t)(kb + 1) * 64;
+    k_oz_panel256<<<dim3((unsigned)cdiv(w, 32), (unsigned)plan.N), 256, kPanelSmem, st>>>(
+        plan.R, plan.ldr, plan.rstride, plan.np, kb0, rows, static_cast<__nv_bfloat16*>(plan.slices), plan.EC);
+    TK_LAUNCH_CHECK();
+    const uint32_t gx = (uint32_t)cdiv(w, OT_M);
+    const OtTiles tl{gx * (gx + 1) / 2 * 4, 1, (uint32_t)plan.N};
+    const OtTri t{1, 0, (int)plan.np, (int)w, plan.rstride, 0, 1.0};
+    k_oz_tc<OZ_S, 4, 32, false><<<ot_grid<OZ_S, 32>(tl), 128 + ot_epi<4>, sizeof(OtSmem<OZ_S, 32>) + 1024, st>>>(
+        plan.mP256, plan.mQ256, plan.EC, plan.EC, w, (int)w, 256, 256, nullptr, plan.R + c0 * (plan.ldr + 1), plan.ldr,
+        nullptr, 0, plan.err, tl, t);
+    TK_LAUNCH_CHECK();
+    return TK_OK;
+  }
   __nv_bfloat16* sl = static_cast<__nv_bfloat16*>(plan.slices);
   k_oz_panel_slice<<<dim3((unsigned)cdiv(w, 32), (unsigned)plan.N), 256, 0, st>>>(plan.R, plan.ldr, plan.rstride,
                                                                                    plan.np, kb, sl, plan.EC);
   TK_LAUNCH_CHECK();
-  const dim3 grid((unsigned)cdiv(w, CS_M), (unsigned)cdiv(w / CS_N, CS_TILES), (unsigned)plan.N);
-  k_oz_syrk<<<grid, 384, sizeof(CsSmem) + 1024, st>>>(plan.mP, plan.mQ, plan.EC, plan.np, kb, plan.R, plan.ldr,
-                                                     plan.rstride, plan.err);
+  const dim3 grid((unsigned)cdiv(rem, CS_M), (unsigned)cdiv(w / CS_N, CS_TILES), (unsigned)plan.N);
+  k_oz_syrk<<<grid, 384, sizeof(CsSmem) + 1024, st>>>(plan.mP, plan.mQ, plan.EC, plan.np, kb, (int)rem, plan.R,
+                                                     plan.ldr, plan.rstride, plan.err);
   TK_LAUNCH_CHECK();
   return TK_OK;
 }
