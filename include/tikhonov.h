@@ -115,7 +115,8 @@ typedef struct {
                              Cholesky trailing updates, and the refinement's r = b - A x and A^T r; FP64:
                              the Gaussian sketch, the Gram matrix and the trailing updates when A has
                              2^16 .. 2^32 elements, and the two products with A of every LSQR step when it
-                             has 2^19 or more.  Costs 32 (MIXED) or 16 (FP64) bytes of workspace per element of
+                             has 2^19 or more; both: the explicit inverse of the factors beyond blocks of
+                             256.  Costs 32 (MIXED) or 16 (FP64) bytes of workspace per element of
                              A for the digit planes; 0 = float64 FMA. */
   const double* x0;       /* [NULL] warm start, device N x n float64 (row i for lambdas[i]; m >= n only):
                              the solve starts from x = x0 instead of 0 and returns the same minimiser of

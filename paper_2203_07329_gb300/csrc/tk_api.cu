@@ -85,8 +85,8 @@ tk_status check_opts(const tk_opts* o) {
 
 // The float64 form with emulate_fp64: whether the solve makes digit planes of A at all.  They pay off
 // for the Gaussian sketch, the Gram matrix and the Cholesky updates (2000 x 64: 25 us to make them, 400
-// us less work on the float64 pipe) and, for larger A, the LSQR products (use_oz); A of more than 2^32 elements keeps the float64 pipe, because the planes
-// take 16 bytes per element.
+// us less work on the float64 pipe) and, for larger A, the LSQR products (use_oz); A of more than 2^32
+// elements keeps the float64 pipe, because the planes take 16 bytes per element.
 bool oz64_wanted(int64_t m, int64_t n) { return m * n >= kOz64MinElems && m * n <= (int64_t(1) << 32); }
 
 tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
