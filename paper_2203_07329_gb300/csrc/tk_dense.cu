@@ -1011,9 +1011,11 @@ tk_status tri_inverse(const double* R, int64_t n, int64_t ldr, int64_t rstride, 
     k_tinv_final<T><<<dim3((unsigned)(bt - k), (unsigned)N, nb), 256, 0, st>>>(M, Mt, np, np * np, k - 1, nt, bt);
     TK_LAUNCH_CHECK();
   }
-  if (work)
+  const int nl = work ? oz_tri_lambdas<T>(np, N, kTriBlock * CB) : 0;
+  for (int l0 = 0; work && l0 < N; l0 += nl)
     for (int64_t h = (int64_t)kTriBlock * CB; h < np; h *= 2)
-      TK_TRY(oz_tri_level<T>(R, ldr, rstride, M, Mt, np, np * np, N, np, (int)h, work, bytes, err, st));
+      TK_TRY(oz_tri_level<T>(R + l0 * rstride, ldr, rstride, M + l0 * np * np, Mt + l0 * np * np, np, np * np,
+                             std::min(nl, N - l0), np, (int)h, work, bytes, err, st));
   return TK_OK;
 }
 template tk_status tri_inverse<float>(const double*, int64_t, int64_t, int64_t, int, float*, float*, void*, size_t, int*,

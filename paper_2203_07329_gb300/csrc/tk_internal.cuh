@@ -313,6 +313,8 @@ template <typename T>
 tk_status oz_lsqr_aw_split(const OzMat& A, const T* W, int64_t ldw, int count, void* Wslices, int* EW, double* partial,
                            int splits, int* err, cudaStream_t st);
 template <typename T>
+int oz_tri_lambdas(int64_t n, int N, int h0);  // lambdas per pass of the levels
+template <typename T>
 tk_status oz_lsqr_atu(const OzMat& A, const T* U, int64_t ldu, int count, void* Uslices, int* EU, double* partial,
                       int splits, int* err, cudaStream_t st);
 // The two products of one LSQR step fused over one read of A's row-exponent digit planes (count <= 32,

@@ -964,11 +964,12 @@ tk_status launch_oz_tc(const OtBig& P, const void* Qs, const int* EQ, int M, int
 // Digit planes (row stride h) and row exponents of the blocks of a level: batch z = (matrix l, pair i),
 // row r: src + l mstride + i pstride + r ld, h values; rows or columns past the matrix (r or k >= n - edge,
 // edge = (2 i + 1) h, where row_edge / col_edge is set) and, with lower, the columns k > r are zero.
+// shift (per matrix n exponents, by the pair's diagonal index): value k counts 2^shift[k] times.
 template <typename T>
 __global__ void __launch_bounds__(256)
     k_oz_block_rows(const T* __restrict__ src, int64_t mstride, int64_t pstride, int64_t ld, int pairs, int h, int n,
-                    int row_edge, int col_edge, int lower, int64_t rows, int planes, int* __restrict__ E,
-                    __nv_bfloat16* __restrict__ out) {
+                    int row_edge, int col_edge, int lower, const int* __restrict__ shift, int64_t rows, int planes,
+                    int* __restrict__ E, __nv_bfloat16* __restrict__ out) {
   __shared__ int sh[8];
   const int z = blockIdx.y, r = blockIdx.x;
   const int left = n - (2 * (z % pairs) + 1) * h;
@@ -979,13 +980,25 @@ __global__ void __launch_bounds__(256)
   if (row_edge && r >= left) K = 0;
   if (K < 0) K = 0;
   bool bad = false;
-  int e = oz_vec_exp<T>(x, nullptr, 0, K, &bad);
+  if (shift) shift += (int64_t)(z / pairs) * n + 2 * (int64_t)(z % pairs) * h;
+  int e = oz_vec_exp<T>(x, shift, 0, K, &bad);
   e = oz_block_exp(e, bad, sh);
   const int64_t row = (int64_t)z * h + r;
   if (threadIdx.x == 0) E[row] = e;
   unsigned* o = reinterpret_cast<unsigned*>(out + row * h);
   for (int k = 2 * threadIdx.x; k < h; k += 2 * blockDim.x)
-    oz_vec_split<T>(x, nullptr, k, K, e, rows * h, planes, o + k / 2);
+    oz_vec_split<T>(x, shift, k, K, e, rows * h, planes, o + k / 2);
+}
+// up[l][k] = the exponent of R_kk, down[l][k] its negative (0 where R_kk is not a positive finite number)
+__global__ void __launch_bounds__(256)
+    k_oz_diag_exp(const double* __restrict__ R, int64_t ldr, int64_t rstride, int n, int* __restrict__ up,
+                  int* __restrict__ down) {
+  const int k = blockIdx.x * 256 + threadIdx.x, l = blockIdx.y;
+  if (k >= n) return;
+  const double d = R[(int64_t)l * rstride + (int64_t)k * (ldr + 1)];
+  const int e = d > 0.0 && d <= 1.7976931348623157e308 ? ilogb(d) : 0;
+  up[(int64_t)l * n + k] = e;
+  down[(int64_t)l * n + k] = -e;
 }
 // M[a + r][a + h + l] = Mt[a + h + l][a + r] for the level's blocks (a = 2 i h): 32 x 32 tiles
 template <typename T>
@@ -2069,7 +2082,9 @@ tk_status oz_lsqr_fused(const OzMat& A, const float* W, int64_t ldw, int count, 
 
 // The level h of M = R^-1 (n a multiple of 64, h of 128): for every pair of diagonal blocks of M that are
 // finished, M12 = -M11 (R12 M22), both products from digits (T = double: 8, float64-accurate; T = float: 4,
-// the 28-bit rounded operands); Mt = M^T receives its block first.
+// the 28-bit rounded operands); Mt = M^T receives its block first.  With R = D U, D its diagonal, M11 is U11^-1
+// D^-1 and R12 M22 has rows of the size of D: in the second product the powers of two of D move from one operand
+// to the other, so that the digits of a row of M11 are not spent on the range of D (small lambda: 1 .. 1e-5).
 template <typename T>
 tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* Mt, int64_t ldm, int64_t mstride, int N,
                        int64_t n, int h, void* work, size_t bytes, int* err, cudaStream_t st) {
@@ -2090,7 +2105,11 @@ tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* M
   int* EP = a.take<int>((size_t)rows);
   int* EQ = a.take<int>((size_t)rows);
   T* Tt = a.take<T>((size_t)rows * h);  // (R12 M22)^T
+  int* up = a.take<int>((size_t)N * n);
+  int* down = a.take<int>((size_t)N * n);
   if (!a.ok()) return TK_ENOMEM;
+  k_oz_diag_exp<<<dim3((unsigned)cdiv(n, 256), (unsigned)N), 256, 0, st>>>(R, ldr, rstride, (int)n, up, down);
+  TK_LAUNCH_CHECK();
   CUtensorMap mP, mQ;
   TK_TRY(make_slice_map(&mP, Ps, rows, h, OT_M, S));
   TK_TRY(make_slice_map(&mQ, Qs, rows, h, NT, S));
@@ -2101,18 +2120,19 @@ tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* M
   const unsigned g = ot_grid<S, NT>(tl);
   const int64_t pr = 2 * (int64_t)h;  // a pair's step along the diagonal
   OtTri t{pairs, 1, h, (int)n, (int64_t)pairs * h * h, (int64_t)h * h, 1.0};
-  k_oz_block_rows<double><<<gs, 256, 0, st>>>(R + h, rstride, pr * (ldr + 1), ldr, pairs, h, (int)n, 0, 1, 0, rows, S,
-                                              EP, Ps);
+  k_oz_block_rows<double><<<gs, 256, 0, st>>>(R + h, rstride, pr * (ldr + 1), ldr, pairs, h, (int)n, 0, 1, 0,
+                                              nullptr, rows, S, EP, Ps);
   TK_LAUNCH_CHECK();
   k_oz_block_rows<T><<<gs, 256, 0, st>>>(Mt + h * (ldm + 1), mstride, pr * (ldm + 1), ldm, pairs, h, (int)n, 1, 1, 1,
-                                         rows, S, EQ, Qs);
+                                         nullptr, rows, S, EQ, Qs);
   TK_LAUNCH_CHECK();
   k_oz_tc<S, 3, NT, false><<<g, 256, smem, st>>>(mP, mQ, EP, EQ, h, h, h, h, nullptr, Tt, h, nullptr, 0, err, tl, t);
   TK_LAUNCH_CHECK();
-  k_oz_block_rows<T><<<gs, 256, 0, st>>>(M, mstride, pr * (ldm + 1), ldm, pairs, h, (int)n, 0, 0, 0, rows, S, EP, Ps);
+  k_oz_block_rows<T><<<gs, 256, 0, st>>>(M, mstride, pr * (ldm + 1), ldm, pairs, h, (int)n, 0, 0, 0, up, rows, S,
+                                         EP, Ps);
   TK_LAUNCH_CHECK();
-  k_oz_block_rows<T><<<gs, 256, 0, st>>>(Tt, (int64_t)pairs * h * h, (int64_t)h * h, h, pairs, h, (int)n, 1, 0, 0, rows,
-                                         S, EQ, Qs);
+  k_oz_block_rows<T><<<gs, 256, 0, st>>>(Tt, (int64_t)pairs * h * h, (int64_t)h * h, h, pairs, h, (int)n, 1, 0, 0, down,
+                                         rows, S, EQ, Qs);
   TK_LAUNCH_CHECK();
   t = OtTri{pairs, 2, h, (int)n, mstride, pr * (ldm + 1), -1.0};
   k_oz_tc<S, 3, NT, false>
@@ -2128,17 +2148,31 @@ template tk_status oz_tri_level<float>(const double*, int64_t, int64_t, float*, 
 template tk_status oz_tri_level<double>(const double*, int64_t, int64_t, double*, double*, int64_t, int64_t, int,
                                         int64_t, int, void*, size_t, int*, cudaStream_t);
 
+// Lambdas per pass of the levels: their planes take 16 to 32 bytes per element of a level, and 2 GiB of them are
+// thousands of tiles already
+template <typename T>
+int oz_tri_lambdas(int64_t n, int N, int h0) {
+  int64_t most = 1;
+  for (int64_t h = h0; h < n; h *= 2)
+    most = std::max(most, cdiv(n - h, 2 * h) * h * h * (int64_t)(4 * oz_digits<T>() + sizeof(T)));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(N, (int64_t(2) << 30) / most));
+}
+template int oz_tri_lambdas<float>(int64_t, int, int);
+template int oz_tri_lambdas<double>(int64_t, int, int);
+
 template <typename T>
 size_t oz_tri_workspace(int64_t n, int N, int h0) {
   size_t most = 0;
   for (int64_t h = h0; h < n; h *= 2) {
-    const size_t rows = (size_t)N * cdiv(n - h, 2 * h) * h;
+    const size_t rows = (size_t)oz_tri_lambdas<T>(n, N, h0) * cdiv(n - h, 2 * h) * h;
     Arena a;
     a.take<__nv_bfloat16>(oz_digits<T>() * rows * h);
     a.take<__nv_bfloat16>(oz_digits<T>() * rows * h);
     a.take<int>(rows);
     a.take<int>(rows);
     a.take<T>(rows * h);
+    a.take<int>((size_t)N * n);
+    a.take<int>((size_t)N * n);
     most = std::max(most, a.used + 256);
   }
   return most;
@@ -2240,9 +2274,18 @@ tk_status oz_gram(const double* Y, int64_t r, int64_t c, double* C, void* work, 
   return TK_OK;
 }
 
+// Lambdas whose panels of 256 rows share a launch: 2 GiB of planes at most
+static int oz_panel_lambdas(int64_t np, int N) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(N, (int64_t(2) << 30) / (np * 256 * OZ_S * 2)));
+}
+// values of a digit plane: of the block rows' planes of 64, or of the panels' of 256
+static size_t oz_chol_plane(int64_t np, int N) {
+  return (size_t)np * std::max(N * 64, np > 256 ? oz_panel_lambdas(np, N) * 256 : 0);
+}
+
 size_t oz_chol_workspace(int64_t np, int N) {
   Arena a;
-  a.take<__nv_bfloat16>((size_t)N * OZ_S * np * (np > 256 ? 256 : 64));
+  a.take<__nv_bfloat16>(OZ_S * oz_chol_plane(np, N));
   a.take<int>((size_t)N * np);
   return a.used + 256;
 }
@@ -2257,7 +2300,7 @@ tk_status oz_chol_begin(double* R, int64_t ldr, int64_t rstride, int N, int64_t 
   a.base = static_cast<char*>(work);
   a.cap = bytes;
   const size_t sb = sizeof(__nv_bfloat16) * (size_t)N * OZ_S * np * 64;
-  plan->slices = a.take<__nv_bfloat16>((size_t)N * OZ_S * np * (np > 256 ? 256 : 64));
+  plan->slices = a.take<__nv_bfloat16>(OZ_S * oz_chol_plane(np, N));
   plan->EC = a.take<int>((size_t)N * np);
   if (!a.ok()) return TK_ENOMEM;
   plan->R = R;
@@ -2287,8 +2330,8 @@ tk_status oz_chol_begin(double* R, int64_t ldr, int64_t rstride, int N, int64_t 
   TK_CUDA(cudaFuncSetAttribute(k_oz_syrk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(CsSmem) + 1024)));
   if (np > 256) {
     // the same memory, as the planes of a panel of 256 rows
-    const int64_t rows = (int64_t)N * np;
-    if (rows > INT32_MAX - 2 * OT_M || (double)N * np * np > 2e9 * OT_M * OT_N) {
+    const int64_t rows = (int64_t)oz_panel_lambdas(np, N) * np;
+    if (rows > INT32_MAX - 2 * OT_M || (double)rows * np > 2e9 * OT_M * OT_N) {
       set_error_msg("emulated Cholesky: unsupported order or lambda count");
       return TK_EINVAL;
     }
@@ -2312,18 +2355,22 @@ tk_status oz_chol_step(const OzCholPlan& plan, int kb, cudaStream_t st) {
   if (w <= 0) return TK_OK;
   const int64_t rem = std::min<int64_t>(w, (3 - kb % 4) * 64);
   if (rem == 0) {
-    const int kb0 = kb - 3;
-    const int64_t rows = (int64_t)plan.N * plan.np, c0 = (int64_t)(kb + 1) * 64;
-    k_oz_panel256<<<dim3((unsigned)cdiv(w, 32), (unsigned)plan.N), 256, kPanelSmem, st>>>(
-        plan.R, plan.ldr, plan.rstride, plan.np, kb0, rows, static_cast<__nv_bfloat16*>(plan.slices), plan.EC);
-    TK_LAUNCH_CHECK();
+    const int kb0 = kb - 3, nl = oz_panel_lambdas(plan.np, plan.N);
+    const int64_t rows = (int64_t)nl * plan.np, c0 = (int64_t)(kb + 1) * 64;
     const uint32_t gx = (uint32_t)cdiv(w, OT_M);
-    const OtTiles tl{gx * (gx + 1) / 2 * 4, 1, (uint32_t)plan.N};
     const OtTri t{1, 0, (int)plan.np, (int)w, plan.rstride, 0, 1.0};
-    k_oz_tc<OZ_S, 4, 32, false><<<ot_grid<OZ_S, 32>(tl), 128 + ot_epi<4>, sizeof(OtSmem<OZ_S, 32>) + 1024, st>>>(
-        plan.mP256, plan.mQ256, plan.EC, plan.EC, w, (int)w, 256, 256, nullptr, plan.R + c0 * (plan.ldr + 1), plan.ldr,
-        nullptr, 0, plan.err, tl, t);
-    TK_LAUNCH_CHECK();
+    for (int l0 = 0; l0 < plan.N; l0 += nl) {
+      const int cnt = std::min(nl, plan.N - l0);
+      double* Rl = plan.R + (int64_t)l0 * plan.rstride;
+      k_oz_panel256<<<dim3((unsigned)cdiv(w, 32), (unsigned)cnt), 256, kPanelSmem, st>>>(
+          Rl, plan.ldr, plan.rstride, plan.np, kb0, rows, static_cast<__nv_bfloat16*>(plan.slices), plan.EC);
+      TK_LAUNCH_CHECK();
+      const OtTiles tl{gx * (gx + 1) / 2 * 4, 1, (uint32_t)cnt};
+      k_oz_tc<OZ_S, 4, 32, false><<<ot_grid<OZ_S, 32>(tl), 128 + ot_epi<4>, sizeof(OtSmem<OZ_S, 32>) + 1024, st>>>(
+          plan.mP256, plan.mQ256, plan.EC, plan.EC, w, (int)w, 256, 256, nullptr, Rl + c0 * (plan.ldr + 1), plan.ldr,
+          nullptr, 0, plan.err, tl, t);
+      TK_LAUNCH_CHECK();
+    }
     return TK_OK;
   }
   __nv_bfloat16* sl = static_cast<__nv_bfloat16*>(plan.slices);

@@ -27,3 +27,25 @@ def test_panel_updates_have_float64_backward_error(n, N):
         err = ((R[i].T @ R[i] - want).abs() / (d[:, None] * d[None, :])).max().item()
         assert err < 4 * (n + 1) * 2.0 ** -53, err
         assert torch.tril(R[i], -1).abs().max().item() == 0.0
+
+
+# More lambdas than the planes of one pass hold (2 GiB: 1638 of order 320): the factors on both sides of the
+# border, same bound; and their inverses, which precondition neighbouring lambdas alike (iterations within 2).
+def test_more_lambdas_than_one_pass():
+    n, N, m = 270, 1650, 600
+    gen = torch.Generator().manual_seed(1)
+    A = torch.randn(m, n, dtype=torch.float64, generator=gen).cuda()
+    b = torch.randn(m, dtype=torch.float64, generator=gen).cuda()
+    C = A.T @ A
+    lams = torch.logspace(-3, 1, N, dtype=torch.float64).numpy()
+    eye = torch.eye(n, dtype=torch.float64, device="cuda")
+    R, brk = tk.tk_cholesky_shifted(C, lams, emulate=True)
+    assert brk == [0] * N
+    for i in (0, 1637, 1638, N - 1):
+        want = C + lams[i] * eye
+        d = want.diagonal().sqrt()
+        err = ((R[i].T @ R[i] - want).abs() / (d[:, None] * d[None, :])).max().item()
+        assert err < 4 * (n + 1) * 2.0 ** -53, (i, err)
+    r = tk.tk_solve(A, b, lams, tk.opts_default(precision=tk.TK_PREC_MIXED, sketch=tk.TK_SKETCH_GAUSS, s=m,
+                                                max_refine=1))
+    assert abs(r.info[1637]["iters"] - r.info[1638]["iters"]) <= 2

@@ -106,3 +106,19 @@ def test_lowrank_apply_shapes(m, n, s, N):
         e = float((r1.X[i] - r0.X[i]).norm() / r0.X[i].norm())
         assert e < 1e-10, (lams[i], e)
         assert r1.info[i]["status"] == 0
+
+
+# A spectrum down to 1e-8 and lambda down to 1e-10 (1e-12): the factors' diagonals span five (six) decades, and
+# the explicit inverse must precondition as the one from the SIMT pipes does (equal iterations up to rounding)
+@pytest.mark.parametrize("mixed,n,lo", [(True, 700, 1e-10), (True, 1500, 1e-10), (False, 1100, 1e-12)])
+def test_digit_inverse_of_small_lambdas(mixed, n, lo):
+    m, N = 6 * n, 6
+    p = datagen.make_ridge_problem(m, n, datagen.spectrum("log", n, hi=1.0, lo=1e-8),
+                                   datagen.log_lambdas(N, lo, 1e-2), seed=n)
+    A, b, lams = p.A.cuda(), p.b.cuda(), p.lambdas.numpy()
+    kw = dict(sketch=tk.TK_SKETCH_GAUSS, s=3 * n, precision=tk.TK_PREC_MIXED if mixed else tk.TK_PREC_FP64)
+    r1 = _solve(A, b, lams, **kw)
+    r0 = _solve(A, b, lams, lsqr_tc=0, emulate_fp64=0, **kw)
+    for i in range(N):
+        assert r1.info[i]["status"] == r0.info[i]["status"], lams[i]
+        assert r1.info[i]["iters"] <= 1.2 * r0.info[i]["iters"] + 3, (lams[i], r1.info[i], r0.info[i])
