@@ -1514,10 +1514,17 @@ TK_API tk_status tk_sketch_draw_sparse(uint64_t seed, int64_t L, int64_t s, int3
   return TK_OK;
 }
 
+// The sketch on its own: on the float64 pipe, because no digit planes of A exist here to form it from.
+static tk_status sketch_plan(const tk_problem* p, const tk_opts* o, Plan& P) {
+  TK_TRY(make_plan(p, 1, o, P));
+  P.oz64 = false;
+  return TK_OK;
+}
+
 TK_API tk_status tk_sketch_apply_workspace(const tk_problem* p, const tk_opts* o, size_t* bytes) {
   if (!bytes) return einval("bytes pointer is NULL");
   Plan P;
-  TK_TRY(make_plan(p, 1, o, P));
+  TK_TRY(sketch_plan(p, o, P));
   Arena a;
   if (P.under) {
     a.take<char>((size_t)P.m * P.n * (P.dt == TK_F64 ? 8 : 4));
@@ -1531,7 +1538,7 @@ TK_API tk_status tk_sketch_apply_workspace(const tk_problem* p, const tk_opts* o
 TK_API tk_status tk_sketch_apply(const tk_problem* p, const tk_opts* o, double* Y, void* work, size_t work_bytes,
                                  void* stream) {
   Plan P;
-  TK_TRY(make_plan(p, 1, o, P));
+  TK_TRY(sketch_plan(p, o, P));
   if (P.mixed && !tc_sketch(P)) return einval("tk_sketch_apply: MIXED selects the tensor-core Gaussian sketch only");
   if (!p->A || !Y) return einval("A and Y must be non-NULL");
   size_t need = 0;

@@ -1,0 +1,36 @@
+"""Host-only checks (no GPU): the workspace queries of calls whose workspace the digit planes dominate stay within
+what the header states for them, so that what fits the GPU as float64 data fits it as a solve."""
+import ctypes as C
+
+import pytest
+
+GIB = float(1 << 30)
+
+
+@pytest.fixture(scope="module")
+def tk():
+    from paper_2203_07329_gb300 import build
+    build.build()
+    from paper_2203_07329_gb300 import tikhonov
+    tikhonov.lib()
+    return tikhonov
+
+
+def _prob(tk, m, n, dtype=None):
+    # fake non-null device addresses: the queries do not touch them
+    return tk.tk_problem(m, n, n, tk.TK_F64 if dtype is None else dtype, 0x1000, 0x2000)
+
+
+def _size(tk, m, n, N, dtype=None, **kw):
+    return tk.workspace_size(_prob(tk, m, n, dtype), N, tk.opts_default(**kw))
+
+
+# tk_sketch_apply forms the float64 Gaussian sketch on the float64 pipe at every size: it has no digit planes of A
+# to read, and its scratch is the embedding (8 s L bytes) and split planes of the small result
+@pytest.mark.parametrize("m,n,s", [(1 << 17, 64, 256), (64, 1 << 17, 256)])
+def test_sketch_apply_has_no_digit_planes(tk, m, n, s):
+    out = C.c_size_t(0)
+    o = tk.opts_default(sketch=tk.TK_SKETCH_GAUSS, s=s)
+    assert tk.lib().tk_sketch_apply_workspace(C.byref(_prob(tk, m, n)), C.byref(o), C.byref(out)) == tk.TK_OK
+    L = max(m, n)
+    assert out.value <= 8 * s * L + 8 * m * n + (64 << 20)
