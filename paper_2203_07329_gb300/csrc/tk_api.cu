@@ -211,8 +211,11 @@ OzMat oz_mat(const Plan& P, const Bufs& B) {
 // otherwise: 462 x 30000 x 1000 takes 31 ms there, 1.6 ms from digits).
 bool oz_gauss(const Plan& P) { return P.oz64 && P.o.sketch == TK_SKETCH_GAUSS && P.s <= 65535; }
 
-size_t sketch_scratch(const Plan& P) {
-  tk_dtype dt = P.mixed ? TK_F32 : P.dt;
+// The type of the copy of A that a solve sketches: float32 in the mixed form, else float64 (float32 data is
+// widened first).
+tk_dtype sketch_dtype(const Plan& P) { return P.mixed ? TK_F32 : TK_F64; }
+
+size_t sketch_scratch(const Plan& P, tk_dtype dt) {
   if (oz_gauss(P)) {
     Arena a;
     a.take<double>((size_t)P.s * P.L);
@@ -241,7 +244,7 @@ void carve(const Plan& P, Arena& a, Arena& t, Bufs& B) {
   B.info = a.take<int>(N);
   B.ones = a.take<double>(N);
   B.Y = ty.take<double>((size_t)P.s * P.c);
-  if (P.under) B.AT = t.take<char>((size_t)P.m * P.n * (P.dt == TK_F64 ? 8 : 4));
+  if (P.under) B.AT = t.take<char>((size_t)P.m * P.n * (sketch_dtype(P) == TK_F64 ? 8 : 4));
   if (P.mixed && P.dt == TK_F64) B.A32 = a.take<float>((size_t)P.m * P.n);
   if (P.lsqr_tc) B.AT32 = a.take<float>((size_t)P.m * P.n);
   if (!P.mixed && P.dt == TK_F32) B.A64 = a.take<double>((size_t)P.m * P.n);
@@ -306,7 +309,7 @@ void carve(const Plan& P, Arena& a, Arena& t, Bufs& B) {
     B.nrm = a.take<double>((size_t)3 * N);
   }
   // the sketch's scratch is free again when the Gram matrix (or the BP2 factorization) is formed
-  size_t sc = std::max(sketch_scratch(P), P.lowrank ? size_t(0) : gram_scratch_bytes(P.s, P.c));
+  size_t sc = std::max(sketch_scratch(P, sketch_dtype(P)), P.lowrank ? size_t(0) : gram_scratch_bytes(P.s, P.c));
   if (P.qr) sc = std::max(sc, bp2_workspace(P.s, P.c, N));
   // and the inverse of the factors, after them
   if (digit_inverse(P))
@@ -1530,7 +1533,7 @@ TK_API tk_status tk_sketch_apply_workspace(const tk_problem* p, const tk_opts* o
     a.take<char>((size_t)P.m * P.n * (P.dt == TK_F64 ? 8 : 4));
     a.take<double>((size_t)P.s * P.c);
   }
-  a.take<char>(sketch_scratch(P));
+  a.take<char>(sketch_scratch(P, P.mixed ? TK_F32 : P.dt));
   *bytes = a.used + 4096;
   return TK_OK;
 }
@@ -1558,7 +1561,7 @@ TK_API tk_status tk_sketch_apply(const tk_problem* p, const tk_opts* o, double* 
   } else {
     B.Y = Y;
   }
-  B.scratch_bytes = sketch_scratch(P);
+  B.scratch_bytes = sketch_scratch(P, P.mixed ? TK_F32 : P.dt);
   B.scratch = a.take<char>(B.scratch_bytes);
   if (!a.ok()) return TK_ENOMEM;
   TK_TRY(do_sketch(P, p->A, P.dt, P.lda, B, st));

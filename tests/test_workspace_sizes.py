@@ -34,3 +34,12 @@ def test_sketch_apply_has_no_digit_planes(tk, m, n, s):
     assert tk.lib().tk_sketch_apply_workspace(C.byref(_prob(tk, m, n)), C.byref(o), C.byref(out)) == tk.TK_OK
     L = max(m, n)
     assert out.value <= 8 * s * L + 8 * m * n + (64 << 20)
+
+
+# the float64 form widens float32 data first: the solve needs everything the same solve of float64 data needs
+# (its sketch's and its transpose's buffers hold float64) and the widened copy
+@pytest.mark.parametrize("sketch", [0, 1, 2, 3])
+@pytest.mark.parametrize("m,n", [(65536, 1024), (4096, 60), (300, 1), (300, 20000), (20, 500)])
+def test_float64_form_of_float32_data(tk, m, n, sketch):
+    kw = dict(sketch=sketch, s=4 * min(m, n))
+    assert _size(tk, m, n, 3, tk.TK_F32, **kw) >= _size(tk, m, n, 3, **kw) + 8 * m * n
