@@ -77,19 +77,12 @@ __device__ __forceinline__ bool jac_angle(double a, double b, double g, double t
   return true;
 }
 
-// The pairs (A, B) and (C, D) of the four rows x[][] held by the block (thread t: values t, t + TH, ..).
-template <int NE, int TH, int A, int B, int C, int D>
-__device__ __forceinline__ void jac_two_pairs(double (&x)[4][NE], int ne, double tol, JacSmem& S, int* nrot) {
+// The angles of the pairs (A, B) and (C, D) of a block's four rows from the threads' parts g0, g1 of their dot
+// products: rotations and flags in S, the norms updated, rotations counted by lanes 0 and 16 of warp 0.
+template <int TH, int A, int B, int C, int D>
+__device__ __forceinline__ void jac_two_angles(double g0, double g1, double tol, JacSmem& S, int* nrot) {
   constexpr int NW = TH / 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  double g0 = 0.0, g1 = 0.0;
-#pragma unroll
-  for (int e = 0; e < NE; ++e) {
-    if (e < ne) {
-      g0 = fma(x[A][e], x[B][e], g0);
-      g1 = fma(x[C][e], x[D][e], g1);
-    }
-  }
   // lanes 0-15 sum g0, lanes 16-31 g1: one exchange, then four steps for both
   const bool up = lane >= 16;
   double v = (up ? g1 : g0) + __shfl_xor_sync(0xffffffffu, up ? g0 : g1, 16);
@@ -118,6 +111,20 @@ __device__ __forceinline__ void jac_two_pairs(double (&x)[4][NE], int ne, double
     }
   }
   __syncthreads();
+}
+
+// The pairs (A, B) and (C, D) of the four rows x[][] held by the block (thread t: values t, t + TH, ..).
+template <int NE, int TH, int A, int B, int C, int D>
+__device__ __forceinline__ void jac_two_pairs(double (&x)[4][NE], int ne, double tol, JacSmem& S, int* nrot) {
+  double g0 = 0.0, g1 = 0.0;
+#pragma unroll
+  for (int e = 0; e < NE; ++e) {
+    if (e < ne) {
+      g0 = fma(x[A][e], x[B][e], g0);
+      g1 = fma(x[C][e], x[D][e], g1);
+    }
+  }
+  jac_two_angles<TH, A, B, C, D>(g0, g1, tol, S, nrot);
   if (S.rot[0]) {
     const double c = S.cs[0], s = S.sn[0];
 #pragma unroll
@@ -140,6 +147,35 @@ __device__ __forceinline__ void jac_two_pairs(double (&x)[4][NE], int ne, double
       }
     }
   }
+}
+
+// The same for rows that stay in memory (x[i]: row i, null if absent): every thread reads and writes its own
+// values t, t + TH, .. throughout.
+template <int TH>
+__device__ __forceinline__ double jac_dot_mem(const double* x, const double* y, int64_t n) {
+  double g = 0.0;
+  if (x && y) {
+#pragma unroll 4
+    for (int64_t j = threadIdx.x; j < n; j += TH) g = fma(x[j], y[j], g);
+  }
+  return g;
+}
+template <int TH>
+__device__ __forceinline__ void jac_rotate_mem(double* x, double* y, int64_t n, double c, double s) {
+#pragma unroll 4
+  for (int64_t j = threadIdx.x; j < n; j += TH) {
+    const double u = x[j], v = y[j];
+    x[j] = c * u - s * v;
+    y[j] = s * u + c * v;
+  }
+}
+template <int TH, int A, int B, int C, int D>
+__device__ __forceinline__ void jac_two_pairs_mem(double* const (&x)[4], int64_t n, double tol, JacSmem& S,
+                                                  int* nrot) {
+  const double g0 = jac_dot_mem<TH>(x[A], x[B], n), g1 = jac_dot_mem<TH>(x[C], x[D], n);
+  jac_two_angles<TH, A, B, C, D>(g0, g1, tol, S, nrot);
+  if (S.rot[0]) jac_rotate_mem<TH>(x[A], x[B], n, S.cs[0], S.sn[0]);  // (an absent row has norm 0: no rotation)
+  if (S.rot[1]) jac_rotate_mem<TH>(x[C], x[D], n, S.cs[1], S.sn[1]);
 }
 
 // Block pair k of a round: rows 2p, 2p + 1 and 2q, 2q + 1 of W (rows >= s: absent, norm 0).  first:
@@ -182,6 +218,29 @@ __device__ __forceinline__ void jac_block_pair(double* __restrict__ W, double* _
   if (threadIdx.x < 4 && r[threadIdx.x] < s) nrm2[r[threadIdx.x]] = S.nr[threadIdx.x];
 }
 
+// The same with the rows in memory, for any n.
+template <int TH>
+__device__ __forceinline__ void jac_block_pair_mem(double* __restrict__ W, double* __restrict__ nrm2, int64_t s,
+                                                   int64_t n, int64_t sp, int64_t round, int64_t k, double tol,
+                                                   int* __restrict__ rotated, JacSmem& S) {
+  int64_t p, q;
+  circle_pair(sp, round, k, &p, &q);
+  const bool first = round == 0;
+  const int64_t r[4] = {2 * p, 2 * p + 1, 2 * q, 2 * q + 1};
+  if (!first && r[2] >= s) return;  // pair with the dummy block
+  double* x[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = r[i] < s ? W + r[i] * n : nullptr;
+  if (threadIdx.x < 4) S.nr[threadIdx.x] = r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0;
+  __syncthreads();
+  int nrot = 0;
+  if (first) jac_two_pairs_mem<TH, 0, 1, 2, 3>(x, n, tol, S, &nrot);
+  jac_two_pairs_mem<TH, 0, 2, 1, 3>(x, n, tol, S, &nrot);
+  jac_two_pairs_mem<TH, 0, 3, 1, 2>(x, n, tol, S, &nrot);
+  if (nrot) atomicAdd(rotated, nrot);
+  if (threadIdx.x < 4 && r[threadIdx.x] < s) nrm2[r[threadIdx.x]] = S.nr[threadIdx.x];
+}
+
 // One round of every matrix: CTA = (matrix, block pair).
 struct SvdDesc {
   double* W;
@@ -201,6 +260,15 @@ __global__ void __launch_bounds__(TH)
   const SvdDesc& d = D[t.job];
   if (d.done || round >= d.sp - 1) return;
   jac_block_pair<NE, TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, d.rotated, S);
+}
+template <int TH>
+__global__ void __launch_bounds__(TH)
+    k_jacobi_round_mem(const SvdDesc* __restrict__ D, const SvdTile* __restrict__ tl, int64_t round, double tol) {
+  __shared__ JacSmem S;
+  const SvdTile t = tl[blockIdx.x];
+  const SvdDesc& d = D[t.job];
+  if (d.done || round >= d.sp - 1) return;
+  jac_block_pair_mem<TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, d.rotated, S);
 }
 
 // Squared row norms at the start of a sweep (a warp to each of the block pair's four rows).
@@ -448,15 +516,16 @@ tk_status svd_start(const double* Y, int64_t s, int64_t n, const SvdBufs& B, cud
   return gemm<double, double, double>(false, false, s, n, s, B.Q, s, Y, n, B.W, n, 1.0, nullptr, nullptr, 0, st);
 }
 
-// Registers hold 4 rows of a block pair: NE values per thread and row; n <= 8192 (the largest short
-// dimension).
+// Registers hold 4 rows of a block pair: NE values per thread and row, up to 16 x 512 = 8192 (the largest short
+// dimension of a solve).  Longer rows (the SVD called on its own) stay in memory.
 tk_status launch_round(int64_t max_n, unsigned tiles, const SvdDesc* dd, const SvdTile* dt, int64_t round, double tol,
                        cudaStream_t st) {
   if (max_n <= 512) k_jacobi_round<4, 128><<<tiles, 128, 0, st>>>(dd, dt, round, tol);
   else if (max_n <= 1024) k_jacobi_round<8, 128><<<tiles, 128, 0, st>>>(dd, dt, round, tol);
   else if (max_n <= 2048) k_jacobi_round<16, 128><<<tiles, 128, 0, st>>>(dd, dt, round, tol);
   else if (max_n <= 4096) k_jacobi_round<16, 256><<<tiles, 256, 0, st>>>(dd, dt, round, tol);
-  else k_jacobi_round<16, 512><<<tiles, 512, 0, st>>>(dd, dt, round, tol);
+  else if (max_n <= 8192) k_jacobi_round<16, 512><<<tiles, 512, 0, st>>>(dd, dt, round, tol);
+  else k_jacobi_round_mem<512><<<tiles, 512, 0, st>>>(dd, dt, round, tol);
   TK_LAUNCH_CHECK();
   return TK_OK;
 }

@@ -1,0 +1,32 @@
+"""The SVD of the sketch at the ends of its range: rows longer than the registers of a block pair hold."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2203_07329_gb300 import tikhonov as tk
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(Y, max_sweeps):
+    s, n = Y.shape
+    sig, V, sweeps = tk.tk_sketch_svd(torch.from_numpy(Y).cuda())
+    sig, V = sig.cpu().numpy(), V.cpu().numpy()
+    ref = np.linalg.svd(Y, compute_uv=False)
+    # the normwise error of an orthogonal transformation, as for the other shapes of this call
+    u = 2.0 ** -53 * ref[0] * np.sqrt(s * n)
+    assert np.max(np.abs(sig - ref)) <= 8 * u
+    live = sig > 1e3 * u
+    G = V[:, live].T @ V[:, live]
+    assert np.max(np.abs(G - np.eye(G.shape[0]))) < 1e-13 * max(1.0, np.sqrt(s))
+    B = (Y / ref[0]) @ V[:, live]
+    assert np.max(np.abs(np.linalg.norm(B, axis=0) - sig[live] / ref[0])) <= 16 * u / ref[0]
+    assert sweeps < max_sweeps
+
+
+# 8192 values are the most that a block pair holds in registers; rows beyond are rotated in memory.  3, 5: fewer
+# rows than two blocks; 66 and 70: from the orthogonal start, an odd and an even number of blocks
+@pytest.mark.parametrize("s,n", [(3, 8192), (5, 8193), (70, 8192), (66, 8193), (6, 20001), (67, 20011)])
+def test_long_rows(s, n):
+    gen = np.random.default_rng(s + n)
+    _check(gen.standard_normal((s, n)) * np.exp(-np.arange(n) / (n / 6.0)), 30)
