@@ -464,8 +464,9 @@ struct SvdBufs {
   SvdDesc* desc;
   SvdTile* tiles;
 };
-// Small matrices start from Y itself: their sweeps are a few dozen launches.
-constexpr int64_t kSvdStartMin = 64;
+// Small matrices start from Y itself: their sweeps are a few dozen launches.  So do those of which not one row of
+// s values fits in the shared memory of the panels' Gram-Schmidt.
+bool svd_orthogonal_start(int64_t s) { return s >= 64 && s <= (int64_t)(kGsSmemCap / sizeof(double)); }
 int64_t block_players(int64_t s) {
   const int64_t nb = cdiv(s, 2);
   return nb + (nb & 1);
@@ -481,16 +482,16 @@ void svd_carve(Arena& a, int64_t s, int64_t n, SvdBufs& B) {
   B.rotated = a.take<int>(1);
   B.desc = a.take<SvdDesc>(1);
   B.tiles = a.take<SvdTile>((size_t)svd_tile_count(s));
-  if (s >= kSvdStartMin) {
+  if (svd_orthogonal_start(s)) {
     B.C = a.take<double>((size_t)s * s);
     B.Q = a.take<double>((size_t)s * s);
     B.H = a.take<double>((size_t)kGsPanel * s);
   }
 }
 
-// W = Q Y (or a copy of Y for few rows).
+// W = Q Y (or a copy of Y).
 tk_status svd_start(const double* Y, int64_t s, int64_t n, const SvdBufs& B, cudaStream_t st) {
-  if (s < kSvdStartMin) {
+  if (!svd_orthogonal_start(s)) {
     TK_CUDA(cudaMemcpyAsync(B.W, Y, sizeof(double) * (size_t)s * n, cudaMemcpyDeviceToDevice, st));
     return TK_OK;
   }

@@ -30,3 +30,15 @@ def _check(Y, max_sweeps):
 def test_long_rows(s, n):
     gen = np.random.default_rng(s + n)
     _check(gen.standard_normal((s, n)) * np.exp(-np.arange(n) / (n / 6.0)), 30)
+
+
+# more rows than the orthogonal start takes (no row of s values fits in shared memory): rows that are orthogonal from
+# the start, so that one sweep ends it
+def test_more_rows_than_the_orthogonal_start_takes():
+    s = 25602
+    d = torch.exp(-torch.arange(s, dtype=torch.float64) / 3000.0)
+    sig, V, sweeps = tk.tk_sketch_svd(torch.diag(d).cuda())
+    assert sweeps == 1
+    assert float((sig.cpu() - d).abs().max()) <= 2.0 ** -50
+    V -= torch.eye(s, dtype=torch.float64, device="cuda")
+    assert float(V.abs().max()) <= 2.0 ** -50

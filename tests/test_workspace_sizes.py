@@ -43,3 +43,12 @@ def test_sketch_apply_has_no_digit_planes(tk, m, n, s):
 def test_float64_form_of_float32_data(tk, m, n, sketch):
     kw = dict(sketch=sketch, s=4 * min(m, n))
     assert _size(tk, m, n, 3, tk.TK_F32, **kw) >= _size(tk, m, n, 3, **kw) + 8 * m * n
+
+
+# the SVD of the sketch from as many rows as any: no more than Y itself and the orthogonal start (two s x s matrices),
+# which needs a row of s values in shared memory and is left out where none fits (s > 25600)
+@pytest.mark.parametrize("s,n", [(25600, 25600), (25601, 25601), (60000, 60001)])
+def test_svd_of_many_rows(tk, s, n):
+    w = tk.lib().tk_sketch_svd_workspace(s, n)
+    most = 8 * s * n + (16 * s * s if s <= 25600 else 0)
+    assert 8 * s * n < w <= most + 8 * 32 * s + (1 << 20)
