@@ -53,11 +53,13 @@ struct JacSmem {
 };
 
 // Rotation that makes rows of squared norms a, b and dot product g orthogonal (rows already orthogonal
-// to tol: false).  t = tan of the angle in float32 from the scaled ratio zeta = (b - a) / (2 g): off by
-// 1e-7 relative it leaves 1e-7 of g for the next sweep; the norms' update a - t g is exact to second
-// order in that.  cos = (1 + t^2)^(-1/2) by two Newton steps from the float32 value.
+// to tol, or one of them zero: false).  t = tan of the angle in float32 from the scaled ratio zeta =
+// (b - a) / (2 g): off by 1e-7 relative it leaves 1e-7 of g for the next sweep; the norms' update a - t g is
+// exact to second order in that.  Where the ratio leaves float32 (a row of nothing but rounding errors
+// against a full one) t = 1 / (2 zeta) in float64: a t lost to zero would rotate the pair in every sweep.
+// cos = (1 + t^2)^(-1/2) by two Newton steps from the float32 value.
 __device__ __forceinline__ bool jac_angle(double a, double b, double g, double tol, double* c, double* s, double* t) {
-  if (a == 0.0 || b == 0.0) return false;
+  if (!(a > 0.0) || !(b > 0.0)) return false;
   if (!(g * g > tol * tol * (a * b))) return false;
   const double d1 = b - a, d2 = 2.0 * g;
   // both scaled by the power of two that brings the larger to [1, 2): float32 then holds their ratio
@@ -68,6 +70,7 @@ __device__ __forceinline__ bool jac_angle(double a, double b, double g, double t
   const float z = f1 / f2, az = fabsf(z);
   const float ta = az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(fmaf(az, az, 1.0f)));
   *t = (double)((f1 >= 0.0f) == (f2 >= 0.0f) ? ta : -ta);
+  if (az > 1e30f) *t = g / d1;
   const double x = fma(*t, *t, 1.0);
   double r = (double)rsqrtf((float)x);
   r = r * fma(-0.5 * x * r, r, 1.5);
@@ -178,11 +181,16 @@ __device__ __forceinline__ void jac_two_pairs_mem(double* const (&x)[4], int64_t
   if (S.rot[1]) jac_rotate_mem<TH>(x[C], x[D], n, S.cs[1], S.sn[1]);
 }
 
+// A row of less than 2^-106 = (2^-53)^2 of the largest norm counts as zero: it is what rounding left of a row that
+// depends on others, and each sweep would rotate the rounding errors of the sweep before (16 rows with 6 nonzero
+// columns: the cap of 80 sweeps, now 19).
+__device__ __forceinline__ double jac_norm2(double nrm2, double top) { return nrm2 > top * 0x1p-212 ? nrm2 : 0.0; }
+
 // Block pair k of a round: rows 2p, 2p + 1 and 2q, 2q + 1 of W (rows >= s: absent, norm 0).  first:
 // also the pairs inside the two blocks (once a sweep).
 template <int NE, int TH>
 __device__ __forceinline__ void jac_block_pair(double* __restrict__ W, double* __restrict__ nrm2, int64_t s,
-                                               int64_t n, int64_t sp, int64_t round, int64_t k, double tol,
+                                               int64_t n, int64_t sp, int64_t round, int64_t k, double tol, double top,
                                                int* __restrict__ rotated, JacSmem& S) {
   int64_t p, q;
   circle_pair(sp, round, k, &p, &q);
@@ -198,7 +206,7 @@ __device__ __forceinline__ void jac_block_pair(double* __restrict__ W, double* _
       const int64_t j = threadIdx.x + (int64_t)TH * e;
       x[i][e] = (r[i] < s && j < n) ? W[r[i] * n + j] : 0.0;
     }
-  if (threadIdx.x < 4) S.nr[threadIdx.x] = r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0;
+  if (threadIdx.x < 4) S.nr[threadIdx.x] = jac_norm2(r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0, top);
   __syncthreads();
   int nrot = 0;
   if (first) jac_two_pairs<NE, TH, 0, 1, 2, 3>(x, ne, tol, S, &nrot);
@@ -222,7 +230,7 @@ __device__ __forceinline__ void jac_block_pair(double* __restrict__ W, double* _
 template <int TH>
 __device__ __forceinline__ void jac_block_pair_mem(double* __restrict__ W, double* __restrict__ nrm2, int64_t s,
                                                    int64_t n, int64_t sp, int64_t round, int64_t k, double tol,
-                                                   int* __restrict__ rotated, JacSmem& S) {
+                                                   double top, int* __restrict__ rotated, JacSmem& S) {
   int64_t p, q;
   circle_pair(sp, round, k, &p, &q);
   const bool first = round == 0;
@@ -231,7 +239,7 @@ __device__ __forceinline__ void jac_block_pair_mem(double* __restrict__ W, doubl
   double* x[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) x[i] = r[i] < s ? W + r[i] * n : nullptr;
-  if (threadIdx.x < 4) S.nr[threadIdx.x] = r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0;
+  if (threadIdx.x < 4) S.nr[threadIdx.x] = jac_norm2(r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0, top);
   __syncthreads();
   int nrot = 0;
   if (first) jac_two_pairs_mem<TH, 0, 1, 2, 3>(x, n, tol, S, &nrot);
@@ -246,6 +254,7 @@ struct SvdDesc {
   double* W;
   double* nrm2;
   int64_t s, n, sp;  // sp: blocks of two rows, rounded up to an even count
+  double* top;       // the largest squared row norm so far (zero before the first sweep)
   int* rotated;
   int done;
 };
@@ -259,7 +268,7 @@ __global__ void __launch_bounds__(TH)
   const SvdTile t = tl[blockIdx.x];
   const SvdDesc& d = D[t.job];
   if (d.done || round >= d.sp - 1) return;
-  jac_block_pair<NE, TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, d.rotated, S);
+  jac_block_pair<NE, TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, *d.top, d.rotated, S);
 }
 template <int TH>
 __global__ void __launch_bounds__(TH)
@@ -268,7 +277,7 @@ __global__ void __launch_bounds__(TH)
   const SvdTile t = tl[blockIdx.x];
   const SvdDesc& d = D[t.job];
   if (d.done || round >= d.sp - 1) return;
-  jac_block_pair_mem<TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, d.rotated, S);
+  jac_block_pair_mem<TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, *d.top, d.rotated, S);
 }
 
 // Squared row norms at the start of a sweep (a warp to each of the block pair's four rows).
@@ -283,7 +292,11 @@ __global__ void __launch_bounds__(128) k_jacobi_norms(const SvdDesc* __restrict_
 #pragma unroll 4
   for (int64_t i = lane; i < d.n; i += 32) a = fma(d.W[r * d.n + i], d.W[r * d.n + i], a);
   a = warp_sum(a);
-  if (lane == 0) d.nrm2[r] = a;
+  if (lane == 0) {
+    d.nrm2[r] = a;
+    // (non-negative doubles order like their bit patterns)
+    atomicMax(reinterpret_cast<unsigned long long*>(d.top), (unsigned long long)__double_as_longlong(a));
+  }
 }
 
 __global__ void k_row_norms(const double* __restrict__ W, int64_t n, double* __restrict__ nrm) {
@@ -459,7 +472,7 @@ int gs_panel_rows(int64_t s) {
 
 // Buffers of one SVD, carved from its scratch.
 struct SvdBufs {
-  double *W, *nrm, *nrm2, *C, *Q, *H;
+  double *W, *nrm, *nrm2, *top, *C, *Q, *H;
   int *perm, *rotated;
   SvdDesc* desc;
   SvdTile* tiles;
@@ -479,6 +492,7 @@ void svd_carve(Arena& a, int64_t s, int64_t n, SvdBufs& B) {
   B.nrm = a.take<double>((size_t)s);
   B.nrm2 = a.take<double>((size_t)s);
   B.perm = a.take<int>((size_t)s);
+  B.top = a.take<double>(1);
   B.rotated = a.take<int>(1);
   B.desc = a.take<SvdDesc>(1);
   B.tiles = a.take<SvdTile>((size_t)svd_tile_count(s));
@@ -552,9 +566,10 @@ tk_status svd_finish(const double* W, int64_t s, int64_t n, double* nrm, int* pe
 }
 
 // Sweeps over all matrices together (one launch per round) until none rotates; sweeps[j] receives the
-// count of matrix j.  dd, dt: device copies of hd and of the tiles are made here.
-tk_status run_sweeps(std::vector<SvdDesc>& hd, SvdDesc* dd, SvdTile* dt, int* rots, std::vector<int>& sweeps,
-                     cudaStream_t st) {
+// count of matrix j.  dd, dt: device copies of hd and of the tiles are made here; tops, rots: what the matrices' top
+// and rotated point to.
+tk_status run_sweeps(std::vector<SvdDesc>& hd, SvdDesc* dd, SvdTile* dt, double* tops, int* rots,
+                     std::vector<int>& sweeps, cudaStream_t st) {
   const int J = (int)hd.size();
   std::vector<SvdTile> tiles;
   int64_t max_rounds = 0, max_n = 0;
@@ -568,6 +583,7 @@ tk_status run_sweeps(std::vector<SvdDesc>& hd, SvdDesc* dd, SvdTile* dt, int* ro
   }
   TK_CUDA(cudaMemcpyAsync(dd, hd.data(), sizeof(SvdDesc) * J, cudaMemcpyHostToDevice, st));
   TK_CUDA(cudaMemcpyAsync(dt, tiles.data(), sizeof(SvdTile) * tiles.size(), cudaMemcpyHostToDevice, st));
+  TK_CUDA(cudaMemsetAsync(tops, 0, sizeof(double) * J, st));
   const double tol = 1e-15;
   const int max_sweeps = 80;
   std::vector<int> hrot(J);
@@ -606,9 +622,9 @@ tk_status jacobi_svd(const double* Y, int64_t s, int64_t n, double* sigma, doubl
   if (!ar.ok()) return TK_ENOMEM;
   if (s == 0) return TK_OK;
   TK_TRY(svd_start(Y, s, n, B, st));
-  std::vector<SvdDesc> hd(1, SvdDesc{B.W, B.nrm2, s, n, block_players(s), B.rotated, s <= 1 ? 1 : 0});
+  std::vector<SvdDesc> hd(1, SvdDesc{B.W, B.nrm2, s, n, block_players(s), B.top, B.rotated, s <= 1 ? 1 : 0});
   std::vector<int> sweeps;
-  TK_TRY(run_sweeps(hd, B.desc, B.tiles, B.rotated, sweeps, st));
+  TK_TRY(run_sweeps(hd, B.desc, B.tiles, B.top, B.rotated, sweeps, st));
   if (sweeps_host) *sweeps_host = std::max(sweeps[0], 1);
   return svd_finish(B.W, s, n, B.nrm, B.perm, sigma, V, st);
 }
@@ -632,6 +648,7 @@ tk_status jacobi_svd_grouped(std::vector<SvdJob>& jobs, void* work, size_t work_
   a.base = (char*)work;
   a.cap = work_bytes;
   SvdDesc* dd = a.take<SvdDesc>(J);
+  double* tops = a.take<double>(J);
   int* rots = a.take<int>(J);
   size_t ntiles = 0;
   for (const auto& j : jobs) ntiles += (size_t)svd_tile_count(j.s);
@@ -647,10 +664,10 @@ tk_status jacobi_svd_grouped(std::vector<SvdJob>& jobs, void* work, size_t work_
     sa.cap = q.scratch_bytes;
     svd_carve(sa, q.s, q.n, bufs[j]);
     if (!sa.ok()) return TK_ENOMEM;
-    hd[j] = SvdDesc{bufs[j].W, bufs[j].nrm2, q.s, q.n, block_players(q.s), rots + j, q.s <= 1 ? 1 : 0};
+    hd[j] = SvdDesc{bufs[j].W, bufs[j].nrm2, q.s, q.n, block_players(q.s), tops + j, rots + j, q.s <= 1 ? 1 : 0};
   }
   std::vector<int> sweeps;
-  TK_TRY(run_sweeps(hd, dd, dt, rots, sweeps, st));
+  TK_TRY(run_sweeps(hd, dd, dt, tops, rots, sweeps, st));
   for (int j = 0; j < J; ++j) {
     SvdJob& q = jobs[j];
     q.sweeps = sweeps[j];
@@ -664,6 +681,7 @@ size_t svd_grouped_workspace(const std::vector<SvdJob>& jobs) {
   size_t ntiles = 0;
   for (const auto& j : jobs) ntiles += (size_t)svd_tile_count(j.s);
   a.take<SvdDesc>(std::max<size_t>(jobs.size(), 1));
+  a.take<double>(std::max<size_t>(jobs.size(), 1));
   a.take<int>(std::max<size_t>(jobs.size(), 1));
   a.take<SvdTile>(std::max<size_t>(ntiles, 1));
   return a.used + 1024;

@@ -1,4 +1,5 @@
-"""The SVD of the sketch at the ends of its range: rows longer than the registers of a block pair hold."""
+"""The SVD of the sketch at the ends of its range: rows longer than the registers of a block pair hold, and rows
+that depend on each other exactly."""
 import numpy as np
 import pytest
 import torch
@@ -30,6 +31,27 @@ def _check(Y, max_sweeps):
 def test_long_rows(s, n):
     gen = np.random.default_rng(s + n)
     _check(gen.standard_normal((s, n)) * np.exp(-np.arange(n) / (n / 6.0)), 30)
+
+
+# rows that depend on each other exactly (fewer nonzero columns than rows, equal columns, equal rows), below and
+# above the 64 rows of the orthogonal start: each sweep leaves rounding errors of the sweep before, which end as
+# zero rows and not as pairs that are rotated for ever (80 sweeps is the cap)
+def _dependent(kind):
+    gen = np.random.default_rng(7)
+    if kind == "ones":
+        return np.ones((30, 40))
+    if kind == "outer":
+        return np.outer(gen.standard_normal(8), gen.standard_normal(40))
+    s, r, n = {"zero columns 16": (16, 6, 36), "zero columns 32": (32, 20, 50), "zero columns 96": (96, 40, 100),
+               "equal columns 40": (40, 5, 50), "equal columns 80": (80, 30, 90)}[kind]
+    X = gen.standard_normal((s, r))
+    return np.tile(X, (1, n // r)) if kind.startswith("equal") else np.hstack([X, np.zeros((s, n - r))])
+
+
+@pytest.mark.parametrize("kind", ["ones", "outer", "zero columns 16", "zero columns 32", "zero columns 96",
+                                  "equal columns 40", "equal columns 80"])
+def test_dependent_rows(kind):
+    _check(_dependent(kind), 30)
 
 
 # more rows than the orthogonal start takes (no row of s values fits in shared memory): rows that are orthogonal from
