@@ -52,6 +52,12 @@ struct JacSmem {
   int rot[2];
 };
 
+// The power of two that brings x > 0 to [1, 2) (2^1023 for subnormal x).
+__device__ __forceinline__ double pow2_inverse(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return __hiloint2double((e > 2045 ? 1 : 2046 - e) << 20, 0);
+}
+
 // Rotation that makes rows of squared norms a, b and dot product g orthogonal (rows already orthogonal
 // to tol, or one of them zero: false).  t = tan of the angle in float32 from the scaled ratio zeta =
 // (b - a) / (2 g): off by 1e-7 relative it leaves 1e-7 of g for the next sweep; the norms' update a - t g is
@@ -60,7 +66,10 @@ struct JacSmem {
 // cos = (1 + t^2)^(-1/2) by two Newton steps from the float32 value.
 __device__ __forceinline__ bool jac_angle(double a, double b, double g, double tol, double* c, double* s, double* t) {
   if (!(a > 0.0) || !(b > 0.0)) return false;
-  if (!(g * g > tol * tol * (a * b))) return false;
+  // g^2 > tol^2 a b, each factor scaled by the power of two that brings a or b to [1, 2): as they are, the fourth
+  // powers of norms of 1e-81 or 1e77 leave float64
+  const double sa = pow2_inverse(a), sb = pow2_inverse(b);
+  if (!((g * sa) * (g * sb) > tol * tol * ((a * sa) * (b * sb)))) return false;
   const double d1 = b - a, d2 = 2.0 * g;
   // both scaled by the power of two that brings the larger to [1, 2): float32 then holds their ratio
   const int e1 = (__double2hiint(d1) >> 20) & 0x7ff, e2 = (__double2hiint(d2) >> 20) & 0x7ff;
@@ -337,14 +346,32 @@ __global__ void __launch_bounds__(256)
 // finished rows and orthogonalized inside (modified Gram-Schmidt), twice.
 constexpr int kGsPanel = 16;
 
+// scale = the power of two that brings the largest C_ii to [1, 2) (one block).
+__global__ void __launch_bounds__(256) k_gs_scale(const double* __restrict__ C, int64_t s, double* __restrict__ scale) {
+  __shared__ double sh[8];
+  double mx = 0.0;
+  for (int64_t i = threadIdx.x; i < s; i += blockDim.x) mx = fmax(mx, C[i * s + i]);
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) mx = fmax(mx, sh[w]);
+    *scale = pow2_inverse(mx);
+  }
+}
+
 // X = C + noise of 2^-50 of sqrt(C_ii C_jj): rows of C that are dependent in float64 keep a direction of
-// their own (its choice is free), so that Q is a complete basis whatever the rank.
-__global__ void k_gs_noise(const double* __restrict__ C, int64_t s, double* __restrict__ X) {
+// their own (its choice is free), so that Q is a complete basis whatever the rank.  Times scale, so that the squares
+// of X, fourth powers of Y, stay in float64's range.
+__global__ void k_gs_noise(const double* __restrict__ C, int64_t s, const double* __restrict__ scale,
+                           double* __restrict__ X) {
   const int64_t i = blockIdx.y;
+  const double sc = *scale;
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < s; j += (int64_t)gridDim.x * blockDim.x) {
     const uint4 r = philox((uint64_t)(i * s + j), 7u, 0x5eedull);
     const double u = ((double)(int)r.x) * 0x1p-31;  // in [-1, 1)
-    X[i * s + j] = fma(u * 0x1p-50, sqrt(C[i * s + i]) * sqrt(C[j * s + j]), C[i * s + j]);
+    X[i * s + j] = sc * fma(u * 0x1p-50, sqrt(C[i * s + i]) * sqrt(C[j * s + j]), C[i * s + j]);
   }
 }
 
@@ -510,7 +537,9 @@ tk_status svd_start(const double* Y, int64_t s, int64_t n, const SvdBufs& B, cud
     return TK_OK;
   }
   TK_TRY((gemm<double, double, double>(false, true, s, s, n, Y, n, Y, n, B.C, s, 1.0, nullptr, nullptr, 0, st)));
-  k_gs_noise<<<dim3((unsigned)cdiv(s, 256), (unsigned)s), 256, 0, st>>>(B.C, s, B.Q);
+  k_gs_scale<<<1, 256, 0, st>>>(B.C, s, B.top);
+  TK_LAUNCH_CHECK();
+  k_gs_noise<<<dim3((unsigned)cdiv(s, 256), (unsigned)s), 256, 0, st>>>(B.C, s, B.top, B.Q);
   TK_LAUNCH_CHECK();
   const int pr = gs_panel_rows(s);
   TK_CUDA(cudaFuncSetAttribute(k_gs_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGsSmemCap));

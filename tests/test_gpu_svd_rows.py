@@ -1,5 +1,5 @@
-"""The SVD of the sketch at the ends of its range: rows longer than the registers of a block pair hold, and rows
-that depend on each other exactly."""
+"""The SVD of the sketch at the ends of its range: rows longer than the registers of a block pair hold, rows that
+depend on each other exactly, and rows far from unit scale."""
 import numpy as np
 import pytest
 import torch
@@ -52,6 +52,15 @@ def _dependent(kind):
                                   "equal columns 40", "equal columns 80"])
 def test_dependent_rows(kind):
     _check(_dependent(kind), 30)
+
+
+# powers of two on the whole matrix: the squares and fourth powers of a row norm leave float64's range long before
+# the norm does
+@pytest.mark.parametrize("e", [-400, -330, -270, 270, 330, 400])
+@pytest.mark.parametrize("s,n", [(20, 30), (80, 130)])
+def test_scales(s, n, e):
+    gen = np.random.default_rng(s)
+    _check(np.ldexp(gen.standard_normal((s, n)), e), 30)
 
 
 # more rows than the orthogonal start takes (no row of s values fits in shared memory): rows that are orthogonal from
