@@ -216,12 +216,7 @@ bool oz_gauss(const Plan& P) { return P.oz64 && P.o.sketch == TK_SKETCH_GAUSS &&
 tk_dtype sketch_dtype(const Plan& P) { return P.mixed ? TK_F32 : TK_F64; }
 
 size_t sketch_scratch(const Plan& P, tk_dtype dt) {
-  if (oz_gauss(P)) {
-    Arena a;
-    a.take<double>((size_t)P.s * P.L);
-    a.take<char>(oz_sketch_workspace(P.L, P.c, P.s));
-    return a.used + 512;
-  }
+  if (oz_gauss(P)) return oz_sketch_workspace(P.L, P.c, P.s);
   if (tc_sketch(P)) return tc_sketch_workspace(P.L, P.c, P.s);
   if (P.o.sketch == TK_SKETCH_SRHT) return srht_rows_workspace(P.L, P.c, dt, P.s);
   if (P.o.sketch == TK_SKETCH_SPARSE) return sparse_rows_workspace(P.L, P.c, P.s);
@@ -449,17 +444,8 @@ inline dim3 rgrid(int64_t len, int rows) {
 tk_status do_sketch(const Plan& P, const void* A_sk, tk_dtype dt_sk, int64_t ld_sk, Bufs& B, cudaStream_t st) {
   const void* src = A_sk;
   int64_t ld = ld_sk;
-  if (oz_gauss(P)) {
-    Arena sa;
-    sa.base = B.scratch;
-    sa.cap = B.scratch_bytes;
-    double* G = sa.take<double>((size_t)P.s * P.L);
-    const size_t wb = oz_sketch_workspace(P.L, P.c, P.s);
-    char* w = sa.take<char>(wb);
-    if (!sa.ok()) return TK_ENOMEM;
-    TK_TRY(gauss_fill(P.o.seed, P.s, P.L, G, st));
-    return oz_sketch(oz_mat(P, B), P.under, G, P.s, B.Y, w, wb, B.oz_err, st);
-  }
+  if (oz_gauss(P))
+    return oz_sketch(oz_mat(P, B), P.under, P.o.seed, P.s, B.Y, B.scratch, B.scratch_bytes, B.oz_err, st);
   if (P.under) {
     TK_TRY(transpose(A_sk, dt_sk, P.m, P.n, ld_sk, B.AT, st));
     src = B.AT;

@@ -196,7 +196,8 @@ size_t srht_rows_workspace(int64_t L, int64_t cols, tk_dtype dt, int64_t s);
 tk_status gauss_rows(const void* A, tk_dtype dt, int64_t L, int64_t cols, int64_t ld, uint64_t seed, int64_t s,
                      double* Y, Arena& ar, cudaStream_t st);
 size_t gauss_rows_workspace(int64_t L, int64_t cols, tk_dtype dt, int64_t s);
-tk_status gauss_fill(uint64_t seed, int64_t s, int64_t L, double* G, cudaStream_t st);  // the s x L embedding itself
+// columns k0 .. k0 + len - 1 of the s x L embedding itself (G: s x len)
+tk_status gauss_fill(uint64_t seed, int64_t s, int64_t L, int64_t k0, int64_t len, double* G, cudaStream_t st);
 // SRDCT (tk_sketch.cu): X = sqrt(Lp/s) S C D [I; 0], C the orthonormal DCT-II of length Lp.
 tk_status srdct_rows(const void* A, tk_dtype dt, int64_t L, int64_t cols, int64_t ld, uint64_t seed, int64_t s,
                      double* Y, Arena& ar, cudaStream_t st);
@@ -341,11 +342,11 @@ tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* M
                        int64_t n, int h, void* work, size_t bytes, int* err, cudaStream_t st);
 template <typename T>
 size_t oz_tri_workspace(int64_t n, int N, int h0);
-// Y (s x c) = G A (m >= n: G s x m, c = n) or G A^T (under: G s x n, c = m) for an embedding G (float64,
+// Y (s x c) = G A (m >= n: G s x m, c = n) or G A^T (under: G s x n, c = m) for the Gaussian embedding G (gauss_fill,
 // s <= 65535) from the digit planes of A, float64-accurate; work: oz_sketch_workspace(L, c, s) bytes, L the
-// length of G's rows.
+// length of G's rows: 2 GiB for a block of its columns at a time, whatever s L is, and planes of Y.
 size_t oz_sketch_workspace(int64_t L, int64_t c, int64_t s);
-tk_status oz_sketch(const OzMat& A, bool under, const double* G, int64_t s, double* Y, void* work, size_t bytes,
+tk_status oz_sketch(const OzMat& A, bool under, uint64_t seed, int64_t s, double* Y, void* work, size_t bytes,
                     int* err, cudaStream_t st);
 // C = Y^T Y (Y: r x c float64, row stride c), the upper triangle (j >= i) of
 // C (c x c) written, float64-accurate; work: oz_gram_workspace(r, c) bytes.

@@ -874,13 +874,16 @@ unsigned ot_grid(const OtTiles& t) {
 }
 
 // 3D map over the slice planes (K fastest, then rows, then the plane index),
-// box = 64 values of K x box_rows x 1 plane, 128-byte swizzle.
-tk_status make_slice_map(CUtensorMap* map, const void* base, int64_t rows, int64_t kp, uint32_t box_rows,
-                         int planes) {  // kp: row stride
+// box = 64 values of K x box_rows x 1 plane, 128-byte swizzle.  ld, plane: values from one row and one plane to the
+// next where the map covers a part of larger planes (0: kp and rows kp).
+tk_status make_slice_map(CUtensorMap* map, const void* base, int64_t rows, int64_t kp, uint32_t box_rows, int planes,
+                         int64_t ld = 0, int64_t plane = 0) {
+  if (ld == 0) ld = kp;
+  if (plane == 0) plane = rows * ld;
   EncodeTiledFn fn;
   TK_TRY(encode_fn(&fn));
   const cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)rows, (cuuint64_t)planes};
-  const cuuint64_t strides[2] = {(cuuint64_t)kp * 2, (cuuint64_t)rows * kp * 2};
+  const cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)plane * 2};
   const cuuint32_t box[3] = {(cuuint32_t)OT_KB, box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
@@ -906,6 +909,7 @@ struct OtBig {
   const int* E;  // exponents of its `rows`
   int64_t rows, K;
   bool trans;
+  int64_t ld = 0, plane = 0;  // strides of larger planes that it is a part of (as make_slice_map)
 };
 
 template <int S, int MODE, int NT, bool TR>
@@ -913,8 +917,8 @@ tk_status launch_oz_tc_nt(const OtBig& P, const void* Qs, const int* EQ, int M, 
                           int sp, const double* b, void* out, int64_t ldo, const double* coef, int* err,
                           cudaStream_t st, int upper_only) {
   CUtensorMap mP, mQ;
-  if (TR) TK_TRY(make_slice_map(&mP, P.planes, P.K, cdiv(P.rows, OZ_KPAD) * OZ_KPAD, OT_KB, OZ_S));
-  else TK_TRY(make_slice_map(&mP, P.planes, P.rows, kp, OT_M, OZ_S));
+  if (TR) TK_TRY(make_slice_map(&mP, P.planes, P.K, cdiv(P.rows, OZ_KPAD) * OZ_KPAD, OT_KB, OZ_S, P.ld, P.plane));
+  else TK_TRY(make_slice_map(&mP, P.planes, P.rows, kp, OT_M, OZ_S, P.ld, P.plane));
   TK_TRY(make_slice_map(&mQ, Qs, M, kp, NT, planesQ));
   const size_t smem = sizeof(OtSmem<S, NT>) + 1024;
   TK_CUDA(cudaFuncSetAttribute(k_oz_tc<S, MODE, NT, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -2184,47 +2188,74 @@ static int oz_sketch_splits(int64_t L, int64_t c, int64_t s) {
   const int64_t tiles = cdiv(c, OT_M) * cdiv(s, OT_N);
   return tiles >= 152 ? (int)cdiv(L, OT_MAX_KPS) : oz_normal_splits(L, c, s);
 }
-__global__ void k_oz_sum_planes(const double* __restrict__ part, int splits, int64_t total, double* __restrict__ Y) {
+// Y (+)= sum_z part[z]
+__global__ void k_oz_sum_planes(const double* __restrict__ part, int splits, int64_t total, double* __restrict__ Y,
+                                int add) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
-    double acc = 0.0;
+    double acc = add ? Y[k] : 0.0;
 #pragma unroll 4
     for (int z = 0; z < splits; ++z) acc += part[(int64_t)z * total + k];
     Y[k] = acc;
   }
 }
 
+// The columns of the embedding whose float64 values and 8 digit planes (24 bytes a value) are held at a time: 2 GiB of
+// them, a product of thousands of values of K for every s.
+static int64_t oz_sketch_block(int64_t L, int64_t s) {
+  const int64_t fit = (int64_t(2) << 30) / (24 * s) / OT_CHUNK * OT_CHUNK;
+  return std::min<int64_t>(L, std::max<int64_t>(fit, OT_CHUNK));
+}
+
+static void oz_sketch_carve(Arena& a, int64_t L, int64_t c, int64_t s, double** G, void** Gs, int** E, double** part) {
+  const int64_t len = oz_sketch_block(L, s);
+  const int sp = oz_sketch_splits(len, c, s);
+  *G = a.take<double>((size_t)s * len);
+  *Gs = a.take<char>(oz_slices_bytes(s, len));
+  *E = a.take<int>(s);
+  *part = sp > 1 || len < L ? a.take<double>((size_t)sp * s * c) : nullptr;
+}
+
 size_t oz_sketch_workspace(int64_t L, int64_t c, int64_t s) {
   Arena a;
-  a.take<char>(oz_slices_bytes(s, L));
-  a.take<int>(s);
-  const int sp = oz_sketch_splits(L, c, s);
-  if (sp > 1) a.take<double>((size_t)sp * s * c);
+  double *G, *part;
+  void* Gs;
+  int* E;
+  oz_sketch_carve(a, L, c, s, &G, &Gs, &E, &part);
   return a.used + 256;
 }
 
-tk_status oz_sketch(const OzMat& A, bool under, const double* G, int64_t s, double* Y, void* work, size_t bytes,
+tk_status oz_sketch(const OzMat& A, bool under, uint64_t seed, int64_t s, double* Y, void* work, size_t bytes,
                     int* err, cudaStream_t st) {
   const int64_t L = under ? A.n : A.m, c = under ? A.m : A.n;
   if (s == 0 || c == 0) return TK_OK;
   Arena a;
   a.base = static_cast<char*>(work);
   a.cap = bytes;
-  void* Gs = a.take<char>(oz_slices_bytes(s, L));
-  int* E = a.take<int>(s);
-  const int sp = oz_sketch_splits(L, c, s);
-  double* part = sp > 1 ? a.take<double>((size_t)sp * s * c) : nullptr;
+  double *G, *part;
+  void* Gs;
+  int* E;
+  oz_sketch_carve(a, L, c, s, &G, &Gs, &E, &part);
   if (!a.ok()) return TK_ENOMEM;
-  TK_TRY(oz_split_vectors(G, TK_F64, s, L, L, under ? A.EC : A.ER, Gs, E, st));
-  double* out = sp > 1 ? part : Y;
-  if (under)
-    TK_TRY((launch_oz_tc<OZ_S, 1, false>({A.planes, A.ER, A.m, A.n, false}, Gs, E, (int)s, OZ_S, sp, nullptr, out, c,
-                                         nullptr, err, st)));
-  else
-    TK_TRY((launch_oz_tc<OZ_S, 1, true>({A.planes, A.EC, A.n, A.m, true}, Gs, E, (int)s, OZ_S, sp, nullptr, out, c,
-                                        nullptr, err, st)));
-  if (sp > 1) {
-    k_oz_sum_planes<<<(unsigned)std::min<int64_t>(cdiv(s * c, 256), 152 * 8), 256, 0, st>>>(part, sp, s * c, Y);
-    TK_LAUNCH_CHECK();
+  const int64_t block = oz_sketch_block(L, s), n64 = cdiv(A.n, OZ_KPAD) * OZ_KPAD;
+  const int sp = oz_sketch_splits(block, c, s);
+  double* out = part ? part : Y;
+  const __nv_bfloat16* planes = static_cast<const __nv_bfloat16*>(A.planes);
+  // blocks of columns of the embedding (rows of A, or its columns where m < n), their products added in order
+  for (int64_t k0 = 0; k0 < L; k0 += block) {
+    const int64_t len = std::min(block, L - k0);
+    TK_TRY(gauss_fill(seed, s, L, k0, len, G, st));
+    TK_TRY(oz_split_vectors(G, TK_F64, s, len, len, (under ? A.EC : A.ER) + k0, Gs, E, st));
+    if (under)
+      TK_TRY((launch_oz_tc<OZ_S, 1, false>({planes + k0, A.ER, A.m, len, false, n64, A.m * n64}, Gs, E, (int)s, OZ_S, sp,
+                                           nullptr, out, c, nullptr, err, st)));
+    else
+      TK_TRY((launch_oz_tc<OZ_S, 1, true>({planes + k0 * n64, A.EC, A.n, len, true, n64, A.m * n64}, Gs, E, (int)s, OZ_S,
+                                          sp, nullptr, out, c, nullptr, err, st)));
+    if (part) {
+      k_oz_sum_planes<<<(unsigned)std::min<int64_t>(cdiv(s * c, 256), 152 * 8), 256, 0, st>>>(part, sp, s * c, Y,
+                                                                                             k0 > 0);
+      TK_LAUNCH_CHECK();
+    }
   }
   return TK_OK;
 }
@@ -2268,7 +2299,7 @@ tk_status oz_gram(const double* Y, int64_t r, int64_t c, double* C, void* work, 
   TK_TRY((launch_oz_tc<OZ_S, 1, false>({Ys, E, c, r, false}, Ys, E, (int)c, OZ_S, sp, nullptr, sp > 1 ? part : C, c,
                                        nullptr, err, st, 1)));
   if (sp > 1) {  // (below the diagonal tiles the planes hold nothing: those sums are not read)
-    k_oz_sum_planes<<<(unsigned)std::min<int64_t>(cdiv(c * c, 256), 152 * 8), 256, 0, st>>>(part, sp, c * c, C);
+    k_oz_sum_planes<<<(unsigned)std::min<int64_t>(cdiv(c * c, 256), 152 * 8), 256, 0, st>>>(part, sp, c * c, C, 0);
     TK_LAUNCH_CHECK();
   }
   return TK_OK;

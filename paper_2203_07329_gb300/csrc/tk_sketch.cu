@@ -389,6 +389,22 @@ __global__ void k_gauss_fill(uint64_t seed, int64_t s, int64_t L, double inv_sqr
   }
 }
 
+// Columns k0 .. k0 + len - 1 of the rows (G: s x len): grid.y over the rows, grid.x over the calls that touch a row's
+// part (the first and the last may start before it or end behind it).
+__global__ void __launch_bounds__(256) k_gauss_fill_block(uint64_t seed, int64_t s, int64_t L, int64_t k0, int64_t len,
+                                                          double inv_sqrt_s, double* __restrict__ G) {
+  for (int64_t i = blockIdx.y; i < s; i += gridDim.y) {
+    const int64_t i0 = i * L + k0, g = (i0 >> 2) + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t c0 = 4 * g - i0;  // the column of the call's first entry
+    if (c0 >= len) continue;
+    double v[4];
+    gauss_entries4(seed, (uint64_t)g, inv_sqrt_s, v);
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (c0 + t >= 0 && c0 + t < len) G[i * len + c0 + t] = v[t];
+  }
+}
+
 template <typename T>
 __global__ void k_transpose(const T* __restrict__ A, int64_t rows, int64_t cols, int64_t lda, T* __restrict__ AT) {
   __shared__ T tileT[32][33];
@@ -544,9 +560,15 @@ tk_status srht_rows(const void* A, tk_dtype dt, int64_t L, int64_t cols, int64_t
   return srht_impl<float, float>((const float*)A, L, cols, ld, seed, s, Y, ar, st);
 }
 
-tk_status gauss_fill(uint64_t seed, int64_t s, int64_t L, double* G, cudaStream_t st) {
-  if (s * L == 0) return TK_OK;
-  k_gauss_fill<double><<<grid_for(cdiv(s * L, 4), 256), 256, 0, st>>>(seed, s, L, 1.0 / sqrt((double)s), G);
+tk_status gauss_fill(uint64_t seed, int64_t s, int64_t L, int64_t k0, int64_t len, double* G, cudaStream_t st) {
+  if (s * len == 0) return TK_OK;
+  const double is = 1.0 / sqrt((double)s);
+  if (len == L) {
+    k_gauss_fill<double><<<grid_for(cdiv(s * L, 4), 256), 256, 0, st>>>(seed, s, L, is, G);
+  } else {
+    const dim3 g((unsigned)cdiv(cdiv(len, 4) + 1, 256), (unsigned)std::min<int64_t>(s, 65535));
+    k_gauss_fill_block<<<g, 256, 0, st>>>(seed, s, L, k0, len, is, G);
+  }
   TK_LAUNCH_CHECK();
   return TK_OK;
 }

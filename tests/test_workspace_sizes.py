@@ -52,3 +52,12 @@ def test_svd_of_many_rows(tk, s, n):
     w = tk.lib().tk_sketch_svd_workspace(s, n)
     most = 8 * s * n + (16 * s * s if s <= 25600 else 0)
     assert 8 * s * n < w <= most + 8 * 32 * s + (1 << 20)
+
+
+# the float64 form's Gaussian sketch from digits holds a bounded block of the embedding and its planes at a time: not
+# 24 bytes for each of its s L values (2^20 x 2048: 192 GiB)
+@pytest.mark.parametrize("m,n,s", [(1 << 20, 2048, 8192), (1 << 21, 2048, 8192), (2048, 1 << 20, 8192),
+                                   (1 << 20, 64, 60000)])
+def test_gaussian_sketch_of_the_float64_form(tk, m, n, s):
+    srht = _size(tk, m, n, 4, sketch=tk.TK_SKETCH_SRHT, s=s)
+    assert _size(tk, m, n, 4, sketch=tk.TK_SKETCH_GAUSS, s=s) <= srht + 4 * GIB
