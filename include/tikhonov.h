@@ -114,12 +114,13 @@ typedef struct {
                              the float64 pipe, with the same float64 accuracy: MIXED: the Gram matrix, the
                              Cholesky trailing updates, and the refinement's r = b - A x and A^T r; FP64:
                              the Gaussian sketch, the Gram matrix and the trailing updates when A has
-                             2^16 .. 2^32 elements, and the two products with A of every LSQR step when it
-                             has 2^19 or more; both: the explicit inverse of the factors beyond blocks of
+                             2^16 .. 2^32 elements (and the LSQR vectors of all lambdas, N max(m, n) values, at
+                             most 2^32), and the two products with A of every LSQR step when it has 2^19 or
+                             more; both: the explicit inverse of the factors beyond blocks of
                              256.  Costs 32 (MIXED) or 16 (FP64) bytes of workspace per element of
-                             A (its rows rounded up to 64) for the digit planes, and at most 2 GiB for the
-                             planes of each other operand (the Gaussian embedding, the panels of the Cholesky
-                             updates, the inverse); 0 = float64 FMA. */
+                             A (its rows rounded up to 64) for the digit planes, 16 per value of the sketch and
+                             of the LSQR vectors, and at most 2 GiB for a block of the Gaussian embedding, of
+                             the Cholesky panels or of the inverse; 0 = float64 FMA. */
   const double* x0;       /* [NULL] warm start, device N x n float64 (row i for lambdas[i]; m >= n only):
                              the solve starts from x = x0 instead of 0 and returns the same minimiser of
                              problem (1.2).  FP64: LSQR solves for the correction d in

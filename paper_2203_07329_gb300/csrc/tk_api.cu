@@ -60,6 +60,7 @@ constexpr int64_t kMaxLong = (int64_t(1) << 30);
 // memory (16 N c^2 bytes, 4 GiB).
 constexpr double kInv64Cost = 8e7, kInv64CostDigits = 2.7e8;
 constexpr int64_t kOz64MinElems = int64_t(1) << 16;  // smallest A (elements) that the float64 form splits into digits
+constexpr int64_t kOz64MaxPlane = int64_t(1) << 32;  // most values of one of its digit planes
 
 tk_status check_opts(const tk_opts* o) {
   if (!o) return einval("options pointer is NULL");
@@ -85,9 +86,14 @@ tk_status check_opts(const tk_opts* o) {
 
 // The float64 form with emulate_fp64: whether the solve makes digit planes of A at all.  They pay off
 // for the Gaussian sketch, the Gram matrix and the Cholesky updates (2000 x 64: 25 us to make them, 400
-// us less work on the float64 pipe) and, for larger A, the LSQR products (use_oz); A of more than 2^32
-// elements keeps the float64 pipe, because the planes take 16 bytes per element.
-bool oz64_wanted(int64_t m, int64_t n) { return m * n >= kOz64MinElems && m * n <= (int64_t(1) << 32); }
+// us less work on the float64 pipe) and, for larger A, the LSQR products (use_oz): also for A of a few
+// columns, whose planes are mostly padding (rows of them are rounded up to 64 values; 2^20 x 4, 16 lambda: 9.4
+// ms, on the pipe 44).  The planes take 16 bytes per value: not made for A of more than 2^32 elements, nor where
+// those of the LSQR vectors of all lambdas would take more than 64 GiB.
+bool oz64_wanted(int64_t m, int64_t n, int N_cap) {
+  return m * n >= kOz64MinElems && m * n <= kOz64MaxPlane &&
+         N_cap * (cdiv(std::max(m, n), 64) * 64) <= kOz64MaxPlane;
+}
 
 tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
   if (!p) return einval("problem pointer is NULL");
@@ -129,7 +135,7 @@ tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
               (P.dt == TK_F64 || P.lda % 4 == 0);
   P.lsqr_oz = P.mixed && (o->lsqr_tc == 2 || o->lsqr_tc == 3) && o->emulate_fp64 && !P.under;
   P.lsqr_fused = P.lsqr_oz && o->lsqr_tc == 3;
-  P.oz64 = !P.mixed && o->emulate_fp64 && oz64_wanted(P.m, P.n);
+  P.oz64 = !P.mixed && o->emulate_fp64 && oz64_wanted(P.m, P.n, P.N_cap);
   P.inv64 = !P.mixed && !P.lowrank &&
             (double)std::max(N, 1) * P.c * P.c <= (P.oz64 ? kInv64CostDigits : kInv64Cost);
   return TK_OK;

@@ -61,3 +61,10 @@ def test_svd_of_many_rows(tk, s, n):
 def test_gaussian_sketch_of_the_float64_form(tk, m, n, s):
     srht = _size(tk, m, n, 4, sketch=tk.TK_SKETCH_SRHT, s=s)
     assert _size(tk, m, n, 4, sketch=tk.TK_SKETCH_GAUSS, s=s) <= srht + 4 * GIB
+
+
+# the LSQR vectors of very many lambdas get no digit planes beyond 64 GiB: the solve takes what it takes without digits
+def test_no_vector_planes_beyond_64_gib(tk):
+    o = dict(s=256)
+    assert _size(tk, 1 << 20, 64, 4097, **o) <= _size(tk, 1 << 20, 64, 4097, emulate_fp64=0, **o) + GIB
+    assert _size(tk, 1 << 20, 64, 4096, **o) >= _size(tk, 1 << 20, 64, 4096, emulate_fp64=0, **o) + 64 * GIB
