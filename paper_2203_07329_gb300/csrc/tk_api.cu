@@ -1107,6 +1107,7 @@ TK_API tk_status tk_solve(const tk_problem* p, const double* lambdas, int N, con
 // stream (joined to the caller's stream by events) and a slice of the
 // workspace, and solves its problems one after another.
 static constexpr int kLanes = 8;
+static constexpr size_t kLaneDigitBytes = size_t(32) << 30;  // digit planes of all lanes together (8 A of 2^28 elements)
 
 static int batched_lanes(int P) { return std::max(1, std::min(P, kLanes)); }
 
@@ -1139,7 +1140,15 @@ tk_status batch_layout(const tk_problem* ps, int P, int N, const tk_opts* o, int
   }
   L.grouped = grouped;
   if (!grouped) {
-    for (int i = 0; i < P; ++i) L.per = std::max(L.per, (plan_bytes(pl[i]) + 255) & ~size_t(255));
+    // Every lane has a slice for the largest problem.  The float64 form's digit planes (16 bytes per element of A,
+    // twice its float64 A) are not multiplied by 8 lanes beyond kLaneDigitBytes: a problem of that size fills
+    // the GPU by itself.
+    size_t digits = 1;
+    for (int i = 0; i < P; ++i) {
+      L.per = std::max(L.per, (plan_bytes(pl[i]) + 255) & ~size_t(255));
+      if (pl[i].oz64) digits = std::max(digits, oz_slices_bytes(pl[i].m, pl[i].n));
+    }
+    L.lanes = (int)std::min<size_t>(L.lanes, std::max<size_t>(1, kLaneDigitBytes / digits));
     L.total = L.per * (size_t)L.lanes;
     return TK_OK;
   }

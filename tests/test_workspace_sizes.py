@@ -68,3 +68,26 @@ def test_no_vector_planes_beyond_64_gib(tk):
     o = dict(s=256)
     assert _size(tk, 1 << 20, 64, 4097, **o) <= _size(tk, 1 << 20, 64, 4097, emulate_fp64=0, **o) + GIB
     assert _size(tk, 1 << 20, 64, 4096, **o) >= _size(tk, 1 << 20, 64, 4096, emulate_fp64=0, **o) + 64 * GIB
+
+
+def _batched(tk, m, n, N, P, **kw):
+    ps = (tk.tk_problem * P)(*[_prob(tk, m, n) for _ in range(P)])
+    o, out = tk.opts_default(**kw), C.c_size_t(0)
+    assert tk.lib().tk_workspace_size_batched(C.byref(ps), P, N, C.byref(o), 1, C.byref(out)) == tk.TK_OK
+    return out.value
+
+
+# float64 problems on the host lanes: the digit planes of all lanes together stay within 32 GiB (or one problem's), so
+# that 8 problems of 8 GiB each still fit the GPU beside their workspace; small ones keep 8 lanes
+def test_lanes_of_large_float64_problems(tk):
+    m, n, N = 1 << 19, 2048, 4
+    for sketch in (tk.TK_SKETCH_SRHT, tk.TK_SKETCH_GAUSS):
+        o = dict(sketch=sketch, s=8192)
+        assert _batched(tk, m, n, N, 8, **o) + 8 * 8 * m * n <= 200 * GIB
+        assert _batched(tk, m, n, N, 8, **o) == 2 * _batched(tk, m, n, N, 1, **o)
+    one = _batched(tk, 4096, 256, N, 1, s=1024)
+    assert _batched(tk, 4096, 256, N, 8, s=1024) == 8 * one
+    one = _batched(tk, 1 << 17, 2048, N, 1, s=8192)  # 2^28 elements
+    assert _batched(tk, 1 << 17, 2048, N, 8, s=8192) == 8 * one
+    one = _batched(tk, m, n, N, 1, s=8192, emulate_fp64=0)
+    assert _batched(tk, m, n, N, 8, s=8192, emulate_fp64=0) == 8 * one
