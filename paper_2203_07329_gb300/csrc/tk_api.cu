@@ -194,11 +194,12 @@ struct Bufs {
 bool tc_sketch(const Plan& P) { return P.mixed && P.o.sketch == TK_SKETCH_GAUSS && !P.under; }
 
 // With emulate_fp64 the mixed form, and the float64 form when it works from digits, make their Gram
-// matrix (m >= n) and their Cholesky updates from exact slices on the tensor cores (float64 accuracy).
-bool emulated_chol(const Plan& P) {
+// matrix and their Cholesky updates from exact slices on the tensor cores (float64 accuracy).
+bool emulated_gram(const Plan& P) {
   return ((P.mixed && P.o.emulate_fp64) || P.oz64) && !P.lowrank && !P.qr;
 }
-bool emulated_gram(const Plan& P) { return emulated_chol(P); }
+// The emulated Cholesky takes kOzCholLambdas lambdas at most; with more, the float64 form factors on the float64 pipe.
+bool emulated_chol(const Plan& P) { return emulated_gram(P) && (P.mixed || P.N <= kOzCholLambdas); }
 // ... and the off-diagonal blocks of the factors' inverse
 bool digit_inverse(const Plan& P) {
   return !P.lowrank && (P.mixed ? P.o.emulate_fp64 != 0 : P.oz64 && P.inv64);
@@ -315,7 +316,8 @@ void carve(const Plan& P, Arena& a, Arena& t, Bufs& B) {
   // and the inverse of the factors, after them
   if (digit_inverse(P))
     sc = std::max(sc, P.mixed ? tri_inverse_workspace<float>(P.np, N) : tri_inverse_workspace<double>(P.np, N));
-  if (emulated_gram(P)) sc = std::max({sc, oz_gram_workspace(P.s, P.c), oz_chol_workspace(P.np, N)});
+  if (emulated_gram(P)) sc = std::max(sc, oz_gram_workspace(P.s, P.c));
+  if (emulated_chol(P)) sc = std::max(sc, oz_chol_workspace(P.np, N));
   B.scratch_bytes = sc;
   B.scratch = t.take<char>(sc);
   if (P.prep_only) return;
@@ -623,7 +625,7 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
       const double M = (double)(P.s + P.c);
       prof_end(tok, st, (double)N * (2.0 * M * P.c * P.c - 2.0 * P.c * P.c * (double)P.c / 3.0),
                8.0 * N * (M * P.c + P.c * P.c / 2.0));
-    } else if (emulated_gram(P)) {  // chol_shifted times its float64 and tensor-core parts itself
+    } else if (emulated_chol(P)) {  // chol_shifted times its float64 and tensor-core parts itself
       TK_TRY(oz_chol_begin(B.R, P.np, P.np * P.np, N, P.np, B.scratch, B.scratch_bytes, B.oz_err, &ozp, st));
       TK_TRY(chol_shifted(B.C, P.c, B.lam, N, B.R, P.np, P.np * P.np, B.info, none, st, &ozp));
     } else {

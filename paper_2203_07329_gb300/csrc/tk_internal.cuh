@@ -297,6 +297,7 @@ struct OzCholPlan {
   int* EC = nullptr;
   int* err = nullptr;
 };
+constexpr int kOzCholLambdas = 8191;  // most lambdas of oz_chol_begin
 size_t oz_chol_workspace(int64_t np, int N);
 tk_status oz_chol_begin(double* R, int64_t ldr, int64_t rstride, int N, int64_t np, void* work, size_t bytes,
                         int* err, OzCholPlan* plan, cudaStream_t st);

@@ -2323,7 +2323,7 @@ size_t oz_chol_workspace(int64_t np, int N) {
 
 tk_status oz_chol_begin(double* R, int64_t ldr, int64_t rstride, int N, int64_t np, void* work, size_t bytes,
                         int* err, OzCholPlan* plan, cudaStream_t st) {
-  if (np % 64 || ldr % 4 || rstride % 4 || (uintptr_t)R % 32 || (int64_t)N * OZ_S > 65535 || np > INT32_MAX) {
+  if (np % 64 || ldr % 4 || rstride % 4 || (uintptr_t)R % 32 || N > kOzCholLambdas || np > INT32_MAX) {
     set_error_msg("emulated Cholesky: unsupported order or lambda count");
     return TK_EINVAL;
   }
