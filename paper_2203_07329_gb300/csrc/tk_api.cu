@@ -57,8 +57,11 @@ constexpr int64_t kMaxLong = (int64_t(1) << 30);
 // apply into one launch (20 us at c = 1024, 16 lambda) where a substitution is a chain of c/32 launches
 // (1.1 ms for the two of a step, about 30 steps).  On the float64 pipe it costs N c^3/3 flops (6.9 ms there),
 // as much as the substitutions at c = 2048, 32 lambda; from digits a quarter of that, and the limit is its
-// memory (16 N c^2 bytes, 4 GiB).
+// memory (16 N c^2 bytes, 4 GiB).  Factors of order 512 and less (m >= n) are inverted whatever N is, as they
+// always were: 300 columns, 3200 lambda: 116 ms, with substitution 202; 128 columns, 17000 lambda: 312, 474;
+// without digits 200 columns, 2100 lambda: 132, 161.
 constexpr double kInv64Cost = 8e7, kInv64CostDigits = 2.7e8;
+constexpr int64_t kInv64Small = 512;
 constexpr int64_t kOz64MinElems = int64_t(1) << 16;  // smallest A (elements) that the float64 form splits into digits
 constexpr int64_t kOz64MaxPlane = int64_t(1) << 32;  // most values of one of its digit planes
 
@@ -137,7 +140,8 @@ tk_status make_plan(const tk_problem* p, int N, const tk_opts* o, Plan& P) {
   P.lsqr_fused = P.lsqr_oz && o->lsqr_tc == 3;
   P.oz64 = !P.mixed && o->emulate_fp64 && oz64_wanted(P.m, P.n, P.N_cap);
   P.inv64 = !P.mixed && !P.lowrank &&
-            (double)std::max(N, 1) * P.c * P.c <= (P.oz64 ? kInv64CostDigits : kInv64Cost);
+            ((P.c <= kInv64Small && !P.under) ||
+             (double)std::max(N, 1) * P.c * P.c <= (P.oz64 ? kInv64CostDigits : kInv64Cost));
   return TK_OK;
 }
 

@@ -29,3 +29,22 @@ def test_many_lambdas(m, n, N):
     for i in (0, 1, N // 2, 8190, N - 1):
         x = _solve_exact(A, b, lams[i])
         assert np.linalg.norm(X[i] - x) <= 1e-10 * np.linalg.norm(x)
+
+
+# factors of order 512 and less are inverted explicitly however many lambdas there are (m >= n; beyond, the inverse of
+# N c^2 > 8e7, or 2.7e8 from digits, makes way for substitution)
+@pytest.mark.parametrize("c,N,emulate", [(200, 2100, 0), (300, 3200, 1)])
+def test_small_factors_are_inverted(c, N, emulate):
+    gen = np.random.default_rng(6)
+    m = 4 * c
+    A = torch.from_numpy(gen.standard_normal((m, c)) / np.sqrt(m)).cuda()
+    b = torch.from_numpy(gen.standard_normal(m)).cuda()
+    tk.tk_profile_collect()
+    tk.tk_profile_enable(True)
+    try:
+        r = tk.tk_solve(A, b, np.geomspace(1e-2, 1.0, N), tk.opts_default(s=4 * c, emulate_fp64=emulate))
+        ph = tk.tk_profile_collect()
+    finally:
+        tk.tk_profile_enable(False)
+    assert r.status == tk.TK_OK
+    assert ph["precond_inverse"]["launches"] == 1
