@@ -87,6 +87,16 @@ tk_status check_opts(const tk_opts* o) {
   return TK_OK;
 }
 
+// An arena over a caller's workspace whatever its alignment: TMA and the 32-byte accesses of the Cholesky update want
+// aligned buffers; the size queries include room for the shift.
+Arena work_arena(void* work, size_t bytes) {
+  Arena a;
+  const size_t shift = (256 - (uintptr_t)work % 256) % 256;
+  a.base = (char*)work + shift;
+  a.cap = bytes > shift ? bytes - shift : 0;
+  return a;
+}
+
 // The float64 form with emulate_fp64: whether the solve makes digit planes of A at all.  They pay off
 // for the Gaussian sketch, the Gram matrix and the Cholesky updates (2000 x 64: 25 us to make them, 400
 // us less work on the float64 pipe) and, for larger A, the LSQR products (use_oz): also for A of a few
@@ -521,21 +531,16 @@ tk_status solve_impl(const tk_problem* p, const double* lambdas, int N, const tk
   for (int i = 0; i < N; ++i)
     if (!(lambdas[i] > 0.0) || !std::isfinite(lambdas[i])) return einval("every lambda must be a positive finite number");
   if (!p->A || !p->b || !X) return einval("A, b and X must be non-NULL");
-  Arena a;
-  a.base = (char*)work;
-  a.cap = work_bytes;
-  Arena t;
-  t.base = (char*)scratch;
-  t.cap = scratch_bytes;
+  if (!gp && (!work || work_bytes < plan_bytes(P))) {
+    set_error_msg("workspace smaller than tk_workspace_size()");
+    return TK_ENOMEM;
+  }
+  Arena a = work_arena(work, work_bytes), t;
   Bufs B;
   if (!gp) {
-    const size_t need = plan_bytes(P);
-    if (!work || work_bytes < need) {
-      set_error_msg("workspace smaller than tk_workspace_size()");
-      return TK_ENOMEM;
-    }
     carve(P, a, a, B);
   } else {
+    t = work_arena(scratch, scratch_bytes);
     carve(P, a, t, B);
   }
   if (!a.ok() || !t.ok()) {
@@ -1651,9 +1656,7 @@ tk_status cholesky_common(const double* C, int64_t n, const double* lambdas, int
   }
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t np = cdiv(n, 64) * 64;
-  Arena a;
-  a.base = (char*)work;
-  a.cap = work_bytes;
+  Arena a = work_arena(work, work_bytes);
   double* lam = a.take<double>(N);
   int* info = a.take<int>(N);
   double* Rp = a.take<double>((size_t)N * np * np);
@@ -1840,14 +1843,14 @@ TK_API tk_status tk_lcurve(const tk_problem* p, const double* lambdas, int N, in
   cudaStream_t st = (cudaStream_t)stream;
   const int Np = N + N_refine;
   // the solve's own buffers (the same carve solve_impl makes) and the L-curve's after them
-  Arena a;
-  a.base = (char*)work;
-  a.cap = plan_b;
+  const Arena all_of_it = work_arena(work, work_bytes);
+  work = all_of_it.base;
+  Arena a = work_arena(work, plan_b);
   Bufs B;
   carve(P, a, a, B);
   Arena la;
   la.base = (char*)work + plan_b;
-  la.cap = work_bytes - plan_b;
+  la.cap = all_of_it.cap - plan_b;
   LcBufs L;
   lc_carve(la, P.m, P.n, Np, L);
   // first sweep: the given lambdas in ascending order
