@@ -31,6 +31,7 @@ void set_error_msg(const char* msg);
 // also counts it (tk_launch_count()).
 void count_launch();
 void count_launches(size_t n);  // n kernels of a replayed graph
+void count_capture(bool on);    // this thread's launches go into a graph: its replays count them
 #define TK_LAUNCH_CHECK()   \
   do {                      \
     ::tk::count_launch();   \

@@ -770,7 +770,9 @@ tk_status Lsqr<T>::replay(int nact, int count) {
   if (!e) {
     TK_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
     tk_status r = TK_OK;
+    count_capture(true);
     for (int c = 0; c < count && r == TK_OK; ++c) r = step(nact);
+    count_capture(false);
     cudaGraph_t g = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(st, &g);
     if (r != TK_OK || ce != cudaSuccess) {
@@ -781,6 +783,13 @@ tk_status Lsqr<T>::replay(int nact, int count) {
     }
     size_t nodes = 0;
     cudaGraphGetNodes(g, nullptr, &nodes);
+    std::vector<cudaGraphNode_t> list(nodes);
+    cudaGraphGetNodes(g, list.data(), &nodes);
+    size_t kernels = 0;
+    for (cudaGraphNode_t n : list) {
+      cudaGraphNodeType type;
+      if (cudaGraphNodeGetType(n, &type) == cudaSuccess && type == cudaGraphNodeTypeKernel) ++kernels;
+    }
     cudaGraphExec_t ge = nullptr;
     const cudaError_t ie = cudaGraphInstantiate(&ge, g, 0);
     cudaGraphDestroy(g);
@@ -788,11 +797,11 @@ tk_status Lsqr<T>::replay(int nact, int count) {
       set_error(ie, __FILE__, __LINE__);
       return TK_ECUDA;
     }
-    graphs.entries.push_back({nact, ge, nodes});
+    graphs.entries.push_back({nact, ge, kernels});
     e = &graphs.entries.back();
   }
   TK_CUDA(cudaGraphLaunch(e->exec, st));
-  count_launches(e->nodes);
+  count_launches(e->kernels);
   return TK_OK;
 }
 

@@ -187,7 +187,7 @@ struct StepGraphs {
   struct Entry {
     int slots;
     cudaGraphExec_t exec;
-    size_t nodes;
+    size_t kernels;
   };
   std::vector<Entry> entries;
   StepGraphs() = default;

@@ -38,8 +38,11 @@ std::atomic<unsigned long long> g_launches{0};
 
 }  // namespace
 
-void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
-
+static thread_local bool t_capturing = false;
+void count_capture(bool on) { t_capturing = on; }
+void count_launch() {
+  if (!t_capturing) g_launches.fetch_add(1, std::memory_order_relaxed);
+}
 void count_launches(size_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 bool prof_enabled() {
