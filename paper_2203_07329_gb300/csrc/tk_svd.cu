@@ -52,24 +52,15 @@ struct JacSmem {
   int rot[2];
 };
 
-// The power of two that brings x > 0 to [1, 2) (2^1023 for subnormal x).
-__device__ __forceinline__ double pow2_inverse(double x) {
-  const int e = (__double2hiint(x) >> 20) & 0x7ff;
-  return __hiloint2double((e > 2045 ? 1 : 2046 - e) << 20, 0);
-}
-
 // Rotation that makes rows of squared norms a, b and dot product g orthogonal (rows already orthogonal
 // to tol, or one of them zero: false).  t = tan of the angle in float32 from the scaled ratio zeta =
 // (b - a) / (2 g): off by 1e-7 relative it leaves 1e-7 of g for the next sweep; the norms' update a - t g is
 // exact to second order in that.  Where the ratio leaves float32 (a row of nothing but rounding errors
-// against a full one) t = 1 / (2 zeta) in float64: a t lost to zero would rotate the pair in every sweep.
+// against a full one) t = 1 / (2 zeta) with float64's exponent: a t lost to zero would rotate the pair in every sweep.
 // cos = (1 + t^2)^(-1/2) by two Newton steps from the float32 value.
 __device__ __forceinline__ bool jac_angle(double a, double b, double g, double tol, double* c, double* s, double* t) {
   if (!(a > 0.0) || !(b > 0.0)) return false;
-  // g^2 > tol^2 a b, each factor scaled by the power of two that brings a or b to [1, 2): as they are, the fourth
-  // powers of norms of 1e-81 or 1e77 leave float64
-  const double sa = pow2_inverse(a), sb = pow2_inverse(b);
-  if (!((g * sa) * (g * sb) > tol * tol * ((a * sa) * (b * sb)))) return false;
+  if (!(g * g > tol * tol * (a * b))) return false;  // (in range: the rows are scaled, see svd_start)
   const double d1 = b - a, d2 = 2.0 * g;
   // both scaled by the power of two that brings the larger to [1, 2): float32 then holds their ratio
   const int e1 = (__double2hiint(d1) >> 20) & 0x7ff, e2 = (__double2hiint(d2) >> 20) & 0x7ff;
@@ -79,7 +70,10 @@ __device__ __forceinline__ bool jac_angle(double a, double b, double g, double t
   const float z = f1 / f2, az = fabsf(z);
   const float ta = az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(fmaf(az, az, 1.0f)));
   *t = (double)((f1 >= 0.0f) == (f2 >= 0.0f) ? ta : -ta);
-  if (az > 1e30f) *t = g / d1;
+  if (az > 1e30f) {  // g / d1 from the float32 quotient of the mantissas (d1 the larger: e == e1)
+    const float q = 0.5f * (float)(d2 * __hiloint2double((2046 - e2) << 20, 0)) / f1;
+    *t = (double)q * __hiloint2double((1023 + e2 - e1) << 20, 0);
+  }
   const double x = fma(*t, *t, 1.0);
   double r = (double)rsqrtf((float)x);
   r = r * fma(-0.5 * x * r, r, 1.5);
@@ -190,16 +184,16 @@ __device__ __forceinline__ void jac_two_pairs_mem(double* const (&x)[4], int64_t
   if (S.rot[1]) jac_rotate_mem<TH>(x[C], x[D], n, S.cs[1], S.sn[1]);
 }
 
-// A row of less than 2^-106 = (2^-53)^2 of the largest norm counts as zero: it is what rounding left of a row that
-// depends on others, and each sweep would rotate the rounding errors of the sweep before (16 rows with 6 nonzero
-// columns: the cap of 80 sweeps, now 19).
-__device__ __forceinline__ double jac_norm2(double nrm2, double top) { return nrm2 > top * 0x1p-212 ? nrm2 : 0.0; }
+// A row of less than 2^-106 = (2^-53)^2 of the largest norm, which is scaled to 1, counts as zero: it is what rounding
+// left of a row that depends on others, and each sweep would rotate the rounding errors of the sweep before (16 rows
+// with 6 nonzero columns: the cap of 80 sweeps, now 19).
+__device__ __forceinline__ double jac_norm2(double nrm2) { return nrm2 > 0x1p-212 ? nrm2 : 0.0; }
 
 // Block pair k of a round: rows 2p, 2p + 1 and 2q, 2q + 1 of W (rows >= s: absent, norm 0).  first:
 // also the pairs inside the two blocks (once a sweep).
 template <int NE, int TH>
 __device__ __forceinline__ void jac_block_pair(double* __restrict__ W, double* __restrict__ nrm2, int64_t s,
-                                               int64_t n, int64_t sp, int64_t round, int64_t k, double tol, double top,
+                                               int64_t n, int64_t sp, int64_t round, int64_t k, double tol,
                                                int* __restrict__ rotated, JacSmem& S) {
   int64_t p, q;
   circle_pair(sp, round, k, &p, &q);
@@ -215,7 +209,7 @@ __device__ __forceinline__ void jac_block_pair(double* __restrict__ W, double* _
       const int64_t j = threadIdx.x + (int64_t)TH * e;
       x[i][e] = (r[i] < s && j < n) ? W[r[i] * n + j] : 0.0;
     }
-  if (threadIdx.x < 4) S.nr[threadIdx.x] = jac_norm2(r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0, top);
+  if (threadIdx.x < 4) S.nr[threadIdx.x] = jac_norm2(r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0);
   __syncthreads();
   int nrot = 0;
   if (first) jac_two_pairs<NE, TH, 0, 1, 2, 3>(x, ne, tol, S, &nrot);
@@ -239,7 +233,7 @@ __device__ __forceinline__ void jac_block_pair(double* __restrict__ W, double* _
 template <int TH>
 __device__ __forceinline__ void jac_block_pair_mem(double* __restrict__ W, double* __restrict__ nrm2, int64_t s,
                                                    int64_t n, int64_t sp, int64_t round, int64_t k, double tol,
-                                                   double top, int* __restrict__ rotated, JacSmem& S) {
+                                                   int* __restrict__ rotated, JacSmem& S) {
   int64_t p, q;
   circle_pair(sp, round, k, &p, &q);
   const bool first = round == 0;
@@ -248,7 +242,7 @@ __device__ __forceinline__ void jac_block_pair_mem(double* __restrict__ W, doubl
   double* x[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) x[i] = r[i] < s ? W + r[i] * n : nullptr;
-  if (threadIdx.x < 4) S.nr[threadIdx.x] = jac_norm2(r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0, top);
+  if (threadIdx.x < 4) S.nr[threadIdx.x] = jac_norm2(r[threadIdx.x] < s ? nrm2[r[threadIdx.x]] : 0.0);
   __syncthreads();
   int nrot = 0;
   if (first) jac_two_pairs_mem<TH, 0, 1, 2, 3>(x, n, tol, S, &nrot);
@@ -263,7 +257,6 @@ struct SvdDesc {
   double* W;
   double* nrm2;
   int64_t s, n, sp;  // sp: blocks of two rows, rounded up to an even count
-  double* top;       // the largest squared row norm so far (zero before the first sweep)
   int* rotated;
   int done;
 };
@@ -277,7 +270,7 @@ __global__ void __launch_bounds__(TH)
   const SvdTile t = tl[blockIdx.x];
   const SvdDesc& d = D[t.job];
   if (d.done || round >= d.sp - 1) return;
-  jac_block_pair<NE, TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, *d.top, d.rotated, S);
+  jac_block_pair<NE, TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, d.rotated, S);
 }
 template <int TH>
 __global__ void __launch_bounds__(TH)
@@ -286,7 +279,7 @@ __global__ void __launch_bounds__(TH)
   const SvdTile t = tl[blockIdx.x];
   const SvdDesc& d = D[t.job];
   if (d.done || round >= d.sp - 1) return;
-  jac_block_pair_mem<TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, *d.top, d.rotated, S);
+  jac_block_pair_mem<TH>(d.W, d.nrm2, d.s, d.n, d.sp, round, t.k, tol, d.rotated, S);
 }
 
 // Squared row norms at the start of a sweep (a warp to each of the block pair's four rows).
@@ -301,11 +294,7 @@ __global__ void __launch_bounds__(128) k_jacobi_norms(const SvdDesc* __restrict_
 #pragma unroll 4
   for (int64_t i = lane; i < d.n; i += 32) a = fma(d.W[r * d.n + i], d.W[r * d.n + i], a);
   a = warp_sum(a);
-  if (lane == 0) {
-    d.nrm2[r] = a;
-    // (non-negative doubles order like their bit patterns)
-    atomicMax(reinterpret_cast<unsigned long long*>(d.top), (unsigned long long)__double_as_longlong(a));
-  }
+  if (lane == 0) d.nrm2[r] = a;
 }
 
 __global__ void k_row_norms(const double* __restrict__ W, int64_t n, double* __restrict__ nrm) {
@@ -317,11 +306,11 @@ __global__ void k_row_norms(const double* __restrict__ W, int64_t n, double* __r
   if (threadIdx.x == 0) nrm[p] = sqrt(a);
 }
 
-// V[k*s + j] = W[perm[j]][k] / sigma_j ; sigma[j] = nrm[perm[j]].  32 x 32 tiles through shared memory:
+// V[k*s + j] = W[perm[j]][k] / nrm[perm[j]] ; sigma[j] = nrm[perm[j]] / scale.  32 x 32 tiles through shared memory:
 // rows of W are read and rows of V written contiguously.
 __global__ void __launch_bounds__(256)
     k_write_v(const double* __restrict__ W, const double* __restrict__ nrm, const int* __restrict__ perm, int64_t s,
-              int64_t n, double* __restrict__ V, double* __restrict__ sigma) {
+              int64_t n, const double* __restrict__ scale, double* __restrict__ V, double* __restrict__ sigma) {
   __shared__ double tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t k0 = (int64_t)blockIdx.x * 32, j0 = (int64_t)blockIdx.y * 32;
@@ -331,7 +320,7 @@ __global__ void __launch_bounds__(256)
       const int p = perm[j];
       const double sg = nrm[p];
       tile[r][tx] = W[(int64_t)p * n + k] * (sg > 0.0 ? 1.0 / sg : 0.0);
-      if (blockIdx.x == 0 && tx == 0) sigma[j] = sg;
+      if (blockIdx.x == 0 && tx == 0) sigma[j] = sg / *scale;
     }
   }
   __syncthreads();
@@ -346,24 +335,33 @@ __global__ void __launch_bounds__(256)
 // finished rows and orthogonalized inside (modified Gram-Schmidt), twice.
 constexpr int kGsPanel = 16;
 
-// scale = the power of two that brings the largest C_ii to [1, 2) (one block).
-__global__ void __launch_bounds__(256) k_gs_scale(const double* __restrict__ C, int64_t s, double* __restrict__ scale) {
+// *scale = the power of two that brings the largest of nrm[0 .. s) to [1, 2) (1 if they are zero or not finite); one
+// block.
+__global__ void __launch_bounds__(256) k_svd_scale(const double* __restrict__ nrm, int64_t s,
+                                                   double* __restrict__ scale) {
   __shared__ double sh[8];
   double mx = 0.0;
-  for (int64_t i = threadIdx.x; i < s; i += blockDim.x) mx = fmax(mx, C[i * s + i]);
+  for (int64_t i = threadIdx.x; i < s; i += blockDim.x) mx = fmax(mx, nrm[i]);
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) mx = fmax(mx, sh[w]);
-    *scale = pow2_inverse(mx);
+    const int e = (__double2hiint(mx) >> 20) & 0x7ff;
+    *scale = e > 0 && e < 2046 ? __hiloint2double((2046 - e) << 20, 0) : 1.0;
   }
+}
+// W = scale Y (Y may be W)
+__global__ void k_svd_scaled(const double* Y, int64_t total, const double* __restrict__ scale, double* W) {
+  const double sc = *scale;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x)
+    W[k] = sc * Y[k];
 }
 
 // X = C + noise of 2^-50 of sqrt(C_ii C_jj): rows of C that are dependent in float64 keep a direction of
-// their own (its choice is free), so that Q is a complete basis whatever the rank.  Times scale, so that the squares
-// of X, fourth powers of Y, stay in float64's range.
+// their own (its choice is free), so that Q is a complete basis whatever the rank.  Times scale^2, so that the
+// squares of X, fourth powers of Y, stay in float64's range.
 __global__ void k_gs_noise(const double* __restrict__ C, int64_t s, const double* __restrict__ scale,
                            double* __restrict__ X) {
   const int64_t i = blockIdx.y;
@@ -371,7 +369,7 @@ __global__ void k_gs_noise(const double* __restrict__ C, int64_t s, const double
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < s; j += (int64_t)gridDim.x * blockDim.x) {
     const uint4 r = philox((uint64_t)(i * s + j), 7u, 0x5eedull);
     const double u = ((double)(int)r.x) * 0x1p-31;  // in [-1, 1)
-    X[i * s + j] = sc * fma(u * 0x1p-50, sqrt(C[i * s + i]) * sqrt(C[j * s + j]), C[i * s + j]);
+    X[i * s + j] = sc * (sc * fma(u * 0x1p-50, sqrt(C[i * s + i]) * sqrt(C[j * s + j]), C[i * s + j]));
   }
 }
 
@@ -499,7 +497,7 @@ int gs_panel_rows(int64_t s) {
 
 // Buffers of one SVD, carved from its scratch.
 struct SvdBufs {
-  double *W, *nrm, *nrm2, *top, *C, *Q, *H;
+  double *W, *nrm, *nrm2, *scale, *C, *Q, *H;
   int *perm, *rotated;
   SvdDesc* desc;
   SvdTile* tiles;
@@ -519,7 +517,7 @@ void svd_carve(Arena& a, int64_t s, int64_t n, SvdBufs& B) {
   B.nrm = a.take<double>((size_t)s);
   B.nrm2 = a.take<double>((size_t)s);
   B.perm = a.take<int>((size_t)s);
-  B.top = a.take<double>(1);
+  B.scale = a.take<double>(1);
   B.rotated = a.take<int>(1);
   B.desc = a.take<SvdDesc>(1);
   B.tiles = a.take<SvdTile>((size_t)svd_tile_count(s));
@@ -530,16 +528,22 @@ void svd_carve(Arena& a, int64_t s, int64_t n, SvdBufs& B) {
   }
 }
 
-// W = Q Y (or a copy of Y).
+// W = scale Q Y (or scale Y), scale the power of two that brings the largest row norm of Y to [1, 2): squares of the
+// rotations' dot products and products of squared norms, fourth powers of the rows, leave float64's range for norms
+// of 1e-81 or 1e77 otherwise.  svd_finish divides sigma by it.
 tk_status svd_start(const double* Y, int64_t s, int64_t n, const SvdBufs& B, cudaStream_t st) {
+  k_row_norms<<<(unsigned)s, 256, 0, st>>>(Y, n, B.nrm);
+  TK_LAUNCH_CHECK();
+  k_svd_scale<<<1, 256, 0, st>>>(B.nrm, s, B.scale);
+  TK_LAUNCH_CHECK();
+  const unsigned gw = (unsigned)std::min<int64_t>(cdiv(s * n, 256), 152 * 8);
   if (!svd_orthogonal_start(s)) {
-    TK_CUDA(cudaMemcpyAsync(B.W, Y, sizeof(double) * (size_t)s * n, cudaMemcpyDeviceToDevice, st));
+    k_svd_scaled<<<gw, 256, 0, st>>>(Y, s * n, B.scale, B.W);
+    TK_LAUNCH_CHECK();
     return TK_OK;
   }
   TK_TRY((gemm<double, double, double>(false, true, s, s, n, Y, n, Y, n, B.C, s, 1.0, nullptr, nullptr, 0, st)));
-  k_gs_scale<<<1, 256, 0, st>>>(B.C, s, B.top);
-  TK_LAUNCH_CHECK();
-  k_gs_noise<<<dim3((unsigned)cdiv(s, 256), (unsigned)s), 256, 0, st>>>(B.C, s, B.top, B.Q);
+  k_gs_noise<<<dim3((unsigned)cdiv(s, 256), (unsigned)s), 256, 0, st>>>(B.C, s, B.scale, B.Q);
   TK_LAUNCH_CHECK();
   const int pr = gs_panel_rows(s);
   TK_CUDA(cudaFuncSetAttribute(k_gs_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGsSmemCap));
@@ -557,7 +561,10 @@ tk_status svd_start(const double* Y, int64_t s, int64_t n, const SvdBufs& B, cud
       TK_LAUNCH_CHECK();
     }
   }
-  return gemm<double, double, double>(false, false, s, n, s, B.Q, s, Y, n, B.W, n, 1.0, nullptr, nullptr, 0, st);
+  TK_TRY((gemm<double, double, double>(false, false, s, n, s, B.Q, s, Y, n, B.W, n, 1.0, nullptr, nullptr, 0, st)));
+  k_svd_scaled<<<gw, 256, 0, st>>>(B.W, s * n, B.scale, B.W);
+  TK_LAUNCH_CHECK();
+  return TK_OK;
 }
 
 // Registers hold 4 rows of a block pair: NE values per thread and row, up to 16 x 512 = 8192 (the largest short
@@ -575,9 +582,9 @@ tk_status launch_round(int64_t max_n, unsigned tiles, const SvdDesc* dd, const S
 }
 
 // The sorted singular values and right singular vectors from the rotated
-// rows: sigma_j = ||W_perm[j]||, V[:, j] = W_perm[j] / sigma_j.
-tk_status svd_finish(const double* W, int64_t s, int64_t n, double* nrm, int* perm, double* sigma, double* V,
-                     cudaStream_t st) {
+// rows: sigma_j = ||W_perm[j]|| / scale, V[:, j] = W_perm[j] / ||W_perm[j]||.
+tk_status svd_finish(const double* W, int64_t s, int64_t n, double* nrm, int* perm, const double* scale,
+                     double* sigma, double* V, cudaStream_t st) {
   k_row_norms<<<(unsigned)s, 256, 0, st>>>(W, n, nrm);
   TK_LAUNCH_CHECK();
   std::vector<double> h(s);
@@ -588,17 +595,16 @@ tk_status svd_finish(const double* W, int64_t s, int64_t n, double* nrm, int* pe
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return h[a] > h[b]; });
   TK_CUDA(cudaMemcpyAsync(perm, order.data(), sizeof(int) * s, cudaMemcpyHostToDevice, st));
   const dim3 g((unsigned)cdiv(n, 32), (unsigned)cdiv(s, 32));
-  k_write_v<<<g, 256, 0, st>>>(W, nrm, perm, s, n, V, sigma);
+  k_write_v<<<g, 256, 0, st>>>(W, nrm, perm, s, n, scale, V, sigma);
   TK_LAUNCH_CHECK();
   TK_CUDA(cudaStreamSynchronize(st));  // `order` is a host temporary
   return TK_OK;
 }
 
 // Sweeps over all matrices together (one launch per round) until none rotates; sweeps[j] receives the
-// count of matrix j.  dd, dt: device copies of hd and of the tiles are made here; tops, rots: what the matrices' top
-// and rotated point to.
-tk_status run_sweeps(std::vector<SvdDesc>& hd, SvdDesc* dd, SvdTile* dt, double* tops, int* rots,
-                     std::vector<int>& sweeps, cudaStream_t st) {
+// count of matrix j.  dd, dt: device copies of hd and of the tiles are made here.
+tk_status run_sweeps(std::vector<SvdDesc>& hd, SvdDesc* dd, SvdTile* dt, int* rots, std::vector<int>& sweeps,
+                     cudaStream_t st) {
   const int J = (int)hd.size();
   std::vector<SvdTile> tiles;
   int64_t max_rounds = 0, max_n = 0;
@@ -612,7 +618,6 @@ tk_status run_sweeps(std::vector<SvdDesc>& hd, SvdDesc* dd, SvdTile* dt, double*
   }
   TK_CUDA(cudaMemcpyAsync(dd, hd.data(), sizeof(SvdDesc) * J, cudaMemcpyHostToDevice, st));
   TK_CUDA(cudaMemcpyAsync(dt, tiles.data(), sizeof(SvdTile) * tiles.size(), cudaMemcpyHostToDevice, st));
-  TK_CUDA(cudaMemsetAsync(tops, 0, sizeof(double) * J, st));
   const double tol = 1e-15;
   const int max_sweeps = 80;
   std::vector<int> hrot(J);
@@ -651,11 +656,11 @@ tk_status jacobi_svd(const double* Y, int64_t s, int64_t n, double* sigma, doubl
   if (!ar.ok()) return TK_ENOMEM;
   if (s == 0) return TK_OK;
   TK_TRY(svd_start(Y, s, n, B, st));
-  std::vector<SvdDesc> hd(1, SvdDesc{B.W, B.nrm2, s, n, block_players(s), B.top, B.rotated, s <= 1 ? 1 : 0});
+  std::vector<SvdDesc> hd(1, SvdDesc{B.W, B.nrm2, s, n, block_players(s), B.rotated, s <= 1 ? 1 : 0});
   std::vector<int> sweeps;
-  TK_TRY(run_sweeps(hd, B.desc, B.tiles, B.top, B.rotated, sweeps, st));
+  TK_TRY(run_sweeps(hd, B.desc, B.tiles, B.rotated, sweeps, st));
   if (sweeps_host) *sweeps_host = std::max(sweeps[0], 1);
-  return svd_finish(B.W, s, n, B.nrm, B.perm, sigma, V, st);
+  return svd_finish(B.W, s, n, B.nrm, B.perm, B.scale, sigma, V, st);
 }
 
 tk_status jacobi_svd_begin(SvdJob& q, cudaStream_t st) {
@@ -677,7 +682,6 @@ tk_status jacobi_svd_grouped(std::vector<SvdJob>& jobs, void* work, size_t work_
   a.base = (char*)work;
   a.cap = work_bytes;
   SvdDesc* dd = a.take<SvdDesc>(J);
-  double* tops = a.take<double>(J);
   int* rots = a.take<int>(J);
   size_t ntiles = 0;
   for (const auto& j : jobs) ntiles += (size_t)svd_tile_count(j.s);
@@ -693,14 +697,15 @@ tk_status jacobi_svd_grouped(std::vector<SvdJob>& jobs, void* work, size_t work_
     sa.cap = q.scratch_bytes;
     svd_carve(sa, q.s, q.n, bufs[j]);
     if (!sa.ok()) return TK_ENOMEM;
-    hd[j] = SvdDesc{bufs[j].W, bufs[j].nrm2, q.s, q.n, block_players(q.s), tops + j, rots + j, q.s <= 1 ? 1 : 0};
+    hd[j] = SvdDesc{bufs[j].W, bufs[j].nrm2, q.s, q.n, block_players(q.s), rots + j, q.s <= 1 ? 1 : 0};
   }
   std::vector<int> sweeps;
-  TK_TRY(run_sweeps(hd, dd, dt, tops, rots, sweeps, st));
+  TK_TRY(run_sweeps(hd, dd, dt, rots, sweeps, st));
   for (int j = 0; j < J; ++j) {
     SvdJob& q = jobs[j];
     q.sweeps = sweeps[j];
-    if (q.s > 0) TK_TRY(svd_finish(bufs[j].W, q.s, q.n, bufs[j].nrm, bufs[j].perm, q.sigma, q.V, st));
+    if (q.s > 0) TK_TRY(svd_finish(bufs[j].W, q.s, q.n, bufs[j].nrm, bufs[j].perm, bufs[j].scale, q.sigma, q.V,
+                                 st));
   }
   return TK_OK;
 }
@@ -710,7 +715,6 @@ size_t svd_grouped_workspace(const std::vector<SvdJob>& jobs) {
   size_t ntiles = 0;
   for (const auto& j : jobs) ntiles += (size_t)svd_tile_count(j.s);
   a.take<SvdDesc>(std::max<size_t>(jobs.size(), 1));
-  a.take<double>(std::max<size_t>(jobs.size(), 1));
   a.take<int>(std::max<size_t>(jobs.size(), 1));
   a.take<SvdTile>(std::max<size_t>(ntiles, 1));
   return a.used + 1024;
