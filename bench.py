@@ -43,11 +43,15 @@ PEAK_FP32_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of the kernel behind a phase, from a
 # capture of the 65536 x 2048 float64 case (profiles/): (elements of A of that case, bytes).  A
 # launch streams every element of A once, so the figure scales with m n; kernels changed since
-# their capture are left out (traffic null).
+# their capture are left out (traffic null), and so are the 8-digit LSQR products of the float64
+# form, which run under the same phase names.
 MEASURED_TRAFFIC = {
-    # profiles/k_oz_tc_lsqr_digits_65536x2048.md: k_oz_tc<4, 2, 32> and k_oz_tc<4, 1, 32> (32 lambda)
-    "A_times_W_digits": (65536 * 2048, 1083622912 + 5114880),
-    "At_times_U_digits": (65536 * 2048, 1091296512 + 1207296),
+    # profiles/k_oz_tc_lsqr_digits_65536x2048.md: k_oz_tc<4, 2, 32> and k_oz_tc<4, 1, 32, TR> (32 lambda)
+    "A_times_W_digits": (65536 * 2048, 1083660800 + 5034496),
+    "At_times_U_digits": (65536 * 2048, 1090696704 + 652288),
+    # the same file: k_oz_tc<8, 0, 32> and k_oz_tc<8, 1, 32, TR>
+    "refine_residual64": (65536 * 2048, 2152889856 + 38767104),
+    "refine_normal64": (65536 * 2048, 2183049216 + 28356864),
 }
 
 # How each phase is bounded: "hbm" phases are compared as algorithmic bytes / time with the
@@ -339,7 +343,7 @@ def roofline_of(prof, peaks, peak_src, a_elems, fp64=False):
     # DRAM bytes (read + write) of one launch from an ncu capture of the same kernel on a smaller
     # case (profiles/), scaled by the elements of A it streams; None for kernels not captured
     traffic = None
-    if name in MEASURED_TRAFFIC:
+    if name in MEASURED_TRAFFIC and not (fp64 and name.endswith("_digits")):
         case_elems, case_bytes = MEASURED_TRAFFIC[name]
         traffic = case_bytes * a_elems / case_elems
     roofline = {"bound": bound if bound in ("hbm", "tensor") else "alu", "kernel": name, "achieved": achieved,
