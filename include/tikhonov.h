@@ -318,7 +318,7 @@ TK_API tk_status tk_gram(const double* Y, int64_t r, int64_t c, int transpose_fi
 /*
  * tk_gram_emulated -- C = Y^T Y as tk_gram with transpose_first, formed on
  * the BF16 tensor cores from exact integer slices of the columns of Y with
- * float64 accuracy (the Gram matrix of the mixed form with emulate_fp64; no
+ * float64 accuracy (the Gram matrix of the solves with emulate_fp64; no
  * counterpart in the paper's algorithms beyond Algorithm 1 step 3 itself).
  * Only the upper triangle (j >= i) of C is defined on return.
  *   work: device, tk_gram_emulated_workspace(r, c) bytes.
@@ -345,8 +345,8 @@ TK_API tk_status tk_cholesky_shifted(const double* C, int64_t n, const double* l
  * tk_cholesky_shifted_emulated -- as tk_cholesky_shifted, with the trailing
  * updates of the blocked factorization (R_22 -= R_12^T R_12) formed on the
  * BF16 tensor cores from exact integer slices with float64 accuracy (the
- * Cholesky of the mixed form with emulate_fp64).  The diagonal blocks and the
- * panel solves stay float64.  work: tk_cholesky_emulated_workspace(n, N)
+ * Cholesky of the solves with emulate_fp64).  At most 8191 lambdas
+ * (TK_EINVAL).  The diagonal blocks and the panel solves stay float64.  work: tk_cholesky_emulated_workspace(n, N)
  * bytes; TK_ETIMEOUT if a device-side pipeline wait gave up.
  */
 TK_API size_t tk_cholesky_emulated_workspace(int64_t n, int N);
@@ -369,7 +369,9 @@ TK_API tk_status tk_bp2_factor(const double* Y, int64_t s, int64_t n, const doub
 /*
  * tk_sketch_svd -- [~, Sigma, V] = svd(Y, 'econ') of Algorithm 3 step 4 by
  * one-sided Jacobi on Y^T (no Gram matrix is formed).  Y: device s x n
- * float64 with s <= n.  sigma: device s (descending).  V: device n x s.
+ * float64 with s <= n.  sigma: device s (descending).  V: device n x s (the
+ * columns of singular values below rounding, and of exact zeros, are not a
+ * basis of the rest).
  * work: device, tk_sketch_svd_workspace(s, n) bytes.  sweeps: host (may be NULL).
  */
 TK_API size_t tk_sketch_svd_workspace(int64_t s, int64_t n);
@@ -394,8 +396,10 @@ TK_API tk_status tk_lowrank_ranks(const double* sigma, int64_t s, const double* 
  * powers of two and split into 8 signed 7-bit integer slices (exact in BF16, 56 bits), the 36
  * slice products whose weight is at least 2^-56 of the row maxima are
  * accumulated exactly in FP32 over chunks of 256 values of K and then
- * exactly in int64, rounded once to float64 per output; the error is at
- * most that of a float64 GEMM (emulate = 1 requires n <= 2^27, else
+ * exactly in int64, rounded once to float64 per output; the error is
+ * normwise that of a float64 GEMM: with A'' = A scaled so (its rows after its
+ * columns) and X' = X in the units of the columns, a few 2^-55 of max_k |A''_ik|
+ * max_k |X'_lk| per product, not of each |a||x| (emulate = 1 requires n <= 2^27, else
  * TK_EINVAL: the exactness limit of the int64 accumulators; R A is split
  * along m so that no split holds more than 2^27 rows).
  *   p:   A (device, m x n, row stride lda, float64 or float32) and b (device, m).
@@ -479,11 +483,13 @@ enum {
   TK_PHASE_ATU = 6,           /* the product with A^T of every LSQR step */
   TK_PHASE_RES64 = 7,         /* MIXED: float64 residual b - A x */
   TK_PHASE_NE64 = 8,          /* MIXED: float64 A^T (b - A x) */
-  TK_PHASE_TRINV = 9,         /* explicit R^-1 and R^-T from the float64 factors (MIXED: float32; FP64: n <= 512) */
-  TK_PHASE_AW_DIGITS = 10,    /* MIXED, lsqr_tc = 2: TK_PHASE_AW on the tensor cores from digits of A */
-  TK_PHASE_ATU_DIGITS = 11,   /* MIXED, lsqr_tc = 2: TK_PHASE_ATU on the tensor cores from digits of A */
-  TK_PHASE_SLICE = 12,        /* MIXED, emulate_fp64: the digit planes of A (rows and columns), once per solve */
-  TK_PHASE_CHOL_UPDATE = 13,  /* MIXED, emulate_fp64: the Cholesky trailing updates on the tensor cores
+  TK_PHASE_TRINV = 9,         /* explicit R^-1 and R^-T from the float64 factors (MIXED: float32; FP64: min(m, n) = c
+                                 <= 512 for m >= n, or N c^2 up to 2.7e8; 8e7 without digits) */
+  TK_PHASE_AW_DIGITS = 10,    /* TK_PHASE_AW on the tensor cores from digits of A: 4 (MIXED, lsqr_tc = 2) or 8 (FP64,
+                                 emulate_fp64) */
+  TK_PHASE_ATU_DIGITS = 11,   /* TK_PHASE_ATU likewise */
+  TK_PHASE_SLICE = 12,        /* emulate_fp64: the digit planes of A, once per solve (MIXED: and its float32 copy) */
+  TK_PHASE_CHOL_UPDATE = 13,  /* emulate_fp64: the Cholesky trailing updates on the tensor cores
                                  (TK_PHASE_CHOLESKY then holds the diagonal blocks and panel solves) */
   TK_PHASE_LSQR_FUSED = 14,   /* MIXED, lsqr_tc = 3: TK_PHASE_AW_DIGITS and TK_PHASE_ATU_DIGITS of a step in one
                                  kernel over one read of the digits of A */

@@ -316,8 +316,6 @@ template <typename T>
 tk_status oz_lsqr_aw_split(const OzMat& A, const T* W, int64_t ldw, int count, void* Wslices, int* EW, double* partial,
                            int splits, int* err, cudaStream_t st);
 template <typename T>
-int oz_tri_lambdas(int64_t n, int N, int h0);  // lambdas per pass of the levels
-template <typename T>
 tk_status oz_lsqr_atu(const OzMat& A, const T* U, int64_t ldu, int count, void* Uslices, int* EU, double* partial,
                       int splits, int* err, cudaStream_t st);
 // The two products of one LSQR step fused over one read of A's row-exponent digit planes (count <= 32,
@@ -342,6 +340,8 @@ tk_status lm_small_atu(const float* A, int64_t lda, int64_t m, int64_t n, const 
 template <typename T>
 tk_status oz_tri_level(const double* R, int64_t ldr, int64_t rstride, T* M, T* Mt, int64_t ldm, int64_t mstride, int N,
                        int64_t n, int h, void* work, size_t bytes, int* err, cudaStream_t st);
+template <typename T>
+int oz_tri_lambdas(int64_t n, int N, int h0);  // lambdas per pass of the levels
 template <typename T>
 size_t oz_tri_workspace(int64_t n, int N, int h0);
 // Y (s x c) = G A (m >= n: G s x m, c = n) or G A^T (under: G s x n, c = m) for the Gaussian embedding G (gauss_fill,
