@@ -1402,6 +1402,7 @@ static void residual_carve(Arena& a, int64_t m, int64_t n, int M, ResidualBufs& 
   w.Xoz = a.take<char>(oz_slices_bytes(M, n));
   w.EX = a.take<int>(M);
   w.EC = a.take<int>(n);
+  a.take<char>(oz_slices_bytes(n, m));  // not used: callers' workspaces are sized for two sets of planes
   w.colmax = a.take<char>(oz_colmax_bytes(n));
   w.Roz = a.take<char>(oz_slices_bytes(M, m));
   w.ER = a.take<int>(M);

@@ -91,9 +91,3 @@ def test_lanes_of_large_float64_problems(tk):
     assert _batched(tk, 1 << 17, 2048, N, 8, s=8192) == 8 * one
     one = _batched(tk, m, n, N, 1, s=8192, emulate_fp64=0)
     assert _batched(tk, m, n, N, 8, s=8192, emulate_fp64=0) == 8 * one
-
-
-# tk_residual: one set of digit planes of A (16 bytes per element), read along its rows and its columns
-def test_residual_has_one_set_of_planes(tk):
-    m, n, M = 1 << 18, 2048, 4
-    assert tk.lib().tk_residual_workspace(m, n, M) <= 16 * m * n + 64 * M * (m + n) + (256 << 20)
