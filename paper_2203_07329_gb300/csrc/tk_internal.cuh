@@ -31,7 +31,7 @@ void set_error_msg(const char* msg);
 // also counts it (tk_launch_count()).
 void count_launch();
 void count_launches(size_t n);  // n kernels of a replayed graph
-void count_capture(bool on);    // this thread's launches go into a graph: its replays count them
+void count_capture(size_t* into);  // this thread's launches go into a graph: counted there (null: as launches again)
 #define TK_LAUNCH_CHECK()   \
   do {                      \
     ::tk::count_launch();   \

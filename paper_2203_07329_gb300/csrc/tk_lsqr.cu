@@ -770,9 +770,10 @@ tk_status Lsqr<T>::replay(int nact, int count) {
   if (!e) {
     TK_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
     tk_status r = TK_OK;
-    count_capture(true);
+    size_t kernels = 0;
+    count_capture(&kernels);
     for (int c = 0; c < count && r == TK_OK; ++c) r = step(nact);
-    count_capture(false);
+    count_capture(nullptr);
     cudaGraph_t g = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(st, &g);
     if (r != TK_OK || ce != cudaSuccess) {
@@ -780,15 +781,6 @@ tk_status Lsqr<T>::replay(int nact, int count) {
       if (r != TK_OK) return r;
       set_error(ce, __FILE__, __LINE__);
       return TK_ECUDA;
-    }
-    size_t nodes = 0;
-    cudaGraphGetNodes(g, nullptr, &nodes);
-    std::vector<cudaGraphNode_t> list(nodes);
-    cudaGraphGetNodes(g, list.data(), &nodes);
-    size_t kernels = 0;
-    for (cudaGraphNode_t n : list) {
-      cudaGraphNodeType type;
-      if (cudaGraphNodeGetType(n, &type) == cudaSuccess && type == cudaGraphNodeTypeKernel) ++kernels;
     }
     cudaGraphExec_t ge = nullptr;
     const cudaError_t ie = cudaGraphInstantiate(&ge, g, 0);

@@ -38,10 +38,11 @@ std::atomic<unsigned long long> g_launches{0};
 
 }  // namespace
 
-static thread_local bool t_capturing = false;
-void count_capture(bool on) { t_capturing = on; }
+static thread_local size_t* t_captured = nullptr;
+void count_capture(size_t* into) { t_captured = into; }
 void count_launch() {
-  if (!t_capturing) g_launches.fetch_add(1, std::memory_order_relaxed);
+  if (t_captured) ++*t_captured;
+  else g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 void count_launches(size_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
