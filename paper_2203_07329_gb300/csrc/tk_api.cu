@@ -1153,7 +1153,7 @@ tk_status batch_layout(const tk_problem* ps, int P, int N, const tk_opts* o, int
   if (!grouped) {
     // Every lane has a slice for the largest problem.  The float64 form's digit planes (16 bytes per element of A,
     // twice its float64 A) are not multiplied by 8 lanes beyond kLaneDigitBytes: a problem of that size fills
-    // the GPU by itself.
+    // the GPU by itself (8 problems of 2^20 x 512: 974 ms on 4 lanes with 49 GiB, 969 on 8 with 98).
     size_t digits = 1;
     for (int i = 0; i < P; ++i) {
       L.per = std::max(L.per, (plan_bytes(pl[i]) + 255) & ~size_t(255));

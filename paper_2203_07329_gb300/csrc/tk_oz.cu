@@ -2206,7 +2206,9 @@ __global__ void k_oz_sum_planes(const double* __restrict__ part, int splits, int
 }
 
 // The columns of the embedding whose float64 values and 8 digit planes (24 bytes a value) are held at a time: 2 GiB of
-// them, a product of thousands of values of K for every s.
+// them, a product of thousands of values of K for every s, so that the blocks cost nothing to speak of (262144 x 2048,
+// s = 8192: 445.8 ms in 25 blocks, 443.4 in one with 48 GiB of scratch; 65536 x 1024, s = 4096: 38.7 and 38.5; on the
+// float64 pipe 7361 and 503).
 static int64_t oz_sketch_block(int64_t L, int64_t s) {
   const int64_t fit = (int64_t(2) << 30) / (24 * s) / OT_CHUNK * OT_CHUNK;
   return std::min<int64_t>(L, std::max<int64_t>(fit, OT_CHUNK));
